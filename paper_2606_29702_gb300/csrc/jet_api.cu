@@ -57,11 +57,11 @@ cudaError_t simt_launch(int cls, bool fp64, const SimtArgs& a, int grid, size_t 
   return cudaErrorInvalidValue;
 }
 
-cudaError_t simt_occupancy(int cls, bool fp64, size_t smem, int* blocks) {
+cudaError_t simt_occupancy(int cls, bool fp64, int ru, int threads, size_t smem, int* blocks) {
   switch (cls) {
 #define CASE(id, cl) \
   case id:           \
-    return simt_max_active_id<id>(fp64, smem, blocks);
+    return simt_max_active_id<id>(fp64, ru, threads, smem, blocks);
     JET_FOR_EACH_CLASS(CASE)
 #undef CASE
   }
@@ -148,24 +148,62 @@ void below(const Alpha& a, std::set<Alpha>& out) {
   }
 }
 
-int tile_points(int wmax, bool fp64) {
-  const int TP = fp64 ? 2 : 4;
-  int q = kSimtThreads / wmax;
-  if (q < 1) q = 1;
-  return TP * q;
+size_t simt_tile_smem(const jet_plan_s* p, int P, int ru, int threads) {
+  const int pitch = simt_pitch(p->C, P, p->wmax, simt_wgrad_rows(ru), threads, p->elem);
+  return simt_smem_bytes(p->C, P, pitch, p->wmax, p->n_out, p->d, p->elem);
 }
 
-int pitch_for(int cols, bool fp64) {
-  // rows are offset by 16 bytes modulo 128: conflict-free 16-byte accesses
-  // by lanes that walk consecutive rows
-  const int mod = fp64 ? 16 : 32, want = fp64 ? 2 : 4;
-  int p = cols;
-  while (p % mod != want) ++p;
-  return p;
+// most points per tile that `ctas` CTAs of `threads` per SM can hold, at most
+// one item of the jet GEMMs per thread (P = threads * ru / wmax)
+int simt_most_points(const jet_plan_s* p, int ru, int threads, int ctas) {
+  int P = std::max(2, threads * ru / p->wmax / 2 * 2);
+  while (P > 2 && (simt_tile_smem(p, P, ru, threads) + 1280) * ctas > (size_t)226 * 1024) P -= 2;
+  return P;
 }
 
-size_t smem_bytes(int C, int P, int pitch, int wmax, int n_out, int d, size_t elem) {
-  return simt_smem_bytes(C, P, pitch, wmax, n_out, d, elem);
+// CTA shape and largest tile of a SIMT plan.  FP32 runs two CTAs of 256 threads
+// per SM (one CTA's barriers and elementwise phases overlap the other's GEMMs)
+// unless shared memory then takes more than an eighth of the points in flight
+// per SM that one CTA of 512 holds (256-wide layers).  Channel sets of 10 or
+// more run one CTA of 256 threads with all registers.  FP64 is bound by its two
+// lanes per SM, not by the tile.
+void simt_shape(jet_plan_s* p, int p8) {
+  p->threads = kSimtThreads;
+  if (p8) {
+    p->P = 8 * p8;
+    p->P_fixed = true;
+    return;
+  }
+  const bool wide = !p->fp64 && p->C >= 10;
+  p->P = simt_most_points(p, p->ru, kSimtThreads, wide ? 1 : 2);
+  if (p->fp64 || wide) return;
+  const int one = simt_most_points(p, p->ru, 2 * kSimtThreads, 1);
+  if (7 * one > 8 * 2 * p->P) {
+    p->P = one;
+    p->threads = 2 * kSimtThreads;
+  }
+}
+
+// Points per tile of one call on N points: the tile that leaves the busiest SM
+// the least work, counted in GEMM warps per tile plus kTileWarps for what a
+// tile costs whatever its size (its barriers and latencies).
+constexpr double kTileWarps = 2.0;
+int simt_call_points(const jet_plan_s* p, long long N) {
+  if (p->P_fixed) return p->P;
+  int best = p->P;
+  double best_cost = 0.0;
+  for (int P = p->P; P >= 2; P -= 2) {
+    const long long tiles = (N + P - 1) / P, per_sm = (tiles + p->sms - 1) / p->sms;
+    const int warps = (p->wmax / p->ru * P + 31) / 32;
+    const double cost = (double)per_sm * (warps + kTileWarps);
+    if (P == p->P || cost < best_cost) {
+      best = P;
+      best_cost = cost;
+    }
+  }
+  // the z-jet store holds whole tiles: near its capacity the largest tile
+  const bool stored = p->store && N <= p->store_max_points;
+  return stored && (N + best - 1) / best * best > p->store_max_points ? p->P : best;
 }
 
 }  // namespace
@@ -330,13 +368,10 @@ static jet_status plan_create(jet_plan_t* out, int n_specs, const jet_residual_s
   p->n_params = off;
 
   // ---- tiling and occupancy of the fused SIMT kernel
-  int wmax = 0;
-  for (int l = 1; l < n_layers; ++l) wmax = std::max(wmax, widths[l]);
-  const int p8 = JET_FLAG_TILE_GET(flags);
-  p->P = p8 ? 8 * p8 : tile_points(wmax, p->fp64);
-  p->S = simt_point_stride(p->C, p->P);
-  p->pitch = pitch_for(p->S * p->P, p->fp64);
-  p->smem = smem_bytes(p->C, p->P, p->pitch, wmax, n_out, d_in, p->elem);
+  for (int l = 1; l < n_layers; ++l) p->wmax = std::max(p->wmax, widths[l]);
+  p->ru = simt_units(widths, n_layers, p->fp64);
+  simt_shape(p, JET_FLAG_TILE_GET(flags));
+  p->smem = simt_tile_smem(p, p->P, p->ru, p->threads);
   cudaDeviceProp prop;
   cudaError_t e = cudaGetDeviceProperties(&prop, p->device);
   if (e != cudaSuccess) {
@@ -345,11 +380,13 @@ static jet_status plan_create(jet_plan_t* out, int n_specs, const jet_residual_s
   }
   int per_sm = 0;
   if (!p->tc) {
-    e = simt_occupancy(p->cls, p->fp64, p->smem, &per_sm);
+    p->sms = prop.multiProcessorCount;
+    e = simt_occupancy(p->cls, p->fp64, p->ru, p->threads, p->smem, &per_sm);
     if (e != cudaSuccess || per_sm < 1) {
       delete p;
       return e != cudaSuccess ? cuda_fail(e, "occupancy") : fail(JET_ERR_UNSUPPORTED, "SIMT tile does not fit one SM");
     }
+    per_sm = std::min(per_sm, 2);  // as measured; more CTAs would only add gradient slices
     p->grid = prop.multiProcessorCount * per_sm;
     p->ctas_per_sm = per_sm;
   }
@@ -379,7 +416,6 @@ static jet_status plan_create(jet_plan_t* out, int n_specs, const jet_residual_s
       const size_t per_tile = (size_t)jet_elems * p->elem;
       long long tiles = (long long)(mem_budget_bytes / per_tile);
       if (tiles > 0) {
-        p->store_tile_stride = jet_elems;
         p->store_max_points = tiles * p->P;
         e = cudaMalloc(&p->store, tiles * per_tile);
         p->ws_bytes += tiles * per_tile;
@@ -465,7 +501,7 @@ jet_status jet_plan_get_info(jet_plan_t p, jet_plan_info* info) {
   info->grid_ctas = p->tc ? tc_grid(p->tcp) : p->grid;
   info->workspace_bytes = p->tc ? tc_workspace_bytes(p->tcp) : p->ws_bytes;
   info->ctas_per_sm = p->tc ? tc_ctas_per_sm(p->tcp) : p->ctas_per_sm;
-  info->cta_threads = p->tc ? tc_threads(p->tcp) : kSimtThreads;
+  info->cta_threads = p->tc ? tc_threads(p->tcp) : p->threads;
   info->wgrad_chunk_fp32 = p->tc ? tc_wgrad_chunk_fp32(p->tcp) : (p->wacc_off >= 0 ? 1 : 0);
   return JET_OK;
 }
@@ -507,9 +543,10 @@ jet_status jet_plan_destroy(jet_plan_t p) {
 
 namespace {
 
-// Fill the per-call instance descriptor of the SIMT kernel.
+// Fill the per-call instance descriptor of the SIMT kernel, for tiles of P
+// points in CTAs of `threads` with ru units per GEMM thread.
 void fill_instance(const jet_plan_s* p, const void* params, const void* X, long long N, const void* source,
-                   void* r_out, int max_chunks, DevInstance& I) {
+                   void* r_out, int P, int ru, int threads, int max_chunks, DevInstance& I) {
   memset(&I, 0, sizeof(I));
   I.L = p->L;
   I.d = p->d;
@@ -534,19 +571,15 @@ void fill_instance(const jet_plan_s* p, const void* params, const void* X, long 
     I.inv_N = 1.0;  // each term's mean is in its scale
     I.n_groups = fill_groups(p, I.groups);
   }
-  I.P = p->P;
-  I.pitch = p->pitch;
-  I.S = p->S;
-  I.n_tiles = (N + p->P - 1) / p->P;
-  long long chunks = std::min<long long>(std::max<long long>(I.n_tiles, 1), max_chunks);
-  I.tiles_per_chunk = (int)((I.n_tiles + chunks - 1) / chunks);
-  if (I.tiles_per_chunk < 1) I.tiles_per_chunk = 1;
-  I.n_chunks = (int)((I.n_tiles + I.tiles_per_chunk - 1) / I.tiles_per_chunk);
+  I.P = P;
+  I.pitch = simt_pitch(p->C, P, p->wmax, simt_wgrad_rows(ru), threads, p->elem);
+  I.n_tiles = (N + I.P - 1) / I.P;
+  simt_set_chunks(I, max_chunks);
   I.chunk_base = 0;
   I.grad_slices = p->grad_slices;
   I.loss_slices = p->loss_slices;
   I.store = nullptr;
-  I.store_tile_stride = p->store_tile_stride;
+  for (int l = 1; l < p->L; ++l) I.store_tile_stride += (long long)p->C * P * p->widths[l];
   I.wacc_off = p->wacc_off;
 }
 
@@ -578,6 +611,8 @@ jet_status run_simt(jet_plan_s* p, int mode, const DevInstance& I, cudaStream_t 
   a.item_inst = nullptr;
   a.scratch = p->scratch;
   a.scratch_stride = p->scratch_stride;
+  a.ru = p->ru;
+  a.threads = p->threads;
   int grid = std::min(p->grid, I.n_chunks);
   ProfScope prof(p, s);
   CK(simt_launch(p->cls, p->fp64, a, grid, p->smem, s));
@@ -612,7 +647,7 @@ jet_status jet_forward_residual(jet_plan_t p, const void* params, const void* X,
     return JET_OK;
   }
   DevInstance I;
-  fill_instance(p, params, X, N, source, r_out, p->grid, I);
+  fill_instance(p, params, X, N, source, r_out, simt_call_points(p, N), p->ru, p->threads, p->grid, I);
   const bool store = p->store && N <= p->store_max_points;
   if (store) I.store = p->store;
   CK(launch_transpose_weights(I, p->fp64, p->Wt, s));
@@ -641,7 +676,7 @@ jet_status jet_backward_params(jet_plan_t p, const void* params, const void* X, 
     return JET_OK;
   }
   DevInstance I;
-  fill_instance(p, params, X, N, source, r_out, p->grid, I);
+  fill_instance(p, params, X, N, source, r_out, simt_call_points(p, N), p->ru, p->threads, p->grid, I);
   const bool from_store = p->st_valid && p->st_params == params && p->st_X == X && p->st_N == N &&
                           p->st_src == source;
   if (from_store) I.store = p->store;
@@ -666,7 +701,7 @@ static jet_status train_step(jet_plan_t p, void* params, void* adam_m, void* ada
   p->st_valid = false;  // params change in place
   if (p->tc) return tc_train_step(p, p->tcp, params, adam_m, adam_v, step, step_ctr, lr, X, N, source, loss_out, s);
   DevInstance I;
-  fill_instance(p, params, X, N, source, nullptr, p->grid, I);
+  fill_instance(p, params, X, N, source, nullptr, simt_call_points(p, N), p->ru, p->threads, p->grid, I);
   CK(launch_transpose_weights(I, p->fp64, p->Wt, s));
   st = run_simt(p, MODE_FWD_BWD, I, s);
   if (st != JET_OK) return st;
@@ -713,6 +748,8 @@ struct jet_batch_s {
   bool tc = false;
   int grid = 0;
   size_t smem = 0;
+  int ru = 0;
+  std::vector<int> P;  // points per tile of every member
   int max_chunks_per_inst = 16;
   // device workspace
   DevInstance* d_insts = nullptr;
@@ -761,36 +798,40 @@ void free_batch(jet_batch_s* b) {
 jet_status batch_prepare(jet_batch_s* b, const void* const* params, const void* const* X, const int64_t* N,
                          const void* const* source, void* const* r_out, int* n_items_out, cudaStream_t s) {
   const int n = (int)b->plans.size();
-  long long total_tiles = 0;
+  auto tile_cost = [&](int i) {
+    const jet_plan_s* p = b->plans[i];
+    double c = 64.0;
+    for (int l = 2; l < p->L; ++l) c += (double)p->widths[l - 1] * p->widths[l];
+    return c * p->C * b->P[i];
+  };
+  double total_cost = 0.0;
   for (int i = 0; i < n; ++i) {
     jet_status st = check_call(b->plans[i], params[i], X[i], N[i], source ? source[i] : nullptr);
     if (st != JET_OK) return st;
-    total_tiles += (N[i] + b->plans[i]->P - 1) / b->plans[i]->P;
+    total_cost += tile_cost(i) * (double)((N[i] + b->P[i] - 1) / b->P[i]);
   }
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   cudaStreamIsCapturing(s, &cs);
   if (b->have_prev && cs == cudaStreamCaptureStatusNone) cudaEventSynchronize(b->copied);
-  // target about four items per CTA
-  long long target_tiles = std::max<long long>(1, (total_tiles + 4LL * b->grid - 1) / (4LL * b->grid));
+  const double target = total_cost / (4.0 * b->grid);  // about four items of equal cost per CTA
   std::vector<std::pair<double, int>> cost;  // (cost, item) for ordering
   std::vector<int> item_inst;
   int chunk_base = 0;
   for (int i = 0; i < n; ++i) {
     jet_plan_s* p = b->plans[i];
     DevInstance& I = b->h_insts[i];
-    const long long tiles = (N[i] + p->P - 1) / p->P;
-    long long want = std::min<long long>(b->max_chunks_per_inst, std::max<long long>(1, (tiles + target_tiles - 1) / target_tiles));
-    fill_instance(p, params[i], X[i], N[i], source ? source[i] : nullptr, r_out ? r_out[i] : nullptr, (int)want, I);
+    const long long tiles = (N[i] + b->P[i] - 1) / b->P[i];
+    const double per_tile = tile_cost(i);
+    const long long want = std::min<long long>(
+        b->max_chunks_per_inst, std::max<long long>(1, (long long)(per_tile * (double)tiles / target + 0.5)));
+    fill_instance(p, params[i], X[i], N[i], source ? source[i] : nullptr, r_out ? r_out[i] : nullptr, b->P[i], b->ru,
+                  kSimtThreads, (int)want, I);
     I.Wt = (char*)b->Wt + b->wt_off[i] * p->elem;
     I.grad_slices = b->grad_slices + b->slice_off[i];
     I.loss_slices = b->loss_slices + (long long)i * b->max_chunks_per_inst;
     I.chunk_base = chunk_base;
-    double per_tile = 0;
-    for (int l = 2; l < p->L; ++l) per_tile += (double)p->widths[l - 1] * p->widths[l];
-    per_tile = (per_tile + 64.0) * p->C * p->P;
     for (int c = 0; c < I.n_chunks; ++c) {
-      const long long t0 = (long long)c * I.tiles_per_chunk;
-      const long long nt = std::min<long long>(tiles, t0 + I.tiles_per_chunk) - t0;
+      const long long nt = I.tiles_per_chunk + (c < I.chunk_rem ? 1 : 0);
       cost.push_back({per_tile * (double)nt, chunk_base + c});
       item_inst.push_back(i);
     }
@@ -841,27 +882,41 @@ jet_status jet_batch_create(jet_batch_t* out, int32_t n, const jet_plan_t* plans
     *out = b;
     return JET_OK;
   }
+  // members share the launch: CTAs of kSimtThreads, the units per thread that
+  // every member's widths allow, two CTAs per SM where the tiles let them
+  b->ru = plans[0]->ru;
+  for (int i = 1; i < n; ++i) b->ru = std::min(b->ru, plans[i]->ru);
   size_t smem = 0;
-  long long scr = 0, slices = 0, wt = 0;
   for (int i = 0; i < n; ++i) {
-    smem = std::max(smem, plans[i]->smem);
-    scr = std::max(scr, plans[i]->scratch_stride);
-    b->slice_off.push_back(slices);
-    slices += (long long)b->max_chunks_per_inst * plans[i]->n_params;
-    b->wt_off.push_back(wt);
-    wt += weight_ws_elems(plans[i]->n_params);
+    int P = plans[i]->P;
+    if (!plans[i]->P_fixed)
+      P = std::min(P, simt_most_points(plans[i], b->ru, kSimtThreads, !b->fp64 && plans[i]->C >= 10 ? 1 : 2));
+    b->P.push_back(P);
+    smem = std::max(smem, simt_tile_smem(plans[i], P, b->ru, kSimtThreads));
   }
   b->smem = smem;
   int per_sm = 0, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceProp prop;
   cudaError_t e = cudaGetDeviceProperties(&prop, dev);
-  if (e == cudaSuccess) e = simt_occupancy(b->cls, b->fp64, smem, &per_sm);
+  if (e == cudaSuccess) e = simt_occupancy(b->cls, b->fp64, b->ru, kSimtThreads, smem, &per_sm);
   if (e != cudaSuccess || per_sm < 1) {
     delete b;
     return e != cudaSuccess ? cuda_fail(e, "batch occupancy") : fail(JET_ERR_UNSUPPORTED, "batch tile does not fit");
   }
-  b->grid = prop.multiProcessorCount * per_sm;
+  b->grid = prop.multiProcessorCount * std::min(per_sm, 2);
+  // the work list holds about four items per CTA, shared by cost: a member may
+  // take twice its share (with 16 members a fixed 16 chunks left the largest
+  // member's chunks running alone: 26.4 ms against 5.0 ms)
+  b->max_chunks_per_inst = std::min(256, std::max(16, 8 * b->grid / n));
+  long long scr = 0, slices = 0, wt = 0;
+  for (int i = 0; i < n; ++i) {
+    scr = std::max(scr, plans[i]->scratch_stride);
+    b->slice_off.push_back(slices);
+    slices += (long long)b->max_chunks_per_inst * plans[i]->n_params;
+    b->wt_off.push_back(wt);
+    wt += weight_ws_elems(plans[i]->n_params);
+  }
   b->scratch_stride = scr;
   b->max_items = n * b->max_chunks_per_inst;
   const size_t elem = b->fp64 ? 8 : 4;
@@ -904,6 +959,8 @@ static jet_status batch_run(jet_batch_t b, const void* const* params, void* cons
   a.scratch = b->scratch;
   a.scratch_stride = b->scratch_stride;
   a.item_next = b->d_next;
+  a.ru = b->ru;
+  a.threads = kSimtThreads;
   CK(cudaMemsetAsync(b->d_next, 0, sizeof(int), s));
   CK(simt_launch(b->cls, b->fp64, a, std::min(b->grid, n_items), b->smem, s));
   long long maxp = 0;

@@ -67,10 +67,10 @@ struct DevInstance {
   DevGroup groups[kMaxGroups];
   // tiling
   int P;               // points per tile
-  int pitch;           // smem row pitch (elements) of a jet buffer, >= S * P
-  int S;               // point stride within a jet row (SIMT forms)
+  int pitch;           // smem row pitch (elements) of a jet buffer, >= C * P
   long long n_tiles;
-  int tiles_per_chunk;
+  int tiles_per_chunk;  // of every chunk; the first chunk_rem chunks take one more
+  int chunk_rem;
   int n_chunks;
   int chunk_base;      // first work-item index of this instance
   // outputs of the chunk reduction (FP64): [n_chunks][n_params], [n_chunks]
@@ -92,6 +92,8 @@ struct SimtArgs {
   const DevInstance* insts;   // device array (batched) or null
   DevInstance inst0;          // single-instance launches pass it by value
   int n_items;                // total work items (instance, chunk)
+  int ru;                     // units per thread of the jet GEMMs (simt_units)
+  int threads;                // CTA size
   const int* item_inst;       // [n_items] instance of each item (batched) or null
   void* scratch;              // per-CTA z-jet scratch
   long long scratch_stride;   // elements per CTA slot
@@ -101,15 +103,43 @@ struct SimtArgs {
   int* item_next;
 };
 
-constexpr int kSimtThreads = 256;
-// Point stride S of a SIMT shared-memory jet row [unit][n * S + alpha]: the
-// lanes of a warp walk min(P, 32) points and must hit distinct banks, so S = C
-// when C's power-of-two factor times those lanes fits in 32 banks (C = 6 at
-// P = 16), else the odd C | 1 (pad columns stay zero).
-inline int simt_point_stride(int C, int P) {
-  const int lanes = P < 32 ? P : 32;
-  return (C & -C) * lanes <= 32 ? C : (C | 1);
+constexpr int kSimtThreads = 256;  // CTA of the no-alloc path and of batches
+constexpr int kSimtRed = 128;      // doubles of the SIMT kernels' reduction area
+// Weights of a jet GEMM pass through shared memory in two row slabs of at most
+// this many bytes (a 64 x 64 FP32 layer takes two, a 256 x 256 one 32); larger
+// slabs would cost tile points at width 256.
+constexpr int kSimtSlabBytes = 8192;
+__host__ __device__ inline int simt_slab_elems(int wmax, size_t elem) {
+  const int cap = kSimtSlabBytes / (int)elem, need = wmax * wmax;
+  return need < cap ? need : cap;
 }
+// Adjacent lanes that share a weight-gradient item (wr rows x 4 columns), each
+// summing every NS-th vector of jet columns: as many as fill the CTA.  FP32
+// items keep at least 4 sums per lane (one vector reduction).
+__host__ __device__ inline int simt_wgrad_slices(int items, int wr, bool f32, int threads) {
+  const int most = f32 && wr == 4 ? 4 : 8;
+  int ns = 1;
+  while (ns < most && items * ns * 2 <= threads) ns *= 2;
+  return ns;
+}
+// Row pitch (elements) of a SIMT jet buffer of C * P columns.  The weight
+// gradient's 16-byte loads walk 8 / NS rows x NS vectors per quarter warp: the
+// pitch in 16-byte units is NS modulo 2 NS, so that they hit distinct banks.
+inline int simt_pitch(int C, int P, int wmax, int wr, int threads, size_t elem) {
+  const int v = 16 / (int)elem;
+  const int ns = simt_wgrad_slices((wmax / wr) * (wmax / 4), wr, elem == 4, threads);
+  int p = (C * P + v - 1) / v * v;
+  while ((p / v) % (2 * ns) != ns % (2 * ns)) p += v;
+  return p;
+}
+// consecutive units per thread of the SIMT jet GEMMs
+inline int simt_units(const int* widths, int L, bool fp64) {
+  if (fp64) return 2;
+  for (int l = 1; l < L; ++l)
+    if (widths[l] % 8) return 4;
+  return 8;
+}
+inline int simt_wgrad_rows(int ru) { return ru == 8 ? 8 : 4; }
 // share of L2 the per-chunk FP64 gradient slices may take before the kernels
 // accumulate a chunk's weight gradients in FP32 instead of adding per tile
 constexpr double kSimtSliceL2Bytes = 48.0 * 1024 * 1024;
@@ -125,15 +155,23 @@ inline long long simt_wacc_elems(const int* widths, int L, bool fp64) {
 // elements of the SIMT weight workspace: transposed copy, then aligned copy
 __host__ __device__ inline long long weight_copy_offset(long long n_params) { return (n_params + 3) & ~3LL; }
 __host__ __device__ inline long long weight_ws_elems(long long n_params) { return 2 * weight_copy_offset(n_params); }
-// Dynamic shared memory of the fused SIMT kernel: three jet buffers
-// [wmax][pitch], output jets and adjoints [n_out*C][P], tile points [P][d],
-// and a small reduction area.
+// Dynamic shared memory of the fused SIMT kernel: two jet buffers
+// [wmax][pitch], two weight slabs, output jets and adjoints [n_out*C][P], tile
+// points [P][d], and a small reduction area.
 inline size_t simt_smem_bytes(int C, int P, int pitch, int wmax, int n_out, int d, size_t elem) {
-  size_t e = 3 * (size_t)wmax * pitch + 2 * (size_t)n_out * C * P + (size_t)P * d;
+  size_t e = 2 * (size_t)wmax * pitch + 2 * (size_t)simt_slab_elems(wmax, elem) + 2 * (size_t)n_out * C * P +
+             (size_t)P * d;
   size_t bytes = (e * elem + 15) / 16 * 16;
-  return bytes + 64 * sizeof(double);
+  return bytes + kSimtRed * sizeof(double);
 }
-
+// the chunks of a call: n_tiles tiles over n_chunks CTAs or work items
+inline void simt_set_chunks(DevInstance& I, long long n_chunks) {
+  if (n_chunks > I.n_tiles) n_chunks = I.n_tiles;
+  if (n_chunks < 1) n_chunks = 1;
+  I.n_chunks = (int)n_chunks;
+  I.tiles_per_chunk = (int)(I.n_tiles / n_chunks);
+  I.chunk_rem = (int)(I.n_tiles % n_chunks);
+}
 
 // Reductions and elementwise kernels (jet_reduce.cu)
 // One reduction job per instance: grad[p] = sum_c slices[c][p] in FP64 (fixed
@@ -166,7 +204,7 @@ void set_last_error(const char* msg);
 
 // Per-class entry points, one explicit specialisation per instantiation unit.
 template <int ID> cudaError_t simt_launch_id(bool fp64, const SimtArgs& a, int grid, size_t smem, cudaStream_t s);
-template <int ID> cudaError_t simt_max_active_id(bool fp64, size_t smem, int* blocks);
+template <int ID> cudaError_t simt_max_active_id(bool fp64, int ru, int threads, size_t smem, int* blocks);
 template <int ID> cudaError_t debug_activation_id(int kind, long long n, const double* z, const double* v,
                                                   double* out, cudaStream_t s);
 }  // namespace jet

@@ -97,11 +97,11 @@ cudaError_t launch_by_class(int cls, bool fp64, const jet::SimtArgs& a, int grid
   return cudaErrorInvalidValue;
 }
 
-cudaError_t occupancy_by_class(int cls, bool fp64, size_t smem, int* blocks) {
+cudaError_t occupancy_by_class(int cls, bool fp64, int ru, size_t smem, int* blocks) {
   switch (cls) {
 #define CASE(id, cl) \
   case id:           \
-    return jet::simt_max_active_id<id>(fp64, smem, blocks);
+    return jet::simt_max_active_id<id>(fp64, ru, jet::kSimtThreads, smem, blocks);
     JET_FOR_EACH_CLASS(CASE)
 #undef CASE
   }
@@ -204,15 +204,13 @@ extern "C" jet_status jet_backward_params_noalloc(const jet_residual_spec* spec,
   I.r_out = nullptr;
   I.N = N;
   I.inv_N = 1.0 / (double)N;
-  // tiling: same rule as the plan path
+  // tiling: the largest tile whose jet scratch keeps the accepted shapes
   const int TP = fp64 ? 2 : 4;
   const int P = TP * (kSimtThreads / wmax > 0 ? kSimtThreads / wmax : 1);
-  const int S = simt_point_stride(C, P);
-  int pitch = S * P;
-  while (pitch % (fp64 ? 16 : 32) != (fp64 ? 2 : 4)) ++pitch;
+  const int ru = simt_units(widths, n_layers, fp64);
+  const int pitch = simt_pitch(C, P, wmax, simt_wgrad_rows(ru), kSimtThreads, elem);
   I.P = P;
   I.pitch = pitch;
-  I.S = S;
   I.n_tiles = (N + P - 1) / P;
   const size_t smem = simt_smem_bytes(C, P, pitch, wmax, n_out, d_in, elem);
   long long jet_elems = 0;
@@ -228,15 +226,14 @@ extern "C" jet_status jet_backward_params_noalloc(const jet_residual_spec* spec,
   int per_sm = 0, dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = occupancy_by_class(best, fp64, smem, &per_sm);
+  if (e == cudaSuccess) e = occupancy_by_class(best, fp64, ru, smem, &per_sm);
   if (e != cudaSuccess) return nfail_cuda(e, "occupancy");
   if (per_sm < 1) return nfail(JET_ERR_UNSUPPORTED, "tile does not fit one SM");
   long long fit = (long long)((kStaticScratchBytes - fixed) / per_chunk);
   long long chunks = I.n_tiles;
   if (chunks > (long long)sms * per_sm) chunks = (long long)sms * per_sm;
   if (chunks > fit) chunks = fit;
-  I.tiles_per_chunk = (int)((I.n_tiles + chunks - 1) / chunks);
-  I.n_chunks = (int)((I.n_tiles + I.tiles_per_chunk - 1) / I.tiles_per_chunk);
+  simt_set_chunks(I, chunks);
 
   void* base = nullptr;
   jet_status st = scratch_address(&base);
@@ -266,6 +263,8 @@ extern "C" jet_status jet_backward_params_noalloc(const jet_residual_spec* spec,
   a.n_inst = 1;
   a.inst0 = I;
   a.n_items = I.n_chunks;
+  a.ru = ru;
+  a.threads = kSimtThreads;
   a.scratch = scr;
   a.scratch_stride = jet_elems;
   e = launch_by_class(best, fp64, a, I.n_chunks, smem, s);

@@ -31,7 +31,10 @@ struct jet_plan_s {
   std::vector<long long> group_counts;
   long long n_params = 0;
   std::vector<long long> off_W, off_b;
-  int P = 0, pitch = 0, S = 0;
+  int P = 0;               // points per tile (SIMT forms: the most a call takes)
+  bool P_fixed = false;    // SIMT forms: every call takes P (tile override)
+  int ru = 0, threads = 0, wmax = 0;  // SIMT forms: units per thread, CTA size, widest layer
+  int sms = 0;
   size_t smem = 0;
   int grid = 0, ctas_per_sm = 0;
   size_t elem = 4;
@@ -44,7 +47,6 @@ struct jet_plan_s {
   long long wacc_off = -1;  // FP32 weight-gradient accumulator in a scratch slot (elements)
   void* store = nullptr;
   long long store_max_points = 0;
-  long long store_tile_stride = 0;
   size_t ws_bytes = 0;
   // identity of the forward call whose jets the store holds
   bool st_valid = false;

@@ -16,18 +16,27 @@
 //             the value channel, data gradient W^T Zb.
 //
 // Jets live in shared memory as [unit][point-major column] rows: column =
-// n * S + alpha with an odd point stride S >= C (the pad columns stay zero).
-// A thread owns one point and TP consecutive units with every channel, so the
-// composition and its adjoint are thread-local and each jet-GEMM activation
-// load is one conflict-free wavefront.  The hidden z-jets of a tile are
-// written to a per-CTA global scratch slot (or to a full-size store) as
-// [unit][alpha * P + n] in the forward and read back in the backward, cached
-// in L2 only so that L1 keeps the layer's weights: the memory of the backward
-// is bounded by the number of CTAs, not by N.
+// n * C + alpha (columns past C * P stay zero).  In the jet GEMMs a thread owns
+// one point and RU consecutive units with every channel, so the composition
+// and its adjoint are thread-local; the layer's weights pass through shared
+// memory in row slabs.  The hidden z-jets of a tile are written to a per-CTA
+// global scratch slot (or to a full-size store) as [unit][alpha * P + n] in the
+// forward and read back in the backward, with tanh z in place of the value
+// channel (the activation rule and its adjoint read z_0 only through tanh z_0):
+// the memory of the backward is bounded by the number of CTAs, not by N.
 // Gradient partial sums go to a per-(instance, chunk) FP64 slice; every slice
 // element is added by one thread in tile order (fire-and-forget FP64 adds),
 // so the final FP64 reduction is deterministic.
+//
+// What bounds it: the FP32 pipe and shared-memory reads in the jet GEMMs
+// (about 80% of the time), the FP64 pipe in the FP64 form.  Against the form
+// with three jet buffers, 4 units per thread, weights read through L1, one
+// lane per weight-gradient item and tiles that did not depend on N:
+// 3->256x8->1 FP32 at N = 16385 19.29 -> 12.79 ms, 2->64x5->1 (C = 6) FP32 at
+// 65536 1.769 -> 1.637 ms, 2->20x4->1 FP64 at 1000 342 -> 105 us.
 #pragma once
+
+#include <type_traits>
 
 #include "jet_closures_gen.h"
 #include "jet_f2.cuh"
@@ -46,8 +55,7 @@ template <> __device__ __forceinline__ double dev_tanh<double>(double z) { retur
 
 // p[k] = tanh^(k)(z) for k < NP, as polynomials of a = tanh z and s = 1 - a^2.
 template <class T, int NP>
-__device__ __forceinline__ void tanh_derivs(T z, T* p) {
-  const T a = dev_tanh<T>(z);
+__device__ __forceinline__ void tanh_polys(T a, T* p) {
   const T a2 = a * a;
   const T s = T(1) - a2;
   p[0] = a;
@@ -58,11 +66,14 @@ __device__ __forceinline__ void tanh_derivs(T z, T* p) {
   if (NP > 5) p[5] = T(8) * s * (T(15) * a2 * a2 - T(15) * a2 + T(2));
 }
 
-// tanh_derivs of two values in a packed pair (accurate tanhf per value, the
-// derivative polynomials in a and s packed)
+template <class T, int NP>
+__device__ __forceinline__ void tanh_derivs(T z, T* p) {
+  tanh_polys<T, NP>(dev_tanh<T>(z), p);
+}
+
+// tanh_polys of two values in a packed pair
 template <int NP>
-__device__ __forceinline__ void tanh_derivs_pair(f2 z, f2* p) {
-  const f2 a(tanhf(z.v.x), tanhf(z.v.y));
+__device__ __forceinline__ void tanh_polys_pair(f2 a, f2* p) {
   const f2 a2 = a * a;
   const f2 s = jfma(f2(-1.0f), a2, f2(1.0f));
   p[0] = a;
@@ -82,25 +93,60 @@ __device__ __forceinline__ void vload(const T* p, T* out) {
   for (int j = 0; j < Vec<T>::N; ++j) out[j] = q[j];
 }
 
-// Vec<T>::N consecutive values through the read-only path (16-byte aligned)
-template <class T>
-__device__ __forceinline__ void vldg(const T* p, T* out) {
-  using V = typename Vec<T>::type;
-  V v = __ldg(reinterpret_cast<const V*>(p));
-  const T* q = reinterpret_cast<const T*>(&v);
+// the C channels of one (unit, point) in a jet row: 16-byte accesses where the
+// element count divides, else 8-byte or scalar ones (rows start on 16 bytes)
+template <class T, int C>
+__device__ __forceinline__ void load_chan(const T* p, T* v) {
+  if constexpr (sizeof(T) == 4 && C % 4 != 0 && C % 2 == 0) {
 #pragma unroll
-  for (int j = 0; j < Vec<T>::N; ++j) out[j] = q[j];
+    for (int c = 0; c < C; c += 2) {
+      const float2 t = *reinterpret_cast<const float2*>(p + c);
+      v[c] = t.x;
+      v[c + 1] = t.y;
+    }
+  } else if constexpr (C % Vec<T>::N == 0) {
+#pragma unroll
+    for (int c = 0; c < C; c += Vec<T>::N) vload<T>(p + c, v + c);
+  } else {
+#pragma unroll
+    for (int c = 0; c < C; ++c) v[c] = p[c];
+  }
+}
+template <class T, int C>
+__device__ __forceinline__ void store_chan(T* p, const T* v) {
+  if constexpr (sizeof(T) == 4 && C % 4 == 0) {
+#pragma unroll
+    for (int c = 0; c < C; c += 4) *reinterpret_cast<float4*>(p + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
+  } else if constexpr (sizeof(T) == 4 && C % 2 == 0) {
+#pragma unroll
+    for (int c = 0; c < C; c += 2) *reinterpret_cast<float2*>(p + c) = make_float2(v[c], v[c + 1]);
+  } else if constexpr (sizeof(T) == 8 && C % 2 == 0) {
+#pragma unroll
+    for (int c = 0; c < C; c += 2) *reinterpret_cast<double2*>(p + c) = make_double2(v[c], v[c + 1]);
+  } else {
+#pragma unroll
+    for (int c = 0; c < C; ++c) p[c] = v[c];
+  }
 }
 
-template <class T>
-__device__ __forceinline__ void vstore(T* p, const T* in) {
-  using V = typename Vec<T>::type;
-  V v;
-  T* q = reinterpret_cast<T*>(&v);
-#pragma unroll
-  for (int j = 0; j < Vec<T>::N; ++j) q[j] = in[j];
-  *reinterpret_cast<V*>(p) = v;
+// Value-preserving float -> double on the integer pipe.  The FP64 pipe, which
+// executes the conversion instruction, takes two lanes a clock per SM, and a
+// tile converts every weight gradient; subnormals take the instruction.
+__device__ __forceinline__ double widen(float f) {
+  const unsigned b = __float_as_uint(f), e = (b >> 23) & 0xffu, m = b & 0x7fffffu;
+  if (e == 0u && m != 0u) return (double)f;
+  const unsigned ed = e == 0u ? 0u : e == 255u ? 2047u : e + 896u;
+  return __hiloint2double((int)((b & 0x80000000u) | (ed << 20) | (m >> 3)), (int)(m << 29));
 }
+__device__ __forceinline__ double widen(double f) { return f; }
+
+// 16 bytes from global to shared memory, asynchronously
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 // p[0..3] += (a, b, c, d) in global memory as one fire-and-forget FP32
 // vector reduction (16-byte aligned; no value comes back, so nothing waits)
@@ -108,30 +154,28 @@ __device__ __forceinline__ void red_add_v4(float* p, float a, float b, float c, 
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
-struct SimtSmem {
-  int P, pitch, wmax, C, nout, d;
-  __device__ size_t buf_elems() const { return (size_t)wmax * pitch; }
-};
-
-template <class Cls, class T>
+template <class Cls, class T, int RU_>
 struct SimtTile {
   static constexpr int C = Cls::C;
   static constexpr int NP = Cls::NP;
   static constexpr int TP = Vec<T>::N;
-  static constexpr int NT = kSimtThreads;
-  static constexpr int RU = TP;  // consecutive units per thread
-  // k-steps of the jet GEMMs unrolled together (loads in flight): wide
-  // channel sets gain from four, KS-sized ones lose (measured)
-  static constexpr int UK = C >= 7 ? 4 : 2;
+  static constexpr bool F32 = sizeof(T) == 4;
+  static constexpr int RU = RU_;  // consecutive units per thread of the jet GEMMs
+  static constexpr int EU = TP;   // consecutive units per thread of the elementwise phases
+  static constexpr int WR = F32 && RU == 8 ? 8 : 4;  // weight-gradient rows per thread (times 4 columns)
 
   const DevInstance& I;
   const SimtArgs& A;
-  T* B[3];   // jet buffers [wmax][pitch]
+  const int NT;  // threads of the CTA
+  T* B[2];   // jet buffers [wmax][pitch]
+  T* WS;     // two weight slabs
   T* UO;     // output jets [n_out*C][P]
   T* UB;     // output adjoints [n_out*C][P]
   T* XS;     // tile points [P][d]
   double* RED;
-  int P, pitch, wmax, S;  // S: point stride within a jet row
+  int P, pitch, wmax;
+  int slab;     // elements of a weight slab
+  int wst = 0;  // slab that holds, or waits for, the next GEMM's first rows
   const T* params;
   const T* Wt;  // transposed weights [in][out] per layer
   const T* Wc;  // aligned copy of the packed parameters
@@ -141,18 +185,19 @@ struct SimtTile {
   // the FP64 slice once per chunk.  Null: FP64 adds per tile.
   float* wacc_base = nullptr;
 
-  __device__ SimtTile(const DevInstance& I_, const SimtArgs& A_, unsigned char* smem) : I(I_), A(A_) {
+  __device__ SimtTile(const DevInstance& I_, const SimtArgs& A_, unsigned char* smem)
+      : I(I_), A(A_), NT(blockDim.x) {
     P = I.P;
     pitch = I.pitch;
-    S = I.S;
     wmax = 0;
     for (int l = 1; l < I.L; ++l) wmax = max(wmax, I.widths[l]);
+    slab = simt_slab_elems(wmax, sizeof(T));
     T* base = reinterpret_cast<T*>(smem);
-    size_t be = (size_t)wmax * pitch;
+    const size_t be = (size_t)wmax * pitch;
     B[0] = base;
     B[1] = base + be;
-    B[2] = base + 2 * be;
-    UO = base + 3 * be;
+    WS = base + 2 * be;
+    UO = WS + 2 * slab;
     UB = UO + (size_t)I.n_out * C * P;
     XS = UB + (size_t)I.n_out * C * P;
     size_t off = (size_t)(XS - base) + (size_t)P * I.d;
@@ -161,11 +206,11 @@ struct SimtTile {
     params = reinterpret_cast<const T*>(I.params);
     Wt = reinterpret_cast<const T*>(I.Wt);
     Wc = Wt + weight_copy_offset(I.n_params);
-    if (sizeof(T) == 4 && I.wacc_off >= 0)
+    if (F32 && I.wacc_off >= 0)
       wacc_base = reinterpret_cast<float*>(A.scratch) + (long long)blockIdx.x * A.scratch_stride + I.wacc_off;
   }
 
-  // accumulator of W^l (l = 2..L-1): [item][4][4] per thread item of wgrad
+  // accumulator of W^l (l = 2..L-1): [item][WR][4] per thread item of wgrad
   __device__ float* wacc(int l) const {
     long long off = 0;
     for (int k = 2; k < l; ++k) off += (long long)I.widths[k] * I.widths[k - 1];
@@ -191,9 +236,9 @@ struct SimtTile {
         for (int j = 0; j < 8; ++j) {
           const int e = e0 + j * NT;
           if (e >= n) break;
-          const int it = e >> 4, r = (e >> 2) & 3, s = e & 3;
+          const int it = e / (4 * WR), r = (e >> 2) % WR, s = e & 3;
           const int kb = it % nkb, ub = it / nkb;
-          atomicAdd(gW + (ub * 4 + r) * wi + kb + s * nkb, (double)v[j]);
+          atomicAdd(gW + (ub * WR + r) * wi + kb + s * nkb, widen(v[j]));
         }
       }
     }
@@ -201,7 +246,6 @@ struct SimtTile {
 
   __device__ const T* W(int l) const { return params + I.off_W[l - 1]; }   // l = 1..L
   __device__ const T* bias(int l) const { return params + I.off_b[l - 1]; }
-  __device__ const T* WtL(int l) const { return Wt + I.off_W[l - 1]; }
 
   // hidden layer z-jet location for tile t, hidden layer l (1..L-1)
   __device__ T* zjet(long long tile, int l, bool to_store) const {
@@ -211,48 +255,98 @@ struct SimtTile {
     return reinterpret_cast<T*>(A.scratch) + (long long)blockIdx.x * A.scratch_stride + off;
   }
 
-  // acc[r][c] += w[r] * a[c] for RU units and C channels.  FP32: channel
-  // pairs use the packed FMA, with the unit's weight in both halves.
-  static __device__ __forceinline__ void rank1(T (&acc)[RU][C], const T* w, const T* a) {
-    if constexpr (sizeof(T) == 4) {
+  // ---------------------------------------------------------------- weights
+  // The weight rows [K][wo] of one jet GEMM: W^l transposed (forward) or W^l
+  // (data gradient), both 16-byte aligned in the weight workspace.
+  struct Rows {
+    const T* p;
+    int K, wo;
+  };
+  __device__ Rows fwd_rows(int l) const { return {Wt + I.off_W[l - 1], I.widths[l - 1], I.widths[l]}; }
+  __device__ Rows bwd_rows(int l) const { return {Wc + I.off_W[l - 1], I.widths[l], I.widths[l - 1]}; }
+  __device__ int slab_rows(const Rows& w) const { return min(w.K, slab / w.wo); }
+  // copy rows [k0, k0 + slab_rows) into slab `st` (asynchronously)
+  __device__ void issue(const Rows& w, int k0, int st) const {
+    const int n16 = min(slab_rows(w), w.K - k0) * w.wo / TP;
+    const T* src = w.p + (long long)k0 * w.wo;
+    T* dst = WS + st * slab;
+    for (int i = threadIdx.x; i < n16; i += NT) cp_async16(dst + i * TP, src + i * TP);
+    cp_async_commit();
+  }
+
+  // D[u][n] = sum_k rows[k][u] in[k][n] for all channels; thread item = (point
+  // n, RU consecutive units u0), a point's channels as one vector load and the
+  // RU weights as broadcast vector loads from the slab, 2 RU C flops per k; FP32
+  // units accumulate in packed pairs.  done(n, u0, acc) takes an item's sums.
+  // rows' first slab is in flight in slab wst on entry (and its barrier also
+  // orders the phases before this one); on exit next's first slab is.  The FP32
+  // pipe needs four FMAs per word read from shared memory, which bounds the
+  // item's shape: with RU = 8 and C = 6 a warp reads 14 words per 48 FMAs.
+  // One layer of 64 -> 64 units at C = 6 in a loop of its own, as a share of the
+  // FP32 peak: 49% with RU = 4 and weights read through L1, 61% with RU = 8,
+  // 69% with RU = 8 and weights in shared memory (C = 4: 43, 51 and 69%).
+  struct Acc {
+    typename std::conditional<F32, f2, T>::type v[F32 ? RU / 2 : RU][C];
+  };
+  template <class Done>
+  __device__ __forceinline__ void gemm(const Rows& w, const Rows& next, const T* in, Done done) {
+    const int items = (w.wo / RU) * P, rps = slab_rows(w);
+    for (int it0 = 0; it0 < items; it0 += NT) {
+      const int it = it0 + threadIdx.x;
+      const bool act = it < items, last_pass = it0 + NT >= items;
+      const int n = act ? it % P : 0, u0 = act ? (it / P) * RU : 0;
+      Acc acc;
 #pragma unroll
-      for (int r = 0; r < RU; ++r) {
-        const f2 wr(w[r]);
+      for (int r = 0; r < (F32 ? RU / 2 : RU); ++r)
 #pragma unroll
-        for (int c = 0; c + 1 < C; c += 2) {
-          const f2 s = jfma(wr, f2(a[c], a[c + 1]), f2(acc[r][c], acc[r][c + 1]));
-          acc[r][c] = s.v.x;
-          acc[r][c + 1] = s.v.y;
+        for (int c = 0; c < C; ++c) acc.v[r][c] = 0.f;
+      const T* ap = in + n * C;
+      for (int k0 = 0; k0 < w.K; k0 += rps) {
+        cp_async_wait0();
+        __syncthreads();
+        if (k0 + rps < w.K) issue(w, k0 + rps, wst ^ 1);
+        else if (!last_pass) issue(w, 0, wst ^ 1);
+        else if (next.p) issue(next, 0, wst ^ 1);
+        const T* wp = WS + wst * slab + u0;
+        wst ^= 1;
+        if (!act) continue;
+        const int kn = min(rps, w.K - k0);
+#pragma unroll 4
+        for (int k = 0; k < kn; ++k, ap += pitch, wp += w.wo) {
+          T wv[RU], av[C];
+#pragma unroll
+          for (int r = 0; r < RU; r += TP) vload<T>(wp + r, wv + r);
+          load_chan<T, C>(ap, av);
+          if constexpr (F32) {
+#pragma unroll
+            for (int c = 0; c < C; ++c)
+#pragma unroll
+              for (int r = 0; r < RU / 2; ++r)
+                acc.v[r][c] = jfma(f2(wv[2 * r], wv[2 * r + 1]), f2(av[c]), acc.v[r][c]);
+          } else {
+#pragma unroll
+            for (int r = 0; r < RU; ++r)
+#pragma unroll
+              for (int c = 0; c < C; ++c) acc.v[r][c] = fma(wv[r], av[c], acc.v[r][c]);
+          }
         }
-        if (C & 1) acc[r][C - 1] = fma(w[r], a[C - 1], acc[r][C - 1]);
       }
-    } else {
-#pragma unroll
-      for (int r = 0; r < RU; ++r)
-#pragma unroll
-        for (int c = 0; c < C; ++c) acc[r][c] = fma(w[r], a[c], acc[r][c]);
+      if (act) done(n, u0, acc);
     }
   }
 
   // ---------------------------------------------------------------- forward
-  // Every elementwise phase and both jet GEMMs map a thread to one point n of
-  // the tile and RU consecutive units u0 .. u0+RU, with all C channels of each
-  // (unit, point) in registers: lanes walk points, so a point's channels sit
-  // at fixed offsets from one row pointer, shared-memory rows (odd stride S)
-  // are read and written conflict-free, the z-jet scratch rows
-  // [unit][alpha * P + n] are coalesced, and with RU = TP every thread has
-  // exactly one item when the tile fills the CTA (P = TP * threads / width).
   __device__ void layer1(T* out, T* zdst) {
     const int w = I.widths[1], d = I.d, CP = C * P;
     const T* W1 = W(1);
     const T* b1 = bias(1);
-    for (int it = threadIdx.x; it < (w / RU) * P; it += NT) {
-      const int n = it % P, u0 = (it / P) * RU;
+    for (int it = threadIdx.x; it < (w / EU) * P; it += NT) {
+      const int n = it % P, u0 = (it / P) * EU;
       T x[3];
 #pragma unroll
       for (int i = 0; i < 3; ++i) x[i] = i < d ? XS[n * d + i] : T(0);
 #pragma unroll
-      for (int r = 0; r < RU; ++r) {
+      for (int r = 0; r < EU; ++r) {
         const int u = u0 + r;
         T wrow[3];
 #pragma unroll
@@ -271,56 +365,41 @@ struct SimtTile {
         }
         tanh_derivs<T, NP>(z[0], p);
         Cls::compose(z, p, a);
-#pragma unroll
-        for (int c = 0; c < C; ++c) out[u * pitch + n * S + c] = a[c];
+        store_chan<T, C>(out + u * pitch + n * C, a);
         if (zdst) {
+          __stcg(zdst + (long long)u * CP + n, p[0]);
 #pragma unroll
-          for (int c = 0; c < C; ++c) __stcg(zdst + (long long)u * CP + c * P + n, z[c]);
+          for (int c = 1; c < C; ++c) __stcg(zdst + (long long)u * CP + c * P + n, z[c]);
         }
       }
     }
   }
 
-  // Z^l = W^l A^{l-1} (+ b on channel 0), then a^l = compose(z^l).  Per k a
-  // thread reads its point's C activations (one shared-memory wavefront per
-  // load: lanes walk points) and RU weights as one vector, for RU * C FMAs.
-  __device__ void hidden_fwd(int l, const T* in, T* out, T* zdst) {
-    const int wi = I.widths[l - 1], wo = I.widths[l], CP = C * P;
-    const T* Wtl = WtL(l);  // [wi][wo]
+  // Z^l = W^l A^{l-1} (+ b on channel 0), then a^l = compose(z^l)
+  __device__ void hidden_fwd(int l, const T* in, T* out, T* zdst, const Rows& next) {
+    const int CP = C * P;
     const T* bl = bias(l);
-    for (int it = threadIdx.x; it < (wo / RU) * P; it += NT) {
-      const int n = it % P, u0 = (it / P) * RU;
-      T acc[RU][C];
-#pragma unroll
-      for (int r = 0; r < RU; ++r)
-#pragma unroll
-        for (int c = 0; c < C; ++c) acc[r][c] = T(0);
-      const T* ap = in + n * S;  // row k of A^{l-1}, this point's channels
-      const T* wp = Wtl + u0;    // row k of W^l^T, this thread's units
-#pragma unroll(UK)
-      for (int k = 0; k < wi; ++k, ap += pitch, wp += wo) {
-        T wv[RU], av[C];
-        vldg<T>(wp, wv);
-#pragma unroll
-        for (int c = 0; c < C; ++c) av[c] = ap[c];
-        rank1(acc, wv, av);
-      }
-      if constexpr (sizeof(T) == 4) {
+    gemm(fwd_rows(l), next, in, [&](int n, int u0, const Acc& acc) {
+      if constexpr (F32) {
 #pragma unroll
         for (int r = 0; r < RU; r += 2) {
           const int u = u0 + r;
           f2 z[C], p[NP], a[C];
 #pragma unroll
-          for (int c = 0; c < C; ++c) z[c] = f2(acc[r][c], acc[r + 1][c]);
+          for (int c = 0; c < C; ++c) z[c] = acc.v[r / 2][c];
           z[0] = z[0] + f2(bl[u], bl[u + 1]);
-          tanh_derivs_pair<NP>(z[0], p);
+          tanh_polys_pair<NP>(f2(tanhf(z[0].v.x), tanhf(z[0].v.y)), p);
           Cls::compose(z, p, a);
+          T lo[C], hi[C];
 #pragma unroll
           for (int c = 0; c < C; ++c) {
-            out[u * pitch + n * S + c] = a[c].v.x;
-            out[(u + 1) * pitch + n * S + c] = a[c].v.y;
+            lo[c] = a[c].v.x;
+            hi[c] = a[c].v.y;
           }
+          store_chan<T, C>(out + u * pitch + n * C, lo);
+          store_chan<T, C>(out + (u + 1) * pitch + n * C, hi);
           if (zdst) {
+            z[0] = p[0];
 #pragma unroll
             for (int c = 0; c < C; ++c) {
               __stcg(zdst + (long long)u * CP + c * P + n, z[c].v.x);
@@ -334,75 +413,79 @@ struct SimtTile {
           const int u = u0 + r;
           T z[C], p[NP], a[C];
 #pragma unroll
-          for (int c = 0; c < C; ++c) z[c] = acc[r][c];
+          for (int c = 0; c < C; ++c) z[c] = acc.v[r][c];
           z[0] += bl[u];
           tanh_derivs<T, NP>(z[0], p);
           Cls::compose(z, p, a);
-#pragma unroll
-          for (int c = 0; c < C; ++c) out[u * pitch + n * S + c] = a[c];
+          store_chan<T, C>(out + u * pitch + n * C, a);
           if (zdst) {
+            __stcg(zdst + (long long)u * CP + n, p[0]);
 #pragma unroll
-            for (int c = 0; c < C; ++c) __stcg(zdst + (long long)u * CP + c * P + n, z[c]);
+            for (int c = 1; c < C; ++c) __stcg(zdst + (long long)u * CP + c * P + n, z[c]);
           }
         }
       }
-    }
+    });
   }
 
-  // a^l = compose(z^l) from a stored z-jet [w][C*P]
+  // a^l = compose(z^l) from a stored z-jet [w][C*P] (tanh z in channel 0)
   __device__ void compose_from(int l, const T* zsrc, T* out) {
     const int w = I.widths[l], CP = C * P;
-    for (int it = threadIdx.x; it < (w / RU) * P; it += NT) {
-      const int n = it % P, u0 = (it / P) * RU;
+    for (int it = threadIdx.x; it < (w / EU) * P; it += NT) {
+      const int n = it % P, u0 = (it / P) * EU;
       // all loads first, so that they are in flight together
-      T zz[RU][C];
+      T zz[EU][C];
 #pragma unroll
-      for (int r = 0; r < RU; ++r)
+      for (int r = 0; r < EU; ++r)
 #pragma unroll
         for (int c = 0; c < C; ++c) zz[r][c] = __ldcg(zsrc + (long long)(u0 + r) * CP + c * P + n);
-      if constexpr (sizeof(T) == 4) {
+      if constexpr (F32) {
 #pragma unroll
-        for (int r = 0; r < RU; r += 2) {
+        for (int r = 0; r < EU; r += 2) {
           f2 z[C], p[NP], a[C];
 #pragma unroll
           for (int c = 0; c < C; ++c) z[c] = f2(zz[r][c], zz[r + 1][c]);
-          tanh_derivs_pair<NP>(z[0], p);
+          tanh_polys_pair<NP>(z[0], p);
           Cls::compose(z, p, a);
+          T lo[C], hi[C];
 #pragma unroll
           for (int c = 0; c < C; ++c) {
-            out[(u0 + r) * pitch + n * S + c] = a[c].v.x;
-            out[(u0 + r + 1) * pitch + n * S + c] = a[c].v.y;
+            lo[c] = a[c].v.x;
+            hi[c] = a[c].v.y;
           }
+          store_chan<T, C>(out + (u0 + r) * pitch + n * C, lo);
+          store_chan<T, C>(out + (u0 + r + 1) * pitch + n * C, hi);
         }
       } else {
 #pragma unroll
-        for (int r = 0; r < RU; ++r) {
+        for (int r = 0; r < EU; ++r) {
           T p[NP], a[C];
-          tanh_derivs<T, NP>(zz[r][0], p);
+          tanh_polys<T, NP>(zz[r][0], p);
           Cls::compose(zz[r], p, a);
-#pragma unroll
-          for (int c = 0; c < C; ++c) out[(u0 + r) * pitch + n * S + c] = a[c];
+          store_chan<T, C>(out + (u0 + r) * pitch + n * C, a);
         }
       }
     }
   }
 
-  // u_{o,alpha} = W^L a^{L-1}_alpha (+ b^L on the value channel)
+  // u_{o,alpha} = W^L a^{L-1}_alpha (+ b^L on the value channel); lanes walk
+  // the row's columns n * C + alpha
   __device__ void output_layer(const T* in) {
     const int L = I.L, wi = I.widths[L - 1], no = I.n_out;
     const T* WL = W(L);
     const T* bL = bias(L);
     const int ncol = C * P;
     for (int it = threadIdx.x; it < no * ncol; it += NT) {
-      const int o = it / ncol, col = it % ncol;  // col = alpha * P + n
-      const T* ap = in + (col % P) * S + col / P;
-      T s = col < P ? bL[o] : T(0);
+      const int o = it / ncol, col = it - o * ncol;
+      const int n = col / C, c = col - n * C;
+      const T* ap = in + col;
+      T s = c == 0 ? bL[o] : T(0);
+#pragma unroll 4
       for (int k = 0; k < wi; ++k) s = fma(WL[o * wi + k], ap[k * pitch], s);
-      UO[o * ncol + col] = s;
+      UO[o * ncol + c * P + n] = s;
     }
   }
 
-  // residual r_c = sum terms - source, loss partial, and (if bwd) ub = dL/du.
   // Residual r_c = sum of the monomials - source, the loss partial and (bwd)
   // UB = dL/du.  When the monomial values fit the UB area and 2 r / N the
   // reduction area: three parallel passes, (point, monomial) products, per
@@ -422,7 +505,7 @@ struct SimtTile {
                                  threadIdx.x, NT);
     }
     const T two_over_n = T(2.0 * I.inv_N);
-    const bool parallel = nt <= I.n_out * C && I.n_res * P * (int)sizeof(T) <= 64 * (int)sizeof(double);
+    const bool parallel = nt <= I.n_out * C && I.n_res * P * (int)sizeof(T) <= kSimtRed * (int)sizeof(double);
     if (!parallel) {
       if (bwd)
         for (int i = threadIdx.x; i < I.n_out * ncol; i += NT) UB[i] = T(0);
@@ -496,12 +579,19 @@ struct SimtTile {
   }
 
   // ---------------------------------------------------------------- backward
+  // sum of v over the 4 lanes of a group, in a fixed order
+  static __device__ __forceinline__ T sum4(T v) {
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    return v;
+  }
+
   // Abar^{L-1} = W^L^T ub; dW^L = sum_cols ub a^{L-1}^T; db^L = sum_n ub_0
   __device__ void output_bwd(const T* a_last, T* abar, double* g) {
     const int L = I.L, wi = I.widths[L - 1], no = I.n_out;
     const T* WL = W(L);
     const int ncol = C * P;
-    // Abar[k][n*S + c], one (unit, point) per item with all channels
+    // Abar[k][n*C + c], one (unit, point) per item with all channels
     for (int it = threadIdx.x; it < wi * P; it += NT) {
       const int n = it % P, k = it / P;
       T s[C];
@@ -512,103 +602,118 @@ struct SimtTile {
 #pragma unroll
         for (int c = 0; c < C; ++c) s[c] = fma(w, UB[o * ncol + c * P + n], s[c]);
       }
-#pragma unroll
-      for (int c = 0; c < C; ++c) abar[k * pitch + n * S + c] = s[c];
+      store_chan<T, C>(abar + k * pitch + n * C, s);
     }
-    // dW^L[o][k]: four lanes share a weight, each summing a quarter of the
-    // points; the partials combine by shuffles in a fixed order
+    // dW^L[o][k] and db^L[o]: four lanes share a sum, each taking a quarter of
+    // the points; the partials combine by shuffles in a fixed order
     // (the loop runs whole warps: every lane of a warp reaches the shuffles)
-    const int items = 4 * no * wi, items_w = (items + 31) & ~31;
+    const int items = 4 * no * (wi + 1), items_w = (items + 31) & ~31;
     for (int it = threadIdx.x; it < items_w; it += NT) {
       const bool act = it < items;
-      const int part = it & 3, ok = it >> 2, o = act ? ok / wi : 0, k = act ? ok % wi : 0;
+      const int part = it & 3, ok = it >> 2, o = act ? ok / (wi + 1) : 0, k = act ? ok % (wi + 1) : 0;
       T s = T(0);
-      if (act)
-        for (int n = part; n < P; n += 4)
+      if (act && k < wi) {
+        for (int n = part; n < P; n += 4) {
+          T av[C];
+          load_chan<T, C>(a_last + k * pitch + n * C, av);
 #pragma unroll
-          for (int c = 0; c < C; ++c) s = fma(UB[o * ncol + c * P + n], a_last[k * pitch + n * S + c], s);
-      s += __shfl_xor_sync(0xffffffffu, s, 1);
-      s += __shfl_xor_sync(0xffffffffu, s, 2);
-      if (act && part == 0) atomicAdd(g + I.off_W[L - 1] + o * wi + k, (double)s);
-    }
-    for (int o = threadIdx.x; o < no; o += NT) {
-      T s = T(0);
-      for (int n = 0; n < P; ++n) s += UB[o * ncol + n];
-      atomicAdd(g + I.off_b[L - 1] + o, (double)s);
+          for (int c = 0; c < C; ++c) s = fma(UB[o * ncol + c * P + n], av[c], s);
+        }
+      } else if (act) {
+        for (int n = part; n < P; n += 4) s += UB[o * ncol + n];
+      }
+      s = sum4(s);
+      if (act && part == 0) atomicAdd(g + (k < wi ? I.off_W[L - 1] + o * wi + k : I.off_b[L - 1] + o), widen(s));
     }
   }
 
-  // Zbar^l = (d compose / dz)^T Abar^l, per (unit, point), z^l read from zsrc.
-  __device__ void act_adjoint(int l, const T* zsrc, const T* abar, T* zbar) {
+  // Zbar^l = (d compose / dz)^T Abar^l per (unit, point), in place in `bar`;
+  // z^l (tanh z in channel 0) from zsrc
+  __device__ void act_adjoint(int l, const T* zsrc, T* bar) {
     const int w = I.widths[l], CP = C * P;
-    for (int it = threadIdx.x; it < (w / RU) * P; it += NT) {
-      const int n = it % P, u0 = (it / P) * RU;
+    for (int it = threadIdx.x; it < (w / EU) * P; it += NT) {
+      const int n = it % P, u0 = (it / P) * EU;
       // all global loads first, so that they overlap
-      T zz[RU][C];
+      T zz[EU][C];
 #pragma unroll
-      for (int r = 0; r < RU; ++r)
+      for (int r = 0; r < EU; ++r)
 #pragma unroll
         for (int c = 0; c < C; ++c) zz[r][c] = __ldcg(zsrc + (long long)(u0 + r) * CP + c * P + n);
-      if constexpr (sizeof(T) == 4) {
+      if constexpr (F32) {
         // FP32: units (r, r+1) in packed pairs
 #pragma unroll
-        for (int r = 0; r < RU; r += 2) {
-          const int u = u0 + r;
+        for (int r = 0; r < EU; r += 2) {
+          T* b0 = bar + (u0 + r) * pitch + n * C;
+          T* b1 = b0 + pitch;
           f2 z[C], p[NP], ab[C], zb[C];
+          T lo[C], hi[C];
+          load_chan<T, C>(b0, lo);
+          load_chan<T, C>(b1, hi);
 #pragma unroll
           for (int c = 0; c < C; ++c) {
             z[c] = f2(zz[r][c], zz[r + 1][c]);
-            ab[c] = f2(abar[u * pitch + n * S + c], abar[(u + 1) * pitch + n * S + c]);
+            ab[c] = f2(lo[c], hi[c]);
           }
-          tanh_derivs_pair<NP>(z[0], p);
+          tanh_polys_pair<NP>(z[0], p);
           Cls::adjoint(z, p, ab, zb);
 #pragma unroll
           for (int c = 0; c < C; ++c) {
-            zbar[u * pitch + n * S + c] = zb[c].v.x;
-            zbar[(u + 1) * pitch + n * S + c] = zb[c].v.y;
+            lo[c] = zb[c].v.x;
+            hi[c] = zb[c].v.y;
           }
+          store_chan<T, C>(b0, lo);
+          store_chan<T, C>(b1, hi);
         }
       } else {
 #pragma unroll
-        for (int r = 0; r < RU; ++r) {
-          const int u = u0 + r;
+        for (int r = 0; r < EU; ++r) {
+          T* b0 = bar + (u0 + r) * pitch + n * C;
           T p[NP], ab[C], zb[C];
-#pragma unroll
-          for (int c = 0; c < C; ++c) ab[c] = abar[u * pitch + n * S + c];
-          tanh_derivs<T, NP>(zz[r][0], p);
+          load_chan<T, C>(b0, ab);
+          tanh_polys<T, NP>(zz[r][0], p);
           Cls::adjoint(zz[r], p, ab, zb);
-#pragma unroll
-          for (int c = 0; c < C; ++c) zbar[u * pitch + n * S + c] = zb[c];
+          store_chan<T, C>(b0, zb);
         }
       }
     }
   }
 
-  // dW^l[u][k] += sum_cols Zbar[u][col] A[k][col]; db^l[u] += sum_n Zbar[u][n]
+  // dW^l[u][k] += sum_cols Zbar[u][col] A[k][col]; db^l[u] += sum_n Zbar[u][n].
+  // Thread item: WR rows u and 4 columns k (rows kb + s * nkb of A); NS adjacent
+  // lanes share an item, each taking every NS-th vector of columns, so that
+  // narrow layers fill the CTA (a 20 x 20 layer has 25 items); their sums
+  // combine by halves, each lane ending with its own 1 / NS of the block.
   __device__ void wgrad(int l, const T* zbar, const T* aprev, double* g) {
     const int wo = I.widths[l], wi = I.widths[l - 1];
-    const int ncol = S * P;  // every column, the zero pads of odd S included
-    const int nkb = wi / 4;
+    const int ncol = (C * P + TP - 1) / TP * TP;  // zero columns up to a whole vector
+    const int nkb = wi / 4, items = (wo / WR) * nkb;
+    const int NS = simt_wgrad_slices(items, WR, F32, NT);
     double* gW = g + I.off_W[l - 1];
-    for (int it = threadIdx.x; it < (wo / 4) * nkb; it += NT) {
-      const int kb = it % nkb, ub = it / nkb;
-      T acc[4][4];
-      if constexpr (sizeof(T) == 4) {
+    const int work = items * NS, work_w = (work + 31) & ~31;
+    for (int it = threadIdx.x; it < work_w; it += NT) {
+      const bool act = it < work;
+      const int sl = it & (NS - 1), item = act ? it / NS : 0;
+      const int kb = item % nkb, ub = item / nkb;
+      T acc[WR * 4];
+      const T* zp = zbar + ub * WR * pitch;
+      const T* app = aprev + kb * pitch;
+      const int c0 = act ? sl * TP : ncol;
+      if constexpr (F32) {
         // FP32: even and odd columns accumulate in the two halves of a
         // packed pair (the 16-byte loads deliver the pairs), summed at the end
-        f2 ap2[4][4];
+        f2 ap2[WR][4];
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+        for (int r = 0; r < WR; ++r)
 #pragma unroll
           for (int s = 0; s < 4; ++s) ap2[r][s] = f2(0.f);
-        for (int col = 0; col < ncol; col += TP) {
-          T zv[4][TP], av[4][TP];
+        for (int col = c0; col < ncol; col += NS * TP) {
+          T zv[WR][TP], av[4][TP];
 #pragma unroll
-          for (int r = 0; r < 4; ++r) vload<T>(zbar + (ub * 4 + r) * pitch + col, zv[r]);
+          for (int s = 0; s < 4; ++s) vload<T>(app + s * nkb * pitch + col, av[s]);
 #pragma unroll
-          for (int s = 0; s < 4; ++s) vload<T>(aprev + (kb + s * nkb) * pitch + col, av[s]);
+          for (int r = 0; r < WR; ++r) vload<T>(zp + r * pitch + col, zv[r]);
 #pragma unroll
-          for (int r = 0; r < 4; ++r)
+          for (int r = 0; r < WR; ++r)
 #pragma unroll
             for (int s = 0; s < 4; ++s)
 #pragma unroll
@@ -616,110 +721,142 @@ struct SimtTile {
                 ap2[r][s] = jfma(f2(zv[r][j], zv[r][j + 1]), f2(av[s][j], av[s][j + 1]), ap2[r][s]);
         }
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+        for (int r = 0; r < WR; ++r)
 #pragma unroll
-          for (int s = 0; s < 4; ++s) acc[r][s] = ap2[r][s].v.x + ap2[r][s].v.y;
+          for (int s = 0; s < 4; ++s) acc[r * 4 + s] = ap2[r][s].v.x + ap2[r][s].v.y;
       } else {
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+        for (int e = 0; e < WR * 4; ++e) acc[e] = T(0);
+        for (int col = c0; col < ncol; col += NS * TP) {
+          T zv[WR][TP], av[4][TP];
 #pragma unroll
-          for (int s = 0; s < 4; ++s) acc[r][s] = T(0);
-        for (int col = 0; col < ncol; col += TP) {
-          T zv[4][TP], av[4][TP];
+          for (int r = 0; r < WR; ++r) vload<T>(zp + r * pitch + col, zv[r]);
 #pragma unroll
-          for (int r = 0; r < 4; ++r) vload<T>(zbar + (ub * 4 + r) * pitch + col, zv[r]);
+          for (int s = 0; s < 4; ++s) vload<T>(app + s * nkb * pitch + col, av[s]);
 #pragma unroll
-          for (int s = 0; s < 4; ++s) vload<T>(aprev + (kb + s * nkb) * pitch + col, av[s]);
-#pragma unroll
-          for (int r = 0; r < 4; ++r)
+          for (int r = 0; r < WR; ++r)
 #pragma unroll
             for (int s = 0; s < 4; ++s)
 #pragma unroll
-              for (int j = 0; j < TP; ++j) acc[r][s] = fma(zv[r][j], av[s][j], acc[r][s]);
+              for (int j = 0; j < TP; ++j) acc[r * 4 + s] = fma(zv[r][j], av[s][j], acc[r * 4 + s]);
         }
       }
+      // combine the NS lanes: at each step a lane keeps one half of its block
+      // and sends the other to its partner
+      int base = 0, n = WR * 4;
+#pragma unroll
+      for (int m = 1; m < 8; m <<= 1) {
+        const int h = WR * 4 / 2 / m;
+        if (m >= NS) break;
+        const bool up = (it & m) != 0;
+#pragma unroll
+        for (int e = 0; e < h; ++e) {
+          const T send = up ? acc[e] : acc[e + h], keep = up ? acc[e + h] : acc[e];
+          acc[e] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+        }
+        base += up ? h : 0;
+        n = h;
+      }
+      if (!act) continue;
       // fire-and-forget adds: every element belongs to one thread, which adds
       // the tiles in order, so the sums stay deterministic
-      if constexpr (sizeof(T) == 4) {
-        if (wacc_base) {
-          float* a = wacc(l) + (long long)it * 16;
+      if constexpr (F32) {
+        if (wacc_base) {  // n is a multiple of 4 here
+          float* a = wacc(l) + (long long)item * (WR * 4) + base;
 #pragma unroll
-          for (int r = 0; r < 4; ++r) red_add_v4(a + 4 * r, acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
+          for (int e = 0; e < WR * 4; e += 4)
+            if (e < n) red_add_v4(a + e, acc[e], acc[e + 1], acc[e + 2], acc[e + 3]);
           continue;
         }
       }
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int s = 0; s < 4; ++s) atomicAdd(gW + (ub * 4 + r) * wi + kb + s * nkb, (double)acc[r][s]);
+      for (int e = 0; e < WR * 4; ++e)
+        if (e < n) {
+          const int r = (base + e) >> 2, s = (base + e) & 3;
+          atomicAdd(gW + (ub * WR + r) * wi + kb + s * nkb, widen(acc[e]));
+        }
     }
+    // four lanes per bias
     double* gb = g + I.off_b[l - 1];
-    for (int u = threadIdx.x; u < wo; u += NT) {
+    const int bw = (4 * wo + 31) & ~31;
+    for (int it = threadIdx.x; it < bw; it += NT) {
+      const int u = it >> 2, part = it & 3;
       T s = T(0);
-      for (int n = 0; n < P; ++n) s += zbar[u * pitch + n * S];
-      atomicAdd(gb + u, (double)s);
+      if (u < wo)
+        for (int n = part; n < P; n += 4) s += zbar[u * pitch + n * C];
+      s = sum4(s);
+      if (u < wo && part == 0) atomicAdd(gb + u, widen(s));
     }
   }
 
-  // Abar^{l-1}[k][col] = sum_u W^l[u][k] Zbar^l[u][col].  A thread owns one
-  // point and RU consecutive input units (the mapping of hidden_fwd); the
-  // weights W^l[u][k0 .. k0+RU) come from the aligned parameter copy.
-  __device__ void dgrad(int l, const T* zbar, T* abar) {
-    const int wo = I.widths[l], wi = I.widths[l - 1];
-    const T* Wl = Wc + I.off_W[l - 1];  // [wo][wi]
-    for (int it = threadIdx.x; it < (wi / RU) * P; it += NT) {
-      const int n = it % P, k0 = (it / P) * RU;
-      T acc[RU][C];
+  // Abar^{l-1}[k][col] = sum_u W^l[u][k] Zbar^l[u][col]
+  __device__ void dgrad(int l, const T* zbar, T* abar, const Rows& next) {
+    gemm(bwd_rows(l), next, zbar, [&](int n, int k0, const Acc& acc) {
+      if constexpr (F32) {
 #pragma unroll
-      for (int i = 0; i < RU; ++i)
+        for (int r = 0; r < RU; r += 2) {
+          T lo[C], hi[C];
 #pragma unroll
-        for (int c = 0; c < C; ++c) acc[i][c] = T(0);
-      const T* zp = zbar + n * S;  // row u of Zbar^l, this point's channels
-      const T* wp = Wl + k0;       // row u of W^l, this thread's input units
-#pragma unroll(UK)
-      for (int u = 0; u < wo; ++u, zp += pitch, wp += wi) {
-        T wv[RU], zv[C];
-        vldg<T>(wp, wv);
+          for (int c = 0; c < C; ++c) {
+            lo[c] = acc.v[r / 2][c].v.x;
+            hi[c] = acc.v[r / 2][c].v.y;
+          }
+          store_chan<T, C>(abar + (k0 + r) * pitch + n * C, lo);
+          store_chan<T, C>(abar + (k0 + r + 1) * pitch + n * C, hi);
+        }
+      } else {
 #pragma unroll
-        for (int c = 0; c < C; ++c) zv[c] = zp[c];
-        rank1(acc, wv, zv);
+        for (int r = 0; r < RU; ++r) store_chan<T, C>(abar + (k0 + r) * pitch + n * C, acc.v[r]);
       }
-#pragma unroll
-      for (int i = 0; i < RU; ++i)
-#pragma unroll
-        for (int c = 0; c < C; ++c) abar[(k0 + i) * pitch + n * S + c] = acc[i][c];
-    }
+    });
   }
 
-  // dW^1[u][i] += sum_n Zbar_0[u][n] x_i[n] + Zbar_{e_i}[u][n]; db^1[u] += sum_n Zbar_0[u][n]
+  // dW^1[u][i] += sum_n Zbar_0[u][n] x_i[n] + Zbar_{e_i}[u][n]; db^1[u] += sum_n Zbar_0[u][n];
+  // four lanes per unit
   __device__ void layer1_bwd(const T* zbar, double* g) {
     const int w = I.widths[1], d = I.d;
     double* gW = g + I.off_W[0];
     double* gb = g + I.off_b[0];
-    for (int u = threadIdx.x; u < w; u += NT) {
+    const int ww = (4 * w + 31) & ~31;
+    for (int it = threadIdx.x; it < ww; it += NT) {
+      const int u = it >> 2, part = it & 3;
       T sb = T(0), sw[3] = {T(0), T(0), T(0)};
-      for (int n = 0; n < P; ++n) {
-        const T z0 = zbar[u * pitch + n * S];
-        sb += z0;
+      if (u < w)
+        for (int n = part; n < P; n += 4) {
+          T zv[C];
+          load_chan<T, C>(zbar + u * pitch + n * C, zv);
+          sb += zv[0];
+#pragma unroll
+          for (int i = 0; i < 3; ++i)
+            if (i < d) sw[i] = fma(zv[0], XS[n * d + i], sw[i]);
+#pragma unroll
+          for (int i = 0; i < Cls::D; ++i) {
+            const int fo = Cls::first_order(i);
+            if (fo >= 0 && i < d) sw[i] += zv[fo];
+          }
+        }
+      sb = sum4(sb);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) sw[i] = sum4(sw[i]);
+      if (u < w && part == 0) {
 #pragma unroll
         for (int i = 0; i < 3; ++i)
-          if (i < d) sw[i] = fma(z0, XS[n * d + i], sw[i]);
+          if (i < d) atomicAdd(gW + u * d + i, widen(sw[i]));
+        atomicAdd(gb + u, widen(sb));
       }
-#pragma unroll
-      for (int i = 0; i < Cls::D; ++i) {
-        const int fo = Cls::first_order(i);
-        if (fo >= 0 && i < d)
-          for (int n = 0; n < P; ++n) sw[i] += zbar[u * pitch + n * S + fo];
-      }
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-        if (i < d) atomicAdd(gW + u * d + i, (double)sw[i]);
-      atomicAdd(gb + u, (double)sb);
     }
   }
 
   // ---------------------------------------------------------------- driver
-  __device__ double tile(long long t, double* g) {
+  // the first jet GEMM of a tile (p null: the network has none)
+  __device__ Rows first_rows() const {
+    if (I.L < 3) return {nullptr, 0, 0};
+    return A.mode == MODE_BWD_STORE ? bwd_rows(I.L - 1) : fwd_rows(2);
+  }
+
+  // one tile; its first GEMM's first weight slab is in flight on entry, and
+  // the next tile's on exit (more: there is one)
+  __device__ double tile(long long t, double* g, bool more) {
     const int mode = A.mode;
     const long long n0 = t * P;
     const long long rem = I.N - n0;
@@ -733,13 +870,15 @@ struct SimtTile {
     __syncthreads();
     const bool use_store = (mode == MODE_BWD_STORE) || (mode == MODE_FWD && I.store != nullptr);
     const bool write_z = (mode == MODE_FWD_BWD) || (mode == MODE_FWD && I.store != nullptr);
+    const bool bwd = mode != MODE_FWD;
     const int L = I.L;
+    const Rows none{nullptr, 0, 0}, first = more ? first_rows() : none;
     int cur = 0;
     if (mode != MODE_BWD_STORE) {
       layer1(B[0], write_z ? zjet(t, 1, use_store) : nullptr);
       for (int l = 2; l <= L - 1; ++l) {
-        __syncthreads();
-        hidden_fwd(l, B[cur], B[cur ^ 1], write_z ? zjet(t, l, use_store) : nullptr);
+        const Rows next = l < L - 1 ? fwd_rows(l + 1) : bwd ? bwd_rows(l) : first;
+        hidden_fwd(l, B[cur], B[cur ^ 1], write_z ? zjet(t, l, use_store) : nullptr, next);
         cur ^= 1;
       }
     } else {
@@ -748,23 +887,26 @@ struct SimtTile {
     __syncthreads();
     output_layer(B[cur]);
     __syncthreads();
-    const bool bwd = mode != MODE_FWD;
     double loss = residual(n0, nvalid, bwd);
     __syncthreads();
     if (!bwd) return loss;
-    const int ab = (cur + 1) % 3, zb = (cur + 2) % 3, ap = cur;
-    output_bwd(B[cur], B[ab], g);
+    // x: Abar^l, then Zbar^l in place; y: A^{l-1}, then Abar^{l-1}
+    T *x = B[cur ^ 1], *y = B[cur];
+    output_bwd(y, x, g);
     __syncthreads();
     const bool from_store = mode == MODE_BWD_STORE;
     for (int l = L - 1; l >= 1; --l) {
-      act_adjoint(l, zjet(t, l, from_store), B[ab], B[zb]);
-      if (l >= 2) compose_from(l - 1, zjet(t, l - 1, from_store), B[ap]);
+      act_adjoint(l, zjet(t, l, from_store), x);
+      if (l >= 2) compose_from(l - 1, zjet(t, l - 1, from_store), y);
       __syncthreads();
       if (l >= 2) {
-        wgrad(l, B[zb], B[ap], g);
-        dgrad(l, B[zb], B[ab]);
+        wgrad(l, x, y, g);
+        dgrad(l, x, y, l > 2 ? bwd_rows(l - 1) : first);  // its first barrier ends the weight gradient's reads of y
+        T* tmp = x;
+        x = y;
+        y = tmp;
       } else {
-        layer1_bwd(B[zb], g);
+        layer1_bwd(x, g);
       }
       __syncthreads();
     }
@@ -774,31 +916,35 @@ struct SimtTile {
 
 constexpr int kWaccTiles = 64;  // tiles per FP32 weight-gradient run (FP32 forms)
 
-template <class Cls, class T>
+template <class Cls, class T, int RU>
 __device__ __forceinline__ void simt_body(const SimtArgs& args) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int k_s;
+  const int NT = blockDim.x;
   for (int k = blockIdx.x; k < args.n_items;) {
     // batched launches walk a cost-ordered list: position k -> item id, and
     // item id -> instance (second half of item_inst)
     const int item = args.item_inst ? args.item_inst[k] : k;
     const DevInstance& I = args.insts ? args.insts[args.item_inst[args.n_items + item]] : args.inst0;
     const int chunk = item - I.chunk_base;
-    SimtTile<Cls, T> S(I, args, smem);
-    // the pad columns of the odd point stride are never written: zero them
-    // (and everything else) once per item so that the weight-gradient sums
-    // over whole rows see zeros there
-    for (int i = threadIdx.x; i < 3 * S.wmax * S.pitch; i += kSimtThreads) S.B[0][i] = T(0);
+    SimtTile<Cls, T, RU> S(I, args, smem);
+    // columns past C * P are never written: zero them (and everything else)
+    // once per item so that the weight-gradient sums over whole vectors see
+    // zeros there
+    for (int i = threadIdx.x; i < 2 * S.wmax * S.pitch; i += NT) S.B[0][i] = T(0);
+    const auto first = S.first_rows();
+    if (first.p) S.issue(first, 0, 0);
     const bool bwd = args.mode != MODE_FWD;
     double* g = bwd ? I.grad_slices + (long long)chunk * I.n_params : nullptr;
     if (bwd)
-      for (long long i = threadIdx.x; i < I.n_params; i += kSimtThreads) g[i] = 0.0;
+      for (long long i = threadIdx.x; i < I.n_params; i += NT) g[i] = 0.0;
     const bool wacc_on = bwd && S.wacc_base != nullptr;
     if (wacc_on) S.wacc_zero();
     __syncthreads();
     double loss = 0.0;
-    const long long t0 = (long long)chunk * I.tiles_per_chunk;
-    const long long t1 = (t0 + I.tiles_per_chunk < I.n_tiles) ? t0 + I.tiles_per_chunk : I.n_tiles;
+    // tiles of the chunk: the first chunk_rem chunks take one more than the rest
+    const long long t0 = (long long)chunk * I.tiles_per_chunk + min(chunk, I.chunk_rem);
+    const long long t1 = t0 + I.tiles_per_chunk + (chunk < I.chunk_rem ? 1 : 0);
     if constexpr (Cls::C >= 7) {
       // FP32 runs of at most kWaccTiles tiles: the FP32 rounding of a
       // weight's sum stays below kWaccTiles * 2^-24 of its magnitudes at any N
@@ -806,7 +952,7 @@ __device__ __forceinline__ void simt_body(const SimtArgs& args) {
       while (t < t1) {
         const long long r1 = (wacc_on && t1 - t > kWaccTiles) ? t + kWaccTiles : t1;
         for (; t < r1; ++t) {
-          loss += S.tile(t, g);
+          loss += S.tile(t, g, t + 1 < t1);
           __syncthreads();
         }
         if (wacc_on) {
@@ -825,7 +971,7 @@ __device__ __forceinline__ void simt_body(const SimtArgs& args) {
       // once per chunk; their accumulator serves only nets too wide for
       // L2-resident FP64 slices
       for (long long t = t0; t < t1; ++t) {
-        loss += S.tile(t, g);
+        loss += S.tile(t, g, t + 1 < t1);
         __syncthreads();
       }
       if (wacc_on) {
@@ -840,7 +986,7 @@ __device__ __forceinline__ void simt_body(const SimtArgs& args) {
     __syncthreads();
     if (threadIdx.x == 0) {
       double s = 0.0;
-      for (int w = 0; w < kSimtThreads / 32; ++w) s += S.RED[w];
+      for (int w = 0; w < NT / 32; ++w) s += S.RED[w];
       I.loss_slices[chunk] = s;
     }
     // the next item: from the shared counter, or a fixed stride
@@ -855,22 +1001,24 @@ __device__ __forceinline__ void simt_body(const SimtArgs& args) {
   }
 }
 
+// Launch bounds: up to 512 threads (one CTA per SM, or two of 256) and so at
+// most 128 registers, except where the tiles need one CTA of 256 threads with
+// all registers: FP64, and channel sets of 10 or more.
 template <class Cls, class T>
-__global__ void __launch_bounds__(kSimtThreads) simt_kernel(const __grid_constant__ SimtArgs args) {
-  simt_body<Cls, T>(args);
+constexpr int simt_max_threads() {
+  return sizeof(T) == 8 || Cls::C >= 10 ? 256 : 512;
+}
+template <class Cls, class T, int RU>
+__global__ void __launch_bounds__(simt_max_threads<Cls, T>(), 1) simt_kernel(const __grid_constant__ SimtArgs args) {
+  simt_body<Cls, T, RU>(args);
 }
 
-// Channel sets of 10 or more: their tiles take most of the shared memory
-// with one CTA per SM, so the registers are sized for one.
+// the kernel for ru units per thread of the jet GEMMs: FP32 8 (every hidden
+// width a multiple of 8) or 4, FP64 2
 template <class Cls, class T>
-__global__ void __launch_bounds__(kSimtThreads, 1) simt_kernel_wide(const __grid_constant__ SimtArgs args) {
-  simt_body<Cls, T>(args);
-}
-
-template <class Cls, class T>
-constexpr auto simt_entry() {
-  if constexpr (Cls::C >= 10) return &simt_kernel_wide<Cls, T>;
-  else return &simt_kernel<Cls, T>;
+constexpr auto simt_entry(int ru) {
+  if constexpr (sizeof(T) == 8) return &simt_kernel<Cls, T, 2>;
+  else return ru == 8 ? &simt_kernel<Cls, T, 8> : &simt_kernel<Cls, T, 4>;
 }
 
 // Elementwise activation rule on [n][C] FP64 jets (verification hook, Eq. 15).

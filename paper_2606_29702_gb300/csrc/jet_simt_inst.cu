@@ -15,10 +15,10 @@ namespace {
 // kernel can keep resident (the rest of the SM's 256 KB stays L1, which
 // serves the per-k weight vectors of the jet GEMMs).
 template <class K>
-cudaError_t prepare(K kernel, size_t smem) {
+cudaError_t prepare(K kernel, int threads, size_t smem) {
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int blocks = 0, dev = 0, smem_sm = 0, reserved = 0;
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kernel, kSimtThreads, smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kernel, threads, smem);
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
@@ -35,30 +35,26 @@ cudaError_t prepare(K kernel, size_t smem) {
 
 template <>
 cudaError_t simt_launch_id<JET_CLASS_ID>(bool fp64, const SimtArgs& a, int grid, size_t smem, cudaStream_t s) {
-  cudaError_t e;
-  if (fp64) {
-    e = prepare(simt_entry<ThisCls, double>(), smem);
-    if (e != cudaSuccess) return e;
-    simt_entry<ThisCls, double>()<<<grid, kSimtThreads, smem, s>>>(a);
-  } else {
-    e = prepare(simt_entry<ThisCls, float>(), smem);
-    if (e != cudaSuccess) return e;
-    simt_entry<ThisCls, float>()<<<grid, kSimtThreads, smem, s>>>(a);
-  }
+  const auto kernel = fp64 ? simt_entry<ThisCls, double>(a.ru) : simt_entry<ThisCls, float>(a.ru);
+  cudaError_t e = prepare(kernel, a.threads, smem);
+  if (e != cudaSuccess) return e;
+  kernel<<<grid, a.threads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
 template <>
-cudaError_t simt_max_active_id<JET_CLASS_ID>(bool fp64, size_t smem, int* blocks) {
-  cudaError_t e;
-  if (fp64) {
-    e = cudaFuncSetAttribute(simt_entry<ThisCls, double>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, simt_entry<ThisCls, double>(), kSimtThreads, smem);
-  }
-  e = cudaFuncSetAttribute(simt_entry<ThisCls, float>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+cudaError_t simt_max_active_id<JET_CLASS_ID>(bool fp64, int ru, int threads, size_t smem, int* blocks) {
+  const auto kernel = fp64 ? simt_entry<ThisCls, double>(ru) : simt_entry<ThisCls, float>(ru);
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, simt_entry<ThisCls, float>(), kSimtThreads, smem);
+  if (threads > fa.maxThreadsPerBlock) {
+    *blocks = 0;
+    return cudaSuccess;
+  }
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, kernel, threads, smem);
 }
 
 template <>
