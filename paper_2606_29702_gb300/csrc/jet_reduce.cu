@@ -1,6 +1,7 @@
 // Weight transposition (plus an aligned copy of the parameters), deterministic FP64 gradient/loss reduction over the
 // chunk slices, and the fused full-batch Adam update (Sec. 3.1.1).
 #include <cmath>
+#include <type_traits>
 
 #include "jet_internal.h"
 
@@ -51,19 +52,25 @@ struct AdamConst {
   const long long* step_ctr;
 };
 
-// One block takes 32 consecutive parameters (lanes over parameters, so every
-// slice row is read coalesced); its 8 warps sum every 8th chunk slice in FP64
-// and warp 0 adds the 8 partials in a fixed order: deterministic, and enough
-// blocks to fill the GPU when there are many chunks.
+// A block's 8 warps form 8 / G groups; a group takes 32 consecutive parameters
+// (lanes over parameters, so every slice row is read coalesced), its G warps sum
+// every G-th chunk slice in FP64 with eight loads in flight, and the first adds
+// the G partials in a fixed order: deterministic.  Bound by the FP64 adds, which
+// run at 2 a clock per SM.  G = 8 fills the GPU where there are few parameters
+// and many chunks; G = 1 spares the adds of the partials where there are many
+// parameters (a batch).  The chunk losses of a job are summed by all threads of
+// its first block in a fixed tree: one thread adding 304 of them one after
+// another took 22 us (forward pass at 10000 points), the tree 4 us.
 constexpr int kRedWarps = 8;
 
-template <class T, bool ADAM>
+template <class T, bool ADAM, int G>
 __global__ void __launch_bounds__(32 * kRedWarps) reduce_kernel(const __grid_constant__ ReduceJob job0,
                                                                 const ReduceJob* jobs, AdamConst ac) {
   const ReduceJob& J = jobs ? jobs[blockIdx.y] : job0;
   // the grid covers the largest job: blocks past this job's parameters have
   // nothing to do (block 0 stays: it writes the loss, also of loss-only jobs)
-  if (blockIdx.x > 0 && (long long)blockIdx.x * 32 >= J.n_params) return;
+  constexpr int PB = 32 * kRedWarps / G;  // parameters per block
+  if (blockIdx.x > 0 && (long long)blockIdx.x * PB >= J.n_params) return;
   __shared__ double part[kRedWarps][32];
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   const int gc = J.grad_chunks > 0 ? J.grad_chunks : J.n_chunks;
@@ -85,17 +92,28 @@ __global__ void __launch_bounds__(32 * kRedWarps) reduce_kernel(const __grid_con
   }
   const double bc1 = ADAM ? bc_s[0] : 1.0, bc2 = ADAM ? bc_s[1] : 1.0;
   const float bc1_f = (float)bc1, bc2_f = (float)bc2;
-  for (long long p0 = (long long)blockIdx.x * 32; p0 < J.n_params; p0 += (long long)gridDim.x * 32) {
-    const long long p = p0 + lane;
+  for (long long p0 = (long long)blockIdx.x * PB; p0 < J.n_params; p0 += (long long)gridDim.x * PB) {
+    const long long p = p0 + wp / G * 32 + lane;
     double g = 0.0;
-    if (p < J.n_params)
-      for (int c = wp; c < gc; c += kRedWarps) g += J.grad_slices[(long long)c * J.n_params + p];
-    part[wp][lane] = g;
-    __syncthreads();
-    if (wp == 0 && p < J.n_params) {
-      g = 0.0;
+    if (p < J.n_params) {
+      const double* src = J.grad_slices + p;
+      int c = wp % G;
+      for (; c + 7 * G < gc; c += 8 * G) {
+        double v[8];
 #pragma unroll
-      for (int w = 0; w < kRedWarps; ++w) g += part[w][lane];
+        for (int j = 0; j < 8; ++j) v[j] = src[(long long)(c + j * G) * J.n_params];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) g += v[j];
+      }
+      for (; c < gc; c += G) g += src[(long long)c * J.n_params];
+    }
+    if (G > 1) {
+      part[wp][lane] = g;
+      __syncthreads();
+    }
+    if (wp % G == 0 && p < J.n_params) {
+#pragma unroll
+      for (int w = 1; w < G; ++w) g += part[wp + w][lane];
       if (J.grad_out) reinterpret_cast<T*>(J.grad_out)[p] = (T)g;
       if (ADAM) {
         T* th = reinterpret_cast<T*>(J.params);
@@ -118,12 +136,20 @@ __global__ void __launch_bounds__(32 * kRedWarps) reduce_kernel(const __grid_con
         }
       }
     }
-    __syncthreads();
+    if (G > 1) __syncthreads();
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0 && J.loss_out) {
+  if (blockIdx.x == 0 && J.loss_out) {
     double s = 0.0;
-    for (int c = 0; c < J.n_chunks; ++c) s += J.loss_slices[c];
-    *J.loss_out = s * J.inv_N;
+    for (int c = threadIdx.x; c < J.n_chunks; c += 32 * kRedWarps) s += J.loss_slices[c];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) part[wp][0] = s;  // part's last readers passed a barrier
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      s = 0.0;
+#pragma unroll
+      for (int w = 0; w < kRedWarps; ++w) s += part[w][0];
+      *J.loss_out = s * J.inv_N;
+    }
   }
 }
 
@@ -145,18 +171,27 @@ cudaError_t launch_reduce(const ReduceJob* dev_jobs, const ReduceJob& job0, int 
   ac.eps_f = 1e-8f;
   ac.step = step < 1 ? 1 : step;
   ac.step_ctr = adam ? step_ctr : nullptr;
-  long long gx = (max_params + 31) / 32;
+  // G = 1 once a warp per 32 parameters is 16 warps per SM and more
+  const bool many = max_params * (n > 0 ? n : 1) >= 32LL * 16 * 152;
+  const int per_block = many ? 32 * kRedWarps : 32;
+  long long gx = (max_params + per_block - 1) / per_block;
   if (gx > 4096) gx = 4096;
   if (gx < 1) gx = 1;
-  dim3 grid((unsigned)gx, (unsigned)(n > 0 ? n : 1));
+  const dim3 grid((unsigned)gx, (unsigned)(n > 0 ? n : 1));
   const ReduceJob* jobs = n == 1 ? nullptr : dev_jobs;
   const int threads = 32 * kRedWarps;
+  auto launch = [&](auto t, auto a) {
+    using T = decltype(t);
+    constexpr bool ADAM = decltype(a)::value;
+    if (many) reduce_kernel<T, ADAM, 1><<<grid, threads, 0, s>>>(job0, jobs, ac);
+    else reduce_kernel<T, ADAM, kRedWarps><<<grid, threads, 0, s>>>(job0, jobs, ac);
+  };
   if (fp64) {
-    if (adam) reduce_kernel<double, true><<<grid, threads, 0, s>>>(job0, jobs, ac);
-    else reduce_kernel<double, false><<<grid, threads, 0, s>>>(job0, jobs, ac);
+    if (adam) launch(double(), std::true_type());
+    else launch(double(), std::false_type());
   } else {
-    if (adam) reduce_kernel<float, true><<<grid, threads, 0, s>>>(job0, jobs, ac);
-    else reduce_kernel<float, false><<<grid, threads, 0, s>>>(job0, jobs, ac);
+    if (adam) launch(float(), std::true_type());
+    else launch(float(), std::false_type());
   }
   if (adam && step_ctr) {
     cudaError_t e = cudaGetLastError();

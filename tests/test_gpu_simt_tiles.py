@@ -15,7 +15,8 @@ TOL = {"fp64": (1e-12, 1e-10), "fp32": (1e-5, 1e-5)}
 CASES = [("burgers_2x20x4", [2, 64, 1]), ("burgers_2x20x4", [2, 12, 40, 8, 1]), ("burgers_2x20x4", [2, 32, 64, 32, 1]),
          ("ks_2x64x5", [2, 20, 20, 1]), ("ks_2x64x5", [2, 128, 16, 1]), ("ns_uvp_2x64x6", [2, 4, 36, 3]),
          ("helmholtz_3x256x8", [3, 256, 8, 256, 1]), ("helmholtz_3x256x8", [3, 252, 24, 1]),
-         ("ns_psi_3x128x6", [3, 64, 40, 2])]
+         ("ns_psi_3x128x6", [3, 64, 40, 2]),
+         ("burgers_2x20x4", [2] + [128] * 7 + [1])]  # enough parameters for a warp per 32 of them in the reduction
 
 
 def _plan(jet, specs, spec, prec, tile=None):
