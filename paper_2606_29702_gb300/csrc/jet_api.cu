@@ -154,10 +154,10 @@ size_t simt_tile_smem(const jet_plan_s* p, int P, int ru, int threads) {
 }
 
 // most points per tile that `ctas` CTAs of `threads` per SM can hold, at most
-// one item of the jet GEMMs per thread (P = threads * ru / wmax)
+// one item of the jet GEMMs per thread (FP64: two)
 int simt_most_points(const jet_plan_s* p, int ru, int threads, int ctas) {
-  int P = std::max(2, threads * ru / p->wmax / 2 * 2);
-  while (P > 2 && (simt_tile_smem(p, P, ru, threads) + 1280) * ctas > (size_t)226 * 1024) P -= 2;
+  int P = std::max(2, threads * std::max(ru, 2) / p->wmax / 2 * 2);
+  while (P > 2 && (simt_tile_smem(p, P, ru, threads) + kSimtCtaBytes) * ctas > kSimtSmBytes) P -= 2;
   return P;
 }
 
@@ -186,7 +186,8 @@ void simt_shape(jet_plan_s* p, int p8) {
 
 // Points per tile of one call on N points: the tile that leaves the busiest SM
 // the least work, counted in GEMM warps per tile plus kTileWarps for what a
-// tile costs whatever its size (its barriers and latencies).
+// tile costs whatever its size (its barriers and latencies).  FP32 warps count
+// in fours, one per scheduler of the SM: six warps take as long as eight.
 constexpr double kTileWarps = 2.0;
 int simt_call_points(const jet_plan_s* p, long long N) {
   if (p->P_fixed) return p->P;
@@ -194,7 +195,8 @@ int simt_call_points(const jet_plan_s* p, long long N) {
   double best_cost = 0.0;
   for (int P = p->P; P >= 2; P -= 2) {
     const long long tiles = (N + P - 1) / P, per_sm = (tiles + p->sms - 1) / p->sms;
-    const int warps = (p->wmax / p->ru * P + 31) / 32;
+    int warps = (p->wmax / p->ru * P + 31) / 32;
+    if (!p->fp64) warps = (warps + 3) / 4 * 4;
     const double cost = (double)per_sm * (warps + kTileWarps);
     if (P == p->P || cost < best_cost) {
       best = P;
@@ -613,6 +615,7 @@ jet_status run_simt(jet_plan_s* p, int mode, const DevInstance& I, cudaStream_t 
   a.scratch_stride = p->scratch_stride;
   a.ru = p->ru;
   a.threads = p->threads;
+  a.carveout = simt_carveout(p->smem, p->ctas_per_sm);
   int grid = std::min(p->grid, I.n_chunks);
   ProfScope prof(p, s);
   CK(simt_launch(p->cls, p->fp64, a, grid, p->smem, s));
@@ -748,7 +751,7 @@ struct jet_batch_s {
   bool tc = false;
   int grid = 0;
   size_t smem = 0;
-  int ru = 0;
+  int ru = 0, ctas_per_sm = 0;
   std::vector<int> P;  // points per tile of every member
   int max_chunks_per_inst = 16;
   // device workspace
@@ -813,7 +816,7 @@ jet_status batch_prepare(jet_batch_s* b, const void* const* params, const void* 
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   cudaStreamIsCapturing(s, &cs);
   if (b->have_prev && cs == cudaStreamCaptureStatusNone) cudaEventSynchronize(b->copied);
-  const double target = total_cost / (4.0 * b->grid);  // about four items of equal cost per CTA
+  const double target = total_cost / (3.0 * b->grid);  // about three items of equal cost per CTA
   std::vector<std::pair<double, int>> cost;  // (cost, item) for ordering
   std::vector<int> item_inst;
   int chunk_base = 0;
@@ -904,10 +907,11 @@ jet_status jet_batch_create(jet_batch_t* out, int32_t n, const jet_plan_t* plans
     delete b;
     return e != cudaSuccess ? cuda_fail(e, "batch occupancy") : fail(JET_ERR_UNSUPPORTED, "batch tile does not fit");
   }
-  b->grid = prop.multiProcessorCount * std::min(per_sm, 2);
-  // the work list holds about four items per CTA, shared by cost: a member may
-  // take twice its share (with 16 members a fixed 16 chunks left the largest
-  // member's chunks running alone: 26.4 ms against 5.0 ms)
+  b->ctas_per_sm = std::min(per_sm, 2);
+  b->grid = prop.multiProcessorCount * b->ctas_per_sm;
+  // the work list holds about three items per CTA, shared by cost: a member may
+  // take several times its share (with 16 members a fixed 16 chunks left the largest
+  // member's chunks running alone: 26.4 ms against 4.0 ms)
   b->max_chunks_per_inst = std::min(256, std::max(16, 8 * b->grid / n));
   long long scr = 0, slices = 0, wt = 0;
   for (int i = 0; i < n; ++i) {
@@ -961,6 +965,7 @@ static jet_status batch_run(jet_batch_t b, const void* const* params, void* cons
   a.item_next = b->d_next;
   a.ru = b->ru;
   a.threads = kSimtThreads;
+  a.carveout = simt_carveout(b->smem, b->ctas_per_sm);
   CK(cudaMemsetAsync(b->d_next, 0, sizeof(int), s));
   CK(simt_launch(b->cls, b->fp64, a, std::min(b->grid, n_items), b->smem, s));
   long long maxp = 0;

@@ -44,7 +44,7 @@ enum : int {
 };
 
 // Everything a kernel needs to know about one PINN instance for one call.
-struct DevInstance {
+struct alignas(16) DevInstance {
   int L;               // weight layers
   int d, n_out, n_res;
   int widths[kMaxLayers + 1];
@@ -94,6 +94,7 @@ struct SimtArgs {
   int n_items;                // total work items (instance, chunk)
   int ru;                     // units per thread of the jet GEMMs (simt_units)
   int threads;                // CTA size
+  int carveout;               // percent of the SM's 228 KB kept as shared memory (simt_carveout)
   const int* item_inst;       // [n_items] instance of each item (batched) or null
   void* scratch;              // per-CTA z-jet scratch
   long long scratch_stride;   // elements per CTA slot
@@ -105,12 +106,12 @@ struct SimtArgs {
 
 constexpr int kSimtThreads = 256;  // CTA of the no-alloc path and of batches
 constexpr int kSimtRed = 128;      // doubles of the SIMT kernels' reduction area
-// Weights of a jet GEMM pass through shared memory in two row slabs of at most
-// this many bytes (a 64 x 64 FP32 layer takes two, a 256 x 256 one 32); larger
-// slabs would cost tile points at width 256.
-constexpr int kSimtSlabBytes = 8192;
+// Weights of a jet GEMM pass through shared memory in two row slabs: 4 KB each
+// up to width 64 (a 64 x 64 FP32 layer takes four), where two CTAs of 32 points
+// then fit an SM with six channels; 8 KB up to width 128; 16 KB above (a 256 x
+// 256 layer takes 16; with 8 KB its barriers cost 4%).
 __host__ __device__ inline int simt_slab_elems(int wmax, size_t elem) {
-  const int cap = kSimtSlabBytes / (int)elem, need = wmax * wmax;
+  const int cap = (wmax <= 64 ? 4096 : wmax <= 128 ? 8192 : 16384) / (int)elem, need = wmax * wmax;
   return need < cap ? need : cap;
 }
 // Adjacent lanes that share a weight-gradient item (wr rows x 4 columns), each
@@ -132,9 +133,11 @@ inline int simt_pitch(int C, int P, int wmax, int wr, int threads, size_t elem) 
   while ((p / v) % (2 * ns) != ns % (2 * ns)) p += v;
   return p;
 }
-// consecutive units per thread of the SIMT jet GEMMs
+// Consecutive units per thread of the SIMT jet GEMMs.  FP64 takes one: its pipe
+// costs a warp the same however many lanes work, and single units fill the
+// warps of narrow layers (20 units x 8 points: 5 warps of 5, not 2.5 of 3).
 inline int simt_units(const int* widths, int L, bool fp64) {
-  if (fp64) return 2;
+  if (fp64) return 1;
   for (int l = 1; l < L; ++l)
     if (widths[l] % 8) return 4;
   return 8;
@@ -163,6 +166,17 @@ inline size_t simt_smem_bytes(int C, int P, int pitch, int wmax, int n_out, int 
              (size_t)P * d;
   size_t bytes = (e * elem + 15) / 16 * 16;
   return bytes + kSimtRed * sizeof(double);
+}
+// shared memory an SM spends on a CTA besides the dynamic part: the kernel's
+// static arrays (the instance descriptor and the item index) and the reserve
+constexpr size_t kSimtSmBytes = 228 * 1024;
+constexpr size_t kSimtCtaBytes = sizeof(DevInstance) + 16 + 1024;
+// Carve-out that holds `ctas` resident CTAs; the rest of the SM's 256 KB stays
+// L1 (2->64x6->1 composite loss at 12101 points: 364 us with all of it shared
+// memory, 306 us with what two CTAs need).
+inline int simt_carveout(size_t smem, int ctas) {
+  const size_t pct = ((smem + kSimtCtaBytes) * ctas * 100 + kSimtSmBytes - 1) / kSimtSmBytes;
+  return pct > 100 ? 100 : (int)pct;
 }
 // the chunks of a call: n_tiles tiles over n_chunks CTAs or work items
 inline void simt_set_chunks(DevInstance& I, long long n_chunks) {

@@ -265,6 +265,7 @@ extern "C" jet_status jet_backward_params_noalloc(const jet_residual_spec* spec,
   a.n_items = I.n_chunks;
   a.ru = ru;
   a.threads = kSimtThreads;
+  a.carveout = simt_carveout(smem, per_sm < 2 ? per_sm : 2);
   a.scratch = scr;
   a.scratch_stride = jet_elems;
   e = launch_by_class(best, fp64, a, I.n_chunks, smem, s);

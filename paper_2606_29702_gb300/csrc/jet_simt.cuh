@@ -32,8 +32,8 @@
 // (about 80% of the time), the FP64 pipe in the FP64 form.  Against the form
 // with three jet buffers, 4 units per thread, weights read through L1, one
 // lane per weight-gradient item and tiles that did not depend on N:
-// 3->256x8->1 FP32 at N = 16385 19.29 -> 12.79 ms, 2->64x5->1 (C = 6) FP32 at
-// 65536 1.769 -> 1.637 ms, 2->20x4->1 FP64 at 1000 342 -> 105 us.
+// 3->256x8->1 FP32 at N = 16385 19.29 -> 9.86 ms, 2->64x5->1 (C = 6) FP32 at
+// 65536 1.769 -> 1.237 ms, 2->20x4->1 FP64 at 1000 347 -> 84 us.
 #pragma once
 
 #include <type_traits>
@@ -154,6 +154,40 @@ __device__ __forceinline__ void red_add_v4(float* p, float a, float b, float c, 
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
+// The FP32 weight-gradient accumulator of a chunk, [item][WR][4] per layer as
+// the items of SimtTile::wgrad (functions of their own, called once per chunk:
+// inlined they would cost the tile's registers)
+static __device__ __noinline__ void simt_wacc_zero(float* acc, const DevInstance& I) {
+  long long n4 = 0;
+  for (int l = 2; l < I.L; ++l) n4 += (long long)I.widths[l] * I.widths[l - 1] / 4;
+  for (long long i = threadIdx.x; i < n4; i += blockDim.x)
+    reinterpret_cast<float4*>(acc)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+// accumulator -> FP64 slice (consecutive threads read consecutive floats;
+// eight loads in flight before their adds)
+template <int WR>
+static __device__ __noinline__ void simt_wacc_flush(const float* a, const DevInstance& I, double* g) {
+  const int NT = blockDim.x;
+  for (int l = 2; l <= I.L - 1; ++l) {
+    const int wo = I.widths[l], wi = I.widths[l - 1], nkb = wi / 4, n = wo * wi;
+    double* gW = g + I.off_W[l - 1];
+    for (int e0 = threadIdx.x; e0 < n; e0 += 8 * NT) {
+      float v[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = e0 + j * NT < n ? __ldcg(a + e0 + j * NT) : 0.f;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int e = e0 + j * NT;
+        if (e >= n) break;
+        const int it = e / (4 * WR), r = (e >> 2) % WR, s = e & 3;
+        const int kb = it % nkb, ub = it / nkb;
+        atomicAdd(gW + (ub * WR + r) * wi + kb + s * nkb, widen(v[j]));
+      }
+    }
+    a += n;
+  }
+}
+
 template <class Cls, class T, int RU_>
 struct SimtTile {
   static constexpr int C = Cls::C;
@@ -162,12 +196,16 @@ struct SimtTile {
   static constexpr bool F32 = sizeof(T) == 4;
   static constexpr int RU = RU_;  // consecutive units per thread of the jet GEMMs
   static constexpr int EU = TP;   // consecutive units per thread of the elementwise phases
+  // k steps of the jet GEMMs unrolled together: two where the sums and four
+  // steps' operands would exceed the registers (C = 7 at 512 threads: 12.8 ms
+  // with four, 11.8 ms with two), else four
+  static constexpr int UK = C >= 7 ? 2 : 4;
   static constexpr int WR = F32 && RU == 8 ? 8 : 4;  // weight-gradient rows per thread (times 4 columns)
 
   const DevInstance& I;
   const SimtArgs& A;
   const int NT;  // threads of the CTA
-  T* B[2];   // jet buffers [wmax][pitch]
+  T *B0, *B1;  // jet buffers [wmax][pitch]
   T* WS;     // two weight slabs
   T* UO;     // output jets [n_out*C][P]
   T* UB;     // output adjoints [n_out*C][P]
@@ -194,8 +232,8 @@ struct SimtTile {
     slab = simt_slab_elems(wmax, sizeof(T));
     T* base = reinterpret_cast<T*>(smem);
     const size_t be = (size_t)wmax * pitch;
-    B[0] = base;
-    B[1] = base + be;
+    B0 = base;
+    B1 = base + be;
     WS = base + 2 * be;
     UO = WS + 2 * slab;
     UB = UO + (size_t)I.n_out * C * P;
@@ -216,33 +254,8 @@ struct SimtTile {
     for (int k = 2; k < l; ++k) off += (long long)I.widths[k] * I.widths[k - 1];
     return wacc_base + off;
   }
-  __device__ __noinline__ void wacc_zero() {
-    float4* a = reinterpret_cast<float4*>(wacc_base);
-    const long long n4 = (wacc(I.L) - wacc_base) / 4;
-    for (long long i = threadIdx.x; i < n4; i += NT) a[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-  // accumulator -> FP64 slice (consecutive threads read consecutive floats;
-  // eight loads in flight before their adds)
-  __device__ __noinline__ void wacc_flush(double* g) {
-    for (int l = 2; l <= I.L - 1; ++l) {
-      const int wo = I.widths[l], wi = I.widths[l - 1], nkb = wi / 4, n = wo * wi;
-      const float* a = wacc(l);
-      double* gW = g + I.off_W[l - 1];
-      for (int e0 = threadIdx.x; e0 < n; e0 += 8 * NT) {
-        float v[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = e0 + j * NT < n ? __ldcg(a + e0 + j * NT) : 0.f;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int e = e0 + j * NT;
-          if (e >= n) break;
-          const int it = e / (4 * WR), r = (e >> 2) % WR, s = e & 3;
-          const int kb = it % nkb, ub = it / nkb;
-          atomicAdd(gW + (ub * WR + r) * wi + kb + s * nkb, widen(v[j]));
-        }
-      }
-    }
-  }
+  __device__ void wacc_zero() { simt_wacc_zero(wacc_base, I); }
+  __device__ void wacc_flush(double* g) { simt_wacc_flush<WR>(wacc_base, I, g); }
 
   __device__ const T* W(int l) const { return params + I.off_W[l - 1]; }   // l = 1..L
   __device__ const T* bias(int l) const { return params + I.off_b[l - 1]; }
@@ -311,11 +324,16 @@ struct SimtTile {
         wst ^= 1;
         if (!act) continue;
         const int kn = min(rps, w.K - k0);
-#pragma unroll 4
+#pragma unroll(UK)
         for (int k = 0; k < kn; ++k, ap += pitch, wp += w.wo) {
           T wv[RU], av[C];
+          if constexpr (RU % TP == 0) {
 #pragma unroll
-          for (int r = 0; r < RU; r += TP) vload<T>(wp + r, wv + r);
+            for (int r = 0; r < RU; r += TP) vload<T>(wp + r, wv + r);
+          } else {
+#pragma unroll
+            for (int r = 0; r < RU; ++r) wv[r] = wp[r];
+          }
           load_chan<T, C>(ap, av);
           if constexpr (F32) {
 #pragma unroll
@@ -512,21 +530,30 @@ struct SimtTile {
       __syncthreads();
       for (int n = threadIdx.x; n < nvalid; n += NT) {
         T r[kMaxRes];
-        for (int c = 0; c < I.n_res; ++c) r[c] = src ? -src[(n0 + n) * I.n_res + c] : T(0);
+#pragma unroll
+        for (int c = 0; c < kMaxRes; ++c) r[c] = c < I.n_res && src ? -src[(n0 + n) * I.n_res + c] : T(0);
         for (int m = 0; m < nt; ++m) {
           const DevTerm& tm = I.terms[m];
           T prod = T(tm.coef);
           for (int f = 0; f < tm.nfac; ++f) prod *= UO[tm.fac[f] * P + n];
-          r[tm.comp] += prod;
+#pragma unroll
+          for (int c = 0; c < kMaxRes; ++c)
+            if (c == tm.comp) r[c] += prod;
         }
-        for (int c = 0; c < I.n_res; ++c) {
+#pragma unroll
+        for (int c = 0; c < kMaxRes; ++c) {
+          if (c >= I.n_res) break;
           if (rout) rout[(n0 + n) * I.n_res + c] = r[c];
           loss += (double)r[c] * (double)r[c];
         }
         if (bwd)
           for (int m = 0; m < nt; ++m) {
             const DevTerm& tm = I.terms[m];
-            const T g = two_over_n * r[tm.comp] * T(tm.coef);
+            T rc = T(0);
+#pragma unroll
+            for (int c = 0; c < kMaxRes; ++c)
+              if (c == tm.comp) rc = r[c];
+            const T g = two_over_n * rc * T(tm.coef);
             for (int f = 0; f < tm.nfac; ++f) {
               T prod = g;
               for (int h = 0; h < tm.nfac; ++h)
@@ -549,9 +576,18 @@ struct SimtTile {
     __syncthreads();
     for (int n = threadIdx.x; n < nvalid; n += NT) {
       T r[kMaxRes];
-      for (int c = 0; c < I.n_res; ++c) r[c] = src ? -src[(n0 + n) * I.n_res + c] : T(0);
-      for (int m = 0; m < nt; ++m) r[I.terms[m].comp] += prodm[m * P + n];
-      for (int c = 0; c < I.n_res; ++c) {
+#pragma unroll
+      for (int c = 0; c < kMaxRes; ++c) r[c] = c < I.n_res && src ? -src[(n0 + n) * I.n_res + c] : T(0);
+      for (int m = 0; m < nt; ++m) {
+        const int cm = I.terms[m].comp;
+        const T v = prodm[m * P + n];
+#pragma unroll
+        for (int c = 0; c < kMaxRes; ++c)
+          if (c == cm) r[c] += v;
+      }
+#pragma unroll
+      for (int c = 0; c < kMaxRes; ++c) {
+        if (c >= I.n_res) break;
         if (rout) rout[(n0 + n) * I.n_res + c] = r[c];
         loss += (double)r[c] * (double)r[c];
         rg[c * P + n] = two_over_n * r[c];
@@ -707,18 +743,25 @@ struct SimtTile {
 #pragma unroll
           for (int s = 0; s < 4; ++s) ap2[r][s] = f2(0.f);
         for (int col = c0; col < ncol; col += NS * TP) {
-          T zv[WR][TP], av[4][TP];
+          T av[4][TP];
 #pragma unroll
           for (int s = 0; s < 4; ++s) vload<T>(app + s * nkb * pitch + col, av[s]);
+          // four rows' operands at a time: all eight beside 32 packed sums
+          // would spill
 #pragma unroll
-          for (int r = 0; r < WR; ++r) vload<T>(zp + r * pitch + col, zv[r]);
+          for (int r0 = 0; r0 < WR; r0 += 4) {
+            T zv[4][TP];
 #pragma unroll
-          for (int r = 0; r < WR; ++r)
+            for (int r = 0; r < 4; ++r) vload<T>(zp + (r0 + r) * pitch + col, zv[r]);
 #pragma unroll
-            for (int s = 0; s < 4; ++s)
+            for (int r = 0; r < 4; ++r)
 #pragma unroll
-              for (int j = 0; j < TP; j += 2)
-                ap2[r][s] = jfma(f2(zv[r][j], zv[r][j + 1]), f2(av[s][j], av[s][j + 1]), ap2[r][s]);
+              for (int s = 0; s < 4; ++s)
+#pragma unroll
+                for (int j = 0; j < TP; j += 2)
+                  ap2[r0 + r][s] = jfma(f2(zv[r][j], zv[r][j + 1]), f2(av[s][j], av[s][j + 1]), ap2[r0 + r][s]);
+            if (r0 + 4 < WR) asm volatile("" ::: "memory");
+          }
         }
 #pragma unroll
         for (int r = 0; r < WR; ++r)
@@ -873,25 +916,26 @@ struct SimtTile {
     const bool bwd = mode != MODE_FWD;
     const int L = I.L;
     const Rows none{nullptr, 0, 0}, first = more ? first_rows() : none;
-    int cur = 0;
+    T *y = B0, *x = B1;  // y: the newest layer's jets
     if (mode != MODE_BWD_STORE) {
-      layer1(B[0], write_z ? zjet(t, 1, use_store) : nullptr);
+      layer1(y, write_z ? zjet(t, 1, use_store) : nullptr);
       for (int l = 2; l <= L - 1; ++l) {
         const Rows next = l < L - 1 ? fwd_rows(l + 1) : bwd ? bwd_rows(l) : first;
-        hidden_fwd(l, B[cur], B[cur ^ 1], write_z ? zjet(t, l, use_store) : nullptr, next);
-        cur ^= 1;
+        hidden_fwd(l, y, x, write_z ? zjet(t, l, use_store) : nullptr, next);
+        T* tmp = x;
+        x = y;
+        y = tmp;
       }
     } else {
-      compose_from(L - 1, zjet(t, L - 1, true), B[0]);
+      compose_from(L - 1, zjet(t, L - 1, true), y);
     }
     __syncthreads();
-    output_layer(B[cur]);
+    output_layer(y);
     __syncthreads();
     double loss = residual(n0, nvalid, bwd);
     __syncthreads();
     if (!bwd) return loss;
     // x: Abar^l, then Zbar^l in place; y: A^{l-1}, then Abar^{l-1}
-    T *x = B[cur ^ 1], *y = B[cur];
     output_bwd(y, x, g);
     __syncthreads();
     const bool from_store = mode == MODE_BWD_STORE;
@@ -920,18 +964,26 @@ template <class Cls, class T, int RU>
 __device__ __forceinline__ void simt_body(const SimtArgs& args) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int k_s;
+  // the running item's descriptor: read in every phase, through shared memory
+  // rather than a pointer that may be param or global space, which cost
+  // registers that spilled (2->64x5->1, C = 6: 1.32 ms with it, 1.24 ms without)
+  __shared__ DevInstance inst_s;
   const int NT = blockDim.x;
   for (int k = blockIdx.x; k < args.n_items;) {
     // batched launches walk a cost-ordered list: position k -> item id, and
     // item id -> instance (second half of item_inst)
     const int item = args.item_inst ? args.item_inst[k] : k;
-    const DevInstance& I = args.insts ? args.insts[args.item_inst[args.n_items + item]] : args.inst0;
+    const DevInstance* src = args.insts ? args.insts + args.item_inst[args.n_items + item] : &args.inst0;
+    for (int i = threadIdx.x; i < (int)(sizeof(DevInstance) / 16); i += NT)
+      reinterpret_cast<uint4*>(&inst_s)[i] = reinterpret_cast<const uint4*>(src)[i];
+    __syncthreads();
+    const DevInstance& I = inst_s;
     const int chunk = item - I.chunk_base;
     SimtTile<Cls, T, RU> S(I, args, smem);
     // columns past C * P are never written: zero them (and everything else)
     // once per item so that the weight-gradient sums over whole vectors see
     // zeros there
-    for (int i = threadIdx.x; i < 2 * S.wmax * S.pitch; i += NT) S.B[0][i] = T(0);
+    for (int i = threadIdx.x; i < 2 * S.wmax * S.pitch; i += NT) S.B0[i] = T(0);
     const auto first = S.first_rows();
     if (first.p) S.issue(first, 0, 0);
     const bool bwd = args.mode != MODE_FWD;
@@ -1014,10 +1066,10 @@ __global__ void __launch_bounds__(simt_max_threads<Cls, T>(), 1) simt_kernel(con
 }
 
 // the kernel for ru units per thread of the jet GEMMs: FP32 8 (every hidden
-// width a multiple of 8) or 4, FP64 2
+// width a multiple of 8) or 4, FP64 1
 template <class Cls, class T>
 constexpr auto simt_entry(int ru) {
-  if constexpr (sizeof(T) == 8) return &simt_kernel<Cls, T, 2>;
+  if constexpr (sizeof(T) == 8) return &simt_kernel<Cls, T, 1>;
   else return ru == 8 ? &simt_kernel<Cls, T, 8> : &simt_kernel<Cls, T, 4>;
 }
 

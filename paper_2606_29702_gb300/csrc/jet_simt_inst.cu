@@ -10,51 +10,37 @@ namespace jet {
 
 using ThisCls = ClassById<JET_CLASS_ID>::type;
 
-namespace {
-// Dynamic shared memory and an L1/shared split that holds just the CTAs the
-// kernel can keep resident (the rest of the SM's 256 KB stays L1, which
-// serves the per-k weight vectors of the jet GEMMs).
-template <class K>
-cudaError_t prepare(K kernel, int threads, size_t smem) {
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int blocks = 0, dev = 0, smem_sm = 0, reserved = 0;
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kernel, threads, smem);
-  if (e == cudaSuccess) e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-  if (e != cudaSuccess || blocks < 1 || smem_sm < 1) return e;
+// Called when a plan, a batch or the no-alloc path sizes its tile.  The kernel
+// may take all the shared memory the device gives a block, and the query runs
+// with the whole SM's as the preferred carve-out: one left by an earlier launch
+// with a smaller tile would halve the residency it reports.
+template <>
+cudaError_t simt_max_active_id<JET_CLASS_ID>(bool fp64, int ru, int threads, size_t smem, int* blocks) {
+  const auto kernel = fp64 ? simt_entry<ThisCls, double>(ru) : simt_entry<ThisCls, float>(ru);
+  *blocks = 0;
   cudaFuncAttributes fa;
-  e = cudaFuncGetAttributes(&fa, kernel);
+  int dev = 0, most = 0;
+  cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
-  const size_t need = (size_t)blocks * (smem + fa.sharedSizeBytes + (size_t)reserved);
-  int pct = (int)((need * 100 + (size_t)smem_sm - 1) / (size_t)smem_sm);
-  if (pct > 100) pct = 100;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
+  most -= (int)fa.sharedSizeBytes;
+  if (smem > (size_t)most) return cudaErrorInvalidValue;
+  if (threads > fa.maxThreadsPerBlock) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, kernel, threads, smem);
+  return e;
 }
-}  // namespace
 
 template <>
 cudaError_t simt_launch_id<JET_CLASS_ID>(bool fp64, const SimtArgs& a, int grid, size_t smem, cudaStream_t s) {
   const auto kernel = fp64 ? simt_entry<ThisCls, double>(a.ru) : simt_entry<ThisCls, float>(a.ru);
-  cudaError_t e = prepare(kernel, a.threads, smem);
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, a.carveout);
   if (e != cudaSuccess) return e;
   kernel<<<grid, a.threads, smem, s>>>(a);
   return cudaGetLastError();
-}
-
-template <>
-cudaError_t simt_max_active_id<JET_CLASS_ID>(bool fp64, int ru, int threads, size_t smem, int* blocks) {
-  const auto kernel = fp64 ? simt_entry<ThisCls, double>(ru) : simt_entry<ThisCls, float>(ru);
-  cudaFuncAttributes fa;
-  cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
-  if (e != cudaSuccess) return e;
-  if (threads > fa.maxThreadsPerBlock) {
-    *blocks = 0;
-    return cudaSuccess;
-  }
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, kernel, threads, smem);
 }
 
 template <>
