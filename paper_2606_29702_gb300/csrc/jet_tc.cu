@@ -1099,6 +1099,7 @@ jet_status tc_batch_create(const std::vector<jet_plan_s*>& plans, TcBatch** out)
   }
   memset(b->h_insts, 0, sizeof(TcInst) * b->n);
   memset(b->h_prep, 0, sizeof(PrepJob) * b->n);
+  memset(b->h_jobs, 0, sizeof(ReduceJob) * b->n);  // no job of an earlier batch in recycled pinned memory
   *out = b;
   return JET_OK;
 }
