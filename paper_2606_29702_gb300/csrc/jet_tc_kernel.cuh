@@ -260,6 +260,19 @@ struct TcTile {
     }
   }
 
+  // W^l of a 256-wide layer in two loads: part 0 (the first 128 input units)
+  // once the data gradient of the layer above has read that half of W^{l+1},
+  // part 1 once it has read the rest; bar_tma completes with both.  Half of the
+  // 128 KB arrives during the data gradient's second half (3->256x8->1 with the
+  // store, N = 1048576: 43.06 -> 42.58 ms); with the layer input ahead of part 1
+  // the gain was a fifth of that.
+  __device__ void load_hidden_w_half(int l, int part) {
+    const uint32_t box = 64u * rr() * 2u;
+    if (part == 0) tc::mbar_arrive_expect_tx(bar_tma, box * 4u);
+    for (int kc = 2 * part; kc < 2 * part + 2; ++kc)
+      tc::tma_load_3d(sm + I.o_w + kc * box, &Imap->wmap, bar_tma, kc * 64, 0, l - 2);
+  }
+
   __device__ void load_out_w() {  // W^L -> W buffer, 128-row boxes
     const int nck = (ww() + 63) / 64;
     const uint32_t box = 64u * 128u * 2u;
@@ -332,12 +345,12 @@ struct TcTile {
     }
   }
 
-  // D[R1] = W^l^T (MN-major A) x Zbar (MN-major B)
-  __device__ void mma_dgrad(int zi) {
+  // D[R1] = W^l^T (MN-major A) x Zbar (MN-major B), row halves [h0, h1)
+  __device__ void mma_dgrad(int zi, int h0 = 0, int h1 = 2) {
     const uint32_t sW = tc::smem_u32(sm + I.o_w), sZ = tc::smem_u32(ACT(zi));
     const uint32_t chunk = (uint32_t)(rr() / 8) * 1024u;
     const uint32_t id = tc::idesc_bf16(128, cpad(), 1, 1);
-    for (int h = 0; h < hh(); ++h)
+    for (int h = h0; h < (h1 < hh() ? h1 : hh()); ++h)
       for (int s = 0; s < ww() / 16; ++s) {
         const uint64_t ad = tc::sdesc(sW + (uint32_t)(2 * h) * chunk + (uint32_t)s * 2048u, chunk, 1024);
         const uint64_t bd = tc::sdesc(sZ + (uint32_t)s * 2048u, chunk, 1024);
@@ -1098,15 +1111,23 @@ struct TcTile {
           tc::bulk_s2g(zslot(l), ACT(zb), (uint32_t)I.act_bytes);
           tc::bulk_commit();
           ++nz;
-          mma_dgrad(zb);
+          mma_dgrad(zb, 0, ww() == 256 ? 1 : 2);
+          if (ww() == 256) {
+            tc::mma_commit(bar_wg);
+            mma_dgrad(zb, 1, 2);
+          }
           tc::mma_commit(bar_mma);
         }
         part_flush(0, g + I.off_b[l - 1], 1);  // bias gradient of layer l, during the MMA
         if (l == 2) w1b = row_l1(PRELOAD1B);
+        if (tid == 0 && ww() == 256 && wait(bar_wg, ph_wg, 68) && l > 2) load_hidden_w_half(l - 1, 0);
         if (!wait(bar_mma, ph_mma, 66)) break;
         tc::tc_fence_after();
         if (tid == 0) {
-          if (l > 2) load_hidden_w(l - 1);  // W^l is free: W^{l-1} loads while the copy reads
+          if (l > 2) {  // W^l is free: W^{l-1} loads while the copy reads
+            if (ww() == 256) load_hidden_w_half(l - 1, 1);
+            else load_hidden_w(l - 1);
+          }
           tc::bulk_wait_read0();  // ACT(zb) is rewritten by the reload or the next adjoint
           if (l > 2) reload_act(l - 1);
           // the layer input of the next reload, from HBM into L2 a layer ahead
