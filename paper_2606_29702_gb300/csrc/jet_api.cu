@@ -113,13 +113,11 @@ void free_plan_ws(jet_plan_s* p) {
     cudaEventDestroy(e.second);
   }
   p->prof.clear();
-  cudaFree(p->Wt);
-  cudaFree(p->grad_slices);
-  cudaFree(p->loss_slices);
-  cudaFree(p->scratch);
+  cudaFree(p->ws);
   cudaFree(p->store);
-  p->Wt = p->grad_slices = p->loss_slices = nullptr;
-  p->scratch = p->store = nullptr;
+  p->ws = p->Wt = p->scratch = p->store = nullptr;
+  p->grad_slices = p->loss_slices = nullptr;
+  p->wsums = nullptr;
   if (p->tcp) tc_plan_destroy(p->tcp);
   p->tcp = nullptr;
 }
@@ -397,23 +395,25 @@ static jet_status plan_create(jet_plan_t* out, int n_specs, const jet_residual_s
   long long jet_elems = 0;  // hidden z-jets of one tile
   for (int l = 1; l < n_layers; ++l) jet_elems += (long long)p->C * p->P * widths[l];
   if (!p->tc) {
-    // FP32 forms whose per-chunk FP64 slices would not stay in L2 add the
-    // hidden-layer weight gradients of a chunk in an FP32 accumulator and
-    // flush once per chunk; otherwise per-tile FP64 adds into L2-resident
-    // slices are the cheaper of the two
+    // FP32 forms whose per-chunk FP64 slices would not stay in L2 sum the
+    // hidden-layer weights of a chunk in FP32; otherwise per-tile FP64 adds into
+    // L2-resident slices are the cheaper of the two
     const bool slices_fit = (double)p->grid * p->n_params * sizeof(double) <= kSimtSliceL2Bytes;
-    const long long wacc = slices_fit ? 0 : simt_wacc_elems(widths, n_layers, p->fp64);
-    p->scratch_stride = jet_elems + wacc;
-    p->wacc_off = wacc ? jet_elems : -1;
+    p->wsums_stride = slices_fit ? 0 : simt_wacc_elems(widths, n_layers, p->fp64);
+    p->scratch_stride = jet_elems;
+    const size_t b_ws = (size_t)p->grid * p->wsums_stride * sizeof(float);
     size_t b_wt = (size_t)weight_ws_elems(p->n_params) * p->elem;
     size_t b_gs = (size_t)p->grid * p->n_params * sizeof(double);
     size_t b_ls = (size_t)p->grid * sizeof(double);
     size_t b_sc = (size_t)p->grid * p->scratch_stride * p->elem;
-    e = cudaMalloc(&p->Wt, b_wt);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&p->grad_slices, b_gs);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&p->loss_slices, b_ls);
-    if (e == cudaSuccess) e = cudaMalloc(&p->scratch, b_sc);
-    p->ws_bytes = b_wt + b_gs + b_ls + b_sc;
+    Arena arena;
+    arena.add(&p->Wt, b_wt);
+    arena.add(&p->grad_slices, b_gs);
+    arena.add(&p->loss_slices, b_ls);
+    arena.add(&p->scratch, b_sc);
+    arena.add(&p->wsums, b_ws);
+    e = arena.alloc(&p->ws);
+    p->ws_bytes = b_wt + b_gs + b_ls + b_sc + b_ws;
     if (e == cudaSuccess && (flags & JET_FLAG_STORE) && mem_budget_bytes > 0) {
       const size_t per_tile = (size_t)jet_elems * p->elem;
       long long tiles = (long long)(mem_budget_bytes / per_tile);
@@ -504,7 +504,7 @@ jet_status jet_plan_get_info(jet_plan_t p, jet_plan_info* info) {
   info->workspace_bytes = p->tc ? tc_workspace_bytes(p->tcp) : p->ws_bytes;
   info->ctas_per_sm = p->tc ? tc_ctas_per_sm(p->tcp) : p->ctas_per_sm;
   info->cta_threads = p->tc ? tc_threads(p->tcp) : p->threads;
-  info->wgrad_chunk_fp32 = p->tc ? tc_wgrad_chunk_fp32(p->tcp) : (p->wacc_off >= 0 ? 1 : 0);
+  info->wgrad_chunk_fp32 = p->tc ? tc_wgrad_chunk_fp32(p->tcp) : (p->wsums ? 1 : 0);
   return JET_OK;
 }
 
@@ -582,7 +582,7 @@ void fill_instance(const jet_plan_s* p, const void* params, const void* X, long 
   I.loss_slices = p->loss_slices;
   I.store = nullptr;
   for (int l = 1; l < p->L; ++l) I.store_tile_stride += (long long)p->C * P * p->widths[l];
-  I.wacc_off = p->wacc_off;
+  simt_set_sums(I, p->C, p->wsums, p->wsums_stride);
 }
 
 jet_status check_call(const jet_plan_s* p, const void* params, const void* X, long long N, const void* source) {
@@ -622,13 +622,24 @@ jet_status run_simt(jet_plan_s* p, int mode, const DevInstance& I, cudaStream_t 
   return JET_OK;
 }
 
-ReduceJob make_job(const DevInstance& I, void* grad_out, double* loss_out, bool with_grad) {
+ReduceJob make_job(const DevInstance& I, int ru, void* grad_out, double* loss_out, bool with_grad) {
   ReduceJob j;
   memset(&j, 0, sizeof(j));
   j.grad_slices = I.grad_slices;
   j.loss_slices = I.loss_slices;
   j.n_chunks = I.n_chunks;
+  j.n_slice = I.n_slice;
   j.n_params = with_grad ? I.n_params : 0;
+  if (with_grad && I.wsums && I.wsums_direct) {
+    j.hid = HID_SIMT;
+    j.L = I.L;
+    for (int l = 0; l <= I.L; ++l) j.widths[l] = I.widths[l];
+    j.n_hid = (int)I.wsums_stride;
+    j.subs = 1;
+    j.wr = simt_wgrad_rows(ru);
+    j.hid_sums = I.wsums;
+    j.hid_stride = I.wsums_stride;
+  }
   j.inv_N = I.inv_N;
   j.grad_out = grad_out;
   j.loss_out = loss_out;
@@ -656,8 +667,8 @@ jet_status jet_forward_residual(jet_plan_t p, const void* params, const void* X,
   CK(launch_transpose_weights(I, p->fp64, p->Wt, s));
   st = run_simt(p, MODE_FWD, I, s);
   if (st != JET_OK) return st;
-  ReduceJob j = make_job(I, nullptr, loss_out, false);
-  if (loss_out) CK(launch_reduce(nullptr, j, 1, 1, p->fp64, false, 1, 0.f, s));
+  ReduceJob j = make_job(I, p->ru, nullptr, loss_out, false);
+  if (loss_out) CK(launch_reduce(&j, nullptr, 1, p->fp64, false, 1, 0.f, s));
   p->st_valid = store;
   p->st_params = params;
   p->st_X = X;
@@ -686,8 +697,8 @@ jet_status jet_backward_params(jet_plan_t p, const void* params, const void* X, 
   CK(launch_transpose_weights(I, p->fp64, p->Wt, s));
   st = run_simt(p, from_store ? MODE_BWD_STORE : MODE_FWD_BWD, I, s);
   if (st != JET_OK) return st;
-  ReduceJob j = make_job(I, grad_out, loss_out, true);
-  CK(launch_reduce(nullptr, j, 1, I.n_params, p->fp64, false, 1, 0.f, s));
+  ReduceJob j = make_job(I, p->ru, grad_out, loss_out, true);
+  CK(launch_reduce(&j, nullptr, 1, p->fp64, false, 1, 0.f, s));
   return JET_OK;
 }
 
@@ -708,11 +719,11 @@ static jet_status train_step(jet_plan_t p, void* params, void* adam_m, void* ada
   CK(launch_transpose_weights(I, p->fp64, p->Wt, s));
   st = run_simt(p, MODE_FWD_BWD, I, s);
   if (st != JET_OK) return st;
-  ReduceJob j = make_job(I, nullptr, loss_out, true);
+  ReduceJob j = make_job(I, p->ru, nullptr, loss_out, true);
   j.params = params;
   j.m = adam_m;
   j.v = adam_v;
-  CK(launch_reduce(nullptr, j, 1, I.n_params, p->fp64, true, step, lr, s, step_ctr));
+  CK(launch_reduce(&j, nullptr, 1, p->fp64, true, step, lr, s, step_ctr));
   return JET_OK;
 }
 
@@ -764,7 +775,8 @@ struct jet_batch_s {
   void* Wt = nullptr;
   void* scratch = nullptr;
   long long scratch_stride = 0;
-  std::vector<long long> slice_off, wt_off;
+  float* wsums = nullptr;  // FP32 weight-gradient sums per chunk of the members that keep them
+  std::vector<long long> slice_off, wt_off, wsums_off;
   // pinned host staging for the per-call descriptors
   DevInstance* h_insts = nullptr;
   int* h_item_inst = nullptr;
@@ -788,6 +800,7 @@ void free_batch(jet_batch_s* b) {
   cudaFree(b->loss_slices);
   cudaFree(b->Wt);
   cudaFree(b->scratch);
+  cudaFree(b->wsums);
   cudaFreeHost(b->h_insts);
   cudaFreeHost(b->h_item_inst);
   cudaFreeHost(b->h_jobs);
@@ -831,6 +844,7 @@ jet_status batch_prepare(jet_batch_s* b, const void* const* params, const void* 
                   kSimtThreads, (int)want, I);
     I.Wt = (char*)b->Wt + b->wt_off[i] * p->elem;
     I.grad_slices = b->grad_slices + b->slice_off[i];
+    simt_set_sums(I, p->C, p->wsums ? b->wsums + b->wsums_off[i] : nullptr, p->wsums_stride);
     I.loss_slices = b->loss_slices + (long long)i * b->max_chunks_per_inst;
     I.chunk_base = chunk_base;
     for (int c = 0; c < I.n_chunks; ++c) {
@@ -913,9 +927,11 @@ jet_status jet_batch_create(jet_batch_t* out, int32_t n, const jet_plan_t* plans
   // take several times its share (with 16 members a fixed 16 chunks left the largest
   // member's chunks running alone: 26.4 ms against 4.0 ms)
   b->max_chunks_per_inst = std::min(256, std::max(16, 8 * b->grid / n));
-  long long scr = 0, slices = 0, wt = 0;
+  long long scr = 0, slices = 0, wt = 0, sums = 0;
   for (int i = 0; i < n; ++i) {
     scr = std::max(scr, plans[i]->scratch_stride);
+    b->wsums_off.push_back(sums);
+    sums += (long long)b->max_chunks_per_inst * plans[i]->wsums_stride;
     b->slice_off.push_back(slices);
     slices += (long long)b->max_chunks_per_inst * plans[i]->n_params;
     b->wt_off.push_back(wt);
@@ -930,6 +946,7 @@ jet_status jet_batch_create(jet_batch_t* out, int32_t n, const jet_plan_t* plans
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_jobs, sizeof(ReduceJob) * n);
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->grad_slices, sizeof(double) * std::max<long long>(slices, 1));
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->loss_slices, sizeof(double) * b->max_items);
+  if (e == cudaSuccess && sums) e = cudaMalloc((void**)&b->wsums, sizeof(float) * sums);
   if (e == cudaSuccess) e = cudaMalloc(&b->Wt, elem * std::max<long long>(wt, 1));
   if (e == cudaSuccess) e = cudaMalloc(&b->scratch, elem * (size_t)b->grid * std::max<long long>(scr, 1));
   if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_insts, sizeof(DevInstance) * n);
@@ -968,16 +985,14 @@ static jet_status batch_run(jet_batch_t b, const void* const* params, void* cons
   a.carveout = simt_carveout(b->smem, b->ctas_per_sm);
   CK(cudaMemsetAsync(b->d_next, 0, sizeof(int), s));
   CK(simt_launch(b->cls, b->fp64, a, std::min(b->grid, n_items), b->smem, s));
-  long long maxp = 0;
   for (int i = 0; i < n; ++i) {
-    ReduceJob j = make_job(b->h_insts[i], adam ? nullptr : grad_out[i], loss_out ? loss_out + i : nullptr, true);
+    ReduceJob j = make_job(b->h_insts[i], b->ru, adam ? nullptr : grad_out[i], loss_out ? loss_out + i : nullptr, true);
     if (adam) {
       j.params = (void*)params[i];
       j.m = adam_m[i];
       j.v = adam_v[i];
     }
     b->h_jobs[i] = j;
-    maxp = std::max(maxp, j.n_params);
   }
   CK(cudaMemcpyAsync(b->d_jobs, b->h_jobs, sizeof(ReduceJob) * n, cudaMemcpyHostToDevice, s));
   if (!b->copied) CK(cudaEventCreateWithFlags(&b->copied, cudaEventDisableTiming));
@@ -987,7 +1002,7 @@ static jet_status batch_run(jet_batch_t b, const void* const* params, void* cons
     CK(cudaEventRecord(b->copied, s));
     b->have_prev = true;
   }
-  CK(launch_reduce(b->d_jobs, b->h_jobs[0], n, maxp, b->fp64, adam, step, lr, s, step_ctr));
+  CK(launch_reduce(b->h_jobs, b->d_jobs, n, b->fp64, adam, step, lr, s, step_ctr));
   return JET_OK;
 }
 

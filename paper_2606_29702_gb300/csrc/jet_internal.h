@@ -73,17 +73,40 @@ struct alignas(16) DevInstance {
   int chunk_rem;
   int n_chunks;
   int chunk_base;      // first work-item index of this instance
-  // outputs of the chunk reduction (FP64): [n_chunks][n_params], [n_chunks]
+  // outputs of the chunk reduction (FP64): [n_chunks][n_slice], [n_chunks].
+  // A slice holds every parameter (n_slice = n_params), or, with FP32 chunk sums
+  // of the hidden-layer weights (wsums_direct), the others only (SliceMap)
   double* grad_slices;
   double* loss_slices;
+  int n_slice;
+  int goff_b[kMaxLayers];  // offsets of b^l and W^L in a slice (W^1 is first)
+  int goff_WL;
   // z-jet store for MODE_FWD / MODE_BWD_STORE: per tile, per hidden layer,
   // [w][C * P] (as the shared-memory rows); null if not stored
   void* store;
   long long store_tile_stride;  // elements per tile
-  // FP32 forms: element offset, in a CTA's scratch slot, of the chunk's FP32
-  // weight-gradient accumulator (simt_wacc_elems); -1: FP64 adds per tile
-  long long wacc_off;
+  // FP32 forms: FP32 sums of the hidden-layer weight gradients of each chunk
+  // (simt_wacc_elems floats, in the item order of the weight gradient), or null:
+  // FP64 adds per tile.  wsums_direct: the reduction reads them; else the chunk
+  // adds them to its slice after every kWaccTiles tiles
+  float* wsums;
+  long long wsums_stride;
+  int wsums_direct;
 };
+
+// Layout of an FP64 slice without the hidden-layer weights: W^1, b^1, b^2 ..
+// b^{L-1}, W^L, b^L.  Fills the offsets and returns the slice's elements.
+inline int slice_map(const int* widths, int L, int* goff_b, int* goff_WL) {
+  int n = widths[0] * widths[1];
+  for (int l = 1; l < L; ++l) {
+    goff_b[l - 1] = n;
+    n += widths[l];
+  }
+  *goff_WL = n;
+  n += widths[L - 1] * widths[L];
+  goff_b[L - 1] = n;
+  return n + widths[L];
+}
 
 // Per-launch arguments of the fused SIMT kernel.
 struct SimtArgs {
@@ -143,12 +166,12 @@ inline int simt_units(const int* widths, int L, bool fp64) {
   return 8;
 }
 inline int simt_wgrad_rows(int ru) { return ru == 8 ? 8 : 4; }
+constexpr int kWaccTiles = 64;     // tiles per FP32 weight-gradient run (channel sets of 7 or more)
 // share of L2 the per-chunk FP64 gradient slices may take before the kernels
 // accumulate a chunk's weight gradients in FP32 instead of adding per tile
 constexpr double kSimtSliceL2Bytes = 48.0 * 1024 * 1024;
-// FP32 forms: elements of the per-CTA weight-gradient accumulator that
-// follows a tile's z-jets in the CTA's scratch slot, one float per weight of
-// every hidden-to-hidden layer W^l (l = 2 .. L-1, [w_l][w_{l-1}])
+// FP32 forms: elements of a chunk's FP32 weight-gradient sums, one float per
+// weight of every hidden-to-hidden layer W^l (l = 2 .. L-1, [w_l][w_{l-1}])
 inline long long simt_wacc_elems(const int* widths, int L, bool fp64) {
   if (fp64) return 0;
   long long e = 0;
@@ -186,16 +209,46 @@ inline void simt_set_chunks(DevInstance& I, long long n_chunks) {
   I.tiles_per_chunk = (int)(I.n_tiles / n_chunks);
   I.chunk_rem = (int)(I.n_tiles % n_chunks);
 }
+// Where a call's weight-gradient sums go (after simt_set_chunks).  With FP32 sums
+// the reduction reads them, unless a chunk of a wide channel set has more tiles
+// than one run.
+inline void simt_set_sums(DevInstance& I, int C, float* wsums, long long stride) {
+  I.wsums = wsums;
+  I.wsums_stride = stride;
+  I.wsums_direct = wsums && (C < 7 || I.tiles_per_chunk + (I.chunk_rem > 0 ? 1 : 0) <= kWaccTiles) ? 1 : 0;
+  if (I.wsums_direct) {
+    I.n_slice = slice_map(I.widths, I.L, I.goff_b, &I.goff_WL);
+  } else {
+    I.n_slice = (int)I.n_params;
+    for (int l = 0; l < I.L; ++l) I.goff_b[l] = (int)I.off_b[l];
+    I.goff_WL = (int)I.off_W[I.L - 1];
+  }
+}
 
 // Reductions and elementwise kernels (jet_reduce.cu)
 // One reduction job per instance: grad[p] = sum_c slices[c][p] in FP64 (fixed
 // order), loss = inv_N * sum_c loss_slices[c]; optionally fused with Adam.
+// Where the hidden-layer weight gradients of a job are.
+enum : int {
+  HID_SLICES = 0,  // in the FP64 slices, with all other parameters
+  HID_SIMT = 1,    // FP32 sums per chunk, in the item order of the SIMT weight gradient
+  HID_TC = 2,      // FP32 sums per chunk and sub-tile, [k / 4][u][4] per layer (tensor-core kernel)
+  HID_DONE = 3,    // one FP64 sum each, in parameter order (weight-gradient GEMM)
+};
 struct ReduceJob {
-  const double* grad_slices;
+  const double* grad_slices;  // [n_chunks][n_slice]
   const double* loss_slices;
   int n_chunks;
-  int grad_chunks;    // gradient slices to sum (0: n_chunks; 1: one shared accumulator)
+  int n_slice;
   long long n_params;
+  int hid;            // HID_*
+  int L;              // for hid != HID_SLICES: the network's layers and widths,
+  int widths[kMaxLayers + 1];
+  int n_hid;          // its hidden-layer weights,
+  int subs;           // HID_TC: sub-tiles summed in FP32 per chunk
+  int wr;             // HID_SIMT: rows of a weight-gradient item
+  const void* hid_sums;       // float [n_chunks][hid_stride], or HID_DONE double [n_hid]
+  long long hid_stride;
   double inv_N;
   void* grad_out;     // value type T or null
   double* loss_out;   // or null
@@ -204,11 +257,11 @@ struct ReduceJob {
   void* v;
 };
 cudaError_t launch_transpose_weights(const DevInstance& in, bool fp64, void* Wt, cudaStream_t s);
-// jobs: host array copied by value when n == 1, else a device array.  Adam
-// takes step t = `step`, or *step_ctr + 1 with a device counter, which the
-// call then increments on the stream.
-cudaError_t launch_reduce(const ReduceJob* dev_jobs, const ReduceJob& job0, int n, long long max_params, bool fp64,
-                          bool adam, long long step, float lr, cudaStream_t s, long long* step_ctr = nullptr);
+// jobs: host array (copied by value when n == 1); dev_jobs: the same on the
+// device when n > 1.  Adam takes step t = `step`, or *step_ctr + 1 with a device
+// counter, which the call then increments on the stream.
+cudaError_t launch_reduce(const ReduceJob* jobs, const ReduceJob* dev_jobs, int n, bool fp64, bool adam,
+                          long long step, float lr, cudaStream_t s, long long* step_ctr = nullptr);
 
 }  // namespace jet
 

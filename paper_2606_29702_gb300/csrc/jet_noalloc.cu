@@ -249,7 +249,7 @@ extern "C" jet_status jet_backward_params_noalloc(const jet_residual_spec* spec,
   if (scratch_bytes_used) *scratch_bytes_used = used;
   I.chunk_base = 0;
   I.store = nullptr;
-  I.wacc_off = -1;  // its few chunks' FP64 slices stay in L2: FP64 adds per tile
+  simt_set_sums(I, C, nullptr, 0);  // its few chunks' FP64 slices stay in L2: FP64 adds per tile
 
   cudaStream_t s = (cudaStream_t)stream;
   // every buffer below is fully written before it is read: the transpose
@@ -275,11 +275,12 @@ extern "C" jet_status jet_backward_params_noalloc(const jet_residual_spec* spec,
   j.grad_slices = I.grad_slices;
   j.loss_slices = I.loss_slices;
   j.n_chunks = I.n_chunks;
+  j.n_slice = I.n_slice;
   j.n_params = I.n_params;
   j.inv_N = I.inv_N;
   j.grad_out = grad_out;
   j.loss_out = loss_out;
-  e = launch_reduce(nullptr, j, 1, I.n_params, fp64, false, 1, 0.f, s);
+  e = launch_reduce(&j, nullptr, 1, fp64, false, 1, 0.f, s);
   if (e != cudaSuccess) return nfail_cuda(e, "reduce launch");
   return JET_OK;
 }

@@ -13,6 +13,33 @@ namespace jet {
 struct TcPlan;
 }
 
+namespace jet {
+// One device allocation cut into 256-byte aligned parts (a cudaMalloc costs 50
+// to 100 us of plan creation each).
+struct Arena {
+  struct Part {
+    void** ptr;
+    size_t off;
+  };
+  std::vector<Part> parts;
+  size_t bytes = 0;
+  template <class T>
+  void add(T** ptr, size_t n) {
+    *ptr = nullptr;
+    if (n == 0) return;
+    parts.push_back({reinterpret_cast<void**>(ptr), bytes});
+    bytes += (n + 255) / 256 * 256;
+  }
+  cudaError_t alloc(void** base) {
+    *base = nullptr;
+    const cudaError_t e = cudaMalloc(base, bytes > 0 ? bytes : 256);
+    if (e == cudaSuccess)
+      for (const Part& p : parts) *p.ptr = static_cast<char*>(*base) + p.off;
+    return e;
+  }
+};
+}  // namespace jet
+
 struct jet_plan_s {
   int device = 0;
   int d = 0, L = 0, n_out = 0, n_res = 0;
@@ -38,13 +65,15 @@ struct jet_plan_s {
   size_t smem = 0;
   int grid = 0, ctas_per_sm = 0;
   size_t elem = 4;
-  // workspace
+  // workspace (parts of one allocation)
+  void* ws = nullptr;
   void* Wt = nullptr;
   double* grad_slices = nullptr;
   double* loss_slices = nullptr;
   void* scratch = nullptr;
   long long scratch_stride = 0;
-  long long wacc_off = -1;  // FP32 weight-gradient accumulator in a scratch slot (elements)
+  float* wsums = nullptr;   // SIMT FP32 forms: FP32 weight-gradient sums per chunk, or null
+  long long wsums_stride = 0;
   void* store = nullptr;
   long long store_max_points = 0;
   size_t ws_bytes = 0;

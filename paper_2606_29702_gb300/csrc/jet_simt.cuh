@@ -40,6 +40,7 @@
 
 #include "jet_closures_gen.h"
 #include "jet_f2.cuh"
+#include "jet_f64.cuh"
 #include "jet_groups.cuh"
 #include "jet_internal.h"
 
@@ -129,17 +130,6 @@ __device__ __forceinline__ void store_chan(T* p, const T* v) {
   }
 }
 
-// Value-preserving float -> double on the integer pipe.  The FP64 pipe, which
-// executes the conversion instruction, takes two lanes a clock per SM, and a
-// tile converts every weight gradient; subnormals take the instruction.
-__device__ __forceinline__ double widen(float f) {
-  const unsigned b = __float_as_uint(f), e = (b >> 23) & 0xffu, m = b & 0x7fffffu;
-  if (e == 0u && m != 0u) return (double)f;
-  const unsigned ed = e == 0u ? 0u : e == 255u ? 2047u : e + 896u;
-  return __hiloint2double((int)((b & 0x80000000u) | (ed << 20) | (m >> 3)), (int)(m << 29));
-}
-__device__ __forceinline__ double widen(double f) { return f; }
-
 // 16 bytes from global to shared memory, asynchronously
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
@@ -154,9 +144,10 @@ __device__ __forceinline__ void red_add_v4(float* p, float a, float b, float c, 
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
-// The FP32 weight-gradient accumulator of a chunk, [item][WR][4] per layer as
-// the items of SimtTile::wgrad (functions of their own, called once per chunk:
-// inlined they would cost the tile's registers)
+// The FP32 weight-gradient sums of a chunk, [item][WR][4] per layer as the items
+// of SimtTile::wgrad, zeroed and added to the FP64 slice where a chunk is longer
+// than one run (functions of their own, called once per run: inlined they would
+// cost the tile's registers)
 static __device__ __noinline__ void simt_wacc_zero(float* acc, const DevInstance& I) {
   long long n4 = 0;
   for (int l = 2; l < I.L; ++l) n4 += (long long)I.widths[l] * I.widths[l - 1] / 4;
@@ -217,13 +208,13 @@ struct SimtTile {
   const T* params;
   const T* Wt;  // transposed weights [in][out] per layer
   const T* Wc;  // aligned copy of the packed parameters
-  // FP32 forms: the chunk's hidden-layer weight gradients add up in FP32 in
-  // this CTA's scratch slot (fire-and-forget vector reductions; every element
-  // belongs to one thread, which adds the tiles in program order) and reach
-  // the FP64 slice once per chunk.  Null: FP64 adds per tile.
+  // FP32 forms: the chunk's hidden-layer weight gradients add up in FP32
+  // (fire-and-forget vector reductions; every element belongs to one thread,
+  // which adds the tiles in program order).  Null: FP64 adds per tile.
   float* wacc_base = nullptr;
+  bool wacc_first = false;  // the running tile stores its sums instead of adding them
 
-  __device__ SimtTile(const DevInstance& I_, const SimtArgs& A_, unsigned char* smem)
+  __device__ SimtTile(const DevInstance& I_, const SimtArgs& A_, unsigned char* smem, int chunk)
       : I(I_), A(A_), NT(blockDim.x) {
     P = I.P;
     pitch = I.pitch;
@@ -244,8 +235,7 @@ struct SimtTile {
     params = reinterpret_cast<const T*>(I.params);
     Wt = reinterpret_cast<const T*>(I.Wt);
     Wc = Wt + weight_copy_offset(I.n_params);
-    if (F32 && I.wacc_off >= 0)
-      wacc_base = reinterpret_cast<float*>(A.scratch) + (long long)blockIdx.x * A.scratch_stride + I.wacc_off;
+    if (F32 && I.wsums) wacc_base = I.wsums + (long long)chunk * I.wsums_stride;
   }
 
   // accumulator of W^l (l = 2..L-1): [item][WR][4] per thread item of wgrad
@@ -254,9 +244,6 @@ struct SimtTile {
     for (int k = 2; k < l; ++k) off += (long long)I.widths[k] * I.widths[k - 1];
     return wacc_base + off;
   }
-  __device__ void wacc_zero() { simt_wacc_zero(wacc_base, I); }
-  __device__ void wacc_flush(double* g) { simt_wacc_flush<WR>(wacc_base, I, g); }
-
   __device__ const T* W(int l) const { return params + I.off_W[l - 1]; }   // l = 1..L
   __device__ const T* bias(int l) const { return params + I.off_b[l - 1]; }
 
@@ -659,7 +646,7 @@ struct SimtTile {
         for (int n = part; n < P; n += 4) s += UB[o * ncol + n];
       }
       s = sum4(s);
-      if (act && part == 0) atomicAdd(g + (k < wi ? I.off_W[L - 1] + o * wi + k : I.off_b[L - 1] + o), widen(s));
+      if (act && part == 0) atomicAdd(g + (k < wi ? I.goff_WL + o * wi + k : I.goff_b[L - 1] + o), widen(s));
     }
   }
 
@@ -808,7 +795,10 @@ struct SimtTile {
           float* a = wacc(l) + (long long)item * (WR * 4) + base;
 #pragma unroll
           for (int e = 0; e < WR * 4; e += 4)
-            if (e < n) red_add_v4(a + e, acc[e], acc[e + 1], acc[e + 2], acc[e + 3]);
+            if (e < n) {
+              if (wacc_first) __stcg(reinterpret_cast<float4*>(a + e), make_float4(acc[e], acc[e + 1], acc[e + 2], acc[e + 3]));
+              else red_add_v4(a + e, acc[e], acc[e + 1], acc[e + 2], acc[e + 3]);
+            }
           continue;
         }
       }
@@ -820,7 +810,7 @@ struct SimtTile {
         }
     }
     // four lanes per bias
-    double* gb = g + I.off_b[l - 1];
+    double* gb = g + I.goff_b[l - 1];
     const int bw = (4 * wo + 31) & ~31;
     for (int it = threadIdx.x; it < bw; it += NT) {
       const int u = it >> 2, part = it & 3;
@@ -858,8 +848,8 @@ struct SimtTile {
   // four lanes per unit
   __device__ void layer1_bwd(const T* zbar, double* g) {
     const int w = I.widths[1], d = I.d;
-    double* gW = g + I.off_W[0];
-    double* gb = g + I.off_b[0];
+    double* gW = g;
+    double* gb = g + I.goff_b[0];
     const int ww = (4 * w + 31) & ~31;
     for (int it = threadIdx.x; it < ww; it += NT) {
       const int u = it >> 2, part = it & 3;
@@ -958,8 +948,6 @@ struct SimtTile {
   }
 };
 
-constexpr int kWaccTiles = 64;  // tiles per FP32 weight-gradient run (FP32 forms)
-
 template <class Cls, class T, int RU>
 __device__ __forceinline__ void simt_body(const SimtArgs& args) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -979,7 +967,7 @@ __device__ __forceinline__ void simt_body(const SimtArgs& args) {
     __syncthreads();
     const DevInstance& I = inst_s;
     const int chunk = item - I.chunk_base;
-    SimtTile<Cls, T, RU> S(I, args, smem);
+    SimtTile<Cls, T, RU> S(I, args, smem, chunk);
     // columns past C * P are never written: zero them (and everything else)
     // once per item so that the weight-gradient sums over whole vectors see
     // zeros there
@@ -987,49 +975,32 @@ __device__ __forceinline__ void simt_body(const SimtArgs& args) {
     const auto first = S.first_rows();
     if (first.p) S.issue(first, 0, 0);
     const bool bwd = args.mode != MODE_FWD;
-    double* g = bwd ? I.grad_slices + (long long)chunk * I.n_params : nullptr;
+    double* g = bwd ? I.grad_slices + (long long)chunk * I.n_slice : nullptr;
     if (bwd)
-      for (long long i = threadIdx.x; i < I.n_params; i += NT) g[i] = 0.0;
-    const bool wacc_on = bwd && S.wacc_base != nullptr;
-    if (wacc_on) S.wacc_zero();
-    __syncthreads();
+      for (int i = threadIdx.x; i < I.n_slice; i += NT) g[i] = 0.0;
     double loss = 0.0;
     // tiles of the chunk: the first chunk_rem chunks take one more than the rest
     const long long t0 = (long long)chunk * I.tiles_per_chunk + min(chunk, I.chunk_rem);
     const long long t1 = t0 + I.tiles_per_chunk + (chunk < I.chunk_rem ? 1 : 0);
-    if constexpr (Cls::C >= 7) {
-      // FP32 runs of at most kWaccTiles tiles: the FP32 rounding of a
-      // weight's sum stays below kWaccTiles * 2^-24 of its magnitudes at any N
-      long long t = t0;
-      while (t < t1) {
-        const long long r1 = (wacc_on && t1 - t > kWaccTiles) ? t + kWaccTiles : t1;
-        for (; t < r1; ++t) {
-          loss += S.tile(t, g, t + 1 < t1);
-          __syncthreads();
-        }
-        if (wacc_on) {
-          __threadfence();
-          __syncthreads();
-          S.wacc_flush(g);
-          if (t < t1) {
-            __syncthreads();
-            S.wacc_zero();
-            __syncthreads();
-          }
-        }
-      }
-    } else {
-      // smaller channel sets keep every register for the tile and flush
-      // once per chunk; their accumulator serves only nets too wide for
-      // L2-resident FP64 slices
-      for (long long t = t0; t < t1; ++t) {
-        loss += S.tile(t, g, t + 1 < t1);
-        __syncthreads();
-      }
-      if (wacc_on) {
+    // FP32 sums in runs of at most kWaccTiles tiles (wide channel sets): the FP32
+    // rounding of a weight's sum stays below kWaccTiles * 2^-24 of its magnitudes
+    // at any N.  The reduction reads the sums of a single run.
+    const bool runs = bwd && S.wacc_base != nullptr && !I.wsums_direct;
+    if (runs) simt_wacc_zero(S.wacc_base, I);
+    __syncthreads();
+    for (long long t = t0; t < t1; ++t) {
+      S.wacc_first = t == t0 && I.wsums_direct;
+      loss += S.tile(t, g, t + 1 < t1);
+      __syncthreads();
+      if (runs && (t + 1 == t1 || (t + 1 - t0) % kWaccTiles == 0)) {
         __threadfence();
         __syncthreads();
-        S.wacc_flush(g);
+        simt_wacc_flush<SimtTile<Cls, T, RU>::WR>(S.wacc_base, I, g);
+        if (t + 1 < t1) {
+          __syncthreads();
+          simt_wacc_zero(S.wacc_base, I);
+          __syncthreads();
+        }
       }
     }
     // block reduction of the loss partial (fixed order)

@@ -39,10 +39,15 @@ struct TcPlan {
   int o_w, o_wlo, o_a0, o_a1, o_alo0, o_alo1, o_uo, o_ub, o_xs, o_red, o_part;
   int act_bytes = 0, alo_bytes = 0, r0w = 0, r1w = 0;
   long long scratch_stride = 0;
-  // per-CTA scratch slot: A^1..A^{L-3} copies, then (plans that can run the
-  // weight gradient per tile) the chunk's FP32 weight-gradient accumulator
-  long long wacc_off = -1;
-  // workspace
+  // per-CTA scratch slot: A^1..A^{L-3} copies.  FP32 weight-gradient sums of a
+  // chunk (plans that can run the weight gradient per tile), 0: none
+  long long wsums_stride = 0;
+  float* wsums = nullptr;   // [grid][wsums_stride]
+  double* hid64 = nullptr;  // store mode: FP64 sums of the weight-gradient GEMM's items
+  int n_slice = 0, n_hid = 0, goff_WL = 0;
+  int goff_b[kMaxLayers];
+  // workspace (parts of one allocation)
+  void* ws = nullptr;
   __nv_bfloat16* Wh = nullptr;   // hidden weights [L-2][w][w]
   __nv_bfloat16* Wl = nullptr;   // output weights [n_out][w]
   __nv_bfloat16* Wlo = nullptr;  // low parts [L-2][w][w]
@@ -54,22 +59,16 @@ struct TcPlan {
   cudaEvent_t err_ev = nullptr;
   size_t ws_bytes = 0;
   CUtensorMap wmap, wlmap, wlomap;
-  // per-chunk FP64 gradient slices when they fit in a share of L2, else one
-  // accumulator that every chunk adds into (atomic order not fixed)
-  bool shared_acc = false;
   // store mode of the weight gradient (JET_FLAG_STORE with a memory budget):
   // per tile A^1..A^{L-2} and Zbar^2..Zbar^{L-1} in HBM, reduced by the
   // weight-gradient GEMM kernel into one FP64 partial per work item
   unsigned char* wstore = nullptr;
   long long wstore_tile_stride = 0, wstore_tiles = 0;
   size_t wstore_budget = 0;  // grown on demand up to this many bytes
+  void* wg_ws = nullptr;    // wg_out and hid64
   float* wg_out = nullptr;  // [max_items][w*w]
   int wg_max_items = 0, wg_sms = 0;
 };
-
-// budget of the per-chunk gradient slices (their bias, output-layer and
-// first-layer entries take FP64 adds every tile, so they should stay in L2)
-constexpr double kSliceBudgetBytes = 48.0 * 1024 * 1024;
 
 // ------------------------------------------------------------------ weight-gradient GEMM
 // Wbar^l = sum over the tiles of a K range of Zbar^l A^{l-1}^T, both operands
@@ -219,19 +218,12 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_kernel(const __grid_const
   if (warp == 0) tc::tmem_dealloc(tmem, (uint32_t)a.tmem_cols);
 }
 
-// dst[off_W[l-1] + i*wu + k] += sum over the items of layer l and over the
+// dst[(l-2)*wu*wu + i*wu + k] = sum over the items of layer l and over the
 // G diagonal blocks of out[item] (w = G * wu: packed sub-tiles contribute
-// only within their own block)
-struct OffWl {
-  long long v[kMaxLayers];
-};
-
-// Four consecutive elements of a row per thread (hidden widths are multiples
-// of 32), 16-byte loads; each element's items in item order, eight at a time
-// in FP32 before each FP64 add.  offW is a __grid_constant__: read in place,
-// not copied to local memory for its runtime index.
-__global__ void wgrad_sum4_kernel(const float* out, int L, int w, int wu, int G, int ipl,
-                                  const __grid_constant__ OffWl offW, double* dst) {
+// only within their own block).  Four consecutive elements of a row per thread
+// (hidden widths are multiples of 32), 16-byte loads; each element's items in
+// item order, eight at a time in FP32 before each FP64 add.
+__global__ void wgrad_sum4_kernel(const float* out, int L, int w, int wu, int G, int ipl, double* dst) {
   const long long ww = (long long)w * w, uu = (long long)wu * wu, total4 = (long long)(L - 2) * uu / 4;
   for (long long e4 = blockIdx.x * (long long)blockDim.x + threadIdx.x; e4 < total4;
        e4 += (long long)gridDim.x * blockDim.x) {
@@ -271,11 +263,11 @@ __global__ void wgrad_sum4_kernel(const float* out, int L, int w, int wu, int G,
         s3 += (double)v.w;
       }
     }
-    double* d = dst + offW.v[li + 1] + r;
-    d[0] += s0;
-    d[1] += s1;
-    d[2] += s2;
-    d[3] += s3;
+    double* d = dst + e;
+    d[0] = s0;
+    d[1] = s1;
+    d[2] = s2;
+    d[3] = s3;
   }
 }
 
@@ -603,23 +595,25 @@ jet_status tc_plan_create(jet_plan_s* p, TcPlan** out, const cudaDeviceProp& pro
   t->ctas_per_sm = std::min(t->ctas_per_sm, occ);
   t->grid = prop.multiProcessorCount * t->ctas_per_sm;
   t->scratch_stride = ((long long)std::max(0, L - 3) * (t->act_bytes + t->alo_bytes) + 15) / 16 * 16;
-  if (!t->single_act) {
-    t->wacc_off = t->scratch_stride;
-    t->scratch_stride += (long long)std::max(0, L - 2) * t->G * t->wu * t->wu * (long long)sizeof(float);
-  }
+  if (!t->single_act) t->wsums_stride = (long long)(L - 2) * t->G * t->wu * t->wu;
+  t->n_hid = (L - 2) * t->wu * t->wu;
+  t->n_slice = slice_map(p->widths.data(), L, t->goff_b, &t->goff_WL);
   // workspace
   const long long nh = (long long)std::max(0, L - 2) * t->w * t->w, nl = 128LL * t->w;
   size_t b_wh = std::max<long long>(nh, 1) * 2, b_wl = nl * 2, b_wlo = t->split3 ? b_wh : 0;
-  t->shared_acc = (double)t->grid * p->n_params * 8.0 > kSliceBudgetBytes;
-  size_t b_gs = (size_t)(t->shared_acc ? 1 : t->grid) * p->n_params * 8, b_ls = (size_t)t->grid * 8;
+  size_t b_gs = (size_t)t->grid * t->n_slice * 8, b_ls = (size_t)t->grid * 8;
+  size_t b_ws = (size_t)t->grid * t->wsums_stride * sizeof(float);
   size_t b_sc = (size_t)t->grid * std::max<long long>(t->scratch_stride, 16);
-  e = cudaMalloc((void**)&t->Wh, b_wh);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&t->Wl, b_wl);
-  if (e == cudaSuccess && t->split3) e = cudaMalloc((void**)&t->Wlo, b_wlo);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&t->grad_slices, b_gs);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&t->loss_slices, b_ls);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&t->scratch, b_sc);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&t->err, sizeof(int));
+  Arena arena;
+  arena.add(&t->Wh, b_wh);
+  arena.add(&t->Wl, b_wl);
+  arena.add(&t->Wlo, b_wlo);
+  arena.add(&t->grad_slices, b_gs);
+  arena.add(&t->loss_slices, b_ls);
+  arena.add(&t->scratch, b_sc);
+  arena.add(&t->wsums, b_ws);
+  arena.add(&t->err, sizeof(int));
+  e = arena.alloc(&t->ws);
   if (e == cudaSuccess) e = cudaMemset(t->err, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaMallocHost((void**)&t->h_err, sizeof(int));
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&t->err_ev, cudaEventDisableTiming);
@@ -628,7 +622,7 @@ jet_status tc_plan_create(jet_plan_s* p, TcPlan** out, const cudaDeviceProp& pro
     return tcuda(e, "tensor-core workspace");
   }
   *t->h_err = 0;
-  t->ws_bytes = b_wh + b_wl + b_wlo + b_gs + b_ls + b_sc;
+  t->ws_bytes = b_wh + b_wl + b_wlo + b_gs + b_ls + b_sc + b_ws;
   if (want_store) {
     t->wstore_tile_stride = (long long)(L - 2) * (t->act_bytes + t->alo_bytes) + (long long)(L - 2) * t->act_bytes;
     t->wstore_budget = mem_budget;
@@ -646,12 +640,15 @@ jet_status tc_plan_create(jet_plan_s* p, TcPlan** out, const cudaDeviceProp& pro
       const int ipl = std::max(1, t->wg_sms / a);
       t->wg_max_items = (L - 2) * ipl;
       const size_t b_wo = (size_t)t->wg_max_items * t->w * t->w * sizeof(float);
-      e = cudaMalloc((void**)&t->wg_out, b_wo);
+      Arena wg;
+      wg.add(&t->wg_out, b_wo);
+      wg.add(&t->hid64, (size_t)t->n_hid * sizeof(double));
+      e = wg.alloc(&t->wg_ws);
       if (e != cudaSuccess) {
         tc_plan_destroy(t);
         return tcuda(e, "weight-gradient partials");
       }
-      t->ws_bytes += b_wo;
+      t->ws_bytes += b_wo + (size_t)t->n_hid * sizeof(double);
     }
   }
   const int R = 128 * t->H;
@@ -670,15 +667,9 @@ jet_status tc_plan_create(jet_plan_s* p, TcPlan** out, const cudaDeviceProp& pro
 
 void tc_plan_destroy(TcPlan* t) {
   if (!t) return;
-  cudaFree(t->Wh);
-  cudaFree(t->Wl);
-  cudaFree(t->Wlo);
-  cudaFree(t->grad_slices);
-  cudaFree(t->loss_slices);
-  cudaFree(t->scratch);
+  cudaFree(t->ws);
   cudaFree(t->wstore);
-  cudaFree(t->wg_out);
-  cudaFree(t->err);
+  cudaFree(t->wg_ws);
   cudaFreeHost(t->h_err);
   if (t->err_ev) cudaEventDestroy(t->err_ev);
   delete t;
@@ -688,7 +679,7 @@ int tc_tile_points(const TcPlan* t) { return t ? t->P : 0; }
 int tc_grid(const TcPlan* t) { return t ? t->grid : 0; }
 int tc_ctas_per_sm(const TcPlan* t) { return t ? t->ctas_per_sm : 0; }
 int tc_threads(const TcPlan* t) { return t ? t->nthreads : 0; }
-int tc_wgrad_chunk_fp32(const TcPlan* t) { return t && t->wacc_off >= 0 ? 1 : 0; }
+int tc_wgrad_chunk_fp32(const TcPlan* t) { return t && !t->single_act ? 1 : 0; }
 size_t tc_workspace_bytes(const TcPlan* t) { return t ? t->ws_bytes : 0; }
 
 namespace {
@@ -773,7 +764,11 @@ void fill_tc(const jet_plan_s* p, const TcPlan* t, const void* params, const voi
   I.loss_slices = t->loss_slices;
   I.scratch = t->scratch;
   I.scratch_stride = t->scratch_stride;
-  I.wacc_off = t->wacc_off;
+  I.wsums = t->wsums;
+  I.wsums_stride = t->wsums_stride;
+  I.n_slice = t->n_slice;
+  for (int l = 0; l < p->L; ++l) I.goff_b[l] = t->goff_b[l];
+  I.goff_WL = t->goff_WL;
   I.o_w = t->o_w;
   I.o_wlo = t->o_wlo;
   I.o_a0 = t->o_a0;
@@ -789,7 +784,6 @@ void fill_tc(const jet_plan_s* p, const TcPlan* t, const void* params, const voi
   I.alo_bytes = t->alo_bytes;
   I.r0w = t->r0w;
   I.r1w = t->r1w;
-  I.slice_shared = t->shared_acc ? 1 : 0;
   const bool use_store = t->wstore && I.n_tiles <= t->wstore_tiles;
   I.wstore = use_store ? t->wstore : nullptr;
   I.wstore_tile_stride = t->wstore_tile_stride;
@@ -871,10 +865,6 @@ jet_status run(jet_plan_s* p, TcPlan* t, int mode, const TcInst& I, cudaStream_t
   a.tmem_cols = t->tmem_cols;
   a.nthreads = t->nthreads;
   const int grid = std::min(t->grid, I.n_chunks);
-  if (mode != MODE_FWD && t->shared_acc) {
-    cudaError_t z = cudaMemsetAsync(t->grad_slices, 0, (size_t)p->n_params * sizeof(double), s);
-    if (z != cudaSuccess) return tcuda(z, "accumulator reset");
-  }
   jet::plan_prof_begin(p, s);
   cudaError_t e = tc_launch(p->cls, a, grid, t->smem, s);
   if (e == cudaSuccess && mode != MODE_FWD && I.wstore) {
@@ -910,11 +900,9 @@ jet_status run(jet_plan_s* p, TcPlan* t, int mode, const TcInst& I, cudaStream_t
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
-      OffWl ow;
-      for (int l = 0; l < L; ++l) ow.v[l] = p->off_W[l];
       const long long tot = (long long)(L - 2) * t->wu * t->wu;
       wgrad_sum4_kernel<<<(int)std::min<long long>((tot / 4 + 255) / 256, 2048), 256, 0, s>>>(
-          t->wg_out, L, t->w, t->wu, t->G, w.items_per_layer, ow, t->grad_slices);
+          t->wg_out, L, t->w, t->wu, t->G, w.items_per_layer, t->hid64);
       e = cudaGetLastError();
     }
   }
@@ -924,6 +912,26 @@ jet_status run(jet_plan_s* p, TcPlan* t, int mode, const TcInst& I, cudaStream_t
   e = cudaMemcpyAsync(t->h_err, t->err, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaEventRecord(t->err_ev, s);
   return e == cudaSuccess ? JET_OK : tcuda(e, "tc error read-back");
+}
+
+// the gradient reduction of one plan's call
+ReduceJob grad_job(const jet_plan_s* p, const TcPlan* t, const TcInst& I) {
+  ReduceJob j;
+  memset(&j, 0, sizeof(j));
+  j.grad_slices = I.grad_slices;
+  j.loss_slices = I.loss_slices;
+  j.n_chunks = I.n_chunks;
+  j.n_slice = I.n_slice;
+  j.n_params = p->n_params;
+  j.hid = I.wstore ? HID_DONE : HID_TC;
+  j.L = p->L;
+  for (int l = 0; l <= p->L; ++l) j.widths[l] = p->widths[l];
+  j.n_hid = t->n_hid;
+  j.subs = I.wstore ? 1 : t->G;
+  j.hid_sums = I.wstore ? (const void*)t->hid64 : (const void*)I.wsums;
+  j.hid_stride = I.wsums_stride;
+  j.inv_N = I.inv_N;
+  return j;
 }
 
 }  // namespace
@@ -949,7 +957,7 @@ jet_status tc_forward(jet_plan_s* p, TcPlan* t, const void* params, const void* 
     j.n_chunks = I.n_chunks;
     j.inv_N = I.inv_N;
     j.loss_out = loss_out;
-    cudaError_t e = launch_reduce(nullptr, j, 1, 1, false, false, 1, 0.f, s);
+    cudaError_t e = launch_reduce(&j, nullptr, 1, false, false, 1, 0.f, s);
     if (e != cudaSuccess) return tcuda(e, "reduce");
   }
   return JET_OK;
@@ -972,17 +980,10 @@ jet_status tc_backward(jet_plan_s* p, TcPlan* t, const void* params, const void*
   if (t->single_act && !I.wstore) return store_too_small(t, N);
   st = run(p, t, MODE_FWD_BWD, I, s);
   if (st != JET_OK) return st;
-  ReduceJob j;
-  memset(&j, 0, sizeof(j));
-  j.grad_slices = I.grad_slices;
-  j.loss_slices = I.loss_slices;
-  j.n_chunks = I.n_chunks;
-  j.n_params = p->n_params;
-  j.grad_chunks = t->shared_acc ? 1 : 0;
-  j.inv_N = I.inv_N;
+  ReduceJob j = grad_job(p, t, I);
   j.grad_out = grad_out;
   j.loss_out = loss_out;
-  cudaError_t e = launch_reduce(nullptr, j, 1, p->n_params, false, false, 1, 0.f, s);
+  cudaError_t e = launch_reduce(&j, nullptr, 1, false, false, 1, 0.f, s);
   return e == cudaSuccess ? JET_OK : tcuda(e, "reduce");
 }
 
@@ -999,19 +1000,12 @@ jet_status tc_train_step(jet_plan_s* p, TcPlan* t, void* params, void* m, void* 
   if (t->single_act && !I.wstore) return store_too_small(t, N);
   st = run(p, t, MODE_FWD_BWD, I, s);
   if (st != JET_OK) return st;
-  ReduceJob j;
-  memset(&j, 0, sizeof(j));
-  j.grad_slices = I.grad_slices;
-  j.loss_slices = I.loss_slices;
-  j.n_chunks = I.n_chunks;
-  j.n_params = p->n_params;
-  j.grad_chunks = t->shared_acc ? 1 : 0;
-  j.inv_N = I.inv_N;
+  ReduceJob j = grad_job(p, t, I);
   j.loss_out = loss_out;
   j.params = params;
   j.m = m;
   j.v = v;
-  cudaError_t e = launch_reduce(nullptr, j, 1, p->n_params, false, true, step, lr, s, step_ctr);
+  cudaError_t e = launch_reduce(&j, nullptr, 1, false, true, step, lr, s, step_ctr);
   return e == cudaSuccess ? JET_OK : tcuda(e, "reduce/adam");
 }
 
@@ -1037,7 +1031,8 @@ struct TcBatch {
   PrepJob* h_prep = nullptr;
   double* grad_slices = nullptr;
   double* loss_slices = nullptr;
-  std::vector<long long> slice_off;
+  float* wsums = nullptr;  // FP32 weight-gradient sums of every member's chunks
+  std::vector<long long> slice_off, wsums_off;
   unsigned char* scratch = nullptr;
   long long scratch_stride = 0;
   int* err = nullptr;
@@ -1051,7 +1046,7 @@ jet_status tc_batch_create(const std::vector<jet_plan_s*>& plans, TcBatch** out)
   TcBatch* b = new TcBatch();
   b->n = (int)plans.size();
   b->cls = plans[0]->cls;
-  long long slices = 0;
+  long long slices = 0, sums = 0;
   for (jet_plan_s* p : plans)
     if (p->tcp->single_act) {
       delete b;
@@ -1065,7 +1060,9 @@ jet_status tc_batch_create(const std::vector<jet_plan_s*>& plans, TcBatch** out)
     b->nthreads = std::min(b->nthreads, t->nthreads);
     b->scratch_stride = std::max(b->scratch_stride, t->scratch_stride);
     b->slice_off.push_back(slices);
-    slices += (long long)b->max_chunks * p->n_params;
+    slices += (long long)b->max_chunks * t->n_slice;
+    b->wsums_off.push_back(sums);
+    sums += (long long)b->max_chunks * t->wsums_stride;
   }
   int dev = 0, sms = 0, occ = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -1089,6 +1086,7 @@ jet_status tc_batch_create(const std::vector<jet_plan_s*>& plans, TcBatch** out)
   if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_prep, sizeof(PrepJob) * b->n);
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->grad_slices, sizeof(double) * std::max<long long>(slices, 1));
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->loss_slices, sizeof(double) * b->max_items);
+  if (e == cudaSuccess) e = cudaMalloc((void**)&b->wsums, sizeof(float) * std::max<long long>(sums, 4));
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->scratch, (size_t)b->grid * std::max<long long>(b->scratch_stride, 16));
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(b->err, 0, sizeof(int));
@@ -1117,6 +1115,7 @@ void tc_batch_destroy(TcBatch* b) {
   cudaFreeHost(b->h_prep);
   cudaFree(b->grad_slices);
   cudaFree(b->loss_slices);
+  cudaFree(b->wsums);
   cudaFree(b->scratch);
   cudaFree(b->err);
   if (b->copied) cudaEventDestroy(b->copied);
@@ -1166,8 +1165,8 @@ jet_status tc_batch_run(TcBatch* bb, const std::vector<jet_plan_s*>& plans, cons
     I.loss_slices = b->loss_slices + (long long)i * b->max_chunks;
     I.scratch = b->scratch;
     I.scratch_stride = b->scratch_stride;
-    I.slice_shared = 0;  // batches keep one deterministic slice per chunk
-    I.wstore = nullptr;  // and flush weight gradients per tile
+    I.wsums = b->wsums + b->wsums_off[i];
+    I.wstore = nullptr;  // batches run the weight gradient per tile
     double per_tile = (double)(p->L - 1) * t->w * t->w * t->cols_pad + 2000.0 * t->w * t->P * (p->L - 1);
     for (int c = 0; c < I.n_chunks; ++c) {
       const long long t0 = (long long)c * I.tiles_per_chunk;
@@ -1233,16 +1232,9 @@ jet_status tc_batch_run(TcBatch* bb, const std::vector<jet_plan_s*>& plans, cons
   if (e != cudaSuccess) return tcuda(e, "batch item counter reset");
   e = tc_launch(b->cls, a, std::min(b->grid, base), b->smem, s);
   if (e != cudaSuccess) return tcuda(e, "batched tc kernel launch");
-  long long maxp = 0;
   bool jobs_same = !capturing;
   for (int i = 0; i < n; ++i) {
-    ReduceJob j;
-    memset(&j, 0, sizeof(j));
-    j.grad_slices = insts[i].grad_slices;
-    j.loss_slices = insts[i].loss_slices;
-    j.n_chunks = insts[i].n_chunks;
-    j.n_params = plans[i]->n_params;
-    j.inv_N = insts[i].inv_N;
+    ReduceJob j = grad_job(plans[i], plans[i]->tcp, insts[i]);
     j.grad_out = adam ? nullptr : grad_out[i];
     j.loss_out = loss_out ? loss_out + i : nullptr;
     if (adam) {
@@ -1255,14 +1247,13 @@ jet_status tc_batch_run(TcBatch* bb, const std::vector<jet_plan_s*>& plans, cons
       if (b->have_prev && !capturing) cudaEventSynchronize(b->copied);
     }
     if (!jobs_same || capturing) b->h_jobs[i] = j;
-    maxp = std::max(maxp, j.n_params);
   }
   if (!jobs_same || capturing) {
     e = cudaMemcpyAsync(b->d_jobs, b->h_jobs, sizeof(ReduceJob) * n, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess && !capturing) e = cudaEventRecord(b->copied, s);
     if (e != cudaSuccess) return tcuda(e, "batch job upload");
   }
-  e = launch_reduce(b->d_jobs, b->h_jobs[0], n, maxp, false, adam, step, lr, s, step_ctr);
+  e = launch_reduce(b->h_jobs, b->d_jobs, n, false, adam, step, lr, s, step_ctr);
   return e == cudaSuccess ? JET_OK : tcuda(e, "batch reduce");
 }
 

@@ -26,8 +26,8 @@
 //            epilogue (Zbar^l to shared memory), data gradient
 //            Abar^{l-1} = W^l^T Zbar^l (MN-major A) and weight gradient
 //            Wbar^l = Zbar^l A^{l-1}^T (both operands K-major) by MMA; the
-//            weight gradient is added from TMEM into the CTA's FP32
-//            accumulator, which reaches the chunk's FP64 slice once per chunk.
+//            weight gradient is added from TMEM into the chunk's FP32 sums,
+//            which the reduction adds up in FP64 over the chunks.
 //
 // The layer inputs A^l of a tile are saved to a per-CTA global scratch slot by
 // bulk copies during the forward and read back during the backward, so memory
@@ -126,16 +126,18 @@ struct alignas(64) TcInst {
   double* loss_slices;
   unsigned char* scratch;
   long long scratch_stride;  // bytes per CTA slot
-  // FP32 weight-gradient accumulator of the running chunk, at this byte
-  // offset in the CTA's scratch slot (-1: none; such plans never run the
-  // weight gradient per tile)
-  long long wacc_off;
+  // FP32 sums of the hidden-layer weight gradients of each chunk (see wacc),
+  // read by the reduction; unused in store mode
+  float* wsums;
+  long long wsums_stride;
+  int n_slice;              // FP64 slice of a chunk: every other parameter
+  int goff_b[kMaxLayers];   // (slice_map)
+  int goff_WL;
   // shared-memory carve (bytes from the 1024-aligned base)
   int o_w, o_wlo, o_a0, o_a1, o_alo0, o_alo1, o_uo, o_ub, o_xs, o_red;
   int o_part;  // per-warpgroup partial sums, float [warpgroups][4][256]
   int act_bytes, alo_bytes;
   int r0w, r1w;  // TMEM column widths of regions R0 and R1 per half
-  int slice_shared;  // 1: all chunks add into grad_slices[0 .. n_params)
   // store mode: per tile, the layer inputs A^1..A^{L-2} (and their split low
   // parts) and the adjoints Zbar^2..Zbar^{L-1} go to HBM for the separate
   // weight-gradient GEMM; null = per-tile weight-gradient MMA and flush
@@ -216,6 +218,8 @@ struct TcTile {
   float* part;  // per-warpgroup partial sums [nwg][4][256]
   int q, wg, ul;  // TMEM lane quadrant, warpgroup, unit within a 128-row half
   int nwg, nthr;  // warpgroups and threads of the CTA
+  float* wsum;    // FP32 weight-gradient sums of the running chunk
+  bool wfirst;    // the running tile is the chunk's first: it stores its sums instead of adding them
   // descriptor fields of the epilogues' hot accesses, read once per tile: the
   // shared addresses of the operand buffers and the TMEM region widths
   uint32_t act_s0 = tc::smem_u32(sm + I.o_a0), act_s1 = tc::smem_u32(sm + I.o_a1);
@@ -704,12 +708,12 @@ struct TcTile {
       for (int h = 0; h < hh(); ++h) {
         const int k = h * 128 + ul;
         if (k >= wuu()) continue;
-        for (int o = 0; o < I.n_out; ++o) tc::red_add_f64(g + I.off_W[L - 1] + (long long)o * wuu() + k, part_sum(o, k));
+        for (int o = 0; o < I.n_out; ++o) tc::red_add_f64(g + I.goff_WL + o * wuu() + k, part_sum(o, k));
       }
     if (tid < I.n_out) {
       float s = 0.f;
       for (int n = 0; n < P; ++n) s += ub[(tid * C + 0) * P + n];
-      tc::red_add_f64(g + I.off_b[L - 1] + tid, (double)s);
+      tc::red_add_f64(g + I.goff_b[L - 1] + tid, (double)s);
     }
   }
 
@@ -797,22 +801,14 @@ struct TcTile {
     }
   }
 
-  // Weight gradients of a chunk's tiles add up in FP32 in the CTA's scratch
-  // slot and reach the FP64 slice once per chunk (chunk_flush): per-CTA FP32
-  // partials, FP64 across chunks.  Layer l (2..L-1) takes G * wu * wu floats,
-  // laid out [sub][k / 4][u][4], so that the 32 rows of a warp cover 512
-  // contiguous bytes per vector add.  The adds are fire-and-forget FP32
+  // Weight gradients of a chunk's tiles add up in FP32 in the chunk's sums:
+  // FP32 per chunk, FP64 across chunks (the reduction).  Layer l (2..L-1) takes
+  // G * wu * wu floats, laid out [sub][k / 4][u][4], so that the 32 rows of a warp
+  // cover 512 contiguous bytes per vector add.  The adds are fire-and-forget FP32
   // vector reductions; every element belongs to one thread, which adds the
-  // tiles in program order, so the sums are deterministic.
-  __device__ float* wacc(int l) const {
-    return reinterpret_cast<float*>(I.scratch + (long long)blockIdx.x * I.scratch_stride + I.wacc_off) +
-           (long long)(l - 2) * gg() * wuu() * wuu();
-  }
-  __device__ void wacc_zero() {
-    float4* a = reinterpret_cast<float4*>(wacc(2));
-    const long long n4 = (long long)(I.L - 2) * gg() * wuu() * wuu() / 4;
-    for (long long i = tid; i < n4; i += nth()) a[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-  }
+  // tiles in program order, so the sums are deterministic.  The first tile
+  // stores, so nothing has to be zeroed.
+  __device__ float* wacc(int l) const { return wsum + (long long)(l - 2) * gg() * wuu() * wuu(); }
 
   // TMEM columns of lane row (8, from taddr) -> accumulator columns k0 .. k0+7
   // of row u in the [k / 4][u][4] block at acc
@@ -821,8 +817,15 @@ struct TcTile {
     tc::tmem_ld8(taddr, v);
     tc::tmem_wait_ld();
     const int wu = wuu();
-    tc::red_add_v4_hint(acc + ((long long)(k0 / 4) * wu + u) * 4, v[0], v[1], v[2], v[3], pol);
-    tc::red_add_v4_hint(acc + ((long long)(k0 / 4 + 1) * wu + u) * 4, v[4], v[5], v[6], v[7], pol);
+    float* a0 = acc + ((long long)(k0 / 4) * wu + u) * 4;
+    float* a1 = acc + ((long long)(k0 / 4 + 1) * wu + u) * 4;
+    if (wfirst) {
+      tc::st_v4_hint(a0, v[0], v[1], v[2], v[3], pol);
+      tc::st_v4_hint(a1, v[4], v[5], v[6], v[7], pol);
+    } else {
+      tc::red_add_v4_hint(a0, v[0], v[1], v[2], v[3], pol);
+      tc::red_add_v4_hint(a1, v[4], v[5], v[6], v[7], pol);
+    }
   }
 
   // D[R0] (weight-gradient columns nb*NB .. of layer l) -> accumulator.  With
@@ -844,33 +847,6 @@ struct TcTile {
       if (h * 128 + q * 32 >= ww()) continue;  // warp-uniform
       for (int k0 = wg * 8; k0 < NB; k0 += nw() * 8)
         acc8(acc, h * 128 + ul, nb * NB + k0, R0(h) + lane_base() + (uint32_t)k0, pol);
-    }
-  }
-
-  // accumulator (summed over sub-tiles) -> FP64 slice, once per chunk;
-  // consecutive threads take consecutive weights, eight per batch with their
-  // loads in flight before the adds
-  __device__ void chunk_flush(double* g) {
-    const int wu = wuu(), per = wu * wu;
-    for (int l = 2; l <= I.L - 1; ++l) {
-      const float* acc = wacc(l);
-      double* gW = g + I.off_W[l - 1];
-      for (int e0 = tid; e0 < per; e0 += 8 * nth()) {
-        float v[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int e = e0 + j * nth();
-          v[j] = 0.f;
-          if (e < per) {
-            const int u = e / wu, k = e - u * wu;
-            for (int sub = 0; sub < gg(); ++sub)
-              v[j] += __ldcg(acc + ((long long)(sub * (wu / 4) + k / 4) * wu + u) * 4 + (k & 3));
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          if (e0 + j * nth() < per) tc::red_add_f64(gW + e0 + j * nth(), (double)v[j]);
-      }
     }
   }
 
@@ -968,8 +944,8 @@ struct TcTile {
   }
 
   __device__ void layer1_flush(double* g) {
-    for (int i = 0; i < Cls::D; ++i) part_flush(i, g + I.off_W[0] + i, Cls::D);
-    part_flush(3, g + I.off_b[0], 1);
+    for (int i = 0; i < Cls::D; ++i) part_flush(i, g + i, Cls::D);
+    part_flush(3, g + I.goff_b[0], 1);
   }
 
   // ------------------------------------------------------------ one tile
@@ -1118,7 +1094,7 @@ struct TcTile {
           }
           tc::mma_commit(bar_mma);
         }
-        part_flush(0, g + I.off_b[l - 1], 1);  // bias gradient of layer l, during the MMA
+        part_flush(0, g + I.goff_b[l - 1], 1);  // bias gradient of layer l, during the MMA
         if (l == 2) w1b = row_l1(PRELOAD1B);
         if (tid == 0 && ww() == 256 && wait(bar_wg, ph_wg, 68) && l > 2) load_hidden_w_half(l - 1, 0);
         if (!wait(bar_mma, ph_mma, 66)) break;
@@ -1149,7 +1125,7 @@ struct TcTile {
           mma_dgrad(zb);
           tc::mma_commit(bar_mma);
         }
-        part_flush(0, g + I.off_b[l - 1], 1);  // bias gradient of layer l, during the MMAs
+        part_flush(0, g + I.goff_b[l - 1], 1);  // bias gradient of layer l, during the MMAs
         if (!wait(bar_wg, ph_wg, 67)) break;
         tc::tc_fence_after();
         if (tid == 0 && l > 2) reload_act(l - 1);
@@ -1166,7 +1142,7 @@ struct TcTile {
         mma_wgrad(zb, ain, 0, NB);
         tc::mma_commit(bar_mma);
       }
-      part_flush(0, g + I.off_b[l - 1], 1);  // bias gradient of layer l, during the MMAs
+      part_flush(0, g + I.goff_b[l - 1], 1);  // bias gradient of layer l, during the MMAs
       if (l == 2) w1b = row_l1(PRELOAD1B);
       if (!wait(bar_mma, ph_mma, 64)) break;
       tc::tc_fence_after();
@@ -1283,26 +1259,21 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_kernel(const __grid_constant
                   warp >> 2,
                   tid & 127,
                   nwg,
-                  nthr};
+                  nthr,
+                  I.wsums + (long long)chunk * I.wsums_stride,
+                  true};
     const bool bwd = args.mode != MODE_FWD;
-    // one FP64 slice per chunk (fixed summation order), or one accumulator
-    // shared by every chunk, zeroed by the host, when the slices would not
-    // fit in L2
-    double* g = bwd ? I.grad_slices + (I.slice_shared ? 0LL : (long long)chunk * I.n_params) : nullptr;
-    if (bwd && !I.slice_shared)
-      for (long long i = tid; i < I.n_params; i += nthr) g[i] = 0.0;
-    const bool wacc_on = bwd && !I.wstore && I.L >= 3;  // weight gradients per tile
-    if (wacc_on) T.wacc_zero();
+    // one FP64 slice per chunk (fixed summation order)
+    double* g = bwd ? I.grad_slices + (long long)chunk * I.n_slice : nullptr;
+    if (bwd)
+      for (int i = tid; i < I.n_slice; i += nthr) g[i] = 0.0;
     __syncthreads();
     double loss = 0.0;
     const long long t0 = (long long)chunk * I.tiles_per_chunk;
     const long long t1 = (t0 + I.tiles_per_chunk < I.n_tiles) ? t0 + I.tiles_per_chunk : I.n_tiles;
-    for (long long t = t0; t < t1 && !abort_s; ++t) loss += T.tile(t, args.mode, g);
-    // hidden-layer weight gradients of the chunk's tiles -> FP64 slice
-    if (wacc_on && !abort_s) {
-      __threadfence();
-      __syncthreads();
-      T.chunk_flush(g);
+    for (long long t = t0; t < t1 && !abort_s; ++t) {
+      loss += T.tile(t, args.mode, g);
+      T.wfirst = false;
     }
     ph_tma = T.ph_tma;
     ph_mma = T.ph_mma;

@@ -306,6 +306,13 @@ __device__ __forceinline__ void red_add_v4_hint(float* p, float a, float b, floa
                : "memory");
 }
 
+// four FP32 values stored to global memory (16-byte aligned), with an L2 policy
+__device__ __forceinline__ void st_v4_hint(float* p, float a, float b, float c, float d, uint64_t pol) {
+  asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p), "f"(a), "f"(b), "f"(c),
+               "f"(d), "l"(pol)
+               : "memory");
+}
+
 // bulk copies with an L2 policy (same alignment rules as bulk_s2g / bulk_g2s)
 __device__ __forceinline__ void bulk_s2g_hint(void* dst, const void* src, uint32_t bytes, uint64_t pol) {
   asm volatile("cp.async.bulk.global.shared::cta.bulk_group.L2::cache_hint [%0], [%1], %2, %3;" ::"l"(dst),

@@ -66,3 +66,18 @@ def test_simt_batch_of_unequal_widths():
         assert rel_l2(g.cpu().numpy(), g_ref) <= TOL["fp32"][1]
         assert abs(loss - L) <= TOL["fp32"][0] * abs(L)
         assert np.isfinite(loss)
+
+
+@pytest.mark.parametrize("N", [2000, 100000])
+def test_fp32_sums_of_short_and_long_chunks(N):
+    """FP32 weight-gradient sums that the reduction reads (chunks of one run) and that a chunk adds to FP64 slices run
+    by run (more than 64 tiles of 8 points per CTA): repeating 50 points leaves the mean loss and its gradient."""
+    from paper_2606_29702_gb300 import jet, specs
+    spec, X, layers, src = case("ns_psi_3x128x6", 50, widths=[3, 128, 128, 128, 128, 2])
+    L, _, g_ref = reference(spec, X, layers)
+    plan = _plan(jet, specs, spec, "fp32", tile=8)
+    assert plan.info()["wgrad_chunk_fp32"] == 1
+    p, x, _ = _tensors(plan, np.tile(X, (N // 50, 1)), layers, src)
+    g, loss, _ = plan.backward(p, x)
+    assert rel_l2(g.cpu().numpy(), g_ref) <= TOL["fp32"][1]
+    assert abs(float(loss) - L) <= TOL["fp32"][0] * abs(L)
