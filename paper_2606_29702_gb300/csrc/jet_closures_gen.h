@@ -348,11 +348,11 @@ template <> struct ClassById<7> { using type = Cls_ns_uvp; };
 #define JET_TC_SHAPES_0(M) 
 #define JET_TC_SHAPES_1(M) 
 #define JET_TC_SHAPES_2(M) 
-#define JET_TC_SHAPES_3(M) M(64, 2, 1, 128, 512) M(64, 0, 1, 128, 512)
-#define JET_TC_SHAPES_4(M) M(32, 2, 1, 128, 512) M(40, 2, 1, 128, 512) M(16, 2, 1, 128, 256)
+#define JET_TC_SHAPES_3(M) M(64, 2, 1, 128, 512) M(64, 0, 1, 128, 512) M(48, 0, 1, 128, 512) M(32, 0, 1, 128, 512) M(16, 0, 1, 128, 512)
+#define JET_TC_SHAPES_4(M) M(32, 2, 1, 128, 512) M(40, 2, 1, 128, 512) M(16, 2, 1, 128, 256) M(16, 2, 1, 128, 512)
 #define JET_TC_SHAPES_5(M) M(16, 1, 2, 256, 512) M(8, 1, 2, 256, 512)
 #define JET_TC_SHAPES_6(M) M(16, 1, 1, 128, 512) M(8, 1, 1, 128, 512) M(8, 1, 1, 128, 256)
-#define JET_TC_SHAPES_7(M) M(48, 2, 1, 128, 512)
+#define JET_TC_SHAPES_7(M) M(48, 2, 1, 128, 512) M(32, 0, 1, 128, 512) M(16, 0, 1, 128, 512)
 
 // X-macro over the classes: JET_FOR_EACH_CLASS(M) expands M(id, Cls_name)
 #define JET_FOR_EACH_CLASS(M) \

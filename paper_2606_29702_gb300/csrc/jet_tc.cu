@@ -23,6 +23,7 @@ namespace jet {
 template <int ID> cudaError_t tc_launch_id(const TcArgs& a, int grid, size_t smem, cudaStream_t s);
 template <int ID> cudaError_t tc_max_active_id(size_t smem, int threads, int* blocks);
 template <int ID> cudaError_t tc_attrs_id(cudaFuncAttributes* a);
+template <int ID> bool tc_has_shape_id(const int* shape, int threads);
 
 struct TcPlan {
   int w = 0, H = 1, P = 0, cols = 0, cols_pad = 0, top_cols = 0, split3 = 0;
@@ -68,6 +69,9 @@ struct TcPlan {
   void* wg_ws = nullptr;    // wg_out and hid64
   float* wg_out = nullptr;  // [max_items][w*w]
   int wg_max_items = 0, wg_sms = 0;
+  // the same plan with smaller compiled tiles, for calls whose points do not
+  // fill the GPU with the largest (geometry of their own, this plan's workspace)
+  std::vector<TcPlan> smaller;
 };
 
 // ------------------------------------------------------------------ weight-gradient GEMM
@@ -330,6 +334,17 @@ cudaError_t tc_fit(int cls, size_t smem, int threads, int* blocks) {
   return cudaSuccess;
 }
 
+bool tc_has_shape(int cls, const int* shape, int threads) {
+  switch (cls) {
+#define CASE(id, cl) \
+  case id:           \
+    return tc_has_shape_id<id>(shape, threads);
+    JET_FOR_EACH_CLASS(CASE)
+#undef CASE
+  }
+  return false;
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -433,6 +448,21 @@ jet_status tcuda(cudaError_t e, const char* what) {
   return e == cudaErrorMemoryAllocation ? JET_ERR_OOM : JET_ERR_CUDA;
 }
 
+// tile of Pc points per sub-tile: columns of the operands
+void set_tile(TcPlan& t, int C, int ntop, int Pc) {
+  t.Pc = Pc;
+  t.P = t.G * Pc;
+  t.cols = C * Pc;
+  t.cols_pad = (t.cols + 15) / 16 * 16;
+  t.top_cols = ntop * Pc;
+}
+// its TMEM region widths
+void set_regions(TcPlan& t) {
+  const int NB = t.H == 2 ? 128 : t.w;  // N of the weight-gradient MMA (the MMA width)
+  t.r0w = t.single_act ? t.cols_pad : std::max(t.cols_pad, NB);
+  t.r1w = t.cols_pad;
+}
+
 // shared-memory carve for tile size P; returns total bytes (without the 1 KB alignment slack)
 size_t carve(TcPlan& t, int C, int n_out, int d) {
   const int R = 128 * t.H;
@@ -523,12 +553,8 @@ jet_status tc_plan_create(jet_plan_s* p, TcPlan** out, const cudaDeviceProp& pro
       }
       TcPlan c = *t;
       c.nthreads = 512 / ctas;
-      c.P = P;
-      c.Pc = Pc;
-      c.cols = C * Pc;
-      c.cols_pad = (c.cols + 15) / 16 * 16;
+      set_tile(c, C, ntop, Pc);
       if (c.cols_pad > 256) break;
-      c.top_cols = ntop * Pc;
       if (c.split3 && c.top_cols % 16) {
         snprintf(why, sizeof(why), "P=%d: split columns not a multiple of 16", P);
         continue;
@@ -542,9 +568,7 @@ jet_status tc_plan_create(jet_plan_s* p, TcPlan** out, const cudaDeviceProp& pro
         snprintf(why, sizeof(why), "P=%d, %d CTA/SM: %zu B of shared memory", P, ctas, sm);
         continue;
       }
-      const int NB = c.H == 2 ? 128 : c.w;  // N of the weight-gradient MMA (the MMA width)
-      c.r0w = c.single_act ? c.cols_pad : std::max(c.cols_pad, NB);
-      c.r1w = c.cols_pad;
+      set_regions(c);
       const int need = c.H * (c.r0w + c.r1w);
       int tm = 32;
       while (tm < need) tm *= 2;
@@ -661,8 +685,36 @@ jet_status tc_plan_create(jet_plan_s* p, TcPlan** out, const cudaDeviceProp& pro
     return tfail(JET_ERR_UNSUPPORTED, "tensor map encoding failed");
   }
   if (!t->split3) t->wlomap = t->wmap;
+  if (!p8 && !want_store)
+    for (int Pc = t->Pc - 8; Pc >= 8; Pc -= 8) {
+      const int shape[4] = {Pc, t->G, t->H, t->w};
+      if (!tc_has_shape(p->cls, shape, t->nthreads) || (t->split3 && ntop * Pc % 16)) continue;
+      TcPlan v = *t;
+      v.smaller.clear();
+      set_tile(v, C, ntop, Pc);
+      set_regions(v);
+      carve(v, C, p->n_out, p->d);
+      t->smaller.push_back(v);
+    }
   *out = t;
   return JET_OK;
+}
+
+// The tile of one call on N points: the one whose rounds of tiles over the CTAs
+// take the least time.  A tile takes kTcTileCost for its serial chain of layers
+// (barriers, MMA and copy latencies) and the rest in proportion to its points
+// per sub-tile: 2->64x6->1 calls of one round take 63, 69, 76 and 82 us with 16,
+// 32, 48 and 64 of them.  At 1024 points 16 instead of 64: 72 -> 59 us.
+static const TcPlan* tc_call_tile(const TcPlan* t, long long N) {
+  constexpr long long kTcTileCost = 64;
+  auto cost = [&](const TcPlan& v) {
+    const long long tiles = (N + v.P - 1) / v.P;
+    return (tiles + v.grid - 1) / v.grid * (kTcTileCost + v.Pc);
+  };
+  const TcPlan* best = t;
+  for (const TcPlan& v : t->smaller)
+    if (cost(v) < cost(*best)) best = &v;
+  return best;
 }
 
 void tc_plan_destroy(TcPlan* t) {
@@ -947,7 +999,7 @@ jet_status tc_forward(jet_plan_s* p, TcPlan* t, const void* params, const void* 
   st = prep(p, t, params, s);
   if (st != JET_OK) return st;
   TcInst I;
-  fill_tc(p, t, params, X, N, source, r_out, I);
+  fill_tc(p, tc_call_tile(t, N), params, X, N, source, r_out, I);
   st = run(p, t, MODE_FWD, I, s);
   if (st != JET_OK) return st;
   if (loss_out) {
@@ -976,7 +1028,7 @@ jet_status tc_backward(jet_plan_s* p, TcPlan* t, const void* params, const void*
   st = prep(p, t, params, s);
   if (st != JET_OK) return st;
   TcInst I;
-  fill_tc(p, t, params, X, N, source, r_out, I);
+  fill_tc(p, tc_call_tile(t, N), params, X, N, source, r_out, I);
   if (t->single_act && !I.wstore) return store_too_small(t, N);
   st = run(p, t, MODE_FWD_BWD, I, s);
   if (st != JET_OK) return st;
@@ -996,7 +1048,7 @@ jet_status tc_train_step(jet_plan_s* p, TcPlan* t, void* params, void* m, void* 
   st = prep(p, t, params, s);
   if (st != JET_OK) return st;
   TcInst I;
-  fill_tc(p, t, params, X, N, source, nullptr, I);
+  fill_tc(p, tc_call_tile(t, N), params, X, N, source, nullptr, I);
   if (t->single_act && !I.wstore) return store_too_small(t, N);
   st = run(p, t, MODE_FWD_BWD, I, s);
   if (st != JET_OK) return st;

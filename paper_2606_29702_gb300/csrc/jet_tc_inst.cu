@@ -11,6 +11,7 @@ namespace jet {
 template <int ID> cudaError_t tc_launch_id(const TcArgs& a, int grid, size_t smem, cudaStream_t s);
 template <int ID> cudaError_t tc_max_active_id(size_t smem, int threads, int* blocks);
 template <int ID> cudaError_t tc_attrs_id(cudaFuncAttributes* a);
+template <int ID> bool tc_has_shape_id(const int* shape, int threads);
 
 using TcCls = ClassById<JET_CLASS_ID>::type;
 
@@ -37,6 +38,17 @@ cudaError_t tc_launch_id<JET_CLASS_ID>(const TcArgs& a, int grid, size_t smem, c
   JET_CAT(JET_TC_SHAPES_, JET_CLASS_ID)(JET_TRY_SHAPE)
 #undef JET_TRY_SHAPE
   return launch_shape<TcShapeAny>(a, grid, smem, s);
+}
+
+// whether a launch of this tile shape runs a fixed-shape kernel
+template <>
+bool tc_has_shape_id<JET_CLASS_ID>(const int* shape, int threads) {
+#define JET_HAS_SHAPE(PC_, G_, H_, W_, NT_)                                                   \
+  if (shape[0] == (PC_) && ((G_) == 0 || shape[1] == (G_)) && shape[2] == (H_) && shape[3] == (W_) && threads == (NT_)) \
+    return true;
+  JET_CAT(JET_TC_SHAPES_, JET_CLASS_ID)(JET_HAS_SHAPE)
+#undef JET_HAS_SHAPE
+  return false;
 }
 
 // occupancy and attributes of the general kernel (the fixed shapes use the
