@@ -409,6 +409,11 @@ struct TcTile {
   static constexpr bool PRELOAD = Shape::H != 2;    // biases
   static constexpr bool PRELOAD1 = Shape::H != 2;   // W^1, b^1 of the layer-1 forward
   static constexpr bool PRELOAD1B = Shape::H == 2;  // W^1, b^1 of the layer-1 backward
+  // The output layer's adjoints as vector loads, db^L by a warp per output and
+  // the first layer's partial sums by a warpgroup each, widened on the integer
+  // pipe: 2->64x6->3 composite loss 92.7 -> 88.9 us, ensemble 5.97 -> 5.89 ms,
+  // 3->128x6->2 5.18 -> 5.14 ms.  Not for 256-wide shapes: 41.97 -> 42.45 ms.
+  static constexpr bool PAR_FLUSH = Shape::H != 2;
   struct RowBias {
     float v[2];
   };
@@ -677,12 +682,18 @@ struct TcTile {
           const int col = blk(c) * Pc + q8;
           const uint4 raw = tc::lds_v4_b32(act_s(a_buf) + tc::swz_off(r, col, rr()));
           const __nv_bfloat16* bv = reinterpret_cast<const __nv_bfloat16*>(&raw);
-          const float* ubc = ub + c * P + sub * Pc + q8;
+          const float* ubc = ub + c * P + sub * Pc + q8;  // 16-byte aligned: P and Pc are multiples of 8
 #pragma unroll
           for (int o = 0; o < kMaxOut; ++o) {
             if (o >= nout) break;
+            float u[8];
+            if (PAR_FLUSH) {
+              vload<float>(ubc + o * C * P, u);
+              vload<float>(ubc + o * C * P + 4, u + 4);
+            }
 #pragma unroll
-            for (int j = 0; j < 8; ++j) acc[o] = fmaf(__bfloat162float(bv[j]), ubc[o * C * P + j], acc[o]);
+            for (int j = 0; j < 8; ++j)
+              acc[o] = fmaf(__bfloat162float(bv[j]), PAR_FLUSH ? u[j] : ubc[o * C * P + j], acc[o]);
           }
         }
 #pragma unroll
@@ -698,7 +709,7 @@ struct TcTile {
     float s = 0.f;
     for (int sub = 0; sub < gg(); ++sub)
       for (int w2 = 0; w2 < nw(); ++w2) s += PART(w2, k, sub * wuu() + u);
-    return (double)s;
+    return PAR_FLUSH ? widen(s) : (double)s;
   }
 
   __device__ void out_grads_flush(double* g) {
@@ -710,16 +721,28 @@ struct TcTile {
         if (k >= wuu()) continue;
         for (int o = 0; o < I.n_out; ++o) tc::red_add_f64(g + I.goff_WL + o * wuu() + k, part_sum(o, k));
       }
-    if (tid < I.n_out) {
+    if (!PAR_FLUSH) {
+      if (tid < I.n_out) {
+        float s = 0.f;
+        for (int n = 0; n < P; ++n) s += ub[(tid * C + 0) * P + n];
+        tc::red_add_f64(g + I.goff_b[L - 1] + tid, (double)s);
+      }
+      return;
+    }
+    // db^L: one warp per output (the last warps, whose warpgroup has no weights)
+    const int o = (nth() >> 5) - 1 - warp;
+    if (o < I.n_out) {
       float s = 0.f;
-      for (int n = 0; n < P; ++n) s += ub[(tid * C + 0) * P + n];
-      tc::red_add_f64(g + I.goff_b[L - 1] + tid, (double)s);
+      for (int n = tid & 31; n < P; n += 32) s += ub[(o * C + 0) * P + n];
+      for (int m = 16; m > 0; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
+      if ((tid & 31) == 0) tc::red_add_f64(g + I.goff_b[L - 1] + o, widen(s));
     }
   }
 
-  // slot k of PART summed over warpgroups and sub-tiles -> FP64 slice at dst[u * stride]
-  __device__ void part_flush(int k, double* dst, int stride) {
-    if (wg != 0) return;
+  // slot k of PART summed over warpgroups and sub-tiles -> FP64 slice at
+  // dst[u * stride], by warpgroup `by`
+  __device__ void part_flush(int k, double* dst, int stride, int by = 0) {
+    if (wg != (PAR_FLUSH ? by : 0)) return;
     for (int h = 0; h < hh(); ++h) {
       const int u = h * 128 + ul;
       if (u >= wuu()) continue;
@@ -944,8 +967,8 @@ struct TcTile {
   }
 
   __device__ void layer1_flush(double* g) {
-    for (int i = 0; i < Cls::D; ++i) part_flush(i, g + i, Cls::D);
-    part_flush(3, g + I.goff_b[0], 1);
+    for (int i = 0; i < Cls::D; ++i) part_flush(i, g + i, Cls::D, i & (nw() - 1));
+    part_flush(3, g + I.goff_b[0], 1, nw() - 1);
   }
 
   // ------------------------------------------------------------ one tile
