@@ -55,9 +55,9 @@ struct TcPlan {
   double* grad_slices = nullptr;
   double* loss_slices = nullptr;
   unsigned char* scratch = nullptr;
-  int* err = nullptr;
+  // code of a timed-out wait, in pinned host memory that the kernel writes on a
+  // time-out and the next call reads: nothing is copied back per call
   int* h_err = nullptr;
-  cudaEvent_t err_ev = nullptr;
   size_t ws_bytes = 0;
   CUtensorMap wmap, wlmap, wlomap;
   // store mode of the weight gradient (JET_FLAG_STORE with a memory budget):
@@ -636,11 +636,8 @@ jet_status tc_plan_create(jet_plan_s* p, TcPlan** out, const cudaDeviceProp& pro
   arena.add(&t->loss_slices, b_ls);
   arena.add(&t->scratch, b_sc);
   arena.add(&t->wsums, b_ws);
-  arena.add(&t->err, sizeof(int));
   e = arena.alloc(&t->ws);
-  if (e == cudaSuccess) e = cudaMemset(t->err, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaMallocHost((void**)&t->h_err, sizeof(int));
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&t->err_ev, cudaEventDisableTiming);
   if (e != cudaSuccess) {
     tc_plan_destroy(t);
     return tcuda(e, "tensor-core workspace");
@@ -723,7 +720,6 @@ void tc_plan_destroy(TcPlan* t) {
   cudaFree(t->wstore);
   cudaFree(t->wg_ws);
   cudaFreeHost(t->h_err);
-  if (t->err_ev) cudaEventDestroy(t->err_ev);
   delete t;
 }
 
@@ -742,16 +738,15 @@ bool is_capturing(cudaStream_t s) {
 }
 
 // Device-side wait time-outs of an earlier call surface here.  While the
-// stream is being captured into a CUDA graph the event query (and the
-// read-back in run) would invalidate the capture: a time-out inside a replayed
-// graph surfaces at the next call made outside capture.
+// stream is being captured into a CUDA graph nothing is reported (the error
+// path synchronises): a time-out inside a replayed graph surfaces at the next
+// call made outside capture.
 jet_status check_err(TcPlan* t, cudaStream_t s) {
-  if (is_capturing(s)) return JET_OK;
-  if (cudaEventQuery(t->err_ev) == cudaSuccess && *t->h_err != 0) {
+  if (*reinterpret_cast<volatile int*>(t->h_err) != 0 && !is_capturing(s)) {
+    cudaDeviceSynchronize();  // the CTAs that gave up drain and return
     char buf[128];
     snprintf(buf, sizeof(buf), "a bounded device wait timed out in an earlier call (code %d)", *t->h_err);
     *t->h_err = 0;
-    cudaMemset(t->err, 0, sizeof(int));
     jet::set_last_error(buf);
     return JET_ERR_TIMEOUT;
   }
@@ -913,7 +908,7 @@ jet_status run(jet_plan_s* p, TcPlan* t, int mode, const TcInst& I, cudaStream_t
   a.n_items = I.n_chunks;
   a.insts = nullptr;
   a.item_inst = nullptr;
-  a.err = t->err;
+  a.err = t->h_err;
   a.tmem_cols = t->tmem_cols;
   a.nthreads = t->nthreads;
   const int grid = std::min(t->grid, I.n_chunks);
@@ -941,7 +936,7 @@ jet_status run(jet_plan_s* p, TcPlan* t, int mode, const TcInst& I, cudaStream_t
     w.items_per_layer = (int)((I.n_tiles + w.tiles_per_item - 1) / w.tiles_per_item);
     w.n_items = (L - 2) * w.items_per_layer;
     w.out = t->wg_out;
-    w.err = t->err;
+    w.err = t->h_err;
     int tm = 32;
     while (tm < t->H * t->w) tm *= 2;
     w.tmem_cols = tm;
@@ -959,11 +954,7 @@ jet_status run(jet_plan_s* p, TcPlan* t, int mode, const TcInst& I, cudaStream_t
     }
   }
   jet::plan_prof_end(p, s);
-  if (e != cudaSuccess) return tcuda(e, "tc kernel launch");
-  if (is_capturing(s)) return JET_OK;
-  e = cudaMemcpyAsync(t->h_err, t->err, sizeof(int), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaEventRecord(t->err_ev, s);
-  return e == cudaSuccess ? JET_OK : tcuda(e, "tc error read-back");
+  return e == cudaSuccess ? JET_OK : tcuda(e, "tc kernel launch");
 }
 
 // the gradient reduction of one plan's call

@@ -92,7 +92,8 @@ static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parit
     if ((it & 255) == 0 && global_ns() - t0 > budget_ns) break;
   }
   *abort = 1;
-  atomicCAS(err, 0, code);
+  *reinterpret_cast<volatile int*>(err) = code;  // device or pinned host memory
+  __threadfence_system();
   return false;
 }
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort, int* err, int code,
