@@ -4,11 +4,13 @@
 
 #include "jet_f64.cuh"
 #include "jet_internal.h"
+#include "jet_pdl.cuh"
 
 namespace jet {
 
 template <class T>
 __global__ void transpose_weights_kernel(const __grid_constant__ DevInstance I, T* Wt) {
+  dependency_wait();
   const T* P = reinterpret_cast<const T*>(I.params);
   T* Wc = Wt + weight_copy_offset(I.n_params);
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < I.n_params;
@@ -31,9 +33,8 @@ cudaError_t launch_transpose_weights(const DevInstance& in, bool fp64, void* Wt,
   int grid = (int)((in.n_params + 255) / 256);
   if (grid > 2048) grid = 2048;
   if (grid < 1) grid = 1;
-  if (fp64) transpose_weights_kernel<double><<<grid, 256, 0, s>>>(in, reinterpret_cast<double*>(Wt));
-  else transpose_weights_kernel<float><<<grid, 256, 0, s>>>(in, reinterpret_cast<float*>(Wt));
-  return cudaGetLastError();
+  if (fp64) return launch_dependent(&transpose_weights_kernel<double>, grid, 256, 0, s, in, reinterpret_cast<double*>(Wt));
+  return launch_dependent(&transpose_weights_kernel<float>, grid, 256, 0, s, in, reinterpret_cast<float*>(Wt));
 }
 
 // Adam (Kingma & Ba 2015) with beta1 = 0.9, beta2 = 0.999, eps = 1e-8; the
@@ -226,6 +227,7 @@ __device__ __forceinline__ void reduce_elems(const ReduceJob& J, const AdamConst
 template <class T, bool ADAM>
 __global__ void __launch_bounds__(32 * kRedWarps) reduce_kernel(const __grid_constant__ ReduceJob job0,
                                                                 const ReduceJob* jobs, bool many, AdamConst ac) {
+  dependency_wait();
   const ReduceJob& J = jobs ? jobs[blockIdx.y] : job0;
   // the grid covers the largest job: blocks past this job's have nothing to do
   // (block 0 stays: it writes the loss, also of loss-only jobs)
@@ -276,7 +278,10 @@ __global__ void __launch_bounds__(32 * kRedWarps) reduce_kernel(const __grid_con
 }
 
 // the device step counter advances once the update that read it is done
-__global__ void adam_advance_kernel(long long* step_ctr) { *step_ctr += 1; }
+__global__ void adam_advance_kernel(long long* step_ctr) {
+  dependency_wait();
+  *step_ctr += 1;
+}
 
 cudaError_t launch_reduce(const ReduceJob* jobs, const ReduceJob* dev_jobs, int n, bool fp64, bool adam,
                           long long step, float lr, cudaStream_t s, long long* step_ctr) {
@@ -307,19 +312,14 @@ cudaError_t launch_reduce(const ReduceJob* jobs, const ReduceJob* dev_jobs, int 
   const dim3 grid((unsigned)gx, (unsigned)n);
   const ReduceJob* dj = n == 1 ? nullptr : dev_jobs;
   const int threads = 32 * kRedWarps;
+  cudaError_t e;
   if (fp64) {
-    if (adam) reduce_kernel<double, true><<<grid, threads, 0, s>>>(jobs[0], dj, many, ac);
-    else reduce_kernel<double, false><<<grid, threads, 0, s>>>(jobs[0], dj, many, ac);
+    e = launch_dependent(adam ? &reduce_kernel<double, true> : &reduce_kernel<double, false>, grid, threads, 0, s, jobs[0], dj, many, ac);
   } else {
-    if (adam) reduce_kernel<float, true><<<grid, threads, 0, s>>>(jobs[0], dj, many, ac);
-    else reduce_kernel<float, false><<<grid, threads, 0, s>>>(jobs[0], dj, many, ac);
+    e = launch_dependent(adam ? &reduce_kernel<float, true> : &reduce_kernel<float, false>, grid, threads, 0, s, jobs[0], dj, many, ac);
   }
-  if (adam && step_ctr) {
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    adam_advance_kernel<<<1, 1, 0, s>>>(step_ctr);
-  }
-  return cudaGetLastError();
+  if (e == cudaSuccess && adam && step_ctr) e = launch_dependent(&adam_advance_kernel, 1, 1, 0, s, step_ctr);
+  return e;
 }
 
 }  // namespace jet

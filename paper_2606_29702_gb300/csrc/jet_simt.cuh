@@ -43,6 +43,7 @@
 #include "jet_f64.cuh"
 #include "jet_groups.cuh"
 #include "jet_internal.h"
+#include "jet_pdl.cuh"
 
 namespace jet {
 
@@ -951,6 +952,7 @@ struct SimtTile {
 template <class Cls, class T, int RU>
 __device__ __forceinline__ void simt_body(const SimtArgs& args) {
   extern __shared__ __align__(16) unsigned char smem[];
+  dependency_wait();
   __shared__ int k_s;
   // the running item's descriptor: read in every phase, through shared memory
   // rather than a pointer that may be param or global space, which cost

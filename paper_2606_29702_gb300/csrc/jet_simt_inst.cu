@@ -39,8 +39,7 @@ cudaError_t simt_launch_id<JET_CLASS_ID>(bool fp64, const SimtArgs& a, int grid,
   const auto kernel = fp64 ? simt_entry<ThisCls, double>(a.ru) : simt_entry<ThisCls, float>(a.ru);
   const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, a.carveout);
   if (e != cudaSuccess) return e;
-  kernel<<<grid, a.threads, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_dependent(kernel, grid, a.threads, smem, s, a);
 }
 
 template <>

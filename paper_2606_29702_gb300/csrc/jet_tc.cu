@@ -126,6 +126,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_kernel(const __grid_const
   uint32_t fph = 0, eph = 0, dph = 0;
   const int ww = a.w * a.w;
   const uint32_t id = tc::idesc_bf16(128, a.w, 0, 0);
+  dependency_wait();
   for (int item = blockIdx.x; item < a.n_items && !abort_s; item += gridDim.x) {
     const int l = item / a.items_per_layer + 2;
     const long long t0 = (long long)(item % a.items_per_layer) * a.tiles_per_item;
@@ -228,6 +229,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_kernel(const __grid_const
 // (hidden widths are multiples of 32), 16-byte loads; each element's items in
 // item order, eight at a time in FP32 before each FP64 add.
 __global__ void wgrad_sum4_kernel(const float* out, int L, int w, int wu, int G, int ipl, double* dst) {
+  dependency_wait();
   const long long ww = (long long)w * w, uu = (long long)wu * wu, total4 = (long long)(L - 2) * uu / 4;
   for (long long e4 = blockIdx.x * (long long)blockDim.x + threadIdx.x; e4 < total4;
        e4 += (long long)gridDim.x * blockDim.x) {
@@ -416,6 +418,7 @@ __device__ __forceinline__ void prep_element(const PrepJob& j, long long i) {
 }
 
 __global__ void tc_prep_kernel_v(const PrepJob j) {
+  dependency_wait();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < j.nh + j.nl;
        i += (long long)gridDim.x * blockDim.x)
     prep_element(j, i);
@@ -424,6 +427,7 @@ __global__ void tc_prep_kernel_v(const PrepJob j) {
 // all plans of a batch in one launch: element i belongs to the last job
 // whose start is <= i (jobs ordered by start)
 __global__ void tc_prep_batch_kernel(const PrepJob* jobs, int n, long long total) {
+  dependency_wait();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
     int lo = 0, hi = n - 1;
@@ -891,8 +895,7 @@ PrepJob prep_job(const jet_plan_s* p, const TcPlan* t, const void* params, long 
 jet_status prep(const jet_plan_s* p, TcPlan* t, const void* params, cudaStream_t s) {
   const PrepJob j = prep_job(p, t, params, 0);
   int grid = (int)std::min<long long>((j.nh + j.nl + 255) / 256, 1024);
-  tc_prep_kernel_v<<<grid, 256, 0, s>>>(j);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_dependent(&tc_prep_kernel_v, grid, 256, 0, s, j);
   return e == cudaSuccess ? JET_OK : tcuda(e, "tc prep launch");
 }
 
@@ -943,14 +946,12 @@ jet_status run(jet_plan_s* p, TcPlan* t, int mode, const TcInst& I, cudaStream_t
     const size_t smem = (size_t)w.stages * 2 * w.chunk_bytes + 1024;
     e = cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) {
-      wgrad_kernel<<<std::min(w.n_items, t->wg_sms), kWgThreads, smem, s>>>(w);
-      e = cudaGetLastError();
+      e = launch_dependent(&wgrad_kernel, std::min(w.n_items, t->wg_sms), kWgThreads, smem, s, w);
     }
     if (e == cudaSuccess) {
       const long long tot = (long long)(L - 2) * t->wu * t->wu;
-      wgrad_sum4_kernel<<<(int)std::min<long long>((tot / 4 + 255) / 256, 2048), 256, 0, s>>>(
+      e = launch_dependent(&wgrad_sum4_kernel, (int)std::min<long long>((tot / 4 + 255) / 256, 2048), 256, 0, s,
           t->wg_out, L, t->w, t->wu, t->G, w.items_per_layer, t->hid64);
-      e = cudaGetLastError();
     }
   }
   jet::plan_prof_end(p, s);
@@ -1251,8 +1252,7 @@ jet_status tc_batch_run(TcBatch* bb, const std::vector<jet_plan_s*>& plans, cons
   }
   {
     const int pgrid = (int)std::min<long long>((prep_total + 255) / 256, 2048);
-    tc_prep_batch_kernel<<<pgrid, 256, 0, s>>>(b->d_prep, n, prep_total);
-    cudaError_t pe = cudaGetLastError();
+    const cudaError_t pe = launch_dependent(&tc_prep_batch_kernel, pgrid, 256, 0, s, b->d_prep, n, prep_total);
     if (pe != cudaSuccess) return tcuda(pe, "batched weight preparation");
   }
   TcArgs a;

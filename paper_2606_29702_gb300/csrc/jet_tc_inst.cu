@@ -19,8 +19,7 @@ template <class Shape>
 static cudaError_t launch_shape(const TcArgs& a, int grid, size_t smem, cudaStream_t s) {
   cudaError_t e = cudaFuncSetAttribute(tc_kernel<TcCls, Shape>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  tc_kernel<TcCls, Shape><<<grid, a.nthreads, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_dependent(&tc_kernel<TcCls, Shape>, grid, a.nthreads, smem, s, a);
 }
 
 #define JET_CAT2(a, b) a##b

@@ -1223,6 +1223,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_kernel(const __grid_constant
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
+  dependency_wait();  // the weights, and everything the previous call wrote
   uint32_t ph_tma = 0, ph_mma = 0, ph_ld = 0, ph_wg = 0;
   int prev_inst = -1;
   __shared__ int k_s;
