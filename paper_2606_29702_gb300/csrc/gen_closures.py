@@ -28,6 +28,7 @@ Run: python gen_closures.py <out.h>   (the build does this).
 
 import importlib.util
 import itertools
+import math
 import os
 import sys
 from collections import OrderedDict
@@ -254,13 +255,34 @@ def emit_class(name, d, chans):
                 parts.append([fma_sum([factors(c, k, zs) for c, k, zs in J[ai][bi]]), "v[%d]" % bi])
         L.append("    da[%d] = %s;" % (ai, fma_sum(parts)))
     L.append("  }")
-    # adjoint
+    # adjoint, the transposed Jacobian term by term (FP32 forms)
     L.append("  template <class T> static __device__ __forceinline__ void adjoint(const T* z, const T* p, const T* ab, T* zb) {")
     for bi in range(C):
         parts = []
         for ai in range(C):
             if J[ai][bi]:
                 parts.append([fma_sum([factors(c, k, zs) for c, k, zs in J[ai][bi]]), "ab[%d]" % ai])
+        L.append("    zb[%d] = %s;" % (bi, fma_sum(parts)))
+    L.append("  }")
+    # the same as a convolution: d a_alpha / d z_beta = binom(alpha, beta)
+    # c_{alpha - beta} with c = (phi' o u)'s jet (Leibniz: d a_alpha / d z_beta is the
+    # alpha derivative of phi(u) for a perturbation of u's beta channel), i.e. the
+    # composition with every p[k] replaced by p[k + 1].  Half the operations of the
+    # term by term form, whose rounding the FP32 forms keep (2->64x5->1 BF16X3
+    # 314 -> 305 us, 3->128x6->2 BF16, 13 channels, 5.13 -> 5.10 ms).
+    index = {c: i for i, c in enumerate(chans)}
+    L.append("  template <class T> static __device__ __forceinline__ void adjoint_conv(const T* z, const T* p, const T* ab, T* zb) {")
+    L.append("    T c[%d];" % C)
+    for ai in range(C):
+        L.append("    c[%d] = %s;" % (ai, fma_sum([factors(co, k + 1, bl) for co, k, bl in terms[ai]])))
+    for bi, be in enumerate(chans):
+        parts = []
+        for ai, al in enumerate(chans):
+            if any(x < y for x, y in zip(al, be)):
+                continue
+            n = math.prod(math.comb(x, y) for x, y in zip(al, be))
+            diff = index[tuple(x - y for x, y in zip(al, be))]
+            parts.append((["T(%d)" % n] if n > 1 else []) + ["c[%d]" % diff, "ab[%d]" % ai])
         L.append("    zb[%d] = %s;" % (bi, fma_sum(parts)))
     L.append("  }")
     L.append("};")

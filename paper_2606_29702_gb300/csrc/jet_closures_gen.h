@@ -40,6 +40,19 @@ struct Cls_d1o4 {
     zb[3] = jfma(ab[4], T(4)*p[2]*z[1], p[1]*ab[3]);
     zb[4] = p[1]*ab[4];
   }
+  template <class T> static __device__ __forceinline__ void adjoint_conv(const T* z, const T* p, const T* ab, T* zb) {
+    T c[5];
+    c[0] = p[1];
+    c[1] = p[2]*z[1];
+    c[2] = jfma(z[2], p[2], p[3]*z[1]*z[1]);
+    c[3] = jfma(z[3], p[2], jfma(z[2], T(3)*p[3]*z[1], p[4]*z[1]*z[1]*z[1]));
+    c[4] = jfma(z[4], p[2], jfma(z[2], T(3)*p[3]*z[2], jfma(z[3], T(4)*p[3]*z[1], jfma(z[2], T(6)*p[4]*z[1]*z[1], p[5]*z[1]*z[1]*z[1]*z[1]))));
+    zb[0] = jfma(ab[4], c[4], jfma(ab[3], c[3], jfma(ab[2], c[2], jfma(ab[1], c[1], c[0]*ab[0]))));
+    zb[1] = jfma(ab[4], T(4)*c[3], jfma(ab[3], T(3)*c[2], jfma(ab[2], T(2)*c[1], c[0]*ab[1])));
+    zb[2] = jfma(ab[4], T(6)*c[2], jfma(ab[3], T(3)*c[1], c[0]*ab[2]));
+    zb[3] = jfma(ab[4], T(4)*c[1], c[0]*ab[3]);
+    zb[4] = c[0]*ab[4];
+  }
 };
 
 // d2o2: d=2, channels 00 10 01 20 11 02
@@ -75,6 +88,21 @@ struct Cls_d2o2 {
     zb[3] = p[1]*ab[3];
     zb[4] = p[1]*ab[4];
     zb[5] = p[1]*ab[5];
+  }
+  template <class T> static __device__ __forceinline__ void adjoint_conv(const T* z, const T* p, const T* ab, T* zb) {
+    T c[6];
+    c[0] = p[1];
+    c[1] = p[2]*z[1];
+    c[2] = p[2]*z[2];
+    c[3] = jfma(z[3], p[2], p[3]*z[1]*z[1]);
+    c[4] = jfma(z[4], p[2], p[3]*z[1]*z[2]);
+    c[5] = jfma(z[5], p[2], p[3]*z[2]*z[2]);
+    zb[0] = jfma(ab[5], c[5], jfma(ab[4], c[4], jfma(ab[3], c[3], jfma(ab[2], c[2], jfma(ab[1], c[1], c[0]*ab[0])))));
+    zb[1] = jfma(ab[4], c[2], jfma(ab[3], T(2)*c[1], c[0]*ab[1]));
+    zb[2] = jfma(ab[5], T(2)*c[2], jfma(ab[4], c[1], c[0]*ab[2]));
+    zb[3] = c[0]*ab[3];
+    zb[4] = c[0]*ab[4];
+    zb[5] = c[0]*ab[5];
   }
 };
 
@@ -124,6 +152,29 @@ struct Cls_d3o2 {
     zb[8] = p[1]*ab[8];
     zb[9] = p[1]*ab[9];
   }
+  template <class T> static __device__ __forceinline__ void adjoint_conv(const T* z, const T* p, const T* ab, T* zb) {
+    T c[10];
+    c[0] = p[1];
+    c[1] = p[2]*z[1];
+    c[2] = p[2]*z[2];
+    c[3] = p[2]*z[3];
+    c[4] = jfma(z[4], p[2], p[3]*z[1]*z[1]);
+    c[5] = jfma(z[5], p[2], p[3]*z[1]*z[2]);
+    c[6] = jfma(z[6], p[2], p[3]*z[1]*z[3]);
+    c[7] = jfma(z[7], p[2], p[3]*z[2]*z[2]);
+    c[8] = jfma(z[8], p[2], p[3]*z[2]*z[3]);
+    c[9] = jfma(z[9], p[2], p[3]*z[3]*z[3]);
+    zb[0] = jfma(ab[9], c[9], jfma(ab[8], c[8], jfma(ab[7], c[7], jfma(ab[6], c[6], jfma(ab[5], c[5], jfma(ab[4], c[4], jfma(ab[3], c[3], jfma(ab[2], c[2], jfma(ab[1], c[1], c[0]*ab[0])))))))));
+    zb[1] = jfma(ab[6], c[3], jfma(ab[5], c[2], jfma(ab[4], T(2)*c[1], c[0]*ab[1])));
+    zb[2] = jfma(ab[8], c[3], jfma(ab[7], T(2)*c[2], jfma(ab[5], c[1], c[0]*ab[2])));
+    zb[3] = jfma(ab[9], T(2)*c[3], jfma(ab[8], c[2], jfma(ab[6], c[1], c[0]*ab[3])));
+    zb[4] = c[0]*ab[4];
+    zb[5] = c[0]*ab[5];
+    zb[6] = c[0]*ab[6];
+    zb[7] = c[0]*ab[7];
+    zb[8] = c[0]*ab[8];
+    zb[9] = c[0]*ab[9];
+  }
 };
 
 // burgers: d=2, channels 00 10 01 20
@@ -153,6 +204,17 @@ struct Cls_burgers {
     zb[1] = jfma(ab[3], T(2)*p[2]*z[1], p[1]*ab[1]);
     zb[2] = p[1]*ab[2];
     zb[3] = p[1]*ab[3];
+  }
+  template <class T> static __device__ __forceinline__ void adjoint_conv(const T* z, const T* p, const T* ab, T* zb) {
+    T c[4];
+    c[0] = p[1];
+    c[1] = p[2]*z[1];
+    c[2] = p[2]*z[2];
+    c[3] = jfma(z[3], p[2], p[3]*z[1]*z[1]);
+    zb[0] = jfma(ab[3], c[3], jfma(ab[2], c[2], jfma(ab[1], c[1], c[0]*ab[0])));
+    zb[1] = jfma(ab[3], T(2)*c[1], c[0]*ab[1]);
+    zb[2] = c[0]*ab[2];
+    zb[3] = c[0]*ab[3];
   }
 };
 
@@ -189,6 +251,21 @@ struct Cls_ks {
     zb[3] = jfma(ab[5], jfma(z[3], T(6)*p[2], T(6)*p[3]*z[1]*z[1]), jfma(ab[4], T(3)*p[2]*z[1], p[1]*ab[3]));
     zb[4] = jfma(ab[5], T(4)*p[2]*z[1], p[1]*ab[4]);
     zb[5] = p[1]*ab[5];
+  }
+  template <class T> static __device__ __forceinline__ void adjoint_conv(const T* z, const T* p, const T* ab, T* zb) {
+    T c[6];
+    c[0] = p[1];
+    c[1] = p[2]*z[1];
+    c[2] = p[2]*z[2];
+    c[3] = jfma(z[3], p[2], p[3]*z[1]*z[1]);
+    c[4] = jfma(z[4], p[2], jfma(z[3], T(3)*p[3]*z[1], p[4]*z[1]*z[1]*z[1]));
+    c[5] = jfma(z[5], p[2], jfma(z[3], T(3)*p[3]*z[3], jfma(z[4], T(4)*p[3]*z[1], jfma(z[3], T(6)*p[4]*z[1]*z[1], p[5]*z[1]*z[1]*z[1]*z[1]))));
+    zb[0] = jfma(ab[5], c[5], jfma(ab[4], c[4], jfma(ab[3], c[3], jfma(ab[2], c[2], jfma(ab[1], c[1], c[0]*ab[0])))));
+    zb[1] = jfma(ab[5], T(4)*c[4], jfma(ab[4], T(3)*c[3], jfma(ab[3], T(2)*c[1], c[0]*ab[1])));
+    zb[2] = c[0]*ab[2];
+    zb[3] = jfma(ab[5], T(6)*c[3], jfma(ab[4], T(3)*c[1], c[0]*ab[3]));
+    zb[4] = jfma(ab[5], T(4)*c[1], c[0]*ab[4]);
+    zb[5] = c[0]*ab[5];
   }
 };
 
@@ -228,6 +305,23 @@ struct Cls_helmholtz {
     zb[4] = p[1]*ab[4];
     zb[5] = p[1]*ab[5];
     zb[6] = p[1]*ab[6];
+  }
+  template <class T> static __device__ __forceinline__ void adjoint_conv(const T* z, const T* p, const T* ab, T* zb) {
+    T c[7];
+    c[0] = p[1];
+    c[1] = p[2]*z[1];
+    c[2] = p[2]*z[2];
+    c[3] = p[2]*z[3];
+    c[4] = jfma(z[4], p[2], p[3]*z[1]*z[1]);
+    c[5] = jfma(z[5], p[2], p[3]*z[2]*z[2]);
+    c[6] = jfma(z[6], p[2], p[3]*z[3]*z[3]);
+    zb[0] = jfma(ab[6], c[6], jfma(ab[5], c[5], jfma(ab[4], c[4], jfma(ab[3], c[3], jfma(ab[2], c[2], jfma(ab[1], c[1], c[0]*ab[0]))))));
+    zb[1] = jfma(ab[4], T(2)*c[1], c[0]*ab[1]);
+    zb[2] = jfma(ab[5], T(2)*c[2], c[0]*ab[2]);
+    zb[3] = jfma(ab[6], T(2)*c[3], c[0]*ab[3]);
+    zb[4] = c[0]*ab[4];
+    zb[5] = c[0]*ab[5];
+    zb[6] = c[0]*ab[6];
   }
 };
 
@@ -286,6 +380,35 @@ struct Cls_ns_psi {
     zb[11] = p[1]*ab[11];
     zb[12] = p[1]*ab[12];
   }
+  template <class T> static __device__ __forceinline__ void adjoint_conv(const T* z, const T* p, const T* ab, T* zb) {
+    T c[13];
+    c[0] = p[1];
+    c[1] = p[2]*z[1];
+    c[2] = p[2]*z[2];
+    c[3] = p[2]*z[3];
+    c[4] = jfma(z[4], p[2], p[3]*z[1]*z[1]);
+    c[5] = jfma(z[5], p[2], p[3]*z[1]*z[2]);
+    c[6] = jfma(z[6], p[2], p[3]*z[1]*z[3]);
+    c[7] = jfma(z[7], p[2], p[3]*z[2]*z[2]);
+    c[8] = jfma(z[8], p[2], p[3]*z[2]*z[3]);
+    c[9] = jfma(z[9], p[2], jfma(z[4], T(3)*p[3]*z[1], p[4]*z[1]*z[1]*z[1]));
+    c[10] = jfma(z[10], p[2], jfma(z[5], T(2)*p[3]*z[1], jfma(z[4], p[3]*z[2], p[4]*z[1]*z[1]*z[2])));
+    c[11] = jfma(z[11], p[2], jfma(z[7], p[3]*z[1], jfma(z[5], T(2)*p[3]*z[2], p[4]*z[1]*z[2]*z[2])));
+    c[12] = jfma(z[12], p[2], jfma(z[7], T(3)*p[3]*z[2], p[4]*z[2]*z[2]*z[2]));
+    zb[0] = jfma(ab[12], c[12], jfma(ab[11], c[11], jfma(ab[10], c[10], jfma(ab[9], c[9], jfma(ab[8], c[8], jfma(ab[7], c[7], jfma(ab[6], c[6], jfma(ab[5], c[5], jfma(ab[4], c[4], jfma(ab[3], c[3], jfma(ab[2], c[2], jfma(ab[1], c[1], c[0]*ab[0]))))))))))));
+    zb[1] = jfma(ab[11], c[7], jfma(ab[10], T(2)*c[5], jfma(ab[9], T(3)*c[4], jfma(ab[6], c[3], jfma(ab[5], c[2], jfma(ab[4], T(2)*c[1], c[0]*ab[1]))))));
+    zb[2] = jfma(ab[12], T(3)*c[7], jfma(ab[11], T(2)*c[5], jfma(ab[10], c[4], jfma(ab[8], c[3], jfma(ab[7], T(2)*c[2], jfma(ab[5], c[1], c[0]*ab[2]))))));
+    zb[3] = jfma(ab[8], c[2], jfma(ab[6], c[1], c[0]*ab[3]));
+    zb[4] = jfma(ab[10], c[2], jfma(ab[9], T(3)*c[1], c[0]*ab[4]));
+    zb[5] = jfma(ab[11], T(2)*c[2], jfma(ab[10], T(2)*c[1], c[0]*ab[5]));
+    zb[6] = c[0]*ab[6];
+    zb[7] = jfma(ab[12], T(3)*c[2], jfma(ab[11], c[1], c[0]*ab[7]));
+    zb[8] = c[0]*ab[8];
+    zb[9] = c[0]*ab[9];
+    zb[10] = c[0]*ab[10];
+    zb[11] = c[0]*ab[11];
+    zb[12] = c[0]*ab[12];
+  }
 };
 
 // ns_uvp: d=2, channels 00 10 01 20 02
@@ -318,6 +441,19 @@ struct Cls_ns_uvp {
     zb[2] = jfma(ab[4], T(2)*p[2]*z[2], p[1]*ab[2]);
     zb[3] = p[1]*ab[3];
     zb[4] = p[1]*ab[4];
+  }
+  template <class T> static __device__ __forceinline__ void adjoint_conv(const T* z, const T* p, const T* ab, T* zb) {
+    T c[5];
+    c[0] = p[1];
+    c[1] = p[2]*z[1];
+    c[2] = p[2]*z[2];
+    c[3] = jfma(z[3], p[2], p[3]*z[1]*z[1]);
+    c[4] = jfma(z[4], p[2], p[3]*z[2]*z[2]);
+    zb[0] = jfma(ab[4], c[4], jfma(ab[3], c[3], jfma(ab[2], c[2], jfma(ab[1], c[1], c[0]*ab[0]))));
+    zb[1] = jfma(ab[3], T(2)*c[1], c[0]*ab[1]);
+    zb[2] = jfma(ab[4], T(2)*c[2], c[0]*ab[2]);
+    zb[3] = c[0]*ab[3];
+    zb[4] = c[0]*ab[4];
   }
 };
 

@@ -808,7 +808,7 @@ struct TcTile {
           }
           z[0] = z[0] + f2(bu);
           tanh_derivs_fast2<NP>(z[0], p);
-          Cls::adjoint(z, p, ab, zb);
+          Cls::adjoint_conv(z, p, ab, zb);
 #pragma unroll
           for (int c = 0; c < C; ++c) {
             zbv[c][j] = zb[c].v.x;
@@ -942,7 +942,7 @@ struct TcTile {
             if (fo >= 0) z[fo] = f2(w1[i]);
           }
           tanh_derivs_fast2<NP>(z[0], p);
-          Cls::adjoint(z, p, ab, zb);
+          Cls::adjoint_conv(z, p, ab, zb);
           gb += zb[0].v.x;
           gb += zb[0].v.y;
 #pragma unroll
