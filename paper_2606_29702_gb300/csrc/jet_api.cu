@@ -146,16 +146,17 @@ void below(const Alpha& a, std::set<Alpha>& out) {
   }
 }
 
-size_t simt_tile_smem(const jet_plan_s* p, int P, int ru, int threads) {
-  const int pitch = simt_pitch(p->C, P, p->wmax, simt_wgrad_rows(ru), threads, p->elem);
+size_t simt_tile_smem(const jet_plan_s* p, int P, int threads) {
+  const int pitch = simt_pitch(p->C, P, p->wmax, threads, p->elem);
   return simt_smem_bytes(p->C, P, pitch, p->wmax, p->n_out, p->d, p->elem);
 }
 
 // most points per tile that `ctas` CTAs of `threads` per SM can hold, at most
-// one item of the jet GEMMs per thread (FP64: two)
+// one item of the jet GEMMs per thread (FP64: two), in whole groups of points
 int simt_most_points(const jet_plan_s* p, int ru, int threads, int ctas) {
-  int P = std::max(2, threads * std::max(ru, 2) / p->wmax / 2 * 2);
-  while (P > 2 && (simt_tile_smem(p, P, ru, threads) + kSimtCtaBytes) * ctas > kSimtSmBytes) P -= 2;
+  const int step = p->P0 ? p->P0 : 2;
+  int P = std::max(step, threads * std::max(ru, 2) / p->wmax / step * step);
+  while (P > step && (simt_tile_smem(p, P, threads) + kSimtCtaBytes) * ctas > kSimtSmBytes) P -= step;
   return P;
 }
 
@@ -167,6 +168,7 @@ int simt_most_points(const jet_plan_s* p, int ru, int threads, int ctas) {
 // lanes per SM, not by the tile.
 void simt_shape(jet_plan_s* p, int p8) {
   p->threads = kSimtThreads;
+  p->P0 = p->fp64 ? 0 : p8 ? 8 * p8 : simt_group_points(p->wmax);
   if (p8) {
     p->P = 8 * p8;
     p->P_fixed = true;
@@ -187,15 +189,19 @@ void simt_shape(jet_plan_s* p, int p8) {
 // tile costs whatever its size (its barriers and latencies).  FP32 warps count
 // in fours, one per scheduler of the SM: six warps take as long as eight.
 constexpr double kTileWarps = 2.0;
+double simt_tile_cost(const jet_plan_s* p, int P) {
+  int warps = (p->wmax / p->ru * P + 31) / 32;
+  if (!p->fp64) warps = (warps + 3) / 4 * 4;
+  return warps + kTileWarps;
+}
 int simt_call_points(const jet_plan_s* p, long long N) {
   if (p->P_fixed) return p->P;
+  const int step = p->P0 ? p->P0 : 2;
   int best = p->P;
   double best_cost = 0.0;
-  for (int P = p->P; P >= 2; P -= 2) {
+  for (int P = p->P; P >= step; P -= step) {
     const long long tiles = (N + P - 1) / P, per_sm = (tiles + p->sms - 1) / p->sms;
-    int warps = (p->wmax / p->ru * P + 31) / 32;
-    if (!p->fp64) warps = (warps + 3) / 4 * 4;
-    const double cost = (double)per_sm * (warps + kTileWarps);
+    const double cost = (double)per_sm * simt_tile_cost(p, P);
     if (P == p->P || cost < best_cost) {
       best = P;
       best_cost = cost;
@@ -204,6 +210,45 @@ int simt_call_points(const jet_plan_s* p, long long N) {
   // the z-jet store holds whole tiles: near its capacity the largest tile
   const bool stored = p->store && N <= p->store_max_points;
   return stored && (N + best - 1) / best * best > p->store_max_points ? p->P : best;
+}
+
+// Most chunks that FP32 sums are kept for: 2 per SM (1 for channel sets of 10 or
+// more).  With FP32 sums a call's chunks are whole groups of P0 points, N and the
+// plan alone fix them, and a tile takes up to P / P0 groups of one chunk: every
+// sum is formed in the same order whatever the tile.
+int simt_sum_chunks(const jet_plan_s* p) {
+  const int P = p->P0, S0 = simt_swap(p->C, P) ? p->C + 1 : p->C;
+  int pitch = S0 * P;
+  while (pitch % 32 != 4) ++pitch;
+  const size_t smem = (3 * (size_t)p->wmax * pitch + 2 * (size_t)p->n_out * p->C * P + (size_t)P * p->d) * 4 + 512;
+  const int per_sm = p->C >= 10 ? 1 : (int)std::min<size_t>(2, kSimtSmBytes / (smem + 1024));
+  return p->sms * std::max(1, per_sm);
+}
+void simt_sum_tiling(const jet_plan_s* p, DevInstance& I) {
+  I.unit = p->P0;
+  I.n_tiles = (I.N + I.unit - 1) / I.unit;
+  const long long most = std::max<long long>(1, std::min<long long>(I.n_tiles, p->sum_chunks));
+  I.tiles_per_chunk = (int)((I.n_tiles + most - 1) / most);
+  I.chunk_rem = 0;
+  I.n_chunks = (int)((I.n_tiles + I.tiles_per_chunk - 1) / I.tiles_per_chunk);
+  if (p->P_fixed || p->store) {
+    I.P = p->P0;
+    return;
+  }
+  // groups per tile: least time of the busiest SM; whole runs of kWaccTiles
+  // groups where a chunk takes several
+  const long long per_sm = (I.n_chunks + p->sms - 1) / p->sms;
+  const bool runs = p->C >= 7 && I.tiles_per_chunk > kWaccTiles;
+  double best_cost = 0.0;
+  I.P = p->P0;
+  for (int V = p->P / p->P0; V >= 1; --V) {
+    if (runs && kWaccTiles % V) continue;
+    const double cost = (double)per_sm * ((I.tiles_per_chunk + V - 1) / V) * simt_tile_cost(p, V * p->P0);
+    if (best_cost == 0.0 || cost < best_cost) {
+      I.P = V * p->P0;
+      best_cost = cost;
+    }
+  }
 }
 
 }  // namespace
@@ -371,7 +416,7 @@ static jet_status plan_create(jet_plan_t* out, int n_specs, const jet_residual_s
   for (int l = 1; l < n_layers; ++l) p->wmax = std::max(p->wmax, widths[l]);
   p->ru = simt_units(widths, n_layers, p->fp64);
   simt_shape(p, JET_FLAG_TILE_GET(flags));
-  p->smem = simt_tile_smem(p, p->P, p->ru, p->threads);
+  p->smem = simt_tile_smem(p, p->P, p->threads);
   cudaDeviceProp prop;
   cudaError_t e = cudaGetDeviceProperties(&prop, p->device);
   if (e != cudaSuccess) {
@@ -398,13 +443,16 @@ static jet_status plan_create(jet_plan_t* out, int n_specs, const jet_residual_s
     // FP32 forms whose per-chunk FP64 slices would not stay in L2 sum the
     // hidden-layer weights of a chunk in FP32; otherwise per-tile FP64 adds into
     // L2-resident slices are the cheaper of the two
-    const bool slices_fit = (double)p->grid * p->n_params * sizeof(double) <= kSimtSliceL2Bytes;
+    const int chunks = p->fp64 ? p->grid : std::max(p->grid, simt_sum_chunks(p));
+    const bool slices_fit =
+        p->fp64 || (double)simt_sum_chunks(p) * p->n_params * sizeof(double) <= kSimtSliceL2Bytes;
     p->wsums_stride = slices_fit ? 0 : simt_wacc_elems(widths, n_layers, p->fp64);
+    p->sum_chunks = p->wsums_stride ? simt_sum_chunks(p) : 0;
     p->scratch_stride = jet_elems;
-    const size_t b_ws = (size_t)p->grid * p->wsums_stride * sizeof(float);
+    const size_t b_ws = (size_t)chunks * p->wsums_stride * sizeof(float);
     size_t b_wt = (size_t)weight_ws_elems(p->n_params) * p->elem;
-    size_t b_gs = (size_t)p->grid * p->n_params * sizeof(double);
-    size_t b_ls = (size_t)p->grid * sizeof(double);
+    size_t b_gs = (size_t)chunks * p->n_params * sizeof(double);
+    size_t b_ls = (size_t)chunks * sizeof(double);
     size_t b_sc = (size_t)p->grid * p->scratch_stride * p->elem;
     Arena arena;
     arena.add(&p->Wt, b_wt);
@@ -545,10 +593,12 @@ jet_status jet_plan_destroy(jet_plan_t p) {
 
 namespace {
 
-// Fill the per-call instance descriptor of the SIMT kernel, for tiles of P
-// points in CTAs of `threads` with ru units per GEMM thread.
+// Fill the per-call instance descriptor of the SIMT kernel, for CTAs of
+// `threads` with ru units per GEMM thread: the call's own tiles and chunks
+// (want_grad: those of its FP32 sums, if it keeps any; a forward pass without a
+// z-jet store takes any), or (batches) tiles of P points in `chunks` chunks.
 void fill_instance(const jet_plan_s* p, const void* params, const void* X, long long N, const void* source,
-                   void* r_out, int P, int ru, int threads, int max_chunks, DevInstance& I) {
+                   void* r_out, bool want_grad, int ru, int threads, int P, int chunks, DevInstance& I) {
   memset(&I, 0, sizeof(I));
   I.L = p->L;
   I.d = p->d;
@@ -573,15 +623,24 @@ void fill_instance(const jet_plan_s* p, const void* params, const void* X, long 
     I.inv_N = 1.0;  // each term's mean is in its scale
     I.n_groups = fill_groups(p, I.groups);
   }
-  I.P = P;
-  I.pitch = simt_pitch(p->C, P, p->wmax, simt_wgrad_rows(ru), threads, p->elem);
-  I.n_tiles = (N + I.P - 1) / I.P;
-  simt_set_chunks(I, max_chunks);
+  if (P > 0) {
+    I.P = P;
+    simt_set_chunks(I, chunks);
+  } else if (p->sum_chunks && (want_grad || p->store)) {
+    simt_sum_tiling(p, I);
+  } else {
+    I.P = simt_call_points(p, N);
+    simt_set_chunks(I, p->grid);
+  }
+  I.P0 = p->fp64 ? I.P : p->P0;
+  I.swap = p->fp64 ? 0 : simt_swap(p->C, I.P0);
+  I.wr = simt_wgrad_rows(ru, p->wmax, I.P / I.P0, threads, p->fp64);
+  I.pitch = simt_pitch(p->C, I.P, p->wmax, threads, p->elem);
   I.chunk_base = 0;
   I.grad_slices = p->grad_slices;
   I.loss_slices = p->loss_slices;
   I.store = nullptr;
-  for (int l = 1; l < p->L; ++l) I.store_tile_stride += (long long)p->C * P * p->widths[l];
+  for (int l = 1; l < p->L; ++l) I.store_tile_stride += (long long)p->C * I.P * p->widths[l];
   simt_set_sums(I, p->C, p->wsums, p->wsums_stride);
 }
 
@@ -622,7 +681,7 @@ jet_status run_simt(jet_plan_s* p, int mode, const DevInstance& I, cudaStream_t 
   return JET_OK;
 }
 
-ReduceJob make_job(const DevInstance& I, int ru, void* grad_out, double* loss_out, bool with_grad) {
+ReduceJob make_job(const DevInstance& I, void* grad_out, double* loss_out, bool with_grad) {
   ReduceJob j;
   memset(&j, 0, sizeof(j));
   j.grad_slices = I.grad_slices;
@@ -636,7 +695,7 @@ ReduceJob make_job(const DevInstance& I, int ru, void* grad_out, double* loss_ou
     for (int l = 0; l <= I.L; ++l) j.widths[l] = I.widths[l];
     j.n_hid = (int)I.wsums_stride;
     j.subs = 1;
-    j.wr = simt_wgrad_rows(ru);
+    j.wr = I.wr;
     j.hid_sums = I.wsums;
     j.hid_stride = I.wsums_stride;
   }
@@ -661,13 +720,13 @@ jet_status jet_forward_residual(jet_plan_t p, const void* params, const void* X,
     return JET_OK;
   }
   DevInstance I;
-  fill_instance(p, params, X, N, source, r_out, simt_call_points(p, N), p->ru, p->threads, p->grid, I);
+  fill_instance(p, params, X, N, source, r_out, false, p->ru, p->threads, 0, 0, I);
   const bool store = p->store && N <= p->store_max_points;
   if (store) I.store = p->store;
   CK(launch_transpose_weights(I, p->fp64, p->Wt, s));
   st = run_simt(p, MODE_FWD, I, s);
   if (st != JET_OK) return st;
-  ReduceJob j = make_job(I, p->ru, nullptr, loss_out, false);
+  ReduceJob j = make_job(I, nullptr, loss_out, false);
   if (loss_out) CK(launch_reduce(&j, nullptr, 1, p->fp64, false, 1, 0.f, s));
   p->st_valid = store;
   p->st_params = params;
@@ -690,14 +749,14 @@ jet_status jet_backward_params(jet_plan_t p, const void* params, const void* X, 
     return JET_OK;
   }
   DevInstance I;
-  fill_instance(p, params, X, N, source, r_out, simt_call_points(p, N), p->ru, p->threads, p->grid, I);
+  fill_instance(p, params, X, N, source, r_out, true, p->ru, p->threads, 0, 0, I);
   const bool from_store = p->st_valid && p->st_params == params && p->st_X == X && p->st_N == N &&
                           p->st_src == source;
   if (from_store) I.store = p->store;
   CK(launch_transpose_weights(I, p->fp64, p->Wt, s));
   st = run_simt(p, from_store ? MODE_BWD_STORE : MODE_FWD_BWD, I, s);
   if (st != JET_OK) return st;
-  ReduceJob j = make_job(I, p->ru, grad_out, loss_out, true);
+  ReduceJob j = make_job(I, grad_out, loss_out, true);
   CK(launch_reduce(&j, nullptr, 1, p->fp64, false, 1, 0.f, s));
   return JET_OK;
 }
@@ -715,11 +774,11 @@ static jet_status train_step(jet_plan_t p, void* params, void* adam_m, void* ada
   p->st_valid = false;  // params change in place
   if (p->tc) return tc_train_step(p, p->tcp, params, adam_m, adam_v, step, step_ctr, lr, X, N, source, loss_out, s);
   DevInstance I;
-  fill_instance(p, params, X, N, source, nullptr, simt_call_points(p, N), p->ru, p->threads, p->grid, I);
+  fill_instance(p, params, X, N, source, nullptr, true, p->ru, p->threads, 0, 0, I);
   CK(launch_transpose_weights(I, p->fp64, p->Wt, s));
   st = run_simt(p, MODE_FWD_BWD, I, s);
   if (st != JET_OK) return st;
-  ReduceJob j = make_job(I, p->ru, nullptr, loss_out, true);
+  ReduceJob j = make_job(I, nullptr, loss_out, true);
   j.params = params;
   j.m = adam_m;
   j.v = adam_v;
@@ -840,8 +899,8 @@ jet_status batch_prepare(jet_batch_s* b, const void* const* params, const void* 
     const double per_tile = tile_cost(i);
     const long long want = std::min<long long>(
         b->max_chunks_per_inst, std::max<long long>(1, (long long)(per_tile * (double)tiles / target + 0.5)));
-    fill_instance(p, params[i], X[i], N[i], source ? source[i] : nullptr, r_out ? r_out[i] : nullptr, b->P[i], b->ru,
-                  kSimtThreads, (int)want, I);
+    fill_instance(p, params[i], X[i], N[i], source ? source[i] : nullptr, r_out ? r_out[i] : nullptr, true, b->ru,
+                  kSimtThreads, b->P[i], (int)want, I);
     I.Wt = (char*)b->Wt + b->wt_off[i] * p->elem;
     I.grad_slices = b->grad_slices + b->slice_off[i];
     simt_set_sums(I, p->C, p->wsums ? b->wsums + b->wsums_off[i] : nullptr, p->wsums_stride);
@@ -909,7 +968,7 @@ jet_status jet_batch_create(jet_batch_t* out, int32_t n, const jet_plan_t* plans
     if (!plans[i]->P_fixed)
       P = std::min(P, simt_most_points(plans[i], b->ru, kSimtThreads, !b->fp64 && plans[i]->C >= 10 ? 1 : 2));
     b->P.push_back(P);
-    smem = std::max(smem, simt_tile_smem(plans[i], P, b->ru, kSimtThreads));
+    smem = std::max(smem, simt_tile_smem(plans[i], P, kSimtThreads));
   }
   b->smem = smem;
   int per_sm = 0, dev = 0;
@@ -986,7 +1045,7 @@ static jet_status batch_run(jet_batch_t b, const void* const* params, void* cons
   CK(cudaMemsetAsync(b->d_next, 0, sizeof(int), s));
   CK(simt_launch(b->cls, b->fp64, a, std::min(b->grid, n_items), b->smem, s));
   for (int i = 0; i < n; ++i) {
-    ReduceJob j = make_job(b->h_insts[i], b->ru, adam ? nullptr : grad_out[i], loss_out ? loss_out + i : nullptr, true);
+    ReduceJob j = make_job(b->h_insts[i], adam ? nullptr : grad_out[i], loss_out ? loss_out + i : nullptr, true);
     if (adam) {
       j.params = (void*)params[i];
       j.m = adam_m[i];

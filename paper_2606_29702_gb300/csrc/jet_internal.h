@@ -67,9 +67,13 @@ struct alignas(16) DevInstance {
   DevGroup groups[kMaxGroups];
   // tiling
   int P;               // points per tile
+  int P0;              // FP32 SIMT forms: points per weight-gradient group (P = V * P0); FP64: P
+  int swap;            // odd points keep their channels in swapped pairs (simt_swap)
+  int wr;              // rows of a weight-gradient item
+  int unit;            // points per unit of the chunk partition (P or P0)
   int pitch;           // smem row pitch (elements) of a jet buffer, >= C * P
-  long long n_tiles;
-  int tiles_per_chunk;  // of every chunk; the first chunk_rem chunks take one more
+  long long n_tiles;    // partition units
+  int tiles_per_chunk;  // units of every chunk; the first chunk_rem chunks take one more
   int chunk_rem;
   int n_chunks;
   int chunk_base;      // first work-item index of this instance
@@ -137,23 +141,34 @@ __host__ __device__ inline int simt_slab_elems(int wmax, size_t elem) {
   const int cap = (wmax <= 64 ? 4096 : wmax <= 128 ? 8192 : 16384) / (int)elem, need = wmax * wmax;
   return need < cap ? need : cap;
 }
-// Adjacent lanes that share a weight-gradient item (wr rows x 4 columns), each
-// summing every NS-th vector of jet columns: as many as fill the CTA.  FP32
-// items keep at least 4 sums per lane (one vector reduction).
-__host__ __device__ inline int simt_wgrad_slices(int items, int wr, bool f32, int threads) {
-  const int most = f32 && wr == 4 ? 4 : 8;
+// FP64 form: adjacent lanes that share a weight-gradient item (4 x 4), each
+// summing every NS-th vector of jet columns: as many as fill the CTA.
+__host__ __device__ inline int simt_wgrad_slices(int items, int threads) {
   int ns = 1;
-  while (ns < most && items * ns * 2 <= threads) ns *= 2;
+  while (ns < 8 && items * ns * 2 <= threads) ns *= 2;
   return ns;
 }
+// FP32 forms: the FP32 sums of a weight gradient run over groups of P0 points in
+// two chains, the even and the odd columns of a point stride of S0 = C or C | 1,
+// whatever the tile: tiles of V groups leave every sum as a tile of one group
+// forms it, and the rounding of a gradient does not depend on the tile.
+inline int simt_group_points(int wmax) { return 4 * (256 / wmax > 0 ? 256 / wmax : 1); }
+// Where S0 = C | 1 != C (C even), the even columns of an odd point are its odd
+// channels: such points keep their channels in swapped pairs, so that column
+// parity is chain parity at the dense stride C too.
+inline int simt_swap(int C, int P0) {
+  const int lanes = P0 < 32 ? P0 : 32;
+  return C % 2 == 0 && (C & -C) * lanes > 32 ? 1 : 0;
+}
 // Row pitch (elements) of a SIMT jet buffer of C * P columns.  The weight
-// gradient's 16-byte loads walk 8 / NS rows x NS vectors per quarter warp: the
-// pitch in 16-byte units is NS modulo 2 NS, so that they hit distinct banks.
-inline int simt_pitch(int C, int P, int wmax, int wr, int threads, size_t elem) {
+// gradient's 16-byte loads walk 8 rows per quarter warp (FP64: 8 / NS rows x NS
+// vectors): the pitch in 16-byte units is odd (NS modulo 2 NS), so that they hit
+// distinct banks.
+inline int simt_pitch(int C, int P, int wmax, int threads, size_t elem) {
   const int v = 16 / (int)elem;
-  const int ns = simt_wgrad_slices((wmax / wr) * (wmax / 4), wr, elem == 4, threads);
+  const int ns = elem == 4 ? 1 : simt_wgrad_slices((wmax / 4) * (wmax / 4), threads);
   int p = (C * P + v - 1) / v * v;
-  while ((p / v) % (2 * ns) != ns % (2 * ns)) p += v;
+  while ((p / v) % (2 * ns) != ns) p += v;
   return p;
 }
 // Consecutive units per thread of the SIMT jet GEMMs.  FP64 takes one: its pipe
@@ -165,7 +180,13 @@ inline int simt_units(const int* widths, int L, bool fp64) {
     if (widths[l] % 8) return 4;
   return 8;
 }
-inline int simt_wgrad_rows(int ru) { return ru == 8 ? 8 : 4; }
+// Rows of a weight-gradient item (x 4 columns): 4, fewer where that leaves threads
+// without one (8 rows read a quarter fewer words per FMA, but their 32 packed
+// sums spilled: 2->64x5->1, C = 6, 1.37 ms against 1.32 ms).
+inline int simt_wgrad_rows(int ru, int wmax, int V, int threads, bool fp64) {
+  const bool few = (long long)(wmax / 4) * (wmax / 4) * (V > 1 ? 2 : 1) < threads;
+  return fp64 || !few ? 4 : ru == 8 ? 2 : 1;
+}
 constexpr int kWaccTiles = 64;     // tiles per FP32 weight-gradient run (channel sets of 7 or more)
 // share of L2 the per-chunk FP64 gradient slices may take before the kernels
 // accumulate a chunk's weight gradients in FP32 instead of adding per tile
@@ -201,21 +222,24 @@ inline int simt_carveout(size_t smem, int ctas) {
   const size_t pct = ((smem + kSimtCtaBytes) * ctas * 100 + kSimtSmBytes - 1) / kSimtSmBytes;
   return pct > 100 ? 100 : (int)pct;
 }
-// the chunks of a call: n_tiles tiles over n_chunks CTAs or work items
+// the chunks of a call: its units (tiles) over n_chunks CTAs or work items
 inline void simt_set_chunks(DevInstance& I, long long n_chunks) {
+  I.unit = I.P;
+  I.n_tiles = (I.N + I.unit - 1) / I.unit;
   if (n_chunks > I.n_tiles) n_chunks = I.n_tiles;
   if (n_chunks < 1) n_chunks = 1;
   I.n_chunks = (int)n_chunks;
   I.tiles_per_chunk = (int)(I.n_tiles / n_chunks);
   I.chunk_rem = (int)(I.n_tiles % n_chunks);
 }
+
 // Where a call's weight-gradient sums go (after simt_set_chunks).  With FP32 sums
 // the reduction reads them, unless a chunk of a wide channel set has more tiles
 // than one run.
 inline void simt_set_sums(DevInstance& I, int C, float* wsums, long long stride) {
   I.wsums = wsums;
   I.wsums_stride = stride;
-  I.wsums_direct = wsums && (C < 7 || I.tiles_per_chunk + (I.chunk_rem > 0 ? 1 : 0) <= kWaccTiles) ? 1 : 0;
+  I.wsums_direct = wsums && (C < 7 || (I.tiles_per_chunk + (I.chunk_rem > 0 ? 1 : 0)) * (I.unit / I.P0) <= kWaccTiles) ? 1 : 0;
   if (I.wsums_direct) {
     I.n_slice = slice_map(I.widths, I.L, I.goff_b, &I.goff_WL);
   } else {

@@ -208,8 +208,10 @@ extern "C" jet_status jet_backward_params_noalloc(const jet_residual_spec* spec,
   const int TP = fp64 ? 2 : 4;
   const int P = TP * (kSimtThreads / wmax > 0 ? kSimtThreads / wmax : 1);
   const int ru = simt_units(widths, n_layers, fp64);
-  const int pitch = simt_pitch(C, P, wmax, simt_wgrad_rows(ru), kSimtThreads, elem);
-  I.P = P;
+  const int pitch = simt_pitch(C, P, wmax, kSimtThreads, elem);
+  I.P = I.P0 = P;
+  I.swap = fp64 ? 0 : simt_swap(C, P);
+  I.wr = simt_wgrad_rows(ru, wmax, 1, kSimtThreads, fp64);
   I.pitch = pitch;
   I.n_tiles = (N + P - 1) / P;
   const size_t smem = simt_smem_bytes(C, P, pitch, wmax, n_out, d_in, elem);

@@ -61,6 +61,8 @@ struct jet_plan_s {
   int P = 0;               // points per tile (SIMT forms: the most a call takes)
   bool P_fixed = false;    // SIMT forms: every call takes P (tile override)
   int ru = 0, threads = 0, wmax = 0;  // SIMT forms: units per thread, CTA size, widest layer
+  int P0 = 0;              // FP32: points per weight-gradient group (P is a multiple); FP64: 0
+  int sum_chunks = 0;      // FP32 sums: most chunks of a call
   int sms = 0;
   size_t smem = 0;
   int grid = 0, ctas_per_sm = 0;

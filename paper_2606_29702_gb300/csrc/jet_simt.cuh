@@ -16,7 +16,8 @@
 //             the value channel, data gradient W^T Zb.
 //
 // Jets live in shared memory as [unit][point-major column] rows: column =
-// n * C + alpha (columns past C * P stay zero).  In the jet GEMMs a thread owns
+// n * C + alpha (FP32: in swapped channel pairs at odd points where I.swap says so;
+// columns past C * P stay zero).  In the jet GEMMs a thread owns
 // one point and RU consecutive units with every channel, so the composition
 // and its adjoint are thread-local; the layer's weights pass through shared
 // memory in row slabs.  The hidden z-jets of a tile are written to a per-CTA
@@ -157,9 +158,8 @@ static __device__ __noinline__ void simt_wacc_zero(float* acc, const DevInstance
 }
 // accumulator -> FP64 slice (consecutive threads read consecutive floats;
 // eight loads in flight before their adds)
-template <int WR>
 static __device__ __noinline__ void simt_wacc_flush(const float* a, const DevInstance& I, double* g) {
-  const int NT = blockDim.x;
+  const int NT = blockDim.x, WR = I.wr;
   for (int l = 2; l <= I.L - 1; ++l) {
     const int wo = I.widths[l], wi = I.widths[l - 1], nkb = wi / 4, n = wo * wi;
     double* gW = g + I.off_W[l - 1];
@@ -192,7 +192,6 @@ struct SimtTile {
   // steps' operands would exceed the registers (C = 7 at 512 threads: 12.8 ms
   // with four, 11.8 ms with two), else four
   static constexpr int UK = C >= 7 ? 2 : 4;
-  static constexpr int WR = F32 && RU == 8 ? 8 : 4;  // weight-gradient rows per thread (times 4 columns)
 
   const DevInstance& I;
   const SimtArgs& A;
@@ -204,6 +203,8 @@ struct SimtTile {
   T* XS;     // tile points [P][d]
   double* RED;
   int P, pitch, wmax;
+  int P0, V;    // points per weight-gradient group, groups per tile
+  bool swap;    // odd points keep their channels in swapped pairs
   int slab;     // elements of a weight slab
   int wst = 0;  // slab that holds, or waits for, the next GEMM's first rows
   const T* params;
@@ -219,6 +220,9 @@ struct SimtTile {
       : I(I_), A(A_), NT(blockDim.x) {
     P = I.P;
     pitch = I.pitch;
+    P0 = I.P0;
+    V = P / P0;
+    swap = F32 && C % 2 == 0 && I.swap;
     wmax = 0;
     for (int l = 1; l < I.L; ++l) wmax = max(wmax, I.widths[l]);
     slab = simt_slab_elems(wmax, sizeof(T));
@@ -239,7 +243,26 @@ struct SimtTile {
     if (F32 && I.wsums) wacc_base = I.wsums + (long long)chunk * I.wsums_stride;
   }
 
-  // accumulator of W^l (l = 2..L-1): [item][WR][4] per thread item of wgrad
+  // a point's channels in a jet row: exchange of channel pairs (see I.swap)
+  __device__ __forceinline__ bool odd(int n) const { return swap && (n & 1); }
+  static __device__ __forceinline__ void swap_pairs(T* v) {
+#pragma unroll
+    for (int c = 0; c + 1 < C; c += 2) {
+      const T t = v[c];
+      v[c] = v[c + 1];
+      v[c + 1] = t;
+    }
+  }
+  __device__ __forceinline__ void load_point(const T* row, int n, T* v) const {
+    load_chan<T, C>(row + n * C, v);
+    if (odd(n)) swap_pairs(v);
+  }
+  __device__ __forceinline__ void store_point(T* row, int n, T* v) const {
+    if (odd(n)) swap_pairs(v);
+    store_chan<T, C>(row + n * C, v);
+  }
+
+  // accumulator of W^l (l = 2..L-1): [item][wr][4] per thread item of wgrad
   __device__ float* wacc(int l) const {
     long long off = 0;
     for (int k = 2; k < l; ++k) off += (long long)I.widths[k] * I.widths[k - 1];
@@ -337,7 +360,20 @@ struct SimtTile {
           }
         }
       }
-      if (act) done(n, u0, acc);
+      if (!act) continue;
+      if constexpr (F32 && C % 2 == 0) {
+        if (odd(n)) {
+#pragma unroll
+          for (int r = 0; r < RU / 2; ++r)
+#pragma unroll
+            for (int c = 0; c < C; c += 2) {
+              const f2 t = acc.v[r][c];
+              acc.v[r][c] = acc.v[r][c + 1];
+              acc.v[r][c + 1] = t;
+            }
+        }
+      }
+      done(n, u0, acc);
     }
   }
 
@@ -371,7 +407,7 @@ struct SimtTile {
         }
         tanh_derivs<T, NP>(z[0], p);
         Cls::compose(z, p, a);
-        store_chan<T, C>(out + u * pitch + n * C, a);
+        store_point(out + u * pitch, n, a);
         if (zdst) {
           __stcg(zdst + (long long)u * CP + n, p[0]);
 #pragma unroll
@@ -402,8 +438,8 @@ struct SimtTile {
             lo[c] = a[c].v.x;
             hi[c] = a[c].v.y;
           }
-          store_chan<T, C>(out + u * pitch + n * C, lo);
-          store_chan<T, C>(out + (u + 1) * pitch + n * C, hi);
+          store_point(out + u * pitch, n, lo);
+          store_point(out + (u + 1) * pitch, n, hi);
           if (zdst) {
             z[0] = p[0];
 #pragma unroll
@@ -423,7 +459,7 @@ struct SimtTile {
           z[0] += bl[u];
           tanh_derivs<T, NP>(z[0], p);
           Cls::compose(z, p, a);
-          store_chan<T, C>(out + u * pitch + n * C, a);
+          store_point(out + u * pitch, n, a);
           if (zdst) {
             __stcg(zdst + (long long)u * CP + n, p[0]);
 #pragma unroll
@@ -459,8 +495,8 @@ struct SimtTile {
             lo[c] = a[c].v.x;
             hi[c] = a[c].v.y;
           }
-          store_chan<T, C>(out + (u0 + r) * pitch + n * C, lo);
-          store_chan<T, C>(out + (u0 + r + 1) * pitch + n * C, hi);
+          store_point(out + (u0 + r) * pitch, n, lo);
+          store_point(out + (u0 + r + 1) * pitch, n, hi);
         }
       } else {
 #pragma unroll
@@ -468,7 +504,7 @@ struct SimtTile {
           T p[NP], a[C];
           tanh_polys<T, NP>(zz[r][0], p);
           Cls::compose(zz[r], p, a);
-          store_chan<T, C>(out + (u0 + r) * pitch + n * C, a);
+          store_point(out + (u0 + r) * pitch, n, a);
         }
       }
     }
@@ -483,7 +519,7 @@ struct SimtTile {
     const int ncol = C * P;
     for (int it = threadIdx.x; it < no * ncol; it += NT) {
       const int o = it / ncol, col = it - o * ncol;
-      const int n = col / C, c = col - n * C;
+      const int n = col / C, c = (col - n * C) ^ (odd(n) ? 1 : 0);
       const T* ap = in + col;
       T s = c == 0 ? bL[o] : T(0);
 #pragma unroll 4
@@ -603,13 +639,6 @@ struct SimtTile {
   }
 
   // ---------------------------------------------------------------- backward
-  // sum of v over the 4 lanes of a group, in a fixed order
-  static __device__ __forceinline__ T sum4(T v) {
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    v += __shfl_xor_sync(0xffffffffu, v, 2);
-    return v;
-  }
-
   // Abar^{L-1} = W^L^T ub; dW^L = sum_cols ub a^{L-1}^T; db^L = sum_n ub_0
   __device__ void output_bwd(const T* a_last, T* abar, double* g) {
     const int L = I.L, wi = I.widths[L - 1], no = I.n_out;
@@ -626,28 +655,33 @@ struct SimtTile {
 #pragma unroll
         for (int c = 0; c < C; ++c) s[c] = fma(w, UB[o * ncol + c * P + n], s[c]);
       }
-      store_chan<T, C>(abar + k * pitch + n * C, s);
+      store_point(abar + k * pitch, n, s);
     }
-    // dW^L[o][k] and db^L[o]: four lanes share a sum, each taking a quarter of
-    // the points; the partials combine by shuffles in a fixed order
+    // dW^L[o][k] per group of points: four lanes share a sum, each taking a
+    // quarter of the points; the partials combine by shuffles in a fixed order
     // (the loop runs whole warps: every lane of a warp reaches the shuffles)
-    const int items = 4 * no * (wi + 1), items_w = (items + 31) & ~31;
+    const int items = 4 * no * wi * V, items_w = (items + 31) & ~31;
     for (int it = threadIdx.x; it < items_w; it += NT) {
       const bool act = it < items;
-      const int part = it & 3, ok = it >> 2, o = act ? ok / (wi + 1) : 0, k = act ? ok % (wi + 1) : 0;
+      const int part = it & 3, e = act ? it >> 2 : 0, v = e / (no * wi), ok = e - v * (no * wi);
+      const int o = ok / wi, k = ok - o * wi;
       T s = T(0);
-      if (act && k < wi) {
-        for (int n = part; n < P; n += 4) {
+      if (act)
+        for (int n = v * P0 + part; n < (v + 1) * P0; n += 4) {
           T av[C];
-          load_chan<T, C>(a_last + k * pitch + n * C, av);
+          load_point(a_last + k * pitch, n, av);
 #pragma unroll
           for (int c = 0; c < C; ++c) s = fma(UB[o * ncol + c * P + n], av[c], s);
         }
-      } else if (act) {
-        for (int n = part; n < P; n += 4) s += UB[o * ncol + n];
-      }
-      s = sum4(s);
-      if (act && part == 0) atomicAdd(g + (k < wi ? I.goff_WL + o * wi + k : I.goff_b[L - 1] + o), widen(s));
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      if (act && part == 0) atomicAdd(g + I.goff_WL + o * wi + k, widen(s));
+    }
+    for (int e = threadIdx.x; e < no * V; e += NT) {  // db^L per group
+      const int o = e / V, v = e - o * V;
+      T s = T(0);
+      for (int n = v * P0; n < (v + 1) * P0; ++n) s += UB[o * ncol + n];
+      atomicAdd(g + I.goff_b[L - 1] + o, widen(s));
     }
   }
 
@@ -667,12 +701,12 @@ struct SimtTile {
         // FP32: units (r, r+1) in packed pairs
 #pragma unroll
         for (int r = 0; r < EU; r += 2) {
-          T* b0 = bar + (u0 + r) * pitch + n * C;
+          T* b0 = bar + (u0 + r) * pitch;
           T* b1 = b0 + pitch;
           f2 z[C], p[NP], ab[C], zb[C];
           T lo[C], hi[C];
-          load_chan<T, C>(b0, lo);
-          load_chan<T, C>(b1, hi);
+          load_point(b0, n, lo);
+          load_point(b1, n, hi);
 #pragma unroll
           for (int c = 0; c < C; ++c) {
             z[c] = f2(zz[r][c], zz[r + 1][c]);
@@ -685,8 +719,8 @@ struct SimtTile {
             lo[c] = zb[c].v.x;
             hi[c] = zb[c].v.y;
           }
-          store_chan<T, C>(b0, lo);
-          store_chan<T, C>(b1, hi);
+          store_point(b0, n, lo);
+          store_point(b1, n, hi);
         }
       } else {
 #pragma unroll
@@ -703,15 +737,150 @@ struct SimtTile {
   }
 
   // dW^l[u][k] += sum_cols Zbar[u][col] A[k][col]; db^l[u] += sum_n Zbar[u][n].
-  // Thread item: WR rows u and 4 columns k (rows kb + s * nkb of A); NS adjacent
-  // lanes share an item, each taking every NS-th vector of columns, so that
-  // narrow layers fill the CTA (a 20 x 20 layer has 25 items); their sums
-  // combine by halves, each lane ending with its own 1 / NS of the block.
+  // Thread item: WR rows u and 4 columns k (rows kb + s * nkb of A).
   __device__ void wgrad(int l, const T* zbar, const T* aprev, double* g) {
+    if constexpr (!F32) {
+      wgrad64(l, zbar, aprev, g);
+    } else {
+      // several groups added to the chunk's FP32 sums by one thread: the sums
+      // wait in registers, one load and one store per tile instead of a vector
+      // reduction per group (3->256x8->1, three groups a tile: 10.83 -> 10.44 ms)
+      const int items = I.widths[l] / 4 * (I.widths[l - 1] / 4);
+      if (I.wr == 4 && wacc_base && V > 1 && (V % 2 || items * 2 > NT)) wgrad32<4, true>(l, zbar, aprev, g);
+      else if (I.wr == 4) wgrad32<4, false>(l, zbar, aprev, g);
+      else wgrad32<(RU == 8 ? 2 : 1), false>(l, zbar, aprev, g);
+    }
+    // a thread per bias and group of points
+    const int wo = I.widths[l];
+    double* gb = g + I.goff_b[l - 1];
+    for (int it = threadIdx.x; it < wo * V; it += NT) {
+      const int u = it % wo, v = it / wo;
+      const T* zp = zbar + u * pitch;
+      T s = T(0);
+#pragma unroll 4
+      for (int n = v * P0; n < (v + 1) * P0; ++n) s += zp[n * C + (odd(n) ? 1 : 0)];
+      atomicAdd(gb + u, widen(s));
+    }
+  }
+
+  // FP32: the groups of points one after another, their even and odd columns in
+  // the two halves of a packed pair (the 16-byte loads deliver the pairs), summed
+  // at the end of the group.  Where the items leave half the CTA idle, the two
+  // halves of a warp take an item's even and odd groups and then swap half
+  // their blocks, so that every element is added by one thread, group after group.
+  template <int WR, bool HELD>
+  __device__ __forceinline__ void wgrad32(int l, const T* zbar, const T* aprev, double* g) {
+    const int wo = I.widths[l], wi = I.widths[l - 1];
+    const int nkb = wi / 4, items = (wo / WR) * nkb, gcol = P0 * C;
+    const bool two = !HELD && WR >= 2 && V % 2 == 0 && items * 2 <= NT;
+    double* gW = g + I.off_W[l - 1];
+    const int lane = threadIdx.x & 31, sl = two ? lane >> 4 : 0;
+    const int work_w = ((two ? 2 * items : items) + 31) & ~31;  // whole warps: every lane reaches the shuffles
+    for (int it = threadIdx.x; it < work_w; it += NT) {
+      const int item = two ? (it >> 5) * 16 + (lane & 15) : it;
+      const bool act = item < items;
+      const int kb = act ? item % nkb : 0, ub = act ? item / nkb : 0;
+      const T* zp = zbar + ub * WR * pitch;
+      const T* app = aprev + kb * pitch;
+      float* const sums = HELD && act ? wacc(l) + (long long)item * (WR * 4) : nullptr;
+      T run[WR * 4];
+      if constexpr (HELD) {
+#pragma unroll
+        for (int e = 0; e < WR * 4; e += 4) {
+          float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (act && !wacc_first) t = __ldcg(reinterpret_cast<const float4*>(sums + e));
+          run[e] = t.x;
+          run[e + 1] = t.y;
+          run[e + 2] = t.z;
+          run[e + 3] = t.w;
+        }
+      }
+      for (int v0 = 0; v0 < V; v0 += two ? 2 : 1) {
+        const int c0 = (v0 + sl) * gcol, c1 = act ? c0 + gcol : c0;
+        f2 ap2[WR][4];
+#pragma unroll
+        for (int r = 0; r < WR; ++r)
+#pragma unroll
+          for (int s = 0; s < 4; ++s) ap2[r][s] = f2(0.f);
+        for (int col = c0; col < c1; col += TP) {
+          T av[4][TP];
+#pragma unroll
+          for (int s = 0; s < 4; ++s) vload<T>(app + s * nkb * pitch + col, av[s]);
+          T zv[WR][TP];
+#pragma unroll
+          for (int r = 0; r < WR; ++r) vload<T>(zp + r * pitch + col, zv[r]);
+#pragma unroll
+          for (int r = 0; r < WR; ++r)
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+#pragma unroll
+              for (int j = 0; j < TP; j += 2)
+                ap2[r][s] = jfma(f2(zv[r][j], zv[r][j + 1]), f2(av[s][j], av[s][j + 1]), ap2[r][s]);
+        }
+        T acc[WR * 4];
+#pragma unroll
+        for (int r = 0; r < WR; ++r)
+#pragma unroll
+          for (int s = 0; s < 4; ++s) acc[r * 4 + s] = ap2[r][s].v.x + ap2[r][s].v.y;
+        const bool first = wacc_first && v0 == 0;
+        if (!HELD && two) {
+          constexpr int H = WR * 2;  // this thread's half of the block
+#pragma unroll
+          for (int e = 0; e < H; e += 4) {
+            T lo[4], hi[4];  // four elements: group v0, group v0 + 1
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const int k = (e + j) % (WR * 2);
+              const T got = __shfl_xor_sync(0xffffffffu, sl ? acc[k] : acc[k + H], 16);
+              lo[j] = sl ? got : acc[k];
+              hi[j] = sl ? acc[k + H] : got;
+            }
+            if (act) {
+              add4<WR>(l, item, sl * H + e, lo, first, gW, ub, kb, nkb, wi);
+              add4<WR>(l, item, sl * H + e, hi, false, gW, ub, kb, nkb, wi);
+            }
+          }
+        } else if (HELD) {
+#pragma unroll
+          for (int e = 0; e < WR * 4; ++e) run[e] += acc[e];
+        } else if (act) {
+#pragma unroll
+          for (int e = 0; e < WR * 4; e += 4) add4<WR>(l, item, e, acc + e, first, gW, ub, kb, nkb, wi);
+        }
+      }
+      if (HELD && act)
+#pragma unroll
+        for (int e = 0; e < WR * 4; e += 4)
+          __stcg(reinterpret_cast<float4*>(sums + e), make_float4(run[e], run[e + 1], run[e + 2], run[e + 3]));
+    }
+  }
+
+  // one row of an item's block (from element e on) to the chunk's FP32 sums or
+  // the FP64 slice: fire-and-forget adds, one thread per element and in order,
+  // so the sums stay deterministic
+  template <int WR>
+  __device__ __forceinline__ void add4(int l, int item, int e, const T* v, bool first, double* gW, int ub, int kb,
+                                       int nkb, int wi) {
+    if (wacc_base) {
+      float* a = wacc(l) + (long long)item * (WR * 4) + e;
+      if (first) __stcg(reinterpret_cast<float4*>(a), make_float4(v[0], v[1], v[2], v[3]));
+      else red_add_v4(a, v[0], v[1], v[2], v[3]);
+      return;
+    }
+    double* d = gW + (ub * WR + (e >> 2)) * wi + kb;
+#pragma unroll
+    for (int s = 0; s < 4; ++s) atomicAdd(d + s * nkb, widen(v[s]));
+  }
+
+  // FP64: NS adjacent lanes share an item, each taking every NS-th vector of
+  // columns, so that narrow layers fill the CTA (a 20 x 20 layer has 25 items);
+  // their sums combine by halves, each lane ending with its own 1 / NS of the block.
+  __device__ __forceinline__ void wgrad64(int l, const T* zbar, const T* aprev, double* g) {
+    constexpr int WR = 4;
     const int wo = I.widths[l], wi = I.widths[l - 1];
     const int ncol = (C * P + TP - 1) / TP * TP;  // zero columns up to a whole vector
     const int nkb = wi / 4, items = (wo / WR) * nkb;
-    const int NS = simt_wgrad_slices(items, WR, F32, NT);
+    const int NS = simt_wgrad_slices(items, NT);
     double* gW = g + I.off_W[l - 1];
     const int work = items * NS, work_w = (work + 31) & ~31;
     for (int it = threadIdx.x; it < work_w; it += NT) {
@@ -721,56 +890,20 @@ struct SimtTile {
       T acc[WR * 4];
       const T* zp = zbar + ub * WR * pitch;
       const T* app = aprev + kb * pitch;
-      const int c0 = act ? sl * TP : ncol;
-      if constexpr (F32) {
-        // FP32: even and odd columns accumulate in the two halves of a
-        // packed pair (the 16-byte loads deliver the pairs), summed at the end
-        f2 ap2[WR][4];
+#pragma unroll
+      for (int e = 0; e < WR * 4; ++e) acc[e] = T(0);
+      for (int col = act ? sl * TP : ncol; col < ncol; col += NS * TP) {
+        T zv[WR][TP], av[4][TP];
+#pragma unroll
+        for (int r = 0; r < WR; ++r) vload<T>(zp + r * pitch + col, zv[r]);
+#pragma unroll
+        for (int s = 0; s < 4; ++s) vload<T>(app + s * nkb * pitch + col, av[s]);
 #pragma unroll
         for (int r = 0; r < WR; ++r)
 #pragma unroll
-          for (int s = 0; s < 4; ++s) ap2[r][s] = f2(0.f);
-        for (int col = c0; col < ncol; col += NS * TP) {
-          T av[4][TP];
+          for (int s = 0; s < 4; ++s)
 #pragma unroll
-          for (int s = 0; s < 4; ++s) vload<T>(app + s * nkb * pitch + col, av[s]);
-          // four rows' operands at a time: all eight beside 32 packed sums
-          // would spill
-#pragma unroll
-          for (int r0 = 0; r0 < WR; r0 += 4) {
-            T zv[4][TP];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) vload<T>(zp + (r0 + r) * pitch + col, zv[r]);
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-              for (int s = 0; s < 4; ++s)
-#pragma unroll
-                for (int j = 0; j < TP; j += 2)
-                  ap2[r0 + r][s] = jfma(f2(zv[r][j], zv[r][j + 1]), f2(av[s][j], av[s][j + 1]), ap2[r0 + r][s]);
-            if (r0 + 4 < WR) asm volatile("" ::: "memory");
-          }
-        }
-#pragma unroll
-        for (int r = 0; r < WR; ++r)
-#pragma unroll
-          for (int s = 0; s < 4; ++s) acc[r * 4 + s] = ap2[r][s].v.x + ap2[r][s].v.y;
-      } else {
-#pragma unroll
-        for (int e = 0; e < WR * 4; ++e) acc[e] = T(0);
-        for (int col = c0; col < ncol; col += NS * TP) {
-          T zv[WR][TP], av[4][TP];
-#pragma unroll
-          for (int r = 0; r < WR; ++r) vload<T>(zp + r * pitch + col, zv[r]);
-#pragma unroll
-          for (int s = 0; s < 4; ++s) vload<T>(app + s * nkb * pitch + col, av[s]);
-#pragma unroll
-          for (int r = 0; r < WR; ++r)
-#pragma unroll
-            for (int s = 0; s < 4; ++s)
-#pragma unroll
-              for (int j = 0; j < TP; ++j) acc[r * 4 + s] = fma(zv[r][j], av[s][j], acc[r * 4 + s]);
-        }
+            for (int j = 0; j < TP; ++j) acc[r * 4 + s] = fma(zv[r][j], av[s][j], acc[r * 4 + s]);
       }
       // combine the NS lanes: at each step a lane keeps one half of its block
       // and sends the other to its partner
@@ -789,37 +922,12 @@ struct SimtTile {
         n = h;
       }
       if (!act) continue;
-      // fire-and-forget adds: every element belongs to one thread, which adds
-      // the tiles in order, so the sums stay deterministic
-      if constexpr (F32) {
-        if (wacc_base) {  // n is a multiple of 4 here
-          float* a = wacc(l) + (long long)item * (WR * 4) + base;
-#pragma unroll
-          for (int e = 0; e < WR * 4; e += 4)
-            if (e < n) {
-              if (wacc_first) __stcg(reinterpret_cast<float4*>(a + e), make_float4(acc[e], acc[e + 1], acc[e + 2], acc[e + 3]));
-              else red_add_v4(a + e, acc[e], acc[e + 1], acc[e + 2], acc[e + 3]);
-            }
-          continue;
-        }
-      }
 #pragma unroll
       for (int e = 0; e < WR * 4; ++e)
         if (e < n) {
           const int r = (base + e) >> 2, s = (base + e) & 3;
-          atomicAdd(gW + (ub * WR + r) * wi + kb + s * nkb, widen(acc[e]));
+          atomicAdd(gW + (ub * WR + r) * wi + kb + s * nkb, (double)acc[e]);
         }
-    }
-    // four lanes per bias
-    double* gb = g + I.goff_b[l - 1];
-    const int bw = (4 * wo + 31) & ~31;
-    for (int it = threadIdx.x; it < bw; it += NT) {
-      const int u = it >> 2, part = it & 3;
-      T s = T(0);
-      if (u < wo)
-        for (int n = part; n < P; n += 4) s += zbar[u * pitch + n * C];
-      s = sum4(s);
-      if (u < wo && part == 0) atomicAdd(gb + u, widen(s));
     }
   }
 
@@ -835,8 +943,8 @@ struct SimtTile {
             lo[c] = acc.v[r / 2][c].v.x;
             hi[c] = acc.v[r / 2][c].v.y;
           }
-          store_chan<T, C>(abar + (k0 + r) * pitch + n * C, lo);
-          store_chan<T, C>(abar + (k0 + r + 1) * pitch + n * C, hi);
+          store_point(abar + (k0 + r) * pitch, n, lo);
+          store_point(abar + (k0 + r + 1) * pitch, n, hi);
         }
       } else {
 #pragma unroll
@@ -846,38 +954,35 @@ struct SimtTile {
   }
 
   // dW^1[u][i] += sum_n Zbar_0[u][n] x_i[n] + Zbar_{e_i}[u][n]; db^1[u] += sum_n Zbar_0[u][n];
-  // four lanes per unit
+  // a thread per unit and group of points
   __device__ void layer1_bwd(const T* zbar, double* g) {
     const int w = I.widths[1], d = I.d;
     double* gW = g;
     double* gb = g + I.goff_b[0];
-    const int ww = (4 * w + 31) & ~31;
-    for (int it = threadIdx.x; it < ww; it += NT) {
-      const int u = it >> 2, part = it & 3;
+    for (int it = threadIdx.x; it < w * V; it += NT) {
+      const int u = it % w, n0 = it / w * P0;
+      const T* zp = zbar + u * pitch;
       T sb = T(0), sw[3] = {T(0), T(0), T(0)};
-      if (u < w)
-        for (int n = part; n < P; n += 4) {
-          T zv[C];
-          load_chan<T, C>(zbar + u * pitch + n * C, zv);
-          sb += zv[0];
-#pragma unroll
-          for (int i = 0; i < 3; ++i)
-            if (i < d) sw[i] = fma(zv[0], XS[n * d + i], sw[i]);
-#pragma unroll
-          for (int i = 0; i < Cls::D; ++i) {
-            const int fo = Cls::first_order(i);
-            if (fo >= 0 && i < d) sw[i] += zv[fo];
-          }
-        }
-      sb = sum4(sb);
-#pragma unroll
-      for (int i = 0; i < 3; ++i) sw[i] = sum4(sw[i]);
-      if (u < w && part == 0) {
+#pragma unroll 4
+      for (int n = n0; n < n0 + P0; ++n) {
+        const T z0 = zp[n * C + (odd(n) ? 1 : 0)];
+        sb += z0;
 #pragma unroll
         for (int i = 0; i < 3; ++i)
-          if (i < d) atomicAdd(gW + u * d + i, widen(sw[i]));
-        atomicAdd(gb + u, widen(sb));
+          if (i < d) sw[i] = fma(z0, XS[n * d + i], sw[i]);
       }
+#pragma unroll
+      for (int i = 0; i < Cls::D; ++i) {
+        const int fo = Cls::first_order(i);
+        if (fo >= 0 && i < d) {
+#pragma unroll 4
+          for (int n = n0; n < n0 + P0; ++n) sw[i] += zp[n * C + (odd(n) ? fo ^ 1 : fo)];
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+        if (i < d) atomicAdd(gW + u * d + i, widen(sw[i]));
+      atomicAdd(gb + u, widen(sb));
     }
   }
 
@@ -888,12 +993,11 @@ struct SimtTile {
     return A.mode == MODE_BWD_STORE ? bwd_rows(I.L - 1) : fwd_rows(2);
   }
 
-  // one tile; its first GEMM's first weight slab is in flight on entry, and
-  // the next tile's on exit (more: there is one)
-  __device__ double tile(long long t, double* g, bool more) {
+  // the tile of the points [n0, min(n0 + P, n1)); its first GEMM's first weight
+  // slab is in flight on entry, and the next tile's on exit (more: there is one)
+  __device__ double tile(long long n0, long long n1, double* g, bool more) {
     const int mode = A.mode;
-    const long long n0 = t * P;
-    const long long rem = I.N - n0;
+    const long long rem = n1 - n0, t = n0 / P;  // t: the tile's place in the z-jet store
     const int nvalid = rem < (long long)P ? (int)rem : P;
     const int d = I.d;
     const T* X = reinterpret_cast<const T*>(I.X);
@@ -981,24 +1085,29 @@ __device__ __forceinline__ void simt_body(const SimtArgs& args) {
     if (bwd)
       for (int i = threadIdx.x; i < I.n_slice; i += NT) g[i] = 0.0;
     double loss = 0.0;
-    // tiles of the chunk: the first chunk_rem chunks take one more than the rest
-    const long long t0 = (long long)chunk * I.tiles_per_chunk + min(chunk, I.chunk_rem);
-    const long long t1 = t0 + I.tiles_per_chunk + (chunk < I.chunk_rem ? 1 : 0);
-    // FP32 sums in runs of at most kWaccTiles tiles (wide channel sets): the FP32
+    // points of the chunk: the first chunk_rem chunks take one unit more than the rest
+    const long long u0 = (long long)chunk * I.tiles_per_chunk + min(chunk, I.chunk_rem);
+    const long long u1 = u0 + I.tiles_per_chunk + (chunk < I.chunk_rem ? 1 : 0);
+    const long long s0 = u0 * I.unit, s1 = min(u1 * I.unit, I.N);
+    // FP32 sums in runs of at most kWaccTiles groups (wide channel sets): the FP32
     // rounding of a weight's sum stays below kWaccTiles * 2^-24 of its magnitudes
     // at any N.  The reduction reads the sums of a single run.
     const bool runs = bwd && S.wacc_base != nullptr && !I.wsums_direct;
     if (runs) simt_wacc_zero(S.wacc_base, I);
     __syncthreads();
-    for (long long t = t0; t < t1; ++t) {
-      S.wacc_first = t == t0 && I.wsums_direct;
-      loss += S.tile(t, g, t + 1 < t1);
+    int groups = 0;  // of the running FP32 run
+    for (long long n = s0; n < s1; n += S.P) {
+      const bool more = n + S.P < s1;
+      S.wacc_first = n == s0 && I.wsums_direct;
+      loss += S.tile(n, s1, g, more);
       __syncthreads();
-      if (runs && (t + 1 == t1 || (t + 1 - t0) % kWaccTiles == 0)) {
+      groups += S.V;
+      if (runs && (!more || groups + S.V > kWaccTiles)) {
         __threadfence();
         __syncthreads();
-        simt_wacc_flush<SimtTile<Cls, T, RU>::WR>(S.wacc_base, I, g);
-        if (t + 1 < t1) {
+        simt_wacc_flush(S.wacc_base, I, g);
+        groups = 0;
+        if (more) {
           __syncthreads();
           simt_wacc_zero(S.wacc_base, I);
           __syncthreads();
