@@ -81,3 +81,22 @@ def test_fp32_sums_of_short_and_long_chunks(N):
     g, loss, _ = plan.backward(p, x)
     assert rel_l2(g.cpu().numpy(), g_ref) <= TOL["fp32"][1]
     assert abs(float(loss) - L) <= TOL["fp32"][0] * abs(L)
+
+
+@pytest.mark.parametrize("name,widths", [("helmholtz_3x256x8", [3, 256, 256, 256, 1]), ("ns_psi_3x128x6", [3, 128, 128, 128, 128, 2]),
+                                         ("burgers_2x20x4", [2] + [64] * 7 + [1]), ("ks_2x64x5", [2, 32, 32, 32, 1])])
+def test_fp32_gradient_does_not_depend_on_the_tile(name, widths):
+    """A plan with a z-jet store takes tiles of one group of points where it keeps FP32 sums, another takes several:
+    the FP32 sums, and with them the gradient, are the same bits.  Without FP32 sums the FP64 adds of equal tile sums
+    differ in order, at 2^-53 a term: at most the last bit of an FP32 value (2^-24 = 6e-8)."""
+    from paper_2606_29702_gb300 import jet, specs
+    spec, X, layers, src = case(name, 6011, widths=widths)
+    plan = _plan(jet, specs, spec, "fp32")
+    stored = jet.Plan(specs.by_name(spec["family"], **spec["coefs"]), widths, "fp32", store=True, mem_budget=1 << 30)
+    p, x, s = _tensors(plan, X, layers, src)
+    g, loss, _ = plan.backward(p, x, s)
+    g1, loss1, _ = stored.backward(p, x, s)
+    if plan.info()["wgrad_chunk_fp32"]:
+        np.testing.assert_array_equal(g.cpu().numpy(), g1.cpu().numpy())
+    assert rel_l2(g.cpu().numpy(), g1.cpu().numpy()) <= 6e-8
+    assert abs(float(loss) - float(loss1)) <= 1e-12 * abs(float(loss1))
