@@ -470,7 +470,7 @@ void set_regions(TcPlan& t) {
 // shared-memory carve for tile size P; returns total bytes (without the 1 KB alignment slack)
 size_t carve(TcPlan& t, int C, int n_out, int d) {
   const int R = 128 * t.H;
-  const int nck = std::max(2, t.w / 64);
+  const int nck = std::max(2, (t.w + 63) / 64);
   const int ach = (t.cols_pad + 63) / 64;
   const int lch = t.split3 ? (t.top_cols + 63) / 64 : 0;
   size_t off = 0;

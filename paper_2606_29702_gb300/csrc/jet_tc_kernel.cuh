@@ -255,7 +255,7 @@ struct TcTile {
 
   // ------------------------------------------------------------ loads (thread 0)
   __device__ void load_hidden_w(int l) {  // W^l, l = 2..L-1 -> W buffer (and W_lo)
-    const int nck = ww() / 64 > 2 ? ww() / 64 : 2;
+    const int nck = (ww() + 63) / 64 > 2 ? (ww() + 63) / 64 : 2;
     const uint32_t box = 64u * rr() * 2u;
     tc::mbar_arrive_expect_tx(bar_tma, box * nck * (I.split3 ? 2u : 1u));
     for (int kc = 0; kc < nck; ++kc) {
@@ -866,9 +866,10 @@ struct TcTile {
         acc8(a, j, k0, R0(0) + lane_base() + (uint32_t)(sub * wu + k0), pol);
       return;
     }
+    const int nk = ww() % NB != 0 && nb * NB + NB > ww() ? ww() - nb * NB : NB;  // a last block narrower than NB
     for (int h = 0; h < hh(); ++h) {
       if (h * 128 + q * 32 >= ww()) continue;  // warp-uniform
-      for (int k0 = wg * 8; k0 < NB; k0 += nw() * 8)
+      for (int k0 = wg * 8; k0 < nk; k0 += nw() * 8)
         acc8(acc, h * 128 + ul, nb * NB + k0, R0(h) + lane_base() + (uint32_t)k0, pol);
     }
   }
@@ -1136,7 +1137,7 @@ struct TcTile {
         continue;
       }
       const int NB = hh() == 2 ? 128 : ww();
-      const int nblk = ww() / NB;
+      const int nblk = (ww() + NB - 1) / NB;
       if (nblk == 1) {
         // weight gradient first, with its own barrier: its flush from TMEM
         // runs while the data-gradient MMA does, and A^{l-2} reloads into
