@@ -33,8 +33,8 @@
 // (about 80% of the time), the FP64 pipe in the FP64 form.  Against the form
 // with three jet buffers, 4 units per thread, weights read through L1, one
 // lane per weight-gradient item and tiles that did not depend on N:
-// 3->256x8->1 FP32 at N = 16385 19.29 -> 9.86 ms, 2->64x5->1 (C = 6) FP32 at
-// 65536 1.769 -> 1.237 ms, 2->20x4->1 FP64 at 1000 347 -> 84 us.
+// 3->256x8->1 FP32 at N = 16385 19.29 -> 10.13 ms, 2->64x5->1 (C = 6) FP32 at
+// 65536 1.769 -> 1.317 ms, 2->20x4->1 FP64 at 1000 343 -> 77 us.
 #pragma once
 
 #include <type_traits>
