@@ -1060,8 +1060,10 @@ jet_status tc_train_step(jet_plan_s* p, TcPlan* t, void* params, void* m, void* 
 // BF16 weight copies and TMA tensor maps.
 
 namespace jet {
+constexpr int kBatchChunks = 16;  // least bound of a member's chunks
+
 struct TcBatch {
-  int n = 0, cls = 0, grid = 0, tmem_cols = 0, max_chunks = 16, max_items = 0, n_items = 0;
+  int n = 0, cls = 0, grid = 0, tmem_cols = 0, max_chunks = kBatchChunks, max_items = 0, n_items = 0;
   int nthreads = 512;  // smallest CTA of the member plans (their partial-sum areas fit it)
   size_t smem = 0;
   TcInst* d_insts = nullptr;
@@ -1090,7 +1092,6 @@ jet_status tc_batch_create(const std::vector<jet_plan_s*>& plans, TcBatch** out)
   TcBatch* b = new TcBatch();
   b->n = (int)plans.size();
   b->cls = plans[0]->cls;
-  long long slices = 0, sums = 0;
   for (jet_plan_s* p : plans)
     if (p->tcp->single_act) {
       delete b;
@@ -1103,10 +1104,6 @@ jet_status tc_batch_create(const std::vector<jet_plan_s*>& plans, TcBatch** out)
     b->tmem_cols = std::max(b->tmem_cols, t->tmem_cols);
     b->nthreads = std::min(b->nthreads, t->nthreads);
     b->scratch_stride = std::max(b->scratch_stride, t->scratch_stride);
-    b->slice_off.push_back(slices);
-    slices += (long long)b->max_chunks * t->n_slice;
-    b->wsums_off.push_back(sums);
-    sums += (long long)b->max_chunks * t->wsums_stride;
   }
   int dev = 0, sms = 0, occ = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -1118,8 +1115,35 @@ jet_status tc_batch_create(const std::vector<jet_plan_s*>& plans, TcBatch** out)
     return e != cudaSuccess ? tcuda(e, "batch occupancy") : tfail(JET_ERR_UNSUPPORTED, "batch tile does not fit");
   }
   b->grid = sms * std::max(1, std::min(occ, 512 / b->tmem_cols));
+  // Chunks a member may take: about four items per CTA over the members, at least
+  // kBatchChunks.  With 16 for every batch, few members left CTAs idle (one step,
+  // BF16: 4 members 2176 -> 825 us, 6 members 1331 -> 407 us, 9 members 1848 -> 751
+  // us, 16 members 2059 -> 1947 us; from 38 members on the bound is 16 as before).
+  // Eight per CTA measured 891, 484 and 827 us and 4945 against 4872 us at 40
+  // members; items of equal cost 952, 481 and 905 us, and 6190 against 5906 us at 64
+  // (no small items left to fill the tail).
+  b->max_chunks = std::max(kBatchChunks, 4 * b->grid / b->n);
+  for (;;) {
+    long long slices = 0, sums = 0;
+    b->slice_off.clear();
+    b->wsums_off.clear();
+    for (jet_plan_s* p : plans) {
+      b->slice_off.push_back(slices);
+      slices += (long long)b->max_chunks * p->tcp->n_slice;
+      b->wsums_off.push_back(sums);
+      sums += (long long)b->max_chunks * p->tcp->wsums_stride;
+    }
+    e = cudaMalloc((void**)&b->grad_slices, sizeof(double) * std::max<long long>(slices, 1));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&b->wsums, sizeof(float) * std::max<long long>(sums, 4));
+    if (e != cudaErrorMemoryAllocation || b->max_chunks == kBatchChunks) break;
+    // no room for that many chunks: the least bound
+    cudaGetLastError();
+    cudaFree(b->grad_slices);
+    b->grad_slices = nullptr;
+    b->max_chunks = kBatchChunks;
+  }
   b->max_items = b->n * b->max_chunks;
-  e = cudaMalloc((void**)&b->d_insts, sizeof(TcInst) * b->n);
+  if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_insts, sizeof(TcInst) * b->n);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_insts, sizeof(TcInst) * b->n);
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_items, sizeof(int) * 2 * b->max_items);
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_next, sizeof(int));
@@ -1128,9 +1152,7 @@ jet_status tc_batch_create(const std::vector<jet_plan_s*>& plans, TcBatch** out)
   if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_jobs, sizeof(ReduceJob) * b->n);
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_prep, sizeof(PrepJob) * b->n);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_prep, sizeof(PrepJob) * b->n);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b->grad_slices, sizeof(double) * std::max<long long>(slices, 1));
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->loss_slices, sizeof(double) * b->max_items);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b->wsums, sizeof(float) * std::max<long long>(sums, 4));
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->scratch, (size_t)b->grid * std::max<long long>(b->scratch_stride, 16));
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(b->err, 0, sizeof(int));
@@ -1189,7 +1211,7 @@ jet_status tc_batch_run(TcBatch* bb, const std::vector<jet_plan_s*>& plans, cons
     prep_jobs[i] = prep_job(plans[i], plans[i]->tcp, params[i], prep_total);
     prep_total += prep_jobs[i].nh + prep_jobs[i].nl;
   }
-  // work list: about eight items per CTA, cost-ordered, largest first (CTAs take
+  // work list: at most about eight items per CTA, cost-ordered, largest first (CTAs take
   // them from a shared counter, so the smaller ones fill the tail)
   const long long target = std::max<long long>(1, (total_tiles + 8LL * b->grid - 1) / (8LL * b->grid));
   std::vector<TcInst> insts(n);
