@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "../../include/jet.h"
+#include "jet_capture.h"
 #include "jet_closures_gen.h"
 #include "jet_internal.h"
 #include "jet_plan.h"
@@ -836,7 +837,9 @@ struct jet_batch_s {
   long long scratch_stride = 0;
   float* wsums = nullptr;  // FP32 weight-gradient sums per chunk of the members that keep them
   std::vector<long long> slice_off, wt_off, wsums_off;
-  // pinned host staging for the per-call descriptors
+  // the call's descriptors and work list, and their pinned staging (eager calls)
+  std::vector<DevInstance> insts;
+  std::vector<int> items;
   DevInstance* h_insts = nullptr;
   int* h_item_inst = nullptr;
   ReduceJob* h_jobs = nullptr;
@@ -845,7 +848,7 @@ struct jet_batch_s {
   // the pinned staging buffers are rewritten by the next call only after the
   // uploads of this one have read them
   cudaEvent_t copied = nullptr;
-  bool have_prev = false;
+  CaptureStore captured;  // descriptors of captured calls
 };
 
 namespace {
@@ -867,11 +870,11 @@ void free_batch(jet_batch_s* b) {
   if (b->copied) cudaEventDestroy(b->copied);
 }
 
-// Build the per-call work list: every instance is split into chunks of point
-// tiles; items are ordered by estimated cost, largest first, and pulled by the
-// persistent CTAs in that order.
+// Build the per-call descriptors and work list: every instance is split into
+// chunks of point tiles; items are ordered by estimated cost, largest first, and
+// pulled by the persistent CTAs in that order.
 jet_status batch_prepare(jet_batch_s* b, const void* const* params, const void* const* X, const int64_t* N,
-                         const void* const* source, void* const* r_out, int* n_items_out, cudaStream_t s) {
+                         const void* const* source, void* const* r_out) {
   const int n = (int)b->plans.size();
   auto tile_cost = [&](int i) {
     const jet_plan_s* p = b->plans[i];
@@ -885,16 +888,14 @@ jet_status batch_prepare(jet_batch_s* b, const void* const* params, const void* 
     if (st != JET_OK) return st;
     total_cost += tile_cost(i) * (double)((N[i] + b->P[i] - 1) / b->P[i]);
   }
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  cudaStreamIsCapturing(s, &cs);
-  if (b->have_prev && cs == cudaStreamCaptureStatusNone) cudaEventSynchronize(b->copied);
   const double target = total_cost / (3.0 * b->grid);  // about three items of equal cost per CTA
   std::vector<std::pair<double, int>> cost;  // (cost, item) for ordering
   std::vector<int> item_inst;
   int chunk_base = 0;
+  b->insts.resize(n);
   for (int i = 0; i < n; ++i) {
     jet_plan_s* p = b->plans[i];
-    DevInstance& I = b->h_insts[i];
+    DevInstance& I = b->insts[i];
     const long long tiles = (N[i] + b->P[i] - 1) / b->P[i];
     const double per_tile = tile_cost(i);
     const long long want = std::min<long long>(
@@ -918,13 +919,10 @@ jet_status batch_prepare(jet_batch_s* b, const void* const* params, const void* 
   for (int k = 0; k < chunk_base; ++k) order[k] = k;
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost[x].first > cost[y].first; });
   // the kernel walks items in list order; item ids keep their instance chunk
-  // numbering through chunk_base, so list position k maps to item order[k]
-  for (int k = 0; k < chunk_base; ++k) b->h_item_inst[k] = order[k];
-  // h_item_inst[k] holds the global item id; instance lookup table follows it
-  for (int k = 0; k < chunk_base; ++k) b->h_item_inst[chunk_base + k] = item_inst[k];
-  CK(cudaMemcpyAsync(b->d_insts, b->h_insts, sizeof(DevInstance) * n, cudaMemcpyHostToDevice, s));
-  CK(cudaMemcpyAsync(b->d_item_inst, b->h_item_inst, sizeof(int) * 2 * chunk_base, cudaMemcpyHostToDevice, s));
-  *n_items_out = chunk_base;
+  // numbering through chunk_base, so list position k maps to item order[k]; the
+  // instance lookup table of the items follows
+  b->items.assign(order.begin(), order.end());
+  b->items.insert(b->items.end(), item_inst.begin(), item_inst.end());
   return JET_OK;
 }
 
@@ -1025,17 +1023,49 @@ static jet_status batch_run(jet_batch_t b, const void* const* params, void* cons
                             const void* const* source, void* const* grad_out, double* loss_out, bool adam,
                             cudaStream_t s) {
   const int n = (int)b->plans.size();
-  int n_items = 0;
-  jet_status st = batch_prepare(b, params, X, N, source, nullptr, &n_items, s);
+  jet_status st = batch_prepare(b, params, X, N, source, nullptr);
   if (st != JET_OK) return st;
-  for (int i = 0; i < n; ++i) CK(launch_transpose_weights(b->h_insts[i], b->fp64, (void*)b->h_insts[i].Wt, s));
+  const int n_items = (int)b->items.size() / 2;
+  std::vector<ReduceJob> jobs(n);
+  for (int i = 0; i < n; ++i) {
+    jobs[i] = make_job(b->insts[i], adam ? nullptr : grad_out[i], loss_out ? loss_out + i : nullptr, true);
+    if (adam) {
+      jobs[i].params = (void*)params[i];
+      jobs[i].m = adam_m[i];
+      jobs[i].v = adam_v[i];
+    }
+  }
+  const DevInstance* d_insts = b->d_insts;
+  const int* d_items = b->d_item_inst;
+  const ReduceJob* d_jobs = b->d_jobs;
+  const size_t b_insts = sizeof(DevInstance) * n, b_items = sizeof(int) * b->items.size(), b_jobs = sizeof(ReduceJob) * n;
+  if (stream_is_capturing(s)) {
+    const void* src[3] = {b->insts.data(), b->items.data(), jobs.data()};
+    const size_t bytes[3] = {b_insts, b_items, b_jobs};
+    char* dst[3];
+    CK(b->captured.put(s, 3, src, bytes, dst));
+    d_insts = reinterpret_cast<const DevInstance*>(dst[0]);
+    d_items = reinterpret_cast<const int*>(dst[1]);
+    d_jobs = reinterpret_cast<const ReduceJob*>(dst[2]);
+  } else {
+    if (b->copied) CK(cudaEventSynchronize(b->copied));
+    else CK(cudaEventCreateWithFlags(&b->copied, cudaEventDisableTiming));
+    memcpy(b->h_insts, b->insts.data(), b_insts);
+    memcpy(b->h_item_inst, b->items.data(), b_items);
+    memcpy(b->h_jobs, jobs.data(), b_jobs);
+    CK(cudaMemcpyAsync(b->d_insts, b->h_insts, b_insts, cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(b->d_item_inst, b->h_item_inst, b_items, cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(b->d_jobs, b->h_jobs, b_jobs, cudaMemcpyHostToDevice, s));
+    CK(cudaEventRecord(b->copied, s));
+  }
+  for (int i = 0; i < n; ++i) CK(launch_transpose_weights(b->insts[i], b->fp64, (void*)b->insts[i].Wt, s));
   SimtArgs a;
   memset(&a, 0, sizeof(a));
   a.mode = MODE_FWD_BWD;
   a.n_inst = n;
-  a.insts = b->d_insts;
+  a.insts = d_insts;
   a.n_items = n_items;
-  a.item_inst = b->d_item_inst;
+  a.item_inst = d_items;
   a.scratch = b->scratch;
   a.scratch_stride = b->scratch_stride;
   a.item_next = b->d_next;
@@ -1044,24 +1074,7 @@ static jet_status batch_run(jet_batch_t b, const void* const* params, void* cons
   a.carveout = simt_carveout(b->smem, b->ctas_per_sm);
   CK(cudaMemsetAsync(b->d_next, 0, sizeof(int), s));
   CK(simt_launch(b->cls, b->fp64, a, std::min(b->grid, n_items), b->smem, s));
-  for (int i = 0; i < n; ++i) {
-    ReduceJob j = make_job(b->h_insts[i], adam ? nullptr : grad_out[i], loss_out ? loss_out + i : nullptr, true);
-    if (adam) {
-      j.params = (void*)params[i];
-      j.m = adam_m[i];
-      j.v = adam_v[i];
-    }
-    b->h_jobs[i] = j;
-  }
-  CK(cudaMemcpyAsync(b->d_jobs, b->h_jobs, sizeof(ReduceJob) * n, cudaMemcpyHostToDevice, s));
-  if (!b->copied) CK(cudaEventCreateWithFlags(&b->copied, cudaEventDisableTiming));
-  cudaStreamCaptureStatus cs2 = cudaStreamCaptureStatusNone;
-  cudaStreamIsCapturing(s, &cs2);
-  if (cs2 == cudaStreamCaptureStatusNone) {  // a captured upload replays from the staging of the latest call
-    CK(cudaEventRecord(b->copied, s));
-    b->have_prev = true;
-  }
-  CK(launch_reduce(b->h_jobs, b->d_jobs, n, b->fp64, adam, step, lr, s, step_ctr));
+  CK(launch_reduce(jobs.data(), d_jobs, n, b->fp64, adam, step, lr, s, step_ctr));
   return JET_OK;
 }
 

@@ -10,6 +10,7 @@
 #include <cstring>
 #include <vector>
 
+#include "jet_capture.h"
 #include "jet_closures_gen.h"
 #include "jet_internal.h"
 #include "jet_plan.h"
@@ -736,10 +737,7 @@ size_t tc_workspace_bytes(const TcPlan* t) { return t ? t->ws_bytes : 0; }
 
 namespace {
 
-bool is_capturing(cudaStream_t s) {
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone;
-}
+bool is_capturing(cudaStream_t s) { return stream_is_capturing(s); }
 
 // Device-side wait time-outs of an earlier call surface here.  While the
 // stream is being captured into a CUDA graph nothing is reported (the error
@@ -1082,8 +1080,9 @@ struct TcBatch {
   unsigned char* scratch = nullptr;
   long long scratch_stride = 0;
   int* err = nullptr;
-  cudaEvent_t copied = nullptr;  // descriptor upload of the previous call
+  cudaEvent_t copied = nullptr;  // descriptor upload of the previous eager call
   bool have_prev = false;
+  CaptureStore captured;  // descriptors of captured calls
 };
 }  // namespace jet
 
@@ -1161,9 +1160,6 @@ jet_status tc_batch_create(const std::vector<jet_plan_s*>& plans, TcBatch** out)
     tc_batch_destroy(b);
     return tcuda(e, "batch workspace");
   }
-  memset(b->h_insts, 0, sizeof(TcInst) * b->n);
-  memset(b->h_prep, 0, sizeof(PrepJob) * b->n);
-  memset(b->h_jobs, 0, sizeof(ReduceJob) * b->n);  // no job of an earlier batch in recycled pinned memory
   *out = b;
   return JET_OK;
 }
@@ -1245,36 +1241,66 @@ jet_status tc_batch_run(TcBatch* bb, const std::vector<jet_plan_s*>& plans, cons
   std::stable_sort(cost.begin(), cost.end(), [](const std::pair<double, int>& x, const std::pair<double, int>& y) {
     return x.first > y.first;
   });
-  const bool capturing = [&] {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    cudaStreamIsCapturing(s, &cs);
-    return cs != cudaStreamCaptureStatusNone;
-  }();
-  // upload the descriptors only when they changed; wait for the previous
-  // upload to have read the staging buffers before rewriting them
-  bool same = b->have_prev && b->n_items == base && memcmp(b->h_insts, insts.data(), sizeof(TcInst) * n) == 0 &&
-              memcmp(b->h_prep, prep_jobs.data(), sizeof(PrepJob) * n) == 0;
-  if (same)
-    for (int k = 0; k < base && same; ++k) same = b->h_items[k] == cost[k].second && b->h_items[base + k] == inst_of[k];
-  if (!same) {
-    if (b->have_prev && !capturing) cudaEventSynchronize(b->copied);
-    memcpy(b->h_insts, insts.data(), sizeof(TcInst) * n);
-    memcpy(b->h_prep, prep_jobs.data(), sizeof(PrepJob) * n);
-    for (int k = 0; k < base; ++k) {
-      b->h_items[k] = cost[k].second;
-      b->h_items[base + k] = inst_of[k];
+  std::vector<int> items(2 * (size_t)base);  // list position -> item, then item -> instance
+  for (int k = 0; k < base; ++k) {
+    items[k] = cost[k].second;
+    items[base + k] = inst_of[k];
+  }
+  std::vector<ReduceJob> jobs(n);
+  for (int i = 0; i < n; ++i) {
+    jobs[i] = grad_job(plans[i], plans[i]->tcp, insts[i]);
+    jobs[i].grad_out = adam ? nullptr : grad_out[i];
+    jobs[i].loss_out = loss_out ? loss_out + i : nullptr;
+    if (adam) {
+      jobs[i].params = const_cast<void*>(params[i]);
+      jobs[i].m = m[i];
+      jobs[i].v = v[i];
     }
-    b->n_items = base;
-    cudaError_t e = cudaMemcpyAsync(b->d_insts, b->h_insts, sizeof(TcInst) * n, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_items, b->h_items, sizeof(int) * 2 * base, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_prep, b->h_prep, sizeof(PrepJob) * n, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess && !capturing) e = cudaEventRecord(b->copied, s);
+  }
+  const TcInst* d_insts = b->d_insts;
+  const int* d_items = b->d_items;
+  const PrepJob* d_prep = b->d_prep;
+  const ReduceJob* d_jobs = b->d_jobs;
+  if (is_capturing(s)) {
+    const void* src[4] = {insts.data(), items.data(), prep_jobs.data(), jobs.data()};
+    const size_t bytes[4] = {sizeof(TcInst) * n, sizeof(int) * items.size(), sizeof(PrepJob) * n, sizeof(ReduceJob) * n};
+    char* dst[4];
+    const cudaError_t e = b->captured.put(s, 4, src, bytes, dst);
+    if (e != cudaSuccess) return tcuda(e, "descriptors of a captured batch call");
+    d_insts = reinterpret_cast<const TcInst*>(dst[0]);
+    d_items = reinterpret_cast<const int*>(dst[1]);
+    d_prep = reinterpret_cast<const PrepJob*>(dst[2]);
+    d_jobs = reinterpret_cast<const ReduceJob*>(dst[3]);
+  } else {
+    // upload what changed since the previous eager call, whose upload has to have
+    // read the staging buffers before they are rewritten
+    const bool same = b->have_prev && b->n_items == base && memcmp(b->h_insts, insts.data(), sizeof(TcInst) * n) == 0 &&
+                      memcmp(b->h_prep, prep_jobs.data(), sizeof(PrepJob) * n) == 0 &&
+                      memcmp(b->h_items, items.data(), sizeof(int) * items.size()) == 0;
+    const bool jobs_same = b->have_prev && memcmp(b->h_jobs, jobs.data(), sizeof(ReduceJob) * n) == 0;
+    cudaError_t e = cudaSuccess;
+    if ((!same || !jobs_same) && b->have_prev) e = cudaEventSynchronize(b->copied);
+    if (!same && e == cudaSuccess) {
+      memcpy(b->h_insts, insts.data(), sizeof(TcInst) * n);
+      memcpy(b->h_prep, prep_jobs.data(), sizeof(PrepJob) * n);
+      memcpy(b->h_items, items.data(), sizeof(int) * items.size());
+      b->n_items = base;
+      e = cudaMemcpyAsync(b->d_insts, b->h_insts, sizeof(TcInst) * n, cudaMemcpyHostToDevice, s);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_items, b->h_items, sizeof(int) * items.size(), cudaMemcpyHostToDevice, s);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_prep, b->h_prep, sizeof(PrepJob) * n, cudaMemcpyHostToDevice, s);
+    }
+    if (!jobs_same && e == cudaSuccess) {
+      memcpy(b->h_jobs, jobs.data(), sizeof(ReduceJob) * n);
+      e = cudaMemcpyAsync(b->d_jobs, b->h_jobs, sizeof(ReduceJob) * n, cudaMemcpyHostToDevice, s);
+    }
+    if ((!same || !jobs_same) && e == cudaSuccess) e = cudaEventRecord(b->copied, s);
+    // after a failure the staging says nothing about what the device holds
+    b->have_prev = e == cudaSuccess;
     if (e != cudaSuccess) return tcuda(e, "batch descriptor upload");
-    b->have_prev = b->have_prev || !capturing;
   }
   {
     const int pgrid = (int)std::min<long long>((prep_total + 255) / 256, 2048);
-    const cudaError_t pe = launch_dependent(&tc_prep_batch_kernel, pgrid, 256, 0, s, b->d_prep, n, prep_total);
+    const cudaError_t pe = launch_dependent(&tc_prep_batch_kernel, pgrid, 256, 0, s, d_prep, n, prep_total);
     if (pe != cudaSuccess) return tcuda(pe, "batched weight preparation");
   }
   TcArgs a;
@@ -1287,8 +1313,8 @@ jet_status tc_batch_run(TcBatch* bb, const std::vector<jet_plan_s*>& plans, cons
   }
   a.mode = MODE_FWD_BWD;
   a.n_items = base;
-  a.insts = b->d_insts;
-  a.item_inst = b->d_items;
+  a.insts = d_insts;
+  a.item_inst = d_items;
   a.item_next = b->d_next;
   a.err = b->err;
   a.tmem_cols = b->tmem_cols;
@@ -1297,28 +1323,7 @@ jet_status tc_batch_run(TcBatch* bb, const std::vector<jet_plan_s*>& plans, cons
   if (e != cudaSuccess) return tcuda(e, "batch item counter reset");
   e = tc_launch(b->cls, a, std::min(b->grid, base), b->smem, s);
   if (e != cudaSuccess) return tcuda(e, "batched tc kernel launch");
-  bool jobs_same = !capturing;
-  for (int i = 0; i < n; ++i) {
-    ReduceJob j = grad_job(plans[i], plans[i]->tcp, insts[i]);
-    j.grad_out = adam ? nullptr : grad_out[i];
-    j.loss_out = loss_out ? loss_out + i : nullptr;
-    if (adam) {
-      j.params = const_cast<void*>(params[i]);
-      j.m = m[i];
-      j.v = v[i];
-    }
-    if (jobs_same && memcmp(&b->h_jobs[i], &j, sizeof(j)) != 0) {
-      jobs_same = false;
-      if (b->have_prev && !capturing) cudaEventSynchronize(b->copied);
-    }
-    if (!jobs_same || capturing) b->h_jobs[i] = j;
-  }
-  if (!jobs_same || capturing) {
-    e = cudaMemcpyAsync(b->d_jobs, b->h_jobs, sizeof(ReduceJob) * n, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess && !capturing) e = cudaEventRecord(b->copied, s);
-    if (e != cudaSuccess) return tcuda(e, "batch job upload");
-  }
-  e = launch_reduce(b->h_jobs, b->d_jobs, n, false, adam, step, lr, s, step_ctr);
+  e = launch_reduce(jobs.data(), d_jobs, n, false, adam, step, lr, s, step_ctr);
   return e == cudaSuccess ? JET_OK : tcuda(e, "batch reduce");
 }
 
