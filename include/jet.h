@@ -288,7 +288,9 @@ jet_status jet_plan_destroy(jet_plan_t plan);
  * Batched ensemble: n independent plans (same precision; any shapes and
  * residuals) run as ONE persistent launch over a work list of
  * (instance, chunk of point tiles) items.  Arrays are host arrays of n
- * device pointers / sizes.
+ * device pointers / sizes.  Members of the FP64 and FP32 forms may have no
+ * points (N = 0: loss 0 and a zero gradient); the tensor-core forms need
+ * N >= 1 (JET_ERR_INVALID).
  */
 jet_status jet_batch_create(jet_batch_t* out, int32_t n, const jet_plan_t* plans, int32_t flags);
 jet_status jet_batch_backward(jet_batch_t batch, const void* const* params, const void* const* X,

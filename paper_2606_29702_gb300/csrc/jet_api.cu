@@ -898,8 +898,8 @@ jet_status batch_prepare(jet_batch_s* b, const void* const* params, const void* 
     DevInstance& I = b->insts[i];
     const long long tiles = (N[i] + b->P[i] - 1) / b->P[i];
     const double per_tile = tile_cost(i);
-    const long long want = std::min<long long>(
-        b->max_chunks_per_inst, std::max<long long>(1, (long long)(per_tile * (double)tiles / target + 0.5)));
+    const long long share = tiles > 0 ? (long long)(per_tile * (double)tiles / target + 0.5) : 0;
+    const long long want = std::min<long long>(b->max_chunks_per_inst, std::max<long long>(1, share));
     fill_instance(p, params[i], X[i], N[i], source ? source[i] : nullptr, r_out ? r_out[i] : nullptr, true, b->ru,
                   kSimtThreads, b->P[i], (int)want, I);
     I.Wt = (char*)b->Wt + b->wt_off[i] * p->elem;
@@ -1072,8 +1072,10 @@ static jet_status batch_run(jet_batch_t b, const void* const* params, void* cons
   a.ru = b->ru;
   a.threads = kSimtThreads;
   a.carveout = simt_carveout(b->smem, b->ctas_per_sm);
-  CK(cudaMemsetAsync(b->d_next, 0, sizeof(int), s));
-  CK(simt_launch(b->cls, b->fp64, a, std::min(b->grid, n_items), b->smem, s));
+  if (n_items > 0) {  // none: every member is empty
+    CK(cudaMemsetAsync(b->d_next, 0, sizeof(int), s));
+    CK(simt_launch(b->cls, b->fp64, a, std::min(b->grid, n_items), b->smem, s));
+  }
   CK(launch_reduce(jobs.data(), d_jobs, n, b->fp64, adam, step, lr, s, step_ctr));
   return JET_OK;
 }

@@ -222,13 +222,18 @@ inline int simt_carveout(size_t smem, int ctas) {
   const size_t pct = ((smem + kSimtCtaBytes) * ctas * 100 + kSimtSmBytes - 1) / kSimtSmBytes;
   return pct > 100 ? 100 : (int)pct;
 }
-// the chunks of a call: its units (tiles) over n_chunks CTAs or work items
+// the chunks of a call: its units (tiles) over n_chunks CTAs or work items.  No
+// points (an empty member of a batch): no chunk, so every sum over them is zero.
 inline void simt_set_chunks(DevInstance& I, long long n_chunks) {
   I.unit = I.P;
   I.n_tiles = (I.N + I.unit - 1) / I.unit;
-  if (n_chunks > I.n_tiles) n_chunks = I.n_tiles;
   if (n_chunks < 1) n_chunks = 1;
+  if (n_chunks > I.n_tiles) n_chunks = I.n_tiles;
   I.n_chunks = (int)n_chunks;
+  if (n_chunks == 0) {
+    I.tiles_per_chunk = I.chunk_rem = 0;
+    return;
+  }
   I.tiles_per_chunk = (int)(I.n_tiles / n_chunks);
   I.chunk_rem = (int)(I.n_tiles % n_chunks);
 }
