@@ -26,8 +26,12 @@
 // channel (the activation rule and its adjoint read z_0 only through tanh z_0):
 // the memory of the backward is bounded by the number of CTAs, not by N.
 // Gradient partial sums go to a per-(instance, chunk) FP64 slice; every slice
-// element is added by one thread in tile order (fire-and-forget FP64 adds),
-// so the final FP64 reduction is deterministic.
+// element is added by one thread, group of points after group in the order of the
+// tiles (fire-and-forget FP64 adds), so the final FP64 reduction is
+// deterministic.  With a thread per group of a tile the biases, W^1 and W^L had
+// no order: gradients whose sums cancel moved in the fourth digit; one thread per
+// element costs at most 1% (2->64x5->1 FP32 1.319 -> 1.331 ms, 16 FP32 networks
+// 3.80 -> 3.82 ms, 2->64x6->1 composite loss 304 -> 301 us).
 //
 // What bounds it: the FP32 pipe and shared-memory reads in the jet GEMMs
 // (about 80% of the time), the FP64 pipe in the FP64 form.  Against the form
@@ -657,32 +661,34 @@ struct SimtTile {
       }
       store_point(abar + k * pitch, n, s);
     }
-    // dW^L[o][k] per group of points: four lanes share a sum, each taking a
-    // quarter of the points; the partials combine by shuffles in a fixed order
-    // (the loop runs whole warps: every lane of a warp reaches the shuffles)
-    const int items = 4 * no * wi * V, items_w = (items + 31) & ~31;
+    // dW^L[o][k], the groups of points one after another: four lanes share a sum,
+    // each taking a quarter of a group's points; the partials combine by shuffles
+    // in a fixed order (the loop runs whole warps: every lane reaches the shuffles)
+    const int items = 4 * no * wi, items_w = (items + 31) & ~31;
     for (int it = threadIdx.x; it < items_w; it += NT) {
       const bool act = it < items;
-      const int part = it & 3, e = act ? it >> 2 : 0, v = e / (no * wi), ok = e - v * (no * wi);
-      const int o = ok / wi, k = ok - o * wi;
-      T s = T(0);
-      if (act)
-        for (int n = v * P0 + part; n < (v + 1) * P0; n += 4) {
-          T av[C];
-          load_point(a_last + k * pitch, n, av);
+      const int part = it & 3, ok = act ? it >> 2 : 0, o = ok / wi, k = ok - o * wi;
+      for (int n0 = 0; n0 < P; n0 += P0) {
+        T s = T(0);
+        if (act)
+          for (int n = n0 + part; n < n0 + P0; n += 4) {
+            T av[C];
+            load_point(a_last + k * pitch, n, av);
 #pragma unroll
-          for (int c = 0; c < C; ++c) s = fma(UB[o * ncol + c * P + n], av[c], s);
-        }
-      s += __shfl_xor_sync(0xffffffffu, s, 1);
-      s += __shfl_xor_sync(0xffffffffu, s, 2);
-      if (act && part == 0) atomicAdd(g + I.goff_WL + o * wi + k, widen(s));
+            for (int c = 0; c < C; ++c) s = fma(UB[o * ncol + c * P + n], av[c], s);
+          }
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        if (act && part == 0) atomicAdd(g + I.goff_WL + o * wi + k, widen(s));
+      }
     }
-    for (int e = threadIdx.x; e < no * V; e += NT) {  // db^L per group
-      const int o = e / V, v = e - o * V;
-      T s = T(0);
-      for (int n = v * P0; n < (v + 1) * P0; ++n) s += UB[o * ncol + n];
-      atomicAdd(g + I.goff_b[L - 1] + o, widen(s));
-    }
+    for (int o = NT - 1 - threadIdx.x; o < no; o += NT)  // db^L, by the last threads
+      for (int n0 = 0; n0 < P; n0 += P0) {
+        T s = T(0);
+#pragma unroll 8
+        for (int n = n0; n < n0 + P0; ++n) s += UB[o * ncol + n];
+        atomicAdd(g + I.goff_b[L - 1] + o, widen(s));
+      }
   }
 
   // Zbar^l = (d compose / dz)^T Abar^l per (unit, point), in place in `bar`;
@@ -750,16 +756,17 @@ struct SimtTile {
       else if (I.wr == 4) wgrad32<4, false>(l, zbar, aprev, g);
       else wgrad32<(RU == 8 ? 2 : 1), false>(l, zbar, aprev, g);
     }
-    // a thread per bias and group of points
+    // a thread per bias, its groups one after another
     const int wo = I.widths[l];
     double* gb = g + I.goff_b[l - 1];
-    for (int it = threadIdx.x; it < wo * V; it += NT) {
-      const int u = it % wo, v = it / wo;
+    for (int u = threadIdx.x; u < wo; u += NT) {
       const T* zp = zbar + u * pitch;
-      T s = T(0);
-#pragma unroll 4
-      for (int n = v * P0; n < (v + 1) * P0; ++n) s += zp[n * C + (odd(n) ? 1 : 0)];
-      atomicAdd(gb + u, widen(s));
+      for (int n0 = 0; n0 < P; n0 += P0) {
+        T s = T(0);
+#pragma unroll 8
+        for (int n = n0; n < n0 + P0; ++n) s += zp[n * C + (odd(n) ? 1 : 0)];
+        atomicAdd(gb + u, widen(s));
+      }
     }
   }
 
@@ -954,35 +961,36 @@ struct SimtTile {
   }
 
   // dW^1[u][i] += sum_n Zbar_0[u][n] x_i[n] + Zbar_{e_i}[u][n]; db^1[u] += sum_n Zbar_0[u][n];
-  // a thread per unit and group of points
+  // a thread per unit, its groups of points one after another
   __device__ void layer1_bwd(const T* zbar, double* g) {
     const int w = I.widths[1], d = I.d;
     double* gW = g;
     double* gb = g + I.goff_b[0];
-    for (int it = threadIdx.x; it < w * V; it += NT) {
-      const int u = it % w, n0 = it / w * P0;
+    for (int u = threadIdx.x; u < w; u += NT) {
       const T* zp = zbar + u * pitch;
-      T sb = T(0), sw[3] = {T(0), T(0), T(0)};
+      for (int n0 = 0; n0 < P; n0 += P0) {
+        T sb = T(0), sw[3] = {T(0), T(0), T(0)};
 #pragma unroll 4
-      for (int n = n0; n < n0 + P0; ++n) {
-        const T z0 = zp[n * C + (odd(n) ? 1 : 0)];
-        sb += z0;
+        for (int n = n0; n < n0 + P0; ++n) {
+          const T z0 = zp[n * C + (odd(n) ? 1 : 0)];
+          sb += z0;
+#pragma unroll
+          for (int i = 0; i < 3; ++i)
+            if (i < d) sw[i] = fma(z0, XS[n * d + i], sw[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < Cls::D; ++i) {
+          const int fo = Cls::first_order(i);
+          if (fo >= 0 && i < d) {
+#pragma unroll 4
+            for (int n = n0; n < n0 + P0; ++n) sw[i] += zp[n * C + (odd(n) ? fo ^ 1 : fo)];
+          }
+        }
 #pragma unroll
         for (int i = 0; i < 3; ++i)
-          if (i < d) sw[i] = fma(z0, XS[n * d + i], sw[i]);
+          if (i < d) atomicAdd(gW + u * d + i, widen(sw[i]));
+        atomicAdd(gb + u, widen(sb));
       }
-#pragma unroll
-      for (int i = 0; i < Cls::D; ++i) {
-        const int fo = Cls::first_order(i);
-        if (fo >= 0 && i < d) {
-#pragma unroll 4
-          for (int n = n0; n < n0 + P0; ++n) sw[i] += zp[n * C + (odd(n) ? fo ^ 1 : fo)];
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-        if (i < d) atomicAdd(gW + u * d + i, widen(sw[i]));
-      atomicAdd(gb + u, widen(sb));
     }
   }
 
