@@ -1145,13 +1145,21 @@ __device__ __forceinline__ void simt_body(const SimtArgs& args) {
 
 // Launch bounds: up to 512 threads (one CTA per SM, or two of 256) and so at
 // most 128 registers, except where the tiles need one CTA of 256 threads with
-// all registers: FP64, and channel sets of 10 or more.
+// all registers (FP32 channel sets of 10 or more).  FP64 runs two CTAs of 256
+// where their tiles fit: one CTA's elementwise phases overlap the other's GEMMs
+// (with one of 160 registers 3->64x3->2 took 27.4 ms at 40000 points and
+// 3->256x2->1 10.7 ms at 4096, with two 24.3 and 10.1 ms).
 template <class Cls, class T>
 constexpr int simt_max_threads() {
   return sizeof(T) == 8 || Cls::C >= 10 ? 256 : 512;
 }
+template <class Cls, class T>
+constexpr int simt_min_ctas() {
+  return sizeof(T) == 8 ? 2 : 1;
+}
 template <class Cls, class T, int RU>
-__global__ void __launch_bounds__(simt_max_threads<Cls, T>(), 1) simt_kernel(const __grid_constant__ SimtArgs args) {
+__global__ void __launch_bounds__(simt_max_threads<Cls, T>(), simt_min_ctas<Cls, T>())
+    simt_kernel(const __grid_constant__ SimtArgs args) {
   simt_body<Cls, T, RU>(args);
 }
 
