@@ -291,6 +291,12 @@ jet_status jet_plan_destroy(jet_plan_t plan);
  * device pointers / sizes.  Members of the FP64 and FP32 forms may have no
  * points (N = 0: loss 0 and a zero gradient); the tensor-core forms need
  * N >= 1 (JET_ERR_INVALID).
+ * Device memory: the chunk sums of a call, at most 8 bytes per parameter (4 per
+ * hidden-layer weight where FP32 sums of a chunk suffice) and chunk, for one
+ * chunk per member and about three per CTA more (FP64 and FP32 forms) or
+ * max(16 members, 4 CTAs) chunks (tensor-core forms), beside weight copies and a
+ * scratch slot per CTA.  Where that does not fit, a batch is created with at most
+ * 16 chunks per member; JET_ERR_OOM if that does not fit either.
  */
 jet_status jet_batch_create(jet_batch_t* out, int32_t n, const jet_plan_t* plans, int32_t flags);
 jet_status jet_batch_backward(jet_batch_t batch, const void* const* params, const void* const* X,

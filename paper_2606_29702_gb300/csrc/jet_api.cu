@@ -815,6 +815,9 @@ jet_status jet_debug_activation(jet_plan_t p, int32_t kind, int64_t n, const dou
 
 // ------------------------------------------------------------------ batches
 
+constexpr int kSimtBatchChunks = 16;  // least bound of a member's chunks
+constexpr int kSimtBatchItems = 3;    // work items per CTA that the list aims at
+
 struct jet_batch_s {
   std::vector<jet_plan_t> plans;
   int cls = -1;
@@ -824,19 +827,22 @@ struct jet_batch_s {
   size_t smem = 0;
   int ru = 0, ctas_per_sm = 0;
   std::vector<int> P;  // points per tile of every member
-  int max_chunks_per_inst = 16;
+  int max_chunks_per_inst = kSimtBatchChunks;
   // device workspace
   DevInstance* d_insts = nullptr;
   int* d_item_inst = nullptr;
   int* d_next = nullptr;  // the kernel's item counter
   ReduceJob* d_jobs = nullptr;
-  double* grad_slices = nullptr;
+  // FP64 slices and FP32 weight-gradient sums of a call's chunks, cut out per call
+  // (batch_pool_bytes); loss sums [max_items]
+  char* pool = nullptr;
+  size_t pool_bytes = 0;
   double* loss_slices = nullptr;
   void* Wt = nullptr;
   void* scratch = nullptr;
   long long scratch_stride = 0;
-  float* wsums = nullptr;  // FP32 weight-gradient sums per chunk of the members that keep them
-  std::vector<long long> slice_off, wt_off, wsums_off;
+  float* run_sums = nullptr;  // FP32 sums of a CTA's running chunk, of members whose chunks take several runs
+  std::vector<long long> wt_off;
   // the call's descriptors and work list, and their pinned staging (eager calls)
   std::vector<DevInstance> insts;
   std::vector<int> items;
@@ -858,16 +864,44 @@ void free_batch(jet_batch_s* b) {
   cudaFree(b->d_item_inst);
   cudaFree(b->d_next);
   cudaFree(b->d_jobs);
-  cudaFree(b->grad_slices);
+  cudaFree(b->pool);
   cudaFree(b->loss_slices);
   cudaFree(b->Wt);
   cudaFree(b->scratch);
-  cudaFree(b->wsums);
+  cudaFree(b->run_sums);
   cudaFreeHost(b->h_insts);
   cudaFreeHost(b->h_item_inst);
   cudaFreeHost(b->h_jobs);
   if (b->tcb) tc_batch_destroy(b->tcb);
   if (b->copied) cudaEventDestroy(b->copied);
+}
+
+// Most bytes a chunk of a plan takes in the pool: its FP64 slice, beside FP32 sums
+// that the reduction reads or (channel sets of 7 or more, chunks of several runs)
+// with every parameter.
+size_t batch_chunk_bytes(const jet_plan_s* p) {
+  const size_t all = (size_t)p->n_params * sizeof(double);
+  if (!p->wsums) return all;
+  const size_t direct = (size_t)(p->n_params - p->wsums_stride) * sizeof(double) + (size_t)p->wsums_stride * sizeof(float);
+  return p->C < 7 ? direct : std::max(all, direct);
+}
+
+// Bytes that the chunks of any call fit: the work list gives every member one
+// chunk and shares about kSimtBatchItems per CTA more among them by cost, at most
+// max_chunks each, so the largest members may hold nearly all of them.  (Sized by
+// max_chunks for every member, nine 3->256x8->1 FP32 networks took 12.4 GB; 4 GB so.)
+size_t batch_pool_bytes(const std::vector<jet_plan_t>& plans, int grid, int max_chunks) {
+  std::vector<size_t> per;
+  for (const jet_plan_s* p : plans) per.push_back(batch_chunk_bytes(p));
+  std::sort(per.rbegin(), per.rend());
+  size_t total = 0;
+  long long extra = (long long)kSimtBatchItems * grid;
+  for (size_t b : per) {
+    const long long k = std::min<long long>(max_chunks - 1, extra);
+    extra -= k;
+    total += (size_t)(1 + k) * b + 2 * 256;  // alignment of its two parts
+  }
+  return total;
 }
 
 // Build the per-call descriptors and work list: every instance is split into
@@ -888,10 +922,16 @@ jet_status batch_prepare(jet_batch_s* b, const void* const* params, const void* 
     if (st != JET_OK) return st;
     total_cost += tile_cost(i) * (double)((N[i] + b->P[i] - 1) / b->P[i]);
   }
-  const double target = total_cost / (3.0 * b->grid);  // about three items of equal cost per CTA
+  const double target = total_cost / ((double)kSimtBatchItems * b->grid);  // items of equal cost
   std::vector<std::pair<double, int>> cost;  // (cost, item) for ordering
   std::vector<int> item_inst;
   int chunk_base = 0;
+  size_t pool_off = 0;
+  auto take = [&](size_t bytes) {
+    char* at = b->pool + pool_off;
+    pool_off += (bytes + 255) / 256 * 256;
+    return at;
+  };
   b->insts.resize(n);
   for (int i = 0; i < n; ++i) {
     jet_plan_s* p = b->plans[i];
@@ -903,8 +943,9 @@ jet_status batch_prepare(jet_batch_s* b, const void* const* params, const void* 
     fill_instance(p, params[i], X[i], N[i], source ? source[i] : nullptr, r_out ? r_out[i] : nullptr, true, b->ru,
                   kSimtThreads, b->P[i], (int)want, I);
     I.Wt = (char*)b->Wt + b->wt_off[i] * p->elem;
-    I.grad_slices = b->grad_slices + b->slice_off[i];
-    simt_set_sums(I, p->C, p->wsums ? b->wsums + b->wsums_off[i] : nullptr, p->wsums_stride);
+    simt_set_sums(I, p->C, p->wsums ? b->run_sums : nullptr, p->wsums_stride);
+    I.grad_slices = reinterpret_cast<double*>(take((size_t)I.n_chunks * I.n_slice * sizeof(double)));
+    if (I.wsums_direct) I.wsums = reinterpret_cast<float*>(take((size_t)I.n_chunks * I.wsums_stride * sizeof(float)));
     I.loss_slices = b->loss_slices + (long long)i * b->max_chunks_per_inst;
     I.chunk_base = chunk_base;
     for (int c = 0; c < I.n_chunks; ++c) {
@@ -914,7 +955,7 @@ jet_status batch_prepare(jet_batch_s* b, const void* const* params, const void* 
     }
     chunk_base += I.n_chunks;
   }
-  if (chunk_base > b->max_items) return fail(JET_ERR_INVALID, "internal: work list overflow");
+  if (chunk_base > b->max_items || pool_off > b->pool_bytes) return fail(JET_ERR_INVALID, "internal: work list overflow");
   std::vector<int> order(chunk_base);
   for (int k = 0; k < chunk_base; ++k) order[k] = k;
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost[x].first > cost[y].first; });
@@ -983,14 +1024,11 @@ jet_status jet_batch_create(jet_batch_t* out, int32_t n, const jet_plan_t* plans
   // the work list holds about three items per CTA, shared by cost: a member may
   // take several times its share (with 16 members a fixed 16 chunks left the largest
   // member's chunks running alone: 26.4 ms against 4.0 ms)
-  b->max_chunks_per_inst = std::min(256, std::max(16, 8 * b->grid / n));
-  long long scr = 0, slices = 0, wt = 0, sums = 0;
+  b->max_chunks_per_inst = std::min(256, std::max(kSimtBatchChunks, 8 * b->grid / n));
+  long long scr = 0, wt = 0, runs = 0;
   for (int i = 0; i < n; ++i) {
     scr = std::max(scr, plans[i]->scratch_stride);
-    b->wsums_off.push_back(sums);
-    sums += (long long)b->max_chunks_per_inst * plans[i]->wsums_stride;
-    b->slice_off.push_back(slices);
-    slices += (long long)b->max_chunks_per_inst * plans[i]->n_params;
+    runs = std::max(runs, plans[i]->wsums_stride);
     b->wt_off.push_back(wt);
     wt += weight_ws_elems(plans[i]->n_params);
   }
@@ -1001,14 +1039,22 @@ jet_status jet_batch_create(jet_batch_t* out, int32_t n, const jet_plan_t* plans
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_item_inst, sizeof(int) * 2 * b->max_items);
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_next, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_jobs, sizeof(ReduceJob) * n);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b->grad_slices, sizeof(double) * std::max<long long>(slices, 1));
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->loss_slices, sizeof(double) * b->max_items);
-  if (e == cudaSuccess && sums) e = cudaMalloc((void**)&b->wsums, sizeof(float) * sums);
+  if (e == cudaSuccess && runs) e = cudaMalloc((void**)&b->run_sums, sizeof(float) * b->grid * (size_t)runs);
   if (e == cudaSuccess) e = cudaMalloc(&b->Wt, elem * std::max<long long>(wt, 1));
   if (e == cudaSuccess) e = cudaMalloc(&b->scratch, elem * (size_t)b->grid * std::max<long long>(scr, 1));
   if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_insts, sizeof(DevInstance) * n);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_item_inst, sizeof(int) * 2 * b->max_items);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_jobs, sizeof(ReduceJob) * n);
+  // the pool last: where it does not fit, one for the least bound of chunks
+  while (e == cudaSuccess) {
+    b->pool_bytes = batch_pool_bytes(b->plans, b->grid, b->max_chunks_per_inst);
+    e = cudaMalloc((void**)&b->pool, b->pool_bytes);
+    if (e != cudaErrorMemoryAllocation || b->max_chunks_per_inst == kSimtBatchChunks) break;
+    cudaGetLastError();
+    b->max_chunks_per_inst = kSimtBatchChunks;
+    e = cudaSuccess;
+  }
   if (e != cudaSuccess) {
     free_batch(b);
     delete b;

@@ -89,10 +89,10 @@ struct alignas(16) DevInstance {
   // [w][C * P] (as the shared-memory rows); null if not stored
   void* store;
   long long store_tile_stride;  // elements per tile
-  // FP32 forms: FP32 sums of the hidden-layer weight gradients of each chunk
-  // (simt_wacc_elems floats, in the item order of the weight gradient), or null:
-  // FP64 adds per tile.  wsums_direct: the reduction reads them; else the chunk
-  // adds them to its slice after every kWaccTiles tiles
+  // FP32 forms: FP32 sums of the hidden-layer weight gradients (simt_wacc_elems
+  // floats, in the item order of the weight gradient), or null: FP64 adds per
+  // tile.  wsums_direct: of each chunk, and the reduction reads them; else of each
+  // CTA's running chunk, which adds them to its slice after every kWaccTiles tiles
   float* wsums;
   long long wsums_stride;
   int wsums_direct;

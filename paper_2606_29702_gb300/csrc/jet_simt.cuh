@@ -244,7 +244,7 @@ struct SimtTile {
     params = reinterpret_cast<const T*>(I.params);
     Wt = reinterpret_cast<const T*>(I.Wt);
     Wc = Wt + weight_copy_offset(I.n_params);
-    if (F32 && I.wsums) wacc_base = I.wsums + (long long)chunk * I.wsums_stride;
+    if (F32 && I.wsums) wacc_base = I.wsums + (long long)(I.wsums_direct ? chunk : (int)blockIdx.x) * I.wsums_stride;
   }
 
   // a point's channels in a jet row: exchange of channel pairs (see I.swap)
