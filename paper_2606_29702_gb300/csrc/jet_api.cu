@@ -36,6 +36,7 @@ jet_status fail(jet_status st, const char* fmt, ...) {
 }
 
 jet_status cuda_fail(cudaError_t e, const char* what) {
+  cudaGetLastError();  // reported here: a caller's next check of its own calls does not find it
   return fail(e == cudaErrorMemoryAllocation ? JET_ERR_OOM : JET_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 

@@ -42,6 +42,7 @@ jet_status nfail(jet_status st, const char* msg) {
 }
 
 jet_status nfail_cuda(cudaError_t e, const char* what) {
+  cudaGetLastError();  // reported here: a caller's next check of its own calls does not find it
   char buf[256];
   snprintf(buf, sizeof(buf), "%s: %s", what, cudaGetErrorString(e));
   jet::set_last_error(buf);
