@@ -165,7 +165,10 @@ typedef struct {
  *              that fits shared memory only with the store (one activation
  *              buffer); its jet_backward_params / jet_train_step then return
  *              JET_ERR_OOM when N points do not fit the budget, and it cannot
- *              join a batch (JET_ERR_UNSUPPORTED).
+ *              join a batch (JET_ERR_UNSUPPORTED).  Its store grows with the
+ *              largest N of the calls outside stream capture; one that a CUDA
+ *              graph uses is kept beside the larger one until the graph is
+ *              destroyed.
  * On success *out owns device workspace until jet_plan_destroy.
  */
 jet_status jet_plan_create(jet_plan_t* out, const jet_residual_spec* spec, int32_t d_in, int32_t n_layers,

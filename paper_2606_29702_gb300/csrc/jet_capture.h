@@ -1,12 +1,17 @@
-// Descriptors of batched calls under stream capture.
+// Device memory that captured calls use.
 //
-// An eager call uploads its descriptors through the batch's staging buffers, on
-// the stream.  A captured call runs later and repeatedly, with other calls in
-// between: an upload captured from the staging would replay with the arguments of
-// whichever call wrote it last, on a work list of another length.  So a captured
-// call's descriptors go to device memory of their own, filled at once (nothing of
-// the upload is in the graph).  The graph holds a reference: when the last graph
-// of a block is gone, a later captured call takes it over.
+// A captured call runs later and repeatedly, with other calls in between, on the
+// memory that its graph's nodes name.  GraphUse tells whether a graph that uses a
+// piece of memory is still there: the graph, its clones and its executables hold a
+// reference each, which goes with them.
+//
+// CaptureStore keeps the descriptors of captured batch calls.  An eager call
+// uploads its descriptors through the batch's staging buffers, on the stream; an
+// upload captured from the staging would replay with the arguments of whichever
+// call wrote it last, on a work list of another length.  So a captured call's
+// descriptors go to device memory of their own, filled at once (nothing of the
+// upload is in the graph); when no graph uses a block, a later captured call takes
+// it over.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -17,33 +22,66 @@
 
 namespace jet {
 
+inline bool stream_is_capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone;
+}
+
+class GraphUse {
+  using Count = std::shared_ptr<std::atomic<int>>;
+  Count n = std::make_shared<std::atomic<int>>(0);
+
+  // a graph's reference goes (may run on a thread of the driver, after the plan or batch)
+  static void CUDART_CB release(void* p) {
+    auto* ref = static_cast<Count*>(p);
+    --**ref;
+    delete ref;
+  }
+
+ public:
+  bool live() const { return *n > 0; }
+
+  // the graph that is being captured on s uses the memory
+  cudaError_t add(cudaStream_t s) {
+    cudaStreamCaptureStatus st;
+    cudaGraph_t graph = nullptr;
+    cudaError_t e = cudaStreamGetCaptureInfo(s, &st, nullptr, &graph);
+    if (e != cudaSuccess) return e;
+    if (st != cudaStreamCaptureStatusActive) return cudaErrorStreamCaptureInvalidated;
+    auto* own = new Count(n);
+    ++*n;
+    cudaUserObject_t ref;
+    e = cudaUserObjectCreate(&ref, own, release, 1, cudaUserObjectNoDestructorSync);
+    if (e != cudaSuccess) {
+      release(own);
+      return e;
+    }
+    e = cudaGraphRetainUserObject(graph, ref, 1, cudaGraphUserObjectMove);
+    if (e != cudaSuccess) cudaUserObjectRelease(ref, 1);
+    return e;
+  }
+};
+
 class CaptureStore {
   struct Block {
     char* dev = nullptr;
     size_t bytes = 0;
-    std::atomic<bool> in_graph{false};
+    GraphUse use;
   };
-  std::vector<std::shared_ptr<Block>> blocks;
+  std::vector<Block> blocks;
 
-  // destructor of the graph's reference (may run on a thread of the driver)
-  static void CUDART_CB release(void* p) {
-    auto* ref = static_cast<std::shared_ptr<Block>*>(p);
-    (*ref)->in_graph = false;
-    delete ref;
-  }
-
-  cudaError_t take(size_t bytes, std::shared_ptr<Block>* out) {
-    for (const auto& b : blocks)
-      if (!b->in_graph && b->bytes >= bytes) {
-        *out = b;
+  cudaError_t take(size_t bytes, Block** out) {
+    for (Block& b : blocks)
+      if (!b.use.live() && b.bytes >= bytes) {
+        *out = &b;
         return cudaSuccess;
       }
-    auto b = std::make_shared<Block>();
-    const cudaError_t e = cudaMalloc((void**)&b->dev, bytes);
+    Block b;
+    const cudaError_t e = cudaMalloc((void**)&b.dev, bytes);
     if (e != cudaSuccess) return e;
-    b->bytes = bytes;
+    b.bytes = bytes;
     blocks.push_back(b);
-    *out = b;
+    *out = &blocks.back();
     return cudaSuccess;
   }
 
@@ -74,41 +112,19 @@ class CaptureStore {
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
     if (e != cudaSuccess) return e;
-    std::shared_ptr<Block> b;
+    Block* b = nullptr;
     e = take(total > 0 ? total : 256, &b);
     if (e == cudaSuccess) e = fill(b->dev, src, bytes, off, n);
     cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e == cudaSuccess) e = b->use.add(s);
     if (e != cudaSuccess) return e;
-    cudaStreamCaptureStatus st;
-    cudaGraph_t graph = nullptr;
-    e = cudaStreamGetCaptureInfo(s, &st, nullptr, &graph);
-    if (e != cudaSuccess) return e;
-    if (st != cudaStreamCaptureStatusActive) return cudaErrorStreamCaptureInvalidated;
-    cudaUserObject_t ref;
-    auto* own = new std::shared_ptr<Block>(b);
-    e = cudaUserObjectCreate(&ref, own, release, 1, cudaUserObjectNoDestructorSync);
-    if (e != cudaSuccess) {
-      delete own;
-      return e;
-    }
-    b->in_graph = true;
-    e = cudaGraphRetainUserObject(graph, ref, 1, cudaGraphUserObjectMove);
-    if (e != cudaSuccess) {
-      cudaUserObjectRelease(ref, 1);
-      return e;
-    }
     for (int i = 0; i < n; ++i) dst[i] = b->dev + off[i];
     return cudaSuccess;
   }
 
   ~CaptureStore() {
-    for (const auto& b : blocks) cudaFree(b->dev);
+    for (const Block& b : blocks) cudaFree(b.dev);
   }
 };
-
-inline bool stream_is_capturing(cudaStream_t s) {
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone;
-}
 
 }  // namespace jet

@@ -67,6 +67,15 @@ struct TcPlan {
   unsigned char* wstore = nullptr;
   long long wstore_tile_stride = 0, wstore_tiles = 0;
   size_t wstore_budget = 0;  // grown on demand up to this many bytes
+  // graphs whose replays write the store; stores that were too small for a later
+  // call, kept while a graph uses them
+  GraphUse wstore_use;
+  struct OldStore {
+    unsigned char* dev;
+    size_t bytes;
+    GraphUse use;
+  };
+  std::vector<OldStore> old_stores;
   void* wg_ws = nullptr;    // wg_out and hid64
   float* wg_out = nullptr;  // [max_items][w*w]
   int wg_max_items = 0, wg_sms = 0;
@@ -724,6 +733,7 @@ void tc_plan_destroy(TcPlan* t) {
   if (!t) return;
   cudaFree(t->ws);
   cudaFree(t->wstore);
+  for (const TcPlan::OldStore& o : t->old_stores) cudaFree(o.dev);
   cudaFree(t->wg_ws);
   cudaFreeHost(t->h_err);
   delete t;
@@ -839,10 +849,6 @@ void fill_tc(const jet_plan_s* p, const TcPlan* t, const void* params, const voi
   I.wstore_tile_stride = t->wstore_tile_stride;
 }
 
-// Grow the weight-gradient store to the tiles of N points when the plan's
-// budget allows; otherwise the call runs in per-tile mode.  A call that grows
-// it allocates (and cudaFree synchronises): make the first call with the
-// largest N before any stream capture.
 jet_status store_too_small(const TcPlan* t, long long N) {
   char msg[200];
   snprintf(msg, sizeof(msg),
@@ -852,6 +858,11 @@ jet_status store_too_small(const TcPlan* t, long long N) {
   return tfail(JET_ERR_OOM, msg);
 }
 
+// Grow the weight-gradient store to the tiles of N points when the plan's
+// budget allows; otherwise the call runs in per-tile mode.  A call that grows
+// it allocates (and cudaFree synchronises), which a captured call does not: make
+// a call with its N before the capture.  A store that a graph writes stays beside
+// its successor until the graph is gone.
 void ensure_store(TcPlan* t, long long N, cudaStream_t s) {
   if (!t->wstore_budget || !t->wg_out || N < 1 || is_capturing(s)) return;
   const long long tiles = (N + t->P - 1) / t->P;
@@ -859,11 +870,17 @@ void ensure_store(TcPlan* t, long long N, cudaStream_t s) {
   const size_t need = (size_t)tiles * (size_t)t->wstore_tile_stride;
   if (need > t->wstore_budget) return;
   if (t->wstore) {
-    cudaFree(t->wstore);
-    t->ws_bytes -= (size_t)t->wstore_tiles * (size_t)t->wstore_tile_stride;
+    t->old_stores.push_back({t->wstore, (size_t)t->wstore_tiles * (size_t)t->wstore_tile_stride, t->wstore_use});
     t->wstore = nullptr;
     t->wstore_tiles = 0;
+    t->wstore_use = GraphUse();
   }
+  for (size_t i = t->old_stores.size(); i-- > 0;)
+    if (!t->old_stores[i].use.live()) {
+      cudaFree(t->old_stores[i].dev);
+      t->ws_bytes -= t->old_stores[i].bytes;
+      t->old_stores.erase(t->old_stores.begin() + i);
+    }
   if (cudaMalloc((void**)&t->wstore, need) == cudaSuccess) {
     t->wstore_tiles = tiles;
     t->ws_bytes += need;
@@ -914,8 +931,11 @@ jet_status run(jet_plan_s* p, TcPlan* t, int mode, const TcInst& I, cudaStream_t
   a.tmem_cols = t->tmem_cols;
   a.nthreads = t->nthreads;
   const int grid = std::min(t->grid, I.n_chunks);
+  cudaError_t e = cudaSuccess;
+  if (I.wstore && mode != MODE_FWD && is_capturing(s)) e = t->wstore_use.add(s);
+  if (e != cudaSuccess) return tcuda(e, "captured use of the weight-gradient store");
   jet::plan_prof_begin(p, s);
-  cudaError_t e = tc_launch(p->cls, a, grid, t->smem, s);
+  e = tc_launch(p->cls, a, grid, t->smem, s);
   if (e == cudaSuccess && mode != MODE_FWD && I.wstore) {
     // weight gradients of the hidden-to-hidden layers from the store
     WgArgs w;
