@@ -249,7 +249,8 @@ jet_status jet_forward_residual(jet_plan_t plan, const void* params, const void*
  * The hidden jets are recomputed tile by tile from the inputs, unless the plan
  * stores them and the previous jet_forward_residual on this plan used the same
  * params, X, N and source pointers (the caller must not have changed their
- * contents in between).
+ * contents in between); a captured backward pass uses the store of a forward pass
+ * of the same capture, an eager one no store that a CUDA graph writes too.
  */
 jet_status jet_backward_params(jet_plan_t plan, const void* params, const void* X, int64_t N,
                                const void* source, void* grad_out, void* r_out, double* loss_out,

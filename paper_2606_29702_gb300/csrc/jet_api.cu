@@ -724,13 +724,16 @@ jet_status jet_forward_residual(jet_plan_t p, const void* params, const void* X,
   DevInstance I;
   fill_instance(p, params, X, N, source, r_out, false, p->ru, p->threads, 0, 0, I);
   const bool store = p->store && N <= p->store_max_points;
+  const unsigned long long capture = p->store ? stream_capture_id(s) : 0;
   if (store) I.store = p->store;
+  if (store && capture) CK(p->st_graphs.add(s));
   CK(launch_transpose_weights(I, p->fp64, p->Wt, s));
   st = run_simt(p, MODE_FWD, I, s);
   if (st != JET_OK) return st;
   ReduceJob j = make_job(I, nullptr, loss_out, false);
   if (loss_out) CK(launch_reduce(&j, nullptr, 1, p->fp64, false, 1, 0.f, s));
   p->st_valid = store;
+  p->st_capture = capture;
   p->st_params = params;
   p->st_X = X;
   p->st_src = source;
@@ -752,8 +755,11 @@ jet_status jet_backward_params(jet_plan_t p, const void* params, const void* X, 
   }
   DevInstance I;
   fill_instance(p, params, X, N, source, r_out, true, p->ru, p->threads, 0, 0, I);
+  // a captured forward pass fills the store for its own graph's backward only, and
+  // while a graph writes the store no eager call relies on it
+  const unsigned long long capture = p->st_valid ? stream_capture_id(s) : 0;
   const bool from_store = p->st_valid && p->st_params == params && p->st_X == X && p->st_N == N &&
-                          p->st_src == source;
+                          p->st_src == source && p->st_capture == capture && (capture || !p->st_graphs.live());
   if (from_store) I.store = p->store;
   CK(launch_transpose_weights(I, p->fp64, p->Wt, s));
   st = run_simt(p, from_store ? MODE_BWD_STORE : MODE_FWD_BWD, I, s);

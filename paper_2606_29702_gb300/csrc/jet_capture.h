@@ -27,6 +27,14 @@ inline bool stream_is_capturing(cudaStream_t s) {
   return cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone;
 }
 
+// the capture that s is part of (never 0), 0: none
+inline unsigned long long stream_capture_id(cudaStream_t s) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(s, &cs, &id) != cudaSuccess || cs == cudaStreamCaptureStatusNone) return 0;
+  return id;
+}
+
 class GraphUse {
   using Count = std::shared_ptr<std::atomic<int>>;
   Count n = std::make_shared<std::atomic<int>>(0);

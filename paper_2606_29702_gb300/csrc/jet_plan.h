@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "../../include/jet.h"
+#include "jet_capture.h"
 #include "jet_internal.h"
 
 namespace jet {
@@ -79,8 +80,11 @@ struct jet_plan_s {
   void* store = nullptr;
   long long store_max_points = 0;
   size_t ws_bytes = 0;
-  // identity of the forward call whose jets the store holds
+  // identity of the forward call whose jets the store holds (st_capture: the
+  // capture it is part of, 0: eager), and the graphs whose replays write the store
   bool st_valid = false;
+  unsigned long long st_capture = 0;
+  jet::GraphUse st_graphs;
   const void* st_params = nullptr;
   const void* st_X = nullptr;
   const void* st_src = nullptr;

@@ -46,3 +46,31 @@ def test_graph_keeps_its_store_when_the_plan_grows_one():
     assert both > small
     per_point = (both - small) / xs[1].shape[0]
     assert plan.info()["workspace_bytes"] <= small + 1.05 * per_point * (xs[2].shape[0] - xs[0].shape[0]) + (1 << 22)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_store_of_captured_and_eager_passes(prec):
+    """A backward pass takes the jets of a forward pass that has run on its inputs, or computes its own: not those of a
+    captured pass that has not run, and not what a replay put over an eager pass's."""
+    widths = [2, 20, 20, 20, 1]
+    plan, p, (x, y) = _setup(prec, widths, [700, 900], 1 << 28)
+    want = [plan.backward(p, t)[0].clone() for t in (x, y)]
+    tol = dict(rtol=0, atol=1e-5 * float(want[0].abs().max()))
+    g, _ = _capture(lambda s: plan.forward(p, x, stream=s))
+    assert torch.allclose(plan.backward(p, x)[0], want[0], **tol)  # the captured pass has not run
+    plan.forward(p, y)
+    g.replay()  # the graph's pass over the eager one's
+    assert torch.allclose(plan.backward(p, y)[0], want[1], **tol)
+    plan.forward(p, y)
+    both, (grad, _, _) = _capture(lambda s: (plan.forward(p, x, stream=s), plan.backward(p, x, stream=s))[1])
+    plan.forward(p, y)
+    for _ in range(2):
+        grad.zero_()
+        both.replay()
+        torch.cuda.synchronize()
+        assert torch.allclose(grad, want[0], **tol)
+    captured, (grad, _, _) = _capture(lambda s: plan.backward(p, y, stream=s))  # after an eager forward pass on y
+    plan.forward(p, x)
+    captured.replay()
+    torch.cuda.synchronize()
+    assert torch.allclose(grad, want[1], **tol)
