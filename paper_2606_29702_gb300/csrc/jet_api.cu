@@ -199,19 +199,20 @@ double simt_tile_cost(const jet_plan_s* p, int P) {
 int simt_call_points(const jet_plan_s* p, long long N) {
   if (p->P_fixed) return p->P;
   const int step = p->P0 ? p->P0 : 2;
-  int best = p->P;
+  // the z-jet store holds whole tiles: near its capacity, tiles that end within it
+  const bool stored = p->store && N <= p->store_max_points;
+  int best = 0;
   double best_cost = 0.0;
   for (int P = p->P; P >= step; P -= step) {
     const long long tiles = (N + P - 1) / P, per_sm = (tiles + p->sms - 1) / p->sms;
+    if (stored && tiles * P > p->store_max_points) continue;
     const double cost = (double)per_sm * simt_tile_cost(p, P);
-    if (P == p->P || cost < best_cost) {
+    if (best == 0 || cost < best_cost) {
       best = P;
       best_cost = cost;
     }
   }
-  // the z-jet store holds whole tiles: near its capacity the largest tile
-  const bool stored = p->store && N <= p->store_max_points;
-  return stored && (N + best - 1) / best * best > p->store_max_points ? p->P : best;
+  return best;
 }
 
 // Most chunks that FP32 sums are kept for: 2 per SM (1 for channel sets of 10 or
@@ -465,12 +466,14 @@ static jet_status plan_create(jet_plan_t* out, int n_specs, const jet_residual_s
     e = arena.alloc(&p->ws);
     p->ws_bytes = b_wt + b_gs + b_ls + b_sc + b_ws;
     if (e == cudaSuccess && (flags & JET_FLAG_STORE) && mem_budget_bytes > 0) {
-      const size_t per_tile = (size_t)jet_elems * p->elem;
-      long long tiles = (long long)(mem_budget_bytes / per_tile);
-      if (tiles > 0) {
-        p->store_max_points = tiles * p->P;
-        e = cudaMalloc(&p->store, tiles * per_tile);
-        p->ws_bytes += tiles * per_tile;
+      // as many points as the budget holds, in the smallest tiles of a call
+      const int step = p->P_fixed ? p->P : p->P0 ? p->P0 : 2;
+      const size_t per_step = (size_t)(jet_elems / p->P) * step * p->elem;
+      const long long steps = (long long)(mem_budget_bytes / per_step);
+      if (steps > 0) {
+        p->store_max_points = steps * step;
+        e = cudaMalloc(&p->store, steps * per_step);
+        p->ws_bytes += steps * per_step;
       }
     }
     if (e != cudaSuccess) {
