@@ -59,3 +59,26 @@ def test_batch_with_little_memory():
     for g, g0 in zip(grads, want):
         assert rel_l2(g.cpu().numpy(), g0.cpu().numpy()) < 1e-6  # other chunks, FP32 sums
     assert torch.allclose(losses, loss, rtol=1e-12, atol=0.0)
+
+
+def test_tensor_core_batch_accepts_any_larger_memory():
+    """A batch that fits some amount of free memory fits every larger one, whichever bound of chunks it ends with."""
+    from paper_2606_29702_gb300 import jet, specs
+    plans = [jet.Plan(specs.helmholtz(), [3] + [256] * 8 + [1], "bf16") for _ in range(9)]
+    torch.cuda.empty_cache()
+    jet.Batch(plans).close()
+    most = torch.empty(_free() - 2 * GIB, dtype=torch.uint8, device="cuda")
+    fits = []
+    for mb in range(200, 1700, 20):
+        fill = torch.empty(_free() - mb * (1 << 20), dtype=torch.uint8, device="cuda")
+        try:
+            jet.Batch(plans).close()
+            fits.append(True)
+        except jet.JetError as e:
+            assert e.status == 4  # JET_ERR_OOM
+            fits.append(False)
+        del fill
+        torch.cuda.empty_cache()
+    del most
+    torch.cuda.empty_cache()
+    assert fits == sorted(fits) and fits[-1]
