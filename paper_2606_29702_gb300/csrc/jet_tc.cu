@@ -1362,6 +1362,10 @@ __global__ void wait_timeout_kernel(unsigned long long budget_ns, int* err) {
   __syncthreads();
   // nothing arrives at the barrier: the bounded wait must give up
   const bool ok = tc::mbar_wait(&bar, 0u, &abort_s, err, 90, budget_ns);
+  // a later wait with a flag of its own, as the kernels' teardown: the first code stays
+  volatile int later = 0;
+  __syncwarp();
+  tc::mbar_wait(&bar, 0u, &later, err, 91, budget_ns);
   if (ok && threadIdx.x == 0) atomicExch(err, -1);  // a wait that "completed" is a failure of the hook
 }
 }  // namespace

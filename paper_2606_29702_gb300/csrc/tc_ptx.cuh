@@ -78,8 +78,8 @@ __device__ __forceinline__ bool mbar_try_wait_hint(uint64_t* bar, uint32_t parit
 }
 
 // Bounded wait on an mbarrier phase.  Gives up after `budget_ns` nanoseconds
-// (or when *abort is set by another thread), records `code` in *err and sets
-// *abort; returns false then.  The polling loop is one function, not inlined at
+// (or when *abort is set by another thread), records `code` in *err unless an
+// earlier one is there and sets *abort; returns false then.  The polling loop is one function, not inlined at
 // the fused kernel's twenty waits (2->64x5->1 BF16X3 334 -> 327 us, 2->64x6->3
 // 95 -> 93 us).  The timer read before the first suspended poll stays: polling at
 // once instead cost the 256-wide store kernel 12%.
@@ -92,7 +92,8 @@ static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parit
     if ((it & 255) == 0 && global_ns() - t0 > budget_ns) break;
   }
   *abort = 1;
-  *reinterpret_cast<volatile int*>(err) = code;  // device or pinned host memory
+  volatile int* first = err;  // device or pinned host memory
+  if (*first == 0) *first = code;
   __threadfence_system();
   return false;
 }
