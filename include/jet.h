@@ -381,6 +381,14 @@ jet_status jet_backward_params_noalloc(const jet_residual_spec* spec, int32_t d_
  */
 jet_status jet_debug_wait_timeout(int64_t budget_ns);
 
+/*
+ * Verification hook for failure detection: records `code` (not 0) as the
+ * kernels of a tensor-core batch record a wait that gave up.  The batch's next
+ * call outside stream capture returns JET_ERR_TIMEOUT and launches nothing; the
+ * one after it runs.
+ */
+jet_status jet_debug_batch_timeout(jet_batch_t batch, int32_t code);
+
 /* Thread-local message for the last failing call on this thread. */
 const char* jet_last_error(void);
 

@@ -1171,6 +1171,13 @@ jet_status jet_batch_train_step_dev(jet_batch_t b, void* const* params, void* co
                      loss_out, (cudaStream_t)stream);
 }
 
+jet_status jet_debug_batch_timeout(jet_batch_t b, int32_t code) {
+  if (!b || code == 0) return fail(JET_ERR_INVALID, "NULL batch or code 0");
+  if (!b->tc) return fail(JET_ERR_UNSUPPORTED, "only the tensor-core forms wait");
+  tc_batch_set_timeout(b->tcb, code);
+  return JET_OK;
+}
+
 jet_status jet_batch_destroy(jet_batch_t b) {
   if (!b) return JET_OK;
   free_batch(b);

@@ -750,16 +750,17 @@ namespace {
 
 bool is_capturing(cudaStream_t s) { return stream_is_capturing(s); }
 
-// Device-side wait time-outs of an earlier call surface here.  While the
+// Device-side wait time-outs of an earlier call of a plan or a batch, whose code
+// the kernel wrote to h_err (pinned host memory), surface here.  While the
 // stream is being captured into a CUDA graph nothing is reported (the error
 // path synchronises): a time-out inside a replayed graph surfaces at the next
 // call made outside capture.
-jet_status check_err(TcPlan* t, cudaStream_t s) {
-  if (*reinterpret_cast<volatile int*>(t->h_err) != 0 && !is_capturing(s)) {
+jet_status check_err(int* h_err, cudaStream_t s) {
+  if (*reinterpret_cast<volatile int*>(h_err) != 0 && !is_capturing(s)) {
     cudaDeviceSynchronize();  // the CTAs that gave up drain and return
     char buf[128];
-    snprintf(buf, sizeof(buf), "a bounded device wait timed out in an earlier call (code %d)", *t->h_err);
-    *t->h_err = 0;
+    snprintf(buf, sizeof(buf), "a bounded device wait timed out in an earlier call (code %d)", *h_err);
+    *h_err = 0;
     jet::set_last_error(buf);
     return JET_ERR_TIMEOUT;
   }
@@ -1001,7 +1002,7 @@ ReduceJob grad_job(const jet_plan_s* p, const TcPlan* t, const TcInst& I) {
 
 jet_status tc_forward(jet_plan_s* p, TcPlan* t, const void* params, const void* X, long long N, const void* source,
                       void* r_out, double* loss_out, cudaStream_t s) {
-  jet_status st = check_err(t, s);
+  jet_status st = check_err(t->h_err, s);
   if (st != JET_OK) return st;
   if (N == 0) {
     if (loss_out && cudaMemsetAsync(loss_out, 0, sizeof(double), s) != cudaSuccess) return tcuda(cudaGetLastError(), "memset");
@@ -1028,7 +1029,7 @@ jet_status tc_forward(jet_plan_s* p, TcPlan* t, const void* params, const void* 
 
 jet_status tc_backward(jet_plan_s* p, TcPlan* t, const void* params, const void* X, long long N, const void* source,
                        void* grad_out, void* r_out, double* loss_out, cudaStream_t s) {
-  jet_status st = check_err(t, s);
+  jet_status st = check_err(t->h_err, s);
   if (st != JET_OK) return st;
   if (N == 0) {
     cudaMemsetAsync(grad_out, 0, p->n_params * 4, s);
@@ -1053,7 +1054,7 @@ jet_status tc_backward(jet_plan_s* p, TcPlan* t, const void* params, const void*
 jet_status tc_train_step(jet_plan_s* p, TcPlan* t, void* params, void* m, void* v, long long step,
                          long long* step_ctr, float lr, const void* X, long long N, const void* source,
                          double* loss_out, cudaStream_t s) {
-  jet_status st = check_err(t, s);
+  jet_status st = check_err(t->h_err, s);
   if (st != JET_OK) return st;
   ensure_store(t, N, s);
   st = prep(p, t, params, s);
@@ -1100,7 +1101,7 @@ struct TcBatch {
   std::vector<long long> slice_off, wsums_off;
   unsigned char* scratch = nullptr;
   long long scratch_stride = 0;
-  int* err = nullptr;
+  int* h_err = nullptr;  // code of a timed-out wait (as TcPlan::h_err)
   cudaEvent_t copied = nullptr;  // descriptor upload of the previous eager call
   bool have_prev = false;
   CaptureStore captured;  // descriptors of captured calls
@@ -1155,8 +1156,8 @@ jet_status tc_batch_create(const std::vector<jet_plan_s*>& plans, TcBatch** out)
   if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_prep, sizeof(PrepJob) * b->n);
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->loss_slices, sizeof(double) * b->max_items);
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->scratch, (size_t)b->grid * std::max<long long>(b->scratch_stride, 16));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b->err, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(b->err, 0, sizeof(int));
+  if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_err, sizeof(int));
+  if (e == cudaSuccess) *b->h_err = 0;
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->copied, cudaEventDisableTiming);
   // the chunk sums last: where they do not fit, those of the least bound of chunks
   while (e == cudaSuccess) {
@@ -1201,7 +1202,7 @@ void tc_batch_destroy(TcBatch* b) {
   cudaFree(b->loss_slices);
   cudaFree(b->wsums);
   cudaFree(b->scratch);
-  cudaFree(b->err);
+  cudaFreeHost(b->h_err);
   if (b->copied) cudaEventDestroy(b->copied);
   delete b;
 }
@@ -1213,6 +1214,8 @@ jet_status tc_batch_run(TcBatch* bb, const std::vector<jet_plan_s*>& plans, cons
                         cudaStream_t s) {
   TcBatch* b = bb;
   const int n = b->n;
+  const jet_status timed_out = check_err(b->h_err, s);
+  if (timed_out != JET_OK) return timed_out;
   long long total_tiles = 0;
   for (int i = 0; i < n; ++i) {
     if (N[i] < 1) return tfail(JET_ERR_INVALID, "batched calls need N >= 1 for every instance");
@@ -1338,7 +1341,7 @@ jet_status tc_batch_run(TcBatch* bb, const std::vector<jet_plan_s*>& plans, cons
   a.insts = d_insts;
   a.item_inst = d_items;
   a.item_next = b->d_next;
-  a.err = b->err;
+  a.err = b->h_err;
   a.tmem_cols = b->tmem_cols;
   a.nthreads = b->nthreads;
   cudaError_t e = cudaMemsetAsync(b->d_next, 0, sizeof(int), s);
@@ -1348,6 +1351,8 @@ jet_status tc_batch_run(TcBatch* bb, const std::vector<jet_plan_s*>& plans, cons
   e = launch_reduce(jobs.data(), d_jobs, n, false, adam, step, lr, s, step_ctr);
   return e == cudaSuccess ? JET_OK : tcuda(e, "batch reduce");
 }
+
+void tc_batch_set_timeout(TcBatch* b, int code) { *b->h_err = code; }
 
 // ------------------------------------------------------------------ failure-detection hook
 namespace {

@@ -32,6 +32,7 @@ jet_status tc_train_step(jet_plan_s* p, jet::TcPlan* t, void* params, void* m, v
                          double* loss_out, cudaStream_t s);
 jet_status tc_batch_create(const std::vector<jet_plan_s*>& plans, jet::TcBatch** out);
 void tc_batch_destroy(jet::TcBatch* b);
+void tc_batch_set_timeout(jet::TcBatch* b, int code);  // verification hook: what a timed-out wait writes
 jet_status tc_batch_run(jet::TcBatch* b, const std::vector<jet_plan_s*>& plans, const void* const* params,
                         void* const* m, void* const* v, long long step, long long* step_ctr, float lr,
                         const void* const* X,

@@ -60,7 +60,7 @@ EXPORTS = ["jet_plan_create", "jet_plan_create_loss", "jet_plan_set_term_points"
            "jet_train_step_dev", "jet_plan_destroy", "jet_batch_create", "jet_batch_backward", "jet_batch_train_step",
            "jet_batch_train_step_dev", "jet_batch_destroy",
            "jet_debug_activation", "jet_plan_profile", "jet_plan_profile_read", "jet_backward_params_noalloc",
-           "jet_debug_wait_timeout", "jet_last_error", "jet_version"]
+           "jet_debug_wait_timeout", "jet_debug_batch_timeout", "jet_last_error", "jet_version"]
 
 _lib = None
 
@@ -100,6 +100,7 @@ def load():
                                               ctypes.POINTER(JetChan), i32, vp, vp, i64, vp, vp, vp, vp,
                                               ctypes.POINTER(sz)]
     L.jet_debug_wait_timeout.argtypes = [i64]
+    L.jet_debug_batch_timeout.argtypes = [vp, i32]
     L.jet_plan_profile.argtypes = [vp, i32]
     L.jet_plan_profile_read.argtypes = [vp, ctypes.POINTER(i64), ctypes.POINTER(ctypes.c_double)]
     L.jet_last_error.restype = ctypes.c_char_p
@@ -386,6 +387,10 @@ class Batch:
                                                _ptr(step_counter), float(lr), _vp_array(X), Ns, src, _ptr(loss),
                                                _stream(stream)))
         return loss
+
+    def debug_timeout(self, code):
+        """Record a timed-out wait for the next call to report (jet_debug_batch_timeout)."""
+        _check(load().jet_debug_batch_timeout(self._h, int(code)))
 
     def close(self):
         if getattr(self, "_h", None) is not None and _lib is not None:
