@@ -25,8 +25,7 @@ cudaError_t simt_max_active_id<JET_CLASS_ID>(bool fp64, int ru, int threads, siz
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
   most -= (int)fa.sharedSizeBytes;
-  if (smem > (size_t)most) return cudaErrorInvalidValue;
-  if (threads > fa.maxThreadsPerBlock) return cudaSuccess;
+  if (smem > (size_t)most || threads > fa.maxThreadsPerBlock) return cudaSuccess;  // no CTA fits
   e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
