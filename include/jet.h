@@ -132,7 +132,8 @@ typedef struct {
   int32_t precision;
   int32_t store_mode;      /* 1 if jet_forward_residual stores z-jets */
   int64_t store_max_points;
-  int32_t tile_points;     /* points per tile of the fused kernel */
+  int32_t tile_points;     /* points per tile of the fused kernel: the most that
+                              a call takes (calls on few points take fewer) */
   int32_t grid_ctas;       /* persistent CTAs per launch */
   size_t workspace_bytes;  /* device memory the plan owns */
   int32_t ctas_per_sm;     /* CTAs of the fused kernel resident per SM */

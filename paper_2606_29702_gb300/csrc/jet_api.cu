@@ -166,8 +166,10 @@ int simt_most_points(const jet_plan_s* p, int ru, int threads, int ctas) {
 // per SM (one CTA's barriers and elementwise phases overlap the other's GEMMs)
 // unless shared memory then takes more than an eighth of the points in flight
 // per SM that one CTA of 512 holds (256-wide layers).  Channel sets of 10 or
-// more run one CTA of 256 threads with all registers.  FP64 is bound by its two
-// lanes per SM, not by the tile.
+// more run one CTA of 256 threads with all registers.  (One CTA of 512 at width
+// 64: 2->64x5->1 1.41 ms against 1.33 ms, forward pass of 2->64x6->3 at 10000
+// points 93 against 83 us, composite loss 276 against 301 us.)  FP64 is bound by
+// its two lanes per SM, not by the tile.
 void simt_shape(jet_plan_s* p, int p8) {
   p->threads = kSimtThreads;
   p->P0 = p->fp64 ? 0 : p8 ? 8 * p8 : simt_group_points(p->wmax);
@@ -215,10 +217,14 @@ int simt_call_points(const jet_plan_s* p, long long N) {
   return best;
 }
 
-// Most chunks that FP32 sums are kept for: 2 per SM (1 for channel sets of 10 or
-// more).  With FP32 sums a call's chunks are whole groups of P0 points, N and the
-// plan alone fix them, and a tile takes up to P / P0 groups of one chunk: every
-// sum is formed in the same order whatever the tile.
+// Most chunks that FP32 sums are kept for.  With FP32 sums a call's chunks are
+// whole groups of P0 points, N and the plan alone fix them, and a tile takes up to
+// P / P0 groups of one chunk: every sum is formed in the same order whatever the
+// tile.  The count is part of the rounding of every gradient, not a residency: it
+// is that of a kernel with three jet buffers (2 per SM where two of its CTAs fit,
+// else 1; 1 for channel sets of 10 or more), kept so that gradients stay as they
+// are.  The present kernel may hold two CTAs where it gives one (large tile
+// overrides), and leaves the second slots empty then.
 int simt_sum_chunks(const jet_plan_s* p) {
   const int P = p->P0, S0 = simt_swap(p->C, P) ? p->C + 1 : p->C;
   int pitch = S0 * P;
@@ -1032,8 +1038,8 @@ jet_status jet_batch_create(jet_batch_t* out, int32_t n, const jet_plan_t* plans
   b->ctas_per_sm = std::min(per_sm, 2);
   b->grid = prop.multiProcessorCount * b->ctas_per_sm;
   // the work list holds about three items per CTA, shared by cost: a member may
-  // take several times its share (with 16 members a fixed 16 chunks left the largest
-  // member's chunks running alone: 26.4 ms against 4.0 ms)
+  // take several times its share (with 16 FP32 members a fixed 16 chunks left the
+  // largest member's chunks running alone: 11.0 ms against 3.8 ms)
   b->max_chunks_per_inst = std::min(256, std::max(kSimtBatchChunks, 8 * b->grid / n));
   long long scr = 0, wt = 0, runs = 0;
   for (int i = 0; i < n; ++i) {

@@ -135,8 +135,10 @@ constexpr int kSimtThreads = 256;  // CTA of the no-alloc path and of batches
 constexpr int kSimtRed = 128;      // doubles of the SIMT kernels' reduction area
 // Weights of a jet GEMM pass through shared memory in two row slabs: 4 KB each
 // up to width 64 (a 64 x 64 FP32 layer takes four), where two CTAs of 32 points
-// then fit an SM with six channels; 8 KB up to width 128; 16 KB above (a 256 x
-// 256 layer takes 16; with 8 KB its barriers cost 4%).
+// then fit an SM with six channels (with 8 KB 2->64x5->1 FP32 takes 1.385 against
+// 1.331 ms); 8 KB up to width 128; 16 KB above (a 256 x 256 layer takes 16; with 8
+// KB its barriers cost 4% when it was set, while 3->256x8->1 now takes 9.86 ms with
+// 8 KB and 10.14 ms with 16).
 __host__ __device__ inline int simt_slab_elems(int wmax, size_t elem) {
   const int cap = (wmax <= 64 ? 4096 : wmax <= 128 ? 8192 : 16384) / (int)elem, need = wmax * wmax;
   return need < cap ? need : cap;
@@ -181,8 +183,9 @@ inline int simt_units(const int* widths, int L, bool fp64) {
   return 8;
 }
 // Rows of a weight-gradient item (x 4 columns): 4, fewer where that leaves threads
-// without one (8 rows read a quarter fewer words per FMA, but their 32 packed
-// sums spilled: 2->64x5->1, C = 6, 1.37 ms against 1.32 ms).
+// without one (4 for all: sixteen FP32 networks of widths 32 to 128 3.88 against
+// 3.82 ms; 8 rows read a quarter fewer words per FMA, but their 32 packed sums
+// spilled: 2->64x5->1, C = 6, 1.37 against 1.32 ms when tried).
 inline int simt_wgrad_rows(int ru, int wmax, int V, int threads, bool fp64) {
   const bool few = (long long)(wmax / 4) * (wmax / 4) * (V > 1 ? 2 : 1) < threads;
   return fp64 || !few ? 4 : ru == 8 ? 2 : 1;
@@ -216,8 +219,8 @@ inline size_t simt_smem_bytes(int C, int P, int pitch, int wmax, int n_out, int 
 constexpr size_t kSimtSmBytes = 228 * 1024;
 constexpr size_t kSimtCtaBytes = sizeof(DevInstance) + 16 + 1024;
 // Carve-out that holds `ctas` resident CTAs; the rest of the SM's 256 KB stays
-// L1 (2->64x6->1 composite loss at 12101 points: 364 us with all of it shared
-// memory, 306 us with what two CTAs need).
+// L1 (sixteen FP32 networks 3.92 ms with all of it shared memory, 3.82 ms with what
+// two CTAs need; 2->64x6->1 composite loss at 12101 points 304 and 301 us).
 inline int simt_carveout(size_t smem, int ctas) {
   const size_t pct = ((smem + kSimtCtaBytes) * ctas * 100 + kSimtSmBytes - 1) / kSimtSmBytes;
   return pct > 100 ? 100 : (int)pct;

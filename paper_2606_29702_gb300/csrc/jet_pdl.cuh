@@ -3,7 +3,7 @@
 // instructions until that one is complete and its writes are visible.  A call is
 // three to five kernels, two of them of a few microseconds: back to back the
 // launches and drains between them cost 7 us a call (2->64x6->1 BF16 step at 1024
-// points 53.3 -> 45.6 us, 2->20x4->1 FP64 gradient at 1000 points 83 -> 75 us).
+// points 53.7 -> 46.0 us, 2->20x4->1 FP64 gradient at 1000 points 84 -> 77 us).
 // A kernel is complete only when all its threads are past the wait, so each
 // kernel's completion implies that of all before it.
 #pragma once

@@ -111,12 +111,11 @@ __device__ __forceinline__ GradElem grad_elem(const ReduceJob& J, long long i) {
 // partials in a fixed order: deterministic.  Bound by the FP64 adds, which run
 // at 2 a clock per SM.  G = 8 fills the GPU where there are few parameters and
 // many chunks; G = 1 spares the adds of the partials where there are many
-// parameters (64 members of 16 chunks, all in FP64 slices: 285 us with G = 8 and
-// a block per 32 parameters, 76 us with G = 1), except for the few elements of
-// many chunks' slices beside FP32 sums, whose serial chains would be the tail.
-// Reading FP32 sums costs this kernel some (the same 64 members 132 us) and
-// spares the fused kernels the flush into FP64 slices (burgers 2->64x6->1 FP32,
-// 304 chunks: 16% of the kernel; 3->256x8->1 FP32: 1.5 of 9.9 ms).
+// parameters (a step of 64 BF16 networks 6.26 ms with G = 8, 5.91 ms so), except
+// for the few elements of many chunks' slices beside FP32 sums, whose serial
+// chains would be the tail.  The fused kernels leave their FP32 sums to this
+// kernel: a flush of every chunk into FP64 slices took 16% of the composite loss
+// 2->64x6->1 FP32 and a fifth of 3->256x8->1 FP32 when it went.
 constexpr int kRedWarps = 8;
 
 // warps per group for the FP32 (or finished) hidden-layer sums and for the
@@ -298,8 +297,9 @@ cudaError_t launch_reduce(const ReduceJob* jobs, const ReduceJob* dev_jobs, int 
   ac.eps_f = 1e-8f;
   ac.step = step < 1 ? 1 : step;
   ac.step_ctr = adam ? step_ctr : nullptr;
-  // G = 1 once a warp per 32 parameters is 64 warps per SM and more (at 17 warps
-  // per SM, 3->128x6->2 with 152 chunks, it takes 45 us)
+  // G = 1 once a warp per 32 parameters is 64 warps on each of 152 SMs and more
+  // (with few it is slower: 2->64x5->1 FP32, 304 chunks, 1.342 ms against 1.331 ms).
+  // A constant, so that the order of a sum does not follow the device.
   long long params = 0, gx = 1;
   for (int i = 0; i < n; ++i) params += jobs[i].n_params;
   const bool many = params >= 32LL * 64 * 152;

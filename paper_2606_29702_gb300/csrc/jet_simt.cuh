@@ -37,8 +37,8 @@
 // (about 80% of the time), the FP64 pipe in the FP64 form.  Against the form
 // with three jet buffers, 4 units per thread, weights read through L1, one
 // lane per weight-gradient item and tiles that did not depend on N:
-// 3->256x8->1 FP32 at N = 16385 19.29 -> 10.13 ms, 2->64x5->1 (C = 6) FP32 at
-// 65536 1.769 -> 1.317 ms, 2->20x4->1 FP64 at 1000 343 -> 77 us.
+// 3->256x8->1 FP32 at N = 16385 19.29 -> 10.14 ms, 2->64x5->1 (C = 6) FP32 at
+// 65536 1.769 -> 1.331 ms, 2->20x4->1 FP64 at 1000 343 -> 77 us.
 #pragma once
 
 #include <type_traits>
@@ -193,8 +193,9 @@ struct SimtTile {
   static constexpr int RU = RU_;  // consecutive units per thread of the jet GEMMs
   static constexpr int EU = TP;   // consecutive units per thread of the elementwise phases
   // k steps of the jet GEMMs unrolled together: two where the sums and four
-  // steps' operands would exceed the registers (C = 7 at 512 threads: 12.8 ms
-  // with four, 11.8 ms with two), else four
+  // steps' operands would exceed the registers, else four (3->256x8->1, C = 7 at
+  // 512 threads, 12.8 ms with four and 11.8 ms with two when it was set; with the
+  // sums of the weight gradient in registers 9.94 and 10.14 ms)
   static constexpr int UK = C >= 7 ? 2 : 4;
 
   const DevInstance& I;
@@ -750,7 +751,7 @@ struct SimtTile {
     } else {
       // several groups added to the chunk's FP32 sums by one thread: the sums
       // wait in registers, one load and one store per tile instead of a vector
-      // reduction per group (3->256x8->1, three groups a tile: 10.83 -> 10.44 ms)
+      // reduction per group (3->256x8->1, three groups a tile: 10.74 -> 10.14 ms)
       const int items = I.widths[l] / 4 * (I.widths[l - 1] / 4);
       if (I.wr == 4 && wacc_base && V > 1 && (V % 2 || items * 2 > NT)) wgrad32<4, true>(l, zbar, aprev, g);
       else if (I.wr == 4) wgrad32<4, false>(l, zbar, aprev, g);
@@ -1068,7 +1069,8 @@ __device__ __forceinline__ void simt_body(const SimtArgs& args) {
   __shared__ int k_s;
   // the running item's descriptor: read in every phase, through shared memory
   // rather than a pointer that may be param or global space, which cost
-  // registers that spilled (2->64x5->1, C = 6: 1.32 ms with it, 1.24 ms without)
+  // registers that spilled (2->64x5->1, C = 6: 1.44 ms with it, 1.33 ms without;
+  // 3->256x8->1 11.5 and 10.1 ms)
   __shared__ DevInstance inst_s;
   const int NT = blockDim.x;
   for (int k = blockIdx.x; k < args.n_items;) {

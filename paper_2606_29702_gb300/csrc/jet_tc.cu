@@ -715,8 +715,10 @@ jet_status tc_plan_create(jet_plan_s* p, TcPlan** out, const cudaDeviceProp& pro
 // The tile of one call on N points: the one whose rounds of tiles over the CTAs
 // take the least time.  A tile takes kTcTileCost for its serial chain of layers
 // (barriers, MMA and copy latencies) and the rest in proportion to its points
-// per sub-tile: 2->64x6->1 calls of one round take 63, 69, 76 and 82 us with 16,
-// 32, 48 and 64 of them.  At 1024 points 16 instead of 64: 72 -> 59 us.
+// per sub-tile: training steps of one round take 45.8, 50.4, 54.9 and 56.6 us with
+// 16, 32, 48 and 64 of them on 2->64x6->1, 25.9 to 29.9 us on 2->64x2->1 and 78.7
+// to 100 us on 2->64x12->1.  The constant was set on the first of these; among
+// tiles of one round any value takes the smallest.
 static const TcPlan* tc_call_tile(const TcPlan* t, long long N) {
   constexpr long long kTcTileCost = 64;
   auto cost = [&](const TcPlan& v) {

@@ -268,8 +268,8 @@ struct TcTile {
   // once the data gradient of the layer above has read that half of W^{l+1},
   // part 1 once it has read the rest; bar_tma completes with both.  Half of the
   // 128 KB arrives during the data gradient's second half (3->256x8->1 with the
-  // store, N = 1048576: 43.06 -> 42.58 ms); with the layer input ahead of part 1
-  // the gain was a fifth of that.
+  // store, N = 1048576, when it came: 43.06 -> 42.58 ms); with the layer input ahead
+  // of part 1 the gain was a fifth of that.
   __device__ void load_hidden_w_half(int l, int part) {
     const uint32_t box = 64u * rr() * 2u;
     if (part == 0) tc::mbar_arrive_expect_tx(bar_tma, box * 4u);
@@ -411,8 +411,9 @@ struct TcTile {
   static constexpr bool PRELOAD1B = Shape::H == 2;  // W^1, b^1 of the layer-1 backward
   // The output layer's adjoints as vector loads, db^L by a warp per output and
   // the first layer's partial sums by a warpgroup each, widened on the integer
-  // pipe: 2->64x6->3 composite loss 92.7 -> 88.9 us, ensemble 5.97 -> 5.89 ms,
-  // 3->128x6->2 5.18 -> 5.14 ms.  Not for 256-wide shapes: 41.97 -> 42.45 ms.
+  // pipe: ensemble 5.99 -> 5.91 ms, 2->64x6->3 composite loss and 3->128x6->2 level
+  // (92.7 -> 88.9 us and 5.18 -> 5.14 ms when it came).  Not for 256-wide shapes:
+  // 41.97 -> 42.45 ms then; with the code of now 42.09 -> 41.59 ms.
   static constexpr bool PAR_FLUSH = Shape::H != 2;
   struct RowBias {
     float v[2];

@@ -80,8 +80,8 @@ __device__ __forceinline__ bool mbar_try_wait_hint(uint64_t* bar, uint32_t parit
 // Bounded wait on an mbarrier phase.  Gives up after `budget_ns` nanoseconds
 // (or when *abort is set by another thread), records `code` in *err unless an
 // earlier one is there and sets *abort; returns false then.  The polling loop is one function, not inlined at
-// the fused kernel's twenty waits (2->64x5->1 BF16X3 334 -> 327 us, 2->64x6->3
-// 95 -> 93 us).  The timer read before the first suspended poll stays: polling at
+// the fused kernel's twenty waits (2->64x5->1 BF16X3 297 -> 291 us, 3->256x8->1 with
+// the store 42.3 -> 42.1 ms, 2->64x6->3 level).  The timer read before the first suspended poll stays: polling at
 // once instead cost the 256-wide store kernel 12%.
 static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, volatile int* abort, int* err,
                                                    int code, uint64_t budget_ns) {
