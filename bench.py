@@ -203,12 +203,12 @@ def fp32_alu_peak_tflops(sm_mhz=2070.0, sms=152):
 TRAFFIC = {
     # N = 65536 capture of both kernels (fused kernel + weight-gradient GEMM): the store's bytes x16; the GEMM's
     # per-item FP32 partials (one per CTA and layer, the same at any N) once
-    ("helmholtz_3x256x8", "bf16", "store"): ((748488704 + 3874912512 + 3758939904) * 16 + 239806720, "f3354e3bbd5e92b3"),
-    ("ns_psi_3x128x6", "bf16", "tile"): (5669632 + 3053145344, "f3354e3bbd5e92b3"),
-    ("ks_2x64x5", "bf16", "tile"): (834304 + 0, "f3354e3bbd5e92b3"),
-    ("ks_2x64x5", "fp32", "tile"): (168746496 + 650558208, "f3354e3bbd5e92b3"),
+    ("helmholtz_3x256x8", "bf16", "store"): ((751430912 + 3875191808 + 3758984448) * 16 + 239715328, "2c6ce83a9f0a7fd1"),
+    ("ns_psi_3x128x6", "bf16", "tile"): (6097664 + 3066404608, "2c6ce83a9f0a7fd1"),
+    ("ks_2x64x5", "bf16", "tile"): (834816 + 0, "2c6ce83a9f0a7fd1"),
+    ("ks_2x64x5", "fp32", "tile"): (169973504 + 653489664, "2c6ce83a9f0a7fd1"),
     # the batched fused kernel of one ensemble step (the step is one graph replay)
-    ("ensemble_64", "bf16", "tile"): (656530688 + 2226216704, "f3354e3bbd5e92b3"),
+    ("ensemble_64", "bf16", "tile"): (401221376 + 1996702208, "2c6ce83a9f0a7fd1"),
 }
 
 
